@@ -84,11 +84,14 @@ enum {
                                 the time means), the face terms are summed in double-float
                                 and the state update is FP64                              */
   RIDG_PREC_MIXED_FP32 = 2,  /* Newton linear solves in FP32 with the residual in FP64
-                                (nonlinear flux)                                          */
-  RIDG_PREC_MIXED_TF32 = 3,  /* Newton linear solves with the Schur-complement block
+                                (nonlinear flux).  In 2D a matrix-free iterative solver in
+                                FP32 takes every region that it converges on; the others
+                                are solved by FP32 block elimination                      */
+  RIDG_PREC_MIXED_TF32 = 3,  /* as MIXED_FP32, where the block elimination of the regions
+                                that the iterative solver leaves has its Schur-complement
                                 updates on the TF32 tensor cores (FP32 accumulation), FP32
                                 pivot inverses, and refinement sweeps against the FP64
-                                residual (nonlinear flux)                                 */
+                                residual (nonlinear flux, 2D)                             */
   RIDG_PREC_MIXED_FP16 = 4   /* as MIXED_BF16 with FP16 digit operands: the balanced
                                 base-256 digits are exact in FP16 as in BF16 and every
                                 digit product and FP32 sum is the same, so the results are
@@ -119,7 +122,9 @@ typedef struct {
   double dt, t;                 /* current step size and time                            */
   long long steps;              /* steps taken since the last ridg_set_state              */
   long long newton_unconverged; /* regions that hit the Newton cap in the last prediction */
-  int newton_iters_max;         /* largest Newton iteration count of the last prediction  */
+  int newton_iters_max;         /* largest Newton iteration count of the last prediction
+                                   (mixed precisions: linearisations, each used for one or
+                                   more solves against the FP64 residual)                 */
   int precision, slices;
   long long newton_iters_total; /* Newton iterations summed over the regions of the last
                                    prediction (or of the steps of the last ridg_step)      */
@@ -242,7 +247,9 @@ typedef struct {
   double predict_ms;     /* average device time of the prediction kernel per step           */
   double correct_ms;     /* average device time of the correction kernel per step           */
   double step_ms;        /* average device time of one whole step                            */
-  int launches_per_step; /* kernels launched per step                                        */
+  int launches_per_step; /* prediction and correction launches per step (a mixed-precision
+                            Newton prediction, the iterative kernel and the block
+                            elimination of what it leaves, counts as one)                    */
 } ridg_profile_t;
 
 /* Run n steps (the same arithmetic as ridg_step) as individual launches bracketed by CUDA
@@ -298,8 +305,10 @@ int ridg_batch_step(ridg_batch_t* b, int n);
 /* The batch's schedule for a nonlinear flux (1: the whole ensemble's Newton prediction in one
  * launch -- every degree's regions, highest degree first, each CTA moving to the next
  * degree's queue as one runs out -- and every instance's correction in one more launch;
- * 0: one Newton launch per degree and one correction per instance) and the kernel launches
- * of one step.  Burgers batches default to 1 unless the autotuner recorded otherwise.     */
+ * 0: one Newton launch per degree and one correction per instance) and the prediction and
+ * correction launches of one step.  In the mixed precisions each Newton launch is the block
+ * elimination of the regions that the iterative solver, one more launch per degree ahead of
+ * it, left; those are not counted.  Burgers batches default to 1 unless the autotuner recorded otherwise.     */
 int ridg_batch_schedule(ridg_batch_t* b, int* schedule, int* launches_per_step);
 /* Time one step in each schedule from the instances' current states (restored afterwards,
  * graphs dropped) and keep the faster; the choice goes into the autotuner's cache (and to

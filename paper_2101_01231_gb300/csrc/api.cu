@@ -326,6 +326,32 @@ int enqueue_newton3(ridg_t* h) {
   return RIDG_OK;
 }
 
+// The matrix-free solver's launch ahead of a block-elimination launch with arguments a (which
+// then takes the regions it lists).
+cudaError_t enqueue_newton_mf(const ridg_t* h, ridg::NewtonArgs& a, int* list, cudaStream_t s) {
+  ridg::NewtonMfArgs f;
+  std::memset(&f, 0, sizeof(f));
+  f.Q = a.Q;
+  f.W = a.W;
+  f.nx = a.nx;
+  f.ny = a.ny;
+  f.ncell = a.ncell;
+  f.lam[0] = a.lam[0];
+  f.lam[1] = a.lam[1];
+  f.gamma = a.gamma;
+  f.max_iters = a.max_iters;
+  f.tol = a.tol;
+  f.stats = a.stats;
+  f.iters_total = a.iters_total;
+  f.inst = a.inst;
+  f.ninst = a.ninst;
+  f.list_count = list;
+  f.list = list + 1;
+  a.list_count = list;
+  a.list = list + 1;
+  return ridg::launch_newton_mf(h->nb, h->m, h->flux.kind, f, s);
+}
+
 int enqueue_newton(ridg_t* h) {
   if (h->dim == 3) return enqueue_newton3(h);
   ridg::NewtonArgs a;
@@ -347,6 +373,7 @@ int enqueue_newton(ridg_t* h) {
   a.counter = h->nl_words;
   a.stats = h->nl_words + 1;
   a.iters_total = (unsigned long long*)(h->nl_words + 6);
+  if (h->nl_list) RIDG_CUDA(h, enqueue_newton_mf(h, a, h->nl_list, h->stream));
   RIDG_CUDA(h, ridg::launch_newton(h->nb, h->m, h->flux.kind, newton_prec(h), a, h->nl_grid,
                                    h->stream));
   return RIDG_OK;
@@ -622,7 +649,9 @@ int ridg_create(const ridg_mesh* mesh, int order, const ridg_flux* flux, double 
     const size_t scratch = h->nl_scratch_cta * (size_t)h->nl_grid_max;
     h->nl_scratch = h->nl_grid_max > 0 ? dev_alloc(h, scratch) : nullptr;
     h->nl_words = (int*)dev_alloc(h, 24 * sizeof(int));
-    if (!tb_mem || !h->nl_scratch || !h->nl_words) {
+    const bool mixed = newton_prec(h) != ridg::kNewtonF64;
+    if (mixed) h->nl_list = (int*)dev_alloc(h, ((size_t)h->ncell + 1) * sizeof(int));
+    if (!tb_mem || !h->nl_scratch || !h->nl_words || (mixed && !h->nl_list)) {
       dev_free(h, tb_mem);
       ridg_destroy(h);
       return RIDG_ENOMEM;
@@ -687,6 +716,7 @@ void ridg_destroy(ridg_t* h) {
   dev_free(h, h->nl.mem);
   if (!h->nl_scratch_shared) dev_free(h, h->nl_scratch);
   dev_free(h, h->nl_words);
+  dev_free(h, h->nl_list);
   dev_free(h, h->nl3_mem);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
@@ -1153,6 +1183,7 @@ struct NlGroup {
   std::vector<ridg::NlInst> host;      // the table, refreshed before every batch launch
   ridg::NlInst* table = nullptr;       // device copy
   int* counter = nullptr;              // region counter of the group's launch
+  int* list = nullptr;                 // mixed: as ridg_handle::nl_list, over the group's regions
   long long regions = 0;
   size_t scratch_off = 0;              // the degree's block storage in the batch's
 };
@@ -1251,13 +1282,18 @@ ridg::NewtonArgs group_args(ridg_batch_t* b, const NlGroup& g) {
   a.iters_total = (unsigned long long*)(h->nl_words + 6);
   a.inst = g.table;
   a.ninst = (int)g.idx.size();
+  if (g.list) {
+    a.list_count = g.list;
+    a.list = g.list + 1;
+  }
   return a;
 }
 
 // One persistent Newton launch over every region of the group's instances.
 int enqueue_newton_group(ridg_batch_t* b, const NlGroup& g) {
   ridg_t* h = b->inst[g.idx[0]];
-  const ridg::NewtonArgs a = group_args(b, g);
+  ridg::NewtonArgs a = group_args(b, g);
+  if (g.list) RIDG_CUDA(h, enqueue_newton_mf(h, a, g.list, b->stream));
   RIDG_CUDA(h, ridg::launch_newton(h->nb, h->m, h->flux.kind, newton_prec(h), a, h->nl_grid,
                                    b->stream));
   return RIDG_OK;
@@ -1287,6 +1323,12 @@ int upload_batch_multi(ridg_batch_t* b) {
 int enqueue_batch_multi(ridg_batch_t* b) {
   ridg_t* h0 = b->inst[0];
   const int grid = ridg::newton_multi_ctas_per_sm(newton_prec(h0)) * sm_count();
+  for (const NlGroup& g : b->groups) {
+    if (!g.list) continue;
+    ridg_t* h = b->inst[g.idx[0]];
+    ridg::NewtonArgs a = group_args(b, g);
+    RIDG_CUDA(h, enqueue_newton_mf(h, a, g.list, b->stream));
+  }
   RIDG_CUDA(h0, ridg::launch_newton_multi(newton_prec(h0), b->multi_host, b->multi_dev, grid,
                                           b->stream));
   ridg::CorrMulti c;
@@ -1378,7 +1420,13 @@ int ridg_batch_create(int count, const ridg_mesh* meshes, const int* orders, con
       g.host.resize(g.idx.size());
       g.table = (ridg::NlInst*)dev_alloc(b->inst[0], g.idx.size() * sizeof(ridg::NlInst));
       g.counter = (int*)dev_alloc(b->inst[0], 4 * sizeof(int));
-      if (!g.table || !g.counter) {
+      const bool mixed = newton_prec(b->inst[0]) != ridg::kNewtonF64;
+      if (mixed) {
+        size_t regions = 0;
+        for (int i : g.idx) regions += (size_t)b->inst[i]->ncell;
+        g.list = (int*)dev_alloc(b->inst[0], (regions + 1) * sizeof(int));
+      }
+      if (!g.table || !g.counter || (mixed && !g.list)) {
         ridg_batch_destroy(b);
         return RIDG_ENOMEM;
       }
@@ -1411,6 +1459,7 @@ void ridg_batch_destroy(ridg_batch_t* b) {
   for (NlGroup& g : b->groups) {
     if (g.table) dev_free(b->inst[0], g.table);
     if (g.counter) dev_free(b->inst[0], g.counter);
+    if (g.list) dev_free(b->inst[0], g.list);
   }
   if (b->corr_table) dev_free(b->inst[0], b->corr_table);
   if (b->multi_dev) dev_free(b->inst[0], b->multi_dev);

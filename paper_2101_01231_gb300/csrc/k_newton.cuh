@@ -1569,12 +1569,16 @@ __device__ void newton_regions(const NewtonArgs& a, unsigned char* smem, uint32_
   }
 
   for (;;) {
-    if (tid == 0) misc[0] = atomicAdd(a.counter, 1);
+    if (tid == 0) {
+      const int k = atomicAdd(a.counter, 1);
+      const long long count = a.list ? *a.list_count : a.ncell;
+      misc[0] = k >= count ? -1 : a.list ? a.list[k] : k;
+    }
     __syncthreads();
     const long long eg = misc[0];
     const bool stop = TC && misc[1] != 0;  // a tensor-core wait timed out
     __syncthreads();
-    if (eg >= a.ncell || stop) break;
+    if (eg < 0 || stop) break;
     // the region's instance: the handle's own mesh (its parameters read from the launch's
     // constant bank), or (batched launch) the last instance of the table whose first region
     // is <= eg, its parameters kept in shared memory

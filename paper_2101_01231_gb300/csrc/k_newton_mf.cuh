@@ -1,0 +1,1009 @@
+// Matrix-free Newton prediction for a nonlinear flux in 2D (Sec. 3): the mixed precisions'
+// first solver, one CTA per region.
+//
+// The region system of eq. pred_full_system is solved by the same outer iteration as in
+// k_newton.cuh -- FP64 residual by quadrature, FP64 iterate, linear solves in FP32, stop when
+// ||dW||_inf <= tol max(1, ||W||_inf) -- but no Jacobian is stored and nothing is factorised:
+//  * the linearised residual is applied in FP32 on the nodal basis of the NB^3 Gauss points
+//    of every cell, where a product with F'(w) is pointwise and a derivative is one NB x NB
+//    matrix per line (the integrals int d Psi_k Psi_l F'(w) by NB points per dimension);
+//  * the time operator (psi_a(1) psi_g(1) - int psi_a' psi_g, one NB x NB matrix) is the
+//    preconditioner.  The step is an integral equation in time, so the preconditioned operator
+//    is a small perturbation of the identity at the scheme's time steps and BiCGStab reaches
+//    1e-4 .. 1e-5 in 3 to 12 iterations (two applications each).
+// A direct solve needs 118 b^3 flop per region and factorisation (b = m theta_T unknowns per
+// cell: 149 MFLOP for Euler Q2) and moves every block through L2; one application here is
+// ~30 kFMA for Euler Q2 and its data stay in shared memory and registers.  What bounds the
+// kernel is the FP64 pipe (2 FMA per clock and SM), on the two or three FP64 residuals that
+// the outer iteration cannot do without; those are evaluated by sum factorisation along lines
+// held in registers, with the even / odd symmetry of the Gauss points (about half the
+// multiplications), one flux evaluation per point for both directions and one per face.
+// Measured against the block elimination alone (one step, tensor-core / FP32 solves): Euler
+// Q2 160^2 214 -> 16.3 ms, Euler Q1 67 x 90 7.7 -> 1.1 ms, eight Burgers problems of up to
+// 72^2 at degrees 1 .. 4 228 -> 13.2 ms.
+//
+// The initial iterate is Q^n extended constant in time, so the first residual is evaluated
+// with one time mode and one time point.
+//
+// A region that does not converge quickly (contraction below 10x per solve, BiCGStab
+// stalled, a non-finite value) is put on a list; the block elimination of k_newton.cuh then
+// solves the listed regions from the start, with its own iteration cap and statistics.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "k_nlflux.cuh"
+#include "ridg_internal.h"
+
+namespace ridg {
+namespace mf {
+
+// 1D tables, passed by value (constant bank).  The Gauss points are symmetric: the FP64
+// rule keeps the lower half, q < H, and the centre point at H - 1 if NQ is odd.
+template <int NB>
+struct Tab {
+  static constexpr int NQ = (3 * (NB - 1) + 2) / 2, H = (NQ + 1) / 2;
+  double V[NB][H];     // phi_b(x_q)
+  double wV[NB][H];    // w_q phi_b(x_q)
+  double wD[NB][H];    // w_q phi_b'(x_q)
+  double ep[NB];       // phi_b(+1)
+  double Mt[NB][NB];   // time operator
+  // the NB-point rule of the linearised operator
+  float N[NB][NB];     // [b][n] phi_b(x_n)
+  float M[NB][NB];     // [b][n] w_n / 2 phi_b(x_n): node values to modes
+  float TN[NB][NB];    // [n][a] node values of (time operator)^-1 psi_a
+  float Ti[NB][NB];    // [n][n'] inverse time operator on node values
+  float D[NB][NB];     // [n][q] w_q sum_b phi_b(x_n) phi_b'(x_q)
+  float E[2][NB];      // [side][n] sum_b phi_b(x_n) phi_b(+-1)
+  float L[2][NB];      // [side][n] w_n / 2 E: trace of node values
+};
+
+template <int NB, int MV>
+struct Cfg {
+  static constexpr int THS = NB * NB, THT = NB * THS, BS = MV * THT, C = 9 * MV;
+  static constexpr int NQ = Tab<NB>::NQ;
+  static constexpr int COL = 9 * THS;               // columns (cell, y, x) of the region
+  static constexpr int NT = (COL + 31) / 32 * 32, NW = NT / 32;
+  static constexpr int VT = NB * MV;                // values per column
+  static constexpr int FL = 24 * NB;                // face lines: 24 faces, NB lines each
+  static constexpr int NG = MV == 1 ? 1 : 2;        // Burgers: one flux for both directions
+  static_assert(FL <= NT, "one thread per face line");
+  // CTAs per SM that the registers are held to (168 / 128 / 96 a thread at Euler, Burgers Q4,
+  // Burgers Q2 and Q3; unbounded they are 127 to 254 and one CTA fewer fits)
+  static constexpr int MINB = MV == 4 ? (NB == 2 ? 5 : 4) : (NB == 2 ? 8 : NB == 3 ? 6 : NB == 4 ? 4 : 2);
+  // FP64 arena: B1, B2 (line buffers), face fluxes; the face traces share B2
+  static constexpr int nB = C * NB * NQ * NQ, nTr = 4 * C * NB * NQ, nH = 24 * MV * NB * NQ;
+  static constexpr int nB2 = nB > nTr ? nB : nTr;
+  static constexpr int nArena64 = nB + nB2 + nH;
+  // FP32 arena: the vector, its fluxes, the face fluxes
+  static constexpr int nP = VT * COL, nF = 24 * VT * NB;
+  static constexpr int nArena32 = (1 + NG) * nP + nF;
+  static constexpr size_t arena = nArena64 * 8 > nArena32 * 4 ? nArena64 * 8 : nArena32 * 4;
+  static constexpr size_t oR = 8 * 9 * BS, oQ = 2 * oR, oRed = oQ + 8 * C * THS, oArena = (oRed + 4 * 2 * 4 * NW + 15) / 16 * 16;
+  static constexpr size_t bytes = oArena + arena;
+};
+
+// ---- FP64 lines ---------------------------------------------------------------------------
+// values at the NQ points of the polynomial with modes a
+template <int NB>
+__device__ __forceinline__ void interp(const Tab<NB>& T, const double (&a)[NB],
+                                       double (&v)[Tab<NB>::NQ]) {
+  constexpr int NQ = Tab<NB>::NQ;
+#pragma unroll
+  for (int q = 0; q < NQ / 2; ++q) {
+    double e = a[0];
+#pragma unroll
+    for (int b = 2; b < NB; b += 2) e = fma(T.V[b][q], a[b], e);
+    if constexpr (NB <= 3) {
+      v[q] = fma(T.V[1][q], a[1], e);
+      v[NQ - 1 - q] = fma(-T.V[1][q], a[1], e);
+    } else {
+      const double o = fma(T.V[3][q], a[3], T.V[1][q] * a[1]);
+      v[q] = e + o;
+      v[NQ - 1 - q] = e - o;
+    }
+  }
+  if constexpr (NQ & 1) {
+    double e = a[0];
+#pragma unroll
+    for (int b = 2; b < NB; b += 2) e = fma(T.V[b][NQ / 2], a[b], e);
+    v[NQ / 2] = e;
+  }
+}
+
+// out[b] = sum_q w_q phi_b(x_q) f[q], or with phi_b'
+template <int NB, bool DERIV>
+__device__ __forceinline__ void project(const Tab<NB>& T, const double (&f)[Tab<NB>::NQ],
+                                        double (&out)[NB]) {
+  constexpr int NQ = Tab<NB>::NQ, HP = NQ / 2;
+  double s[HP], d[HP];
+#pragma unroll
+  for (int q = 0; q < HP; ++q) {
+    s[q] = f[q] + f[NQ - 1 - q];
+    d[q] = f[q] - f[NQ - 1 - q];
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    if constexpr (DERIV) {
+      if (b == 0) {
+        out[b] = 0.0;
+        continue;
+      }
+    }
+    const bool even = DERIV ? (b & 1) : !(b & 1);
+    double acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < HP; ++q) {
+      const double w = DERIV ? T.wD[b][q] : T.wV[b][q];
+      const double x = even ? s[q] : d[q];
+      acc = q == 0 ? w * x : fma(w, x, acc);
+    }
+    if constexpr (NQ & 1)
+      if (even) acc = fma(DERIV ? T.wD[b][HP] : T.wV[b][HP], f[HP], acc);
+    out[b] = acc;
+  }
+}
+
+// phi_b(x_q) at any q (compile-time indices)
+template <int NB>
+__device__ __forceinline__ double vq(const Tab<NB>& T, int b, int q) {
+  constexpr int NQ = Tab<NB>::NQ, H = Tab<NB>::H;
+  return q < H ? T.V[b][q] : ((b & 1) ? -T.V[b][NQ - 1 - q] : T.V[b][NQ - 1 - q]);
+}
+template <int NB>
+__device__ __forceinline__ double wvq(const Tab<NB>& T, int b, int q) {
+  constexpr int NQ = Tab<NB>::NQ, H = Tab<NB>::H;
+  return q < H ? T.wV[b][q] : ((b & 1) ? -T.wV[b][NQ - 1 - q] : T.wV[b][NQ - 1 - q]);
+}
+
+// both directions' fluxes of one state (Euler: one reciprocal)
+template <int FLUX>
+__device__ __forceinline__ void flux2(const double* w, double* fx, double* fy, double g) {
+  if constexpr (FLUX == RIDG_FLUX_BURGERS) {
+    fx[0] = 0.5 * w[0] * w[0];
+  } else {
+    const double ir = 1.0 / w[0], u = w[1] * ir, v = w[2] * ir;
+    const double p = (g - 1.0) * (w[3] - 0.5 * fma(w[1], u, w[2] * v)), h = w[3] + p;
+    fx[0] = w[1];
+    fx[1] = fma(w[1], u, p);
+    fx[2] = w[1] * v;
+    fx[3] = u * h;
+    fy[0] = w[2];
+    fy[1] = fx[2];
+    fy[2] = fma(w[2], v, p);
+    fy[3] = v * h;
+  }
+}
+template <int FLUX>
+__device__ __forceinline__ void flux1(const double* w, int dd, double* f, double g) {
+  if constexpr (FLUX == RIDG_FLUX_BURGERS) {
+    f[0] = 0.5 * w[0] * w[0];
+  } else {
+    const double ir = 1.0 / w[0], u = w[1] * ir, v = w[2] * ir;
+    const double p = (g - 1.0) * (w[3] - 0.5 * fma(w[1], u, w[2] * v));
+    const double un = dd == 0 ? u : v;
+    f[0] = dd == 0 ? w[1] : w[2];
+    f[1] = w[1] * un;
+    f[2] = w[2] * un;
+    if (dd == 0) f[1] += p; else f[2] += p;
+    f[3] = un * (w[3] + p);
+  }
+}
+
+// the cells left and right of region face f (dd * 12 + row * 4 + pos), -1 outside
+__device__ __forceinline__ void face_cells(int f, int& dd, int& cl, int& cr) {
+  dd = f >= 12;
+  const int k = f - 12 * dd, row = k >> 2, pos = k & 3;
+  cl = pos > 0 ? (dd ? (pos - 1) * 3 + row : row * 3 + pos - 1) : -1;
+  cr = pos < 3 ? (dd ? pos * 3 + row : row * 3 + pos) : -1;
+}
+
+// ---------------------------------------------------------------------------------------
+// residual of eq. pred_full_system for the 9 region cells in FP64 (the sums of
+// newton::residual).  FIRST: at the initial iterate (constant in time; the time term and the
+// source cancel), where the face speeds alpha[24] are also taken and frozen.
+// ---------------------------------------------------------------------------------------
+template <int NB, int MV, int FLUX, bool FIRST>
+__device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, double* Rs,
+                         double* alpha, double* arena, const double* lam, double g) {
+  using K = Cfg<NB, MV>;
+  constexpr int NQ = K::NQ, C = K::C, NT = K::NT, THS = K::THS, NA = FIRST ? 1 : NB,
+                NX = NQ * NQ;
+  const int tid = threadIdx.x;
+  double* B1 = arena;              // [c][a][y][x], y and x with NQ slots
+  double* B2 = B1 + K::nB;
+  double* Tr = B2;                 // [dd][side][c][a][NQ]
+  double* Hf = B2 + K::nB2;        // [face][j][a][NQ]
+  // x lines: values at the x points, and the x traces (side 0: +1, 1: -1)
+  for (int i = tid; i < C * NA * NB; i += NT) {
+    const int c = i / (NA * NB), a = (i / NB) % NA, y = i % NB;
+    const double* src = Ws + (c * NB + a) * THS + y * NB;
+    double m[NB], v[NQ];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) m[b] = src[b];
+    interp<NB>(T, m, v);
+    double* dst = B1 + ((c * NB + a) * NQ + y) * NQ;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) dst[q] = v[q];
+    double e = m[0], o = T.ep[1] * m[1];
+#pragma unroll
+    for (int b = 2; b < NB; ++b)
+      if (b & 1) o = fma(T.ep[b], m[b], o); else e = fma(T.ep[b], m[b], e);
+    Tr[((0 * C + c) * NB + a) * NQ + y] = e + o;
+    Tr[((1 * C + c) * NB + a) * NQ + y] = e - o;
+  }
+  // y traces
+  for (int i = tid; i < C * NA * NB; i += NT) {
+    const int c = i / (NA * NB), a = (i / NB) % NA, x = i % NB;
+    const double* src = Ws + (c * NB + a) * THS + x;
+    double e = src[0], o = T.ep[1] * src[NB];
+#pragma unroll
+    for (int b = 2; b < NB; ++b)
+      if (b & 1) o = fma(T.ep[b], src[b * NB], o); else e = fma(T.ep[b], src[b * NB], e);
+    Tr[((2 * C + c) * NB + a) * NQ + x] = e + o;
+    Tr[((3 * C + c) * NB + a) * NQ + x] = e - o;
+  }
+  __syncthreads();
+  // y lines, and the traces along their faces (in place: a line is read and written by the
+  // same thread)
+  for (int i = tid; i < C * NA * NQ; i += NT) {
+    const int c = i / (NA * NQ), a = (i / NQ) % NA, x = i % NQ;
+    double* p = B1 + (c * NB + a) * NX + x;
+    double m[NB], v[NQ];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) m[b] = p[b * NQ];
+    interp<NB>(T, m, v);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) p[q * NQ] = v[q];
+  }
+  for (int i = tid; i < 4 * C * NA; i += NT) {
+    double* p = Tr + (i / NA * NB + i % NA) * NQ;
+    double m[NB], v[NQ];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) m[b] = p[b];
+    interp<NB>(T, m, v);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) p[q] = v[q];
+  }
+  __syncthreads();
+  if constexpr (FIRST) {
+    // Rusanov speeds: the largest of both sides over the face's points (time-constant)
+    for (int f = tid; f < 24; f += NT) {
+      int dd, cl, cr;
+      face_cells(f, dd, cl, cr);
+      double s = 0.0;
+      if (cl >= 0 && cr >= 0) {
+        for (int q = 0; q < NQ; ++q) {
+          double wl[MV], wr[MV];
+          for (int j = 0; j < MV; ++j) {
+            wl[j] = Tr[((dd * 2 * C + cl * MV + j) * NB) * NQ + q];
+            wr[j] = Tr[(((dd * 2 + 1) * C + cr * MV + j) * NB) * NQ + q];
+          }
+          s = fmax(s, fmax(nlflux::speed<FLUX>(wl, dd, g), nlflux::speed<FLUX>(wr, dd, g)));
+        }
+      }
+      alpha[f] = s;
+    }
+    __syncthreads();
+  }
+  // time lines of the face points: both traces, the face flux, projected onto the time modes
+  for (int i = tid; i < 24 * NQ; i += NT) {
+    const int f = i / NQ, qo = i - f * NQ;
+    int dd, cl, cr;
+    face_cells(f, dd, cl, cr);
+    const double* tl = Tr + (dd * 2 * C + (cl < 0 ? cr : cl) * MV) * NB * NQ + qo;
+    const double* tr = Tr + ((dd * 2 + 1) * C + (cr < 0 ? cl : cr) * MV) * NB * NQ + qo;
+    const double al = 0.5 * alpha[f];
+    double* h = Hf + f * MV * NB * NQ + qo;
+    double ml[MV][NA], mr[MV][NA], acc[MV][NA];
+#pragma unroll
+    for (int j = 0; j < MV; ++j)
+#pragma unroll
+      for (int a = 0; a < NA; ++a) {
+        ml[j][a] = tl[(j * NB + a) * NQ];
+        mr[j][a] = tr[(j * NB + a) * NQ];
+        acc[j][a] = 0.0;
+      }
+#pragma unroll
+    for (int q = 0; q < (FIRST ? 1 : NQ); ++q) {
+      double wl[MV], wr[MV], fl[MV], fr[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        wl[j] = ml[j][0];
+        wr[j] = mr[j][0];
+#pragma unroll
+        for (int a = 1; a < NA; ++a) {
+          wl[j] = fma(vq<NB>(T, a, q), ml[j][a], wl[j]);
+          wr[j] = fma(vq<NB>(T, a, q), mr[j][a], wr[j]);
+        }
+      }
+      if (cl >= 0) flux1<FLUX>(wl, dd, fl, g);
+      if (cr >= 0) flux1<FLUX>(wr, dd, fr, g);
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        // region boundary: the interior trace alone
+        const double fh = cl < 0 ? fr[j] : cr < 0 ? fl[j]
+                          : fma(0.5, fl[j] + fr[j], -al * (wr[j] - wl[j]));
+        if constexpr (FIRST) {
+          acc[j][0] = 2.0 * fh;
+        } else {
+#pragma unroll
+          for (int a = 0; a < NA; ++a) acc[j][a] = fma(wvq<NB>(T, a, q), fh, acc[j][a]);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < MV; ++j)
+#pragma unroll
+      for (int a = 0; a < NA; ++a) h[(j * NB + a) * NQ] = acc[j][a];
+  }
+  __syncthreads();  // the traces (in B2) are consumed
+  // time lines of the volume points: values, both fluxes, projected onto the time modes
+  for (int i = tid; i < 9 * NX; i += NT) {
+    const int r = i / NX, yx = i - r * NX;
+    double* p1 = B1 + r * MV * NB * NX + yx;
+    double* p2 = B2 + r * MV * NB * NX + yx;
+    if constexpr (FIRST) {
+      double w[MV], fx[MV], fy[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) w[j] = p1[j * NB * NX];
+      flux2<FLUX>(w, fx, fy, g);
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        p1[j * NB * NX] = 2.0 * fx[j];
+        if constexpr (K::NG == 2) p2[j * NB * NX] = 2.0 * fy[j];
+      }
+    } else if constexpr (MV == 1) {
+      double m[NB], v[NQ];
+#pragma unroll
+      for (int a = 0; a < NB; ++a) m[a] = p1[a * NX];
+      interp<NB>(T, m, v);
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) v[q] = 0.5 * v[q] * v[q];
+      project<NB, false>(T, v, m);
+#pragma unroll
+      for (int a = 0; a < NB; ++a) p1[a * NX] = m[a];
+    } else {
+      double m[MV][NB], ax[MV][NB], ay[MV][NB];
+#pragma unroll
+      for (int j = 0; j < MV; ++j)
+#pragma unroll
+        for (int a = 0; a < NB; ++a) {
+          m[j][a] = p1[(j * NB + a) * NX];
+          ax[j][a] = ay[j][a] = 0.0;
+        }
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        double w[MV], fx[MV], fy[MV];
+#pragma unroll
+        for (int j = 0; j < MV; ++j) {
+          w[j] = m[j][0];
+#pragma unroll
+          for (int a = 1; a < NB; ++a) w[j] = fma(vq<NB>(T, a, q), m[j][a], w[j]);
+        }
+        flux2<FLUX>(w, fx, fy, g);
+#pragma unroll
+        for (int j = 0; j < MV; ++j)
+#pragma unroll
+          for (int a = 0; a < NB; ++a) {
+            ax[j][a] = fma(wvq<NB>(T, a, q), fx[j], ax[j][a]);
+            ay[j][a] = fma(wvq<NB>(T, a, q), fy[j], ay[j][a]);
+          }
+      }
+#pragma unroll
+      for (int j = 0; j < MV; ++j)
+#pragma unroll
+        for (int a = 0; a < NB; ++a) {
+          p1[(j * NB + a) * NX] = ax[j][a];
+          p2[(j * NB + a) * NX] = ay[j][a];
+        }
+    }
+  }
+  __syncthreads();
+  // y lines back: the x flux with phi_y, the y flux with phi_y'; the face lines along them
+  for (int i = tid; i < C * NA * NQ; i += NT) {
+    const int c = i / (NA * NQ), a = (i / NQ) % NA, x = i % NQ;
+    double* p1 = B1 + (c * NB + a) * NX + x;
+    double* p2 = B2 + (c * NB + a) * NX + x;
+    double f[NQ], o1[NB], o2[NB];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) f[q] = p1[q * NQ];
+    project<NB, false>(T, f, o1);
+    if constexpr (K::NG == 2) {
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) f[q] = p2[q * NQ];
+    }
+    project<NB, true>(T, f, o2);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      p1[b * NQ] = o1[b];
+      p2[b * NQ] = o2[b];
+    }
+  }
+  for (int i = tid; i < 24 * MV * NA; i += NT) {
+    double* p = Hf + (i / NA * NB + i % NA) * NQ;
+    double f[NQ], o[NB];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) f[q] = p[q];
+    project<NB, false>(T, f, o);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) p[b] = o[b];
+  }
+  __syncthreads();
+  // x lines back, and R = time term - source - volume + faces
+  const double l0 = 0.25 * lam[0], l1 = 0.25 * lam[1];
+  for (int i = tid; i < C * NB * NB; i += NT) {
+    const int c = i / (NB * NB), a = (i / NB) % NB, y = i % NB;
+    double* out = Rs + (c * NB + a) * THS + y * NB;
+    if (FIRST && a > 0) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b) out[b] = 0.0;
+      continue;
+    }
+    const int r = c / MV, j = c - r * MV, ry = r / 3, rx = r - 3 * ry;
+    const double* p1 = B1 + ((c * NB + a) * NQ + y) * NQ;
+    const double* p2 = B2 + ((c * NB + a) * NQ + y) * NQ;
+    double f[NQ], ox[NB], oy[NB];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) f[q] = p1[q];
+    project<NB, true>(T, f, ox);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) f[q] = p2[q];
+    project<NB, false>(T, f, oy);
+    const double* hx = Hf + (((ry * 4 + rx) * MV + j) * NB + a) * NQ;         // left face
+    const double* hy = Hf + (((12 + rx * 4 + ry) * MV + j) * NB + a) * NQ;    // lower face
+    const double hl = hx[y], hr = hx[MV * NB * NQ + y];
+    const double sx = hr - hl, dx = hr + hl;  // even / odd x modes: ep (hr -+ hl)
+    const double ey = T.ep[y];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const double hb = hy[b], ht = hy[MV * NB * NQ + b];
+      const double fy = (y & 1) ? ht + hb : ht - hb;
+      double acc = l0 * fma(T.ep[b], (b & 1) ? dx : sx, -ox[b]);
+      acc = fma(l1, fma(ey, fy, -oy[b]), acc);
+      if constexpr (!FIRST) {
+        const double* w = Ws + c * K::THT + y * NB + b;
+#pragma unroll
+        for (int e = 0; e < NB; ++e) acc = fma(T.Mt[a][e], w[e * THS], acc);
+        // psi_a(-1) Q
+        acc = fma((a & 1) ? T.ep[a] : -T.ep[a], Qs[c * THS + y * NB + b], acc);
+      }
+      out[b] = acc;
+    }
+  }
+  __syncthreads();
+}
+
+// ---- block reductions: NV sums (or maxima), one barrier; buf alternates between calls -------
+template <int NW, int NV, bool MAX>
+__device__ __forceinline__ void reduce(float (&v)[NV], float* red, int& buf) {
+  static_assert(NV <= 4, "four slots per warp");
+#pragma unroll
+  for (int k = 0; k < NV; ++k)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float t = __shfl_xor_sync(0xffffffffu, v[k], o);
+      v[k] = MAX ? fmaxf(v[k], t) : v[k] + t;
+    }
+  float* p = red + buf * 4 * NW;
+  buf ^= 1;
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) p[(threadIdx.x >> 5) * 4 + k] = v[k];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    v[k] = p[k];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) v[k] = MAX ? fmaxf(v[k], p[w * 4 + k]) : v[k] + p[w * 4 + k];
+  }
+}
+
+// (F' v) for primitives (u, v, H) and both directions, or one
+struct Prim {
+  float u, v, H;
+};
+__device__ __forceinline__ void euler_jv(const Prim& s, const float* d, float g1, float* gx,
+                                         float* gy) {
+  const float k = 0.5f * fmaf(s.u, s.u, s.v * s.v);
+  const float dp = g1 * (fmaf(k, d[0], d[3]) - fmaf(s.u, d[1], s.v * d[2]));
+  const float a = fmaf(-s.u, d[0], d[1]), b = fmaf(-s.v, d[0], d[2]), h = d[3] + dp;
+  gx[0] = d[1];
+  gx[1] = fmaf(s.u, d[1] + a, dp);
+  gx[2] = fmaf(s.v, a, s.u * d[2]);
+  gx[3] = fmaf(s.H, a, s.u * h);
+  gy[0] = d[2];
+  gy[1] = fmaf(s.u, b, s.v * d[1]);
+  gy[2] = fmaf(s.v, d[2] + b, dp);
+  gy[3] = fmaf(s.H, b, s.v * h);
+}
+__device__ __forceinline__ void euler_jv1(const Prim& s, const float* d, float g1, int dd,
+                                          float* f) {
+  const float k = 0.5f * fmaf(s.u, s.u, s.v * s.v);
+  const float dp = g1 * (fmaf(k, d[0], d[3]) - fmaf(s.u, d[1], s.v * d[2]));
+  const float un = dd ? s.v : s.u, dn = dd ? d[2] : d[1];
+  const float a = fmaf(-un, d[0], dn);  // rho d(u_n)
+  f[0] = dn;
+  f[1] = fmaf(s.u, a, un * d[1]);
+  f[2] = fmaf(s.v, a, un * d[2]);
+  if (dd) f[2] += dp; else f[1] += dp;
+  f[3] = fmaf(s.H, a, un * (d[3] + dp));
+}
+__device__ __forceinline__ Prim prim_of(const float* w, float g1) {
+  Prim s;
+  const float ir = 1.0f / w[0];
+  s.u = w[1] * ir;
+  s.v = w[2] * ir;
+  const float p = g1 * (w[3] - 0.5f * fmaf(w[1], s.u, w[2] * s.v));
+  s.H = (w[3] + p) * ir;
+  return s;
+}
+
+// in-place transform of the x or y lines of P: out[i] = sum_b A(b, i) in[b], A = M[i][b] (to
+// modes) or N[b][i] (to nodes)
+template <int NB, int MV, bool TO_NODES>
+__device__ __forceinline__ void lines(const Tab<NB>& T, float* P, bool ydir) {
+  using K = Cfg<NB, MV>;
+  for (int i = threadIdx.x; i < K::VT * 9 * NB; i += K::NT) {
+    const int tj = i / (9 * NB), ro = i - tj * 9 * NB, r = ro / NB, o = ro - r * NB;
+    const int st = ydir ? NB : 1;
+    float* p = P + tj * K::COL + r * K::THS + (ydir ? o : o * NB);
+    float in[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) in[b] = p[b * st];
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+      float s = 0.f;
+#pragma unroll
+      for (int b = 0; b < NB; ++b) s = fmaf(TO_NODES ? T.N[b][n] : T.M[n][b], in[b], s);
+      p[n * st] = s;
+    }
+  }
+}
+
+// modal FP64 field src (scaled) to FP32 values at the (y, x) nodes, time still modal
+template <int NB, int MV>
+__device__ __forceinline__ void to_nodes(const Tab<NB>& T, const double* src, double scale,
+                                         float* P) {
+  using K = Cfg<NB, MV>;
+  for (int i = threadIdx.x; i < K::VT * 9 * NB; i += K::NT) {
+    const int tj = i / (9 * NB), ro = i - tj * 9 * NB, r = ro / NB, y = ro - r * NB;
+    const int a = tj / MV, j = tj - a * MV;
+    const double* s = src + ((r * MV + j) * NB + a) * K::THS + y * NB;
+    float in[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) in[b] = (float)(s[b] * scale);
+    float* p = P + tj * K::COL + r * K::THS + y * NB;
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+      float v = 0.f;
+#pragma unroll
+      for (int b = 0; b < NB; ++b) v = fmaf(T.N[b][n], in[b], v);
+      p[n] = v;
+    }
+  }
+  __syncthreads();
+  lines<NB, MV, true>(T, P, true);
+  __syncthreads();
+}
+
+// The linearisation point of a thread: F' at the nodes of its column and at both sides of
+// its face line (Burgers: the value; Euler: primitives).
+template <int NB, int MV>
+struct Lin {
+  float w[NB], wl[NB], wr[NB];
+};
+template <int NB>
+struct Lin<NB, 4> {
+  Prim w[NB], wl[NB], wr[NB];
+};
+
+// Thread constants of the linearised operator: the thread's column (cell, y, x) and its
+// face line.
+template <int NB>
+struct Rows {
+  float dx[NB], dy[NB], xp, xm, yp, ym;  // -lam D rows, +-lam E of the column's node
+  int gx, gy;                            // its x line (first node) and y line in a flux array
+  int fx, fy;                            // its left / lower face value: (face * VT) * NB + line
+  int dd, bl, br;                        // face line: direction, first nodes (-1: outside)
+  float al;                              // alpha / 2
+};
+
+// out = (time operator)^-1 J v on node values, all 9 cells
+template <int NB, int MV, int FLUX>
+__device__ __forceinline__ void apply(const Tab<NB>& T, const Rows<NB>& R, const Lin<NB, MV>& S,
+                                      const float (&v)[NB * MV], float (&out)[NB * MV], float* P,
+                                      float* G, float* Fh, float g1) {
+  using K = Cfg<NB, MV>;
+  constexpr int VT = K::VT, COL = K::COL;
+  const int tid = threadIdx.x;
+  if (tid < COL) {
+#pragma unroll
+    for (int t = 0; t < NB; ++t) {
+      if constexpr (MV == 1) {
+        P[t * COL + tid] = v[t];
+        G[t * COL + tid] = S.w[t] * v[t];
+      } else {
+        float gx[MV], gy[MV];
+        euler_jv(S.w[t], v + t * MV, g1, gx, gy);
+#pragma unroll
+        for (int j = 0; j < MV; ++j) {
+          P[(t * MV + j) * COL + tid] = v[t * MV + j];
+          G[(t * MV + j) * COL + tid] = gx[j];
+          G[K::nP + (t * MV + j) * COL + tid] = gy[j];
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (tid < K::FL) {
+    const int st = R.dd ? NB : 1, f = tid / NB, o = tid - f * NB;
+    float* h = Fh + f * VT * NB + o;
+#pragma unroll
+    for (int t = 0; t < NB; ++t) {
+      float vl[MV], vr[MV], fl[MV], fr[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        vl[j] = vr[j] = 0.f;
+        const float* p = P + (t * MV + j) * COL;
+        if (R.bl >= 0)
+#pragma unroll
+          for (int n = 0; n < NB; ++n) vl[j] = fmaf(T.L[0][n], p[R.bl + n * st], vl[j]);
+        if (R.br >= 0)
+#pragma unroll
+          for (int n = 0; n < NB; ++n) vr[j] = fmaf(T.L[1][n], p[R.br + n * st], vr[j]);
+      }
+      if constexpr (MV == 1) {
+        fl[0] = S.wl[t] * vl[0];
+        fr[0] = S.wr[t] * vr[0];
+      } else {
+        euler_jv1(S.wl[t], vl, g1, R.dd, fl);
+        euler_jv1(S.wr[t], vr, g1, R.dd, fr);
+      }
+#pragma unroll
+      for (int j = 0; j < MV; ++j)
+        h[(t * MV + j) * NB] = R.bl < 0   ? fr[j]
+                               : R.br < 0 ? fl[j]
+                                          : fmaf(0.5f, fl[j] + fr[j], -R.al * (vr[j] - vl[j]));
+    }
+  }
+  __syncthreads();
+  if (tid < COL) {
+    float acc[VT];
+#pragma unroll
+    for (int tj = 0; tj < VT; ++tj) {
+      const float* gx = G + tj * COL + R.gx;
+      const float* gy = G + (K::NG == 2 ? K::nP : 0) + tj * COL + R.gy;
+      float s = 0.f;
+#pragma unroll
+      for (int n = 0; n < NB; ++n) s = fmaf(R.dx[n], gx[n], s);
+#pragma unroll
+      for (int n = 0; n < NB; ++n) s = fmaf(R.dy[n], gy[n * NB], s);
+      const float* hx = Fh + R.fx + tj * NB;
+      const float* hy = Fh + R.fy + tj * NB;
+      s = fmaf(R.xm, hx[0], s);
+      s = fmaf(R.xp, hx[VT * NB], s);
+      s = fmaf(R.ym, hy[0], s);
+      s = fmaf(R.yp, hy[VT * NB], s);
+      acc[tj] = s;
+    }
+#pragma unroll
+    for (int t = 0; t < NB; ++t)
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        float s = v[t * MV + j];
+#pragma unroll
+        for (int e = 0; e < NB; ++e) s = fmaf(T.Ti[t][e], acc[e * MV + j], s);
+        out[t * MV + j] = s;
+      }
+  }
+}
+
+constexpr int kMaxSolves = 7;   // linear solves of a region before it is left to the list
+constexpr int kMaxInner = 24;   // BiCGStab iterations per solve
+
+template <int NB, int MV, int FLUX, bool BATCH>
+__global__ void __launch_bounds__((Cfg<NB, MV>::NT), (Cfg<NB, MV>::MINB)) newton_mf_kernel(const NewtonMfArgs a,
+                                                                      const Tab<NB> T) {
+  using K = Cfg<NB, MV>;
+  constexpr int VT = K::VT, COL = K::COL, NT = K::NT, NW = K::NW, THS = K::THS, BS = K::BS;
+  extern __shared__ __align__(16) unsigned char smem[];
+  double* Ws = (double*)smem;
+  double* Rs = (double*)(smem + K::oR);
+  double* Qs = (double*)(smem + K::oQ);
+  __shared__ double alpha[24];
+  float* red = (float*)(smem + K::oRed);
+  double* arena = (double*)(smem + K::oArena);
+  float* P = (float*)arena;
+  float* G = P + K::nP;
+  float* Fh = G + K::NG * K::nP;
+  const int tid = threadIdx.x;
+  const long long eg = blockIdx.x;
+  // the region's instance (batched launch: the last whose first region is <= eg)
+  const double* Qg = a.Q;
+  double* Wg = a.W;
+  int* stats = a.stats;
+  unsigned long long* itot = a.iters_total;
+  int nx = a.nx, ny = a.ny;
+  long long e = eg;
+  double lam[2] = {a.lam[0], a.lam[1]};
+  if constexpr (BATCH) {
+    int lo = 0, hi = a.ninst - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (a.inst[mid].cell0 <= eg) lo = mid; else hi = mid - 1;
+    }
+    const NlInst& in = a.inst[lo];
+    Qg = in.Q;
+    Wg = in.W;
+    stats = in.stats;
+    itot = in.iters_total;
+    nx = in.nx;
+    ny = in.ny;
+    e = eg - in.cell0;
+    lam[0] = in.lam[0];
+    lam[1] = in.lam[1];
+  }
+  const unsigned ue = (unsigned)e, uy = ue / (unsigned)nx;
+  const int ix = (int)(ue - uy * (unsigned)nx), iy = (int)uy;
+  for (int i = tid; i < 9 * MV * THS; i += NT) {
+    const int r = i / (MV * THS), rem = i - r * (MV * THS);
+    int cx = ix + r % 3 - 1, cy = iy + r / 3 - 1;
+    cx += cx < 0 ? nx : (cx >= nx ? -nx : 0);
+    cy += cy < 0 ? ny : (cy >= ny ? -ny : 0);
+    const double q = Qg[((long long)cy * nx + cx) * (MV * THS) + rem];
+    Qs[i] = q;
+    const int j = rem / THS, s = rem - j * THS;
+    double* w = Ws + (r * MV + j) * K::THT + s;  // Q^n extended constant in time
+    w[0] = q;
+#pragma unroll
+    for (int t = 1; t < NB; ++t) w[t * THS] = 0.0;
+  }
+  __syncthreads();
+
+  // thread constants
+  Rows<NB> R;
+  {
+    const int c = tid < COL ? tid : 0, r = c / THS, s = c - r * THS, y = s / NB, x = s - y * NB;
+    const int ry = r / 3, rx = r - 3 * ry;
+    const float l0 = (float)lam[0], l1 = (float)lam[1];
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+      R.dx[n] = -l0 * T.D[x][n];
+      R.dy[n] = -l1 * T.D[y][n];
+    }
+    R.xp = l0 * T.E[0][x];
+    R.xm = -l0 * T.E[1][x];
+    R.yp = l1 * T.E[0][y];
+    R.ym = -l1 * T.E[1][y];
+    R.gx = r * THS + y * NB;
+    R.gy = r * THS + x;
+    R.fx = (ry * 4 + rx) * VT * NB + y;
+    R.fy = (12 + rx * 4 + ry) * VT * NB + x;
+    const int f = tid < K::FL ? tid / NB : 0, o = tid < K::FL ? tid - f * NB : 0;
+    int cl, cr;
+    face_cells(f, R.dd, cl, cr);
+    const int st = R.dd ? 1 : NB;
+    R.bl = cl < 0 ? -1 : cl * THS + o * st;
+    R.br = cr < 0 ? -1 : cr * THS + o * st;
+    R.al = 0.f;
+  }
+  Lin<NB, MV> S;
+  const float g1 = (float)(a.gamma - 1.0);
+  int buf = 0, it = 0;
+  bool conv = false, lin = true;
+  double dprev = 0.0;
+  float bprev = 0.f, wnorm = 1.f;
+#pragma unroll 1
+  for (int solve = 0; solve < kMaxSolves; ++solve) {
+    if (solve == 0)
+      residual<NB, MV, FLUX, true>(T, Ws, Qs, Rs, alpha, arena, lam, a.gamma);
+    else
+      residual<NB, MV, FLUX, false>(T, Ws, Qs, Rs, alpha, arena, lam, a.gamma);
+    // scale of the right-hand side (a power of two, so that its squares stay normal in FP32)
+    float m1[1] = {0.f};
+    for (int i = tid; i < 9 * BS; i += NT) {
+      const double x = fabs(Rs[i]);
+      m1[0] = x <= 1e30 ? fmaxf(m1[0], (float)x) : 3e38f;  // (a NaN compares false)
+    }
+    reduce<NW, 1, true>(m1, red, buf);
+    const float rmax = m1[0];
+    if (!(rmax <= 1e30f)) break;
+    const int ex = rmax > 1e-30f ? ilogbf(rmax) : -100;
+    const double scale = scalbn(1.0, -ex), unscale = scalbn(1.0, ex);
+    // a new linearisation where the last one no longer contracts by 3e3 per solve
+    if (solve > 0 && rmax > 3e-4f * bprev && it < a.max_iters) lin = true;
+    bprev = rmax;
+    if (lin) {
+      to_nodes<NB, MV>(T, Ws, 1.0, P);
+      float w[VT];
+      if (tid < COL) {
+        float m[VT];
+#pragma unroll
+        for (int tj = 0; tj < VT; ++tj) m[tj] = P[tj * COL + tid];
+#pragma unroll
+        for (int t = 0; t < NB; ++t)
+#pragma unroll
+          for (int j = 0; j < MV; ++j) {
+            float s = 0.f;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) s = fmaf(T.N[b][t], m[b * MV + j], s);
+            w[t * MV + j] = s;
+          }
+#pragma unroll
+        for (int tj = 0; tj < VT; ++tj) P[tj * COL + tid] = w[tj];
+#pragma unroll
+        for (int t = 0; t < NB; ++t) {
+          if constexpr (MV == 1) S.w[t] = w[t];
+          else S.w[t] = prim_of(w + t * MV, g1);
+        }
+      }
+      __syncthreads();
+      if (tid < K::FL) {
+        const int st = R.dd ? NB : 1;
+        // outside the region the inner trace stands in (its flux is not used)
+        const int bl = R.bl < 0 ? R.br : R.bl, br = R.br < 0 ? R.bl : R.br;
+#pragma unroll
+        for (int t = 0; t < NB; ++t) {
+          float l[MV], r[MV];
+#pragma unroll
+          for (int j = 0; j < MV; ++j) {
+            const float* p = P + (t * MV + j) * COL;
+            l[j] = r[j] = 0.f;
+#pragma unroll
+            for (int n = 0; n < NB; ++n) {
+              l[j] = fmaf(T.L[R.bl < 0][n], p[bl + n * st], l[j]);
+              r[j] = fmaf(T.L[R.br < 0 ? 0 : 1][n], p[br + n * st], r[j]);
+            }
+          }
+          if constexpr (MV == 1) {
+            S.wl[t] = l[0];
+            S.wr[t] = r[0];
+          } else {
+            S.wl[t] = prim_of(l, g1);
+            S.wr[t] = prim_of(r, g1);
+          }
+        }
+        R.al = 0.5f * (float)alpha[tid / NB];
+      }
+      __syncthreads();
+      lin = false;
+      ++it;
+    }
+    // right-hand side: node values of (time operator)^-1 R, scaled
+    to_nodes<NB, MV>(T, Rs, scale, P);
+    float r[VT], rh[VT], p[VT], v[VT], t[VT], x[VT];
+    float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < VT; ++k) r[k] = p[k] = v[k] = t[k] = x[k] = 0.f;
+    if (tid < COL) {
+      float m[VT];
+#pragma unroll
+      for (int tj = 0; tj < VT; ++tj) m[tj] = P[tj * COL + tid];
+#pragma unroll
+      for (int n = 0; n < NB; ++n)
+#pragma unroll
+        for (int j = 0; j < MV; ++j) {
+          float s = 0.f;
+#pragma unroll
+          for (int b = 0; b < NB; ++b) s = fmaf(T.TN[n][b], m[b * MV + j], s);
+          r[n * MV + j] = s;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < VT; ++k) {
+      rh[k] = p[k] = r[k];
+      s4[0] = fmaf(r[k], r[k], s4[0]);
+    }
+    {
+      float s1[1] = {s4[0]};
+      reduce<NW, 1, false>(s1, red, buf);
+      s4[0] = s1[0];
+    }
+    const float bb = s4[0];
+    // relative accuracy: 1e-4 in the first solve (whose result the nonlinearity limits), then
+    // down to an absolute ~1e-15 of the iterate, at most 1e-5 (FP32)
+    const float bmean = sqrtf(bb / (9 * BS)) * (float)unscale;
+    const float tol = solve == 0 ? 1e-4f : fminf(1e-2f, fmaxf(1e-5f, 1e-15f * wnorm / bmean));
+    const float stop = tol * tol * bb;
+    float rho = bb, rr = bb;
+    bool ok = true;
+    int k = 0;
+#pragma unroll 1
+    for (; k < kMaxInner && rr > stop; ++k) {
+      apply<NB, MV, FLUX>(T, R, S, p, v, P, G, Fh, g1);
+      float s1[1] = {0.f};
+      if (tid < COL)
+#pragma unroll
+        for (int q = 0; q < VT; ++q) s1[0] = fmaf(rh[q], v[q], s1[0]);
+      reduce<NW, 1, false>(s1, red, buf);
+      const float al = rho / s1[0];
+#pragma unroll
+      for (int q = 0; q < VT; ++q) r[q] = fmaf(-al, v[q], r[q]);  // s of the method
+      apply<NB, MV, FLUX>(T, R, S, r, t, P, G, Fh, g1);
+      s4[0] = s4[1] = s4[2] = s4[3] = 0.f;
+      if (tid < COL)
+#pragma unroll
+        for (int q = 0; q < VT; ++q) {
+          s4[0] = fmaf(t[q], r[q], s4[0]);
+          s4[1] = fmaf(t[q], t[q], s4[1]);
+          s4[2] = fmaf(rh[q], t[q], s4[2]);
+          s4[3] = fmaf(r[q], r[q], s4[3]);
+        }
+      reduce<NW, 4, false>(s4, red, buf);
+      const float om = s4[1] > 0.f ? s4[0] / s4[1] : 0.f;
+#pragma unroll
+      for (int q = 0; q < VT; ++q) {
+        x[q] = fmaf(al, p[q], fmaf(om, r[q], x[q]));
+        r[q] = fmaf(-om, t[q], r[q]);
+      }
+      rr = fmaxf(0.f, s4[3] - om * s4[0]);
+      const float rho1 = -om * s4[2];  // <rh, r>, <rh, s> = 0
+      const float be = rho1 / rho * (al / om);
+      rho = rho1;
+#pragma unroll
+      for (int q = 0; q < VT; ++q) p[q] = fmaf(be, fmaf(-om, v[q], p[q]), r[q]);
+      if (!(fabsf(al) < 1e30f) || !(rr < 1e30f)) {
+        ok = false;
+        break;
+      }
+      if (rr > stop && !(fabsf(be) < 1e30f)) {  // (a vanished residual leaves be undefined)
+        ok = false;
+        break;
+      }
+    }
+    if (!ok || rr > 1e-2f * bb) break;  // stalled
+    // the update in modes
+    __syncthreads();
+    if (tid < COL) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int j = 0; j < MV; ++j) {
+          float s = 0.f;
+#pragma unroll
+          for (int n = 0; n < NB; ++n) s = fmaf(T.M[b][n], x[n * MV + j], s);
+          P[(b * MV + j) * COL + tid] = s;
+        }
+    }
+    __syncthreads();
+    lines<NB, MV, false>(T, P, true);
+    __syncthreads();
+    lines<NB, MV, false>(T, P, false);
+    __syncthreads();
+    float mx[2] = {0.f, 0.f};
+    for (int i = tid; i < 9 * BS; i += NT) {
+      const int c = i / K::THT, m = i - c * K::THT, aa = m / THS, s = m - aa * THS;
+      const int rg = c / MV, j = c - rg * MV;
+      const double d = unscale * (double)P[(aa * MV + j) * COL + rg * THS + s];
+      const double w = Ws[i] - d;
+      Ws[i] = w;
+      // (rounded up, so that the FP32 comparison below is never the looser one)
+      mx[0] = isfinite(d) ? fmaxf(mx[0], __double2float_ru(fabs(d))) : 3e38f;
+      mx[1] = isfinite(w) ? fmaxf(mx[1], __double2float_rd(fabs(w))) : 3e38f;
+    }
+    reduce<NW, 2, true>(mx, red, buf);
+    if (!(mx[0] < 1e30f) || !(mx[1] < 1e30f)) break;
+    const double dn = mx[0], wn = mx[1];
+    wnorm = fmaxf(1.f, mx[1]);
+    if (dn <= a.tol * fmax(1.0, wn)) {
+      conv = true;
+      break;
+    }
+    if (solve > 0 && dn > 0.1 * dprev) break;
+    dprev = dn;
+  }
+  if (conv) {
+    for (int i = tid; i < BS; i += NT) Wg[e * BS + i] = Ws[4 * BS + i];
+    if (tid == 0) {
+      atomicMax(&stats[1], it);
+      atomicAdd(&stats[7 + (it < 15 ? it : 15)], 1);
+      atomicAdd(itot, (unsigned long long)it);
+    }
+  } else if (tid == 0) {
+    a.list[atomicAdd(a.list_count, 1)] = (int)eg;
+  }
+}
+
+}  // namespace mf
+}  // namespace ridg

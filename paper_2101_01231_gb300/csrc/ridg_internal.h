@@ -218,7 +218,30 @@ struct NewtonArgs {
   unsigned long long* iters_total;  // Newton iterations summed over regions
   const NlInst* inst;  // batched launch: instance table (ncell = total regions), else nullptr
   int ninst;
+  // the regions to solve: list[0 .. *list_count) (left over by the matrix-free solver), or all
+  // of them if list is nullptr
+  const int* list;
+  const int* list_count;
 };
+// The matrix-free Newton prediction (k_newton_mf.cuh), the mixed precisions' first solver: it
+// solves every region it can and lists the others for launch_newton.
+struct NewtonMfArgs {
+  const double* Q;
+  double* W;
+  int nx, ny;
+  long long ncell;     // regions (batched launch: of all instances)
+  double lam[2];
+  double gamma;
+  int max_iters;       // linearisations per region
+  double tol;
+  int* stats;          // as in NewtonArgs
+  unsigned long long* iters_total;
+  const NlInst* inst;  // batched launch: instance table, else nullptr
+  int ninst;
+  int* list;           // regions left over (room for ncell)
+  int* list_count;     // their number (zeroed by the launch)
+};
+cudaError_t launch_newton_mf(int nb, int m, int flux_kind, const NewtonMfArgs& a, cudaStream_t s);
 cudaError_t launch_newton(int nb, int m, int flux_kind, int prec, const NewtonArgs& a, int grid,
                           cudaStream_t s);
 // The batched Burgers ensemble's Newton prediction in one launch: the degrees' region queues
@@ -321,6 +344,8 @@ struct ridg_handle {
   int nl_grid_max = 0;    // CTAs the block storage is allocated for
   int tune_gemm3_slots = 0;   // 3D GEMM plane-operand ring depth (0: as many as fit)
   int tune_corr3_block = 128; // 3D correction block size
+  int* nl_list = nullptr; // mixed precisions: [0] count, [1..] the regions that the matrix-free
+                          // solver leaves to the block elimination
   bool nl_scratch_shared = false;  // block storage owned by the batch
   int* nl_words = nullptr;  // [0] work counter, [1..3] Newton statistics, [4..5] max speed
                             // bits, [6..7] total Newton iterations, [8..23] iteration histogram

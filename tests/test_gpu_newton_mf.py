@@ -1,0 +1,75 @@
+"""The matrix-free Newton solver of the mixed precisions (k_newton_mf.cuh) at the edges of its
+range: the smallest meshes (every region wraps onto itself), every degree and both fluxes,
+and the hand-over of regions that it leaves to the block elimination."""
+import numpy as np
+import pytest
+
+from paper_2101_01231_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+# both precisions stop when the last update is below 1e-10 and contract by at least 10 per
+# solve, as the FP64 form does: the same fixed point to the tolerance of the existing parity
+# tests
+TOL = 1e-11
+
+
+@pytest.fixture(scope="module")
+def R():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2101_01231_gb300 import ridg
+    return ridg
+
+
+def _smooth(flux, n, M):
+    """A well-resolved state on a small mesh (low wave numbers, small amplitude)."""
+    if flux == "euler":
+        w = I.workload("euler2d_n512_q2", n=n, M=M)
+        c = np.array([1.0, 0.3, -0.2, 2.5])
+
+        def f(x, y):
+            p = 0.02 * np.sin(2 * np.pi * x / 10) + 0.01 * np.cos(2 * np.pi * y / 10)
+            return np.stack([c[j] + (1 + 0.3 * j) * p for j in range(4)])
+        return w, np.ascontiguousarray(I.project_tensor(f, w, M + 1, m=4).reshape(-1, 4 * (M + 1) ** 2))
+    w = dict(I.burgers_ensemble(1)[0], M=M, n=n)
+    f = lambda x, y: 0.5 + 0.05 * np.sin(2 * np.pi * x) * np.cos(2 * np.pi * y)
+    return w, np.ascontiguousarray(I.project_tensor(f, w, M + 1).reshape(-1, (M + 1) ** 2))
+
+
+def _predict(R, w, q, prec, **kw):
+    s = R.Solver(2, w["n"], w["M"], flux=w["flux"], cfl=w["cfl"], lo=w["lo"], hi=w["hi"],
+                 gamma=w.get("gamma", 1.4), precision=prec, **kw)
+    s.set_state(q)
+    W = s.predict()
+    info, status = s.info(), s.last_status
+    s.close()
+    return W, info, status
+
+
+@pytest.mark.parametrize("flux,M", [("burgers", 1), ("burgers", 2), ("burgers", 3), ("burgers", 4),
+                                    ("euler", 1), ("euler", 2)])
+@pytest.mark.parametrize("n", [(3, 3), (5, 17)])
+def test_matrix_free_matches_fp64(R, flux, M, n):
+    w, q = _smooth(flux, n, M)
+    ref, _, st = _predict(R, w, q, R.RIDG_PREC_FP64)
+    assert st == R.RIDG_OK
+    for prec in (R.RIDG_PREC_MIXED_FP32, R.RIDG_PREC_MIXED_TF32):
+        W, info, st = _predict(R, w, q, prec)
+        assert st == R.RIDG_OK and info["newton_unconverged"] == 0
+        assert sum(info["newton_hist"]) == n[0] * n[1]
+        assert np.abs(W - ref).max() <= TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("flux,M", [("burgers", 2), ("burgers", 4), ("euler", 2)])
+def test_regions_left_over_are_block_eliminated(R, flux, M):
+    # a tolerance below round-off: no region converges, every one goes through the list to the
+    # block elimination, which stops them at its cap
+    w, q = _smooth(flux, (7, 5), M)
+    ref, _, _ = _predict(R, w, q, R.RIDG_PREC_FP64)
+    for prec in (R.RIDG_PREC_MIXED_FP32, R.RIDG_PREC_MIXED_TF32):
+        W, info, st = _predict(R, w, q, prec, newton_tol=1e-30)
+        assert st == R.RIDG_ENOCONV
+        assert info["newton_unconverged"] == 35 and info["newton_hist"][4] == 35
+        assert np.abs(W - ref).max() <= TOL * np.abs(ref).max()
