@@ -387,7 +387,7 @@ int enqueue_nl_correct(ridg_t* h) {
                                           h->stream));
     return RIDG_OK;
   }
-  RIDG_CUDA(h, ridg::launch_nl_correct(h->nb, h->m, h->flux.kind, h->nl.tb, h->Q, h->W, h->n[0],
+  RIDG_CUDA(h, ridg::launch_nl_correct(h->nb, h->m, h->flux.kind, h->Q, h->W, h->n[0],
                                        h->n[1], h->ncell, h->dt / h->h[0], h->dt / h->h[1],
                                        h->flux.gamma, h->stream));
   return RIDG_OK;
@@ -1201,9 +1201,9 @@ struct ridg_batch {
   // over every instance's cells (schedule 1, the default) or one launch per degree and per
   // instance (schedule 0); the autotuner may pick either
   int schedule = 1;
-  std::vector<ridg::CorrInst> corr_host;  // all instances, cell0 increasing
+  std::vector<ridg::CorrInst> corr_host;  // all instances, block0 increasing
   ridg::CorrInst* corr_table = nullptr;
-  long long corr_cells = 0;
+  long long corr_blocks = 0;
   ridg::NewtonMulti multi_host{};           // the single Newton launch's arguments
   ridg::NewtonMulti* multi_dev = nullptr;   // and their device copy (read by the kernel)
 };
@@ -1235,21 +1235,22 @@ int refresh_nl_tables(ridg_batch_t* b) {
       return RIDG_ECUDA;
   }
   if (b->corr_table) {
-    long long cell0 = 0;
+    long long block0 = 0;
     for (size_t i = 0; i < b->inst.size(); ++i) {
       ridg_t* h = b->inst[i];
       ridg::CorrInst& c = b->corr_host[i];
       c.Q = h->Q;
       c.W = h->W;
-      c.cell0 = cell0;
+      c.block0 = block0;
+      c.ncell = h->ncell;
       c.nx = h->n[0];
       c.ny = h->n[1];
       c.nb = h->nb;
       c.lamx = h->dt / h->h[0];
       c.lamy = h->dt / h->h[1];
-      cell0 += h->ncell;
+      block0 += ridg::nl_correct_blocks(h->nb, h->ncell);
     }
-    b->corr_cells = cell0;
+    b->corr_blocks = block0;
     if (cudaMemcpyAsync(b->corr_table, b->corr_host.data(),
                         b->corr_host.size() * sizeof(ridg::CorrInst), cudaMemcpyHostToDevice,
                         b->stream) != cudaSuccess)
@@ -1332,14 +1333,9 @@ int enqueue_batch_multi(ridg_batch_t* b) {
   RIDG_CUDA(h0, ridg::launch_newton_multi(newton_prec(h0), b->multi_host, b->multi_dev, grid,
                                           b->stream));
   ridg::CorrMulti c;
-  std::memset(&c, 0, sizeof(c));
-  for (const NlGroup& g : b->groups) {
-    ridg_t* h = b->inst[g.idx[0]];
-    c.tb[h->nb - 2] = h->nl.tb;
-  }
   c.inst = b->corr_table;
   c.ninst = (int)b->inst.size();
-  RIDG_CUDA(h0, ridg::launch_nl_correct_multi(c, b->corr_cells, b->stream));
+  RIDG_CUDA(h0, ridg::launch_nl_correct_multi(c, b->corr_blocks, b->stream));
   return RIDG_OK;
 }
 

@@ -6,15 +6,14 @@
 #include "tables.h"
 
 namespace ridg {
-namespace mf {
-namespace {
+namespace nl {
 
 template <int NB>
-Tab<NB> make_tab() {
-  Tab<NB> T{};
+Rule<NB> make_rule() {
+  Rule<NB> T{};
   std::vector<double> x, w, v(NB), dv(NB);
-  gauss_legendre(Tab<NB>::NQ, x, w);
-  for (int q = 0; q < Tab<NB>::H; ++q) {
+  gauss_legendre(Rule<NB>::NQ, x, w);
+  for (int q = 0; q < Rule<NB>::H; ++q) {
     phi_values(NB, x[q], v.data(), dv.data());
     for (int b = 0; b < NB; ++b) {
       T.V[b][q] = v[b];
@@ -22,10 +21,27 @@ Tab<NB> make_tab() {
       T.wD[b][q] = w[q] * dv[b];
     }
   }
+  phi_values(NB, 1.0, T.ep, nullptr);
+  return T;
+}
+template Rule<2> make_rule<2>();
+template Rule<3> make_rule<3>();
+template Rule<4> make_rule<4>();
+template Rule<5> make_rule<5>();
+
+}  // namespace nl
+
+namespace mf {
+namespace {
+
+template <int NB>
+Tab<NB> make_tab() {
+  Tab<NB> T{};
+  (Rule<NB>&)T = make_rule<NB>();
+  std::vector<double> x, w, v(NB), dv(NB);
   const Tables1D t1 = tables1d(NB);
   std::vector<double> A(NB * NB), inv(NB * NB);
   for (int a = 0; a < NB; ++a) {
-    T.ep[a] = t1.ep[a];
     for (int g = 0; g < NB; ++g)
       A[a * NB + g] = T.Mt[a][g] = t1.ep[a] * t1.ep[g] - t1.D[a * NB + g];
   }

@@ -32,21 +32,17 @@
 
 #include <cuda_runtime.h>
 
-#include "k_nlflux.cuh"
+#include "k_nl_lines.cuh"
 #include "ridg_internal.h"
 
 namespace ridg {
 namespace mf {
 
-// 1D tables, passed by value (constant bank).  The Gauss points are symmetric: the FP64
-// rule keeps the lower half, q < H, and the centre point at H - 1 if NQ is odd.
+using namespace nl;
+
+// 1D tables, passed by value (constant bank): the FP64 residual rule, and
 template <int NB>
-struct Tab {
-  static constexpr int NQ = (3 * (NB - 1) + 2) / 2, H = (NQ + 1) / 2;
-  double V[NB][H];     // phi_b(x_q)
-  double wV[NB][H];    // w_q phi_b(x_q)
-  double wD[NB][H];    // w_q phi_b'(x_q)
-  double ep[NB];       // phi_b(+1)
+struct Tab : nl::Rule<NB> {
   double Mt[NB][NB];   // time operator
   // the NB-point rule of the linearised operator
   float N[NB][NB];     // [b][n] phi_b(x_n)
@@ -83,113 +79,6 @@ struct Cfg {
   static constexpr size_t bytes = oArena + arena;
 };
 
-// ---- FP64 lines ---------------------------------------------------------------------------
-// values at the NQ points of the polynomial with modes a
-template <int NB>
-__device__ __forceinline__ void interp(const Tab<NB>& T, const double (&a)[NB],
-                                       double (&v)[Tab<NB>::NQ]) {
-  constexpr int NQ = Tab<NB>::NQ;
-#pragma unroll
-  for (int q = 0; q < NQ / 2; ++q) {
-    double e = a[0];
-#pragma unroll
-    for (int b = 2; b < NB; b += 2) e = fma(T.V[b][q], a[b], e);
-    if constexpr (NB <= 3) {
-      v[q] = fma(T.V[1][q], a[1], e);
-      v[NQ - 1 - q] = fma(-T.V[1][q], a[1], e);
-    } else {
-      const double o = fma(T.V[3][q], a[3], T.V[1][q] * a[1]);
-      v[q] = e + o;
-      v[NQ - 1 - q] = e - o;
-    }
-  }
-  if constexpr (NQ & 1) {
-    double e = a[0];
-#pragma unroll
-    for (int b = 2; b < NB; b += 2) e = fma(T.V[b][NQ / 2], a[b], e);
-    v[NQ / 2] = e;
-  }
-}
-
-// out[b] = sum_q w_q phi_b(x_q) f[q], or with phi_b'
-template <int NB, bool DERIV>
-__device__ __forceinline__ void project(const Tab<NB>& T, const double (&f)[Tab<NB>::NQ],
-                                        double (&out)[NB]) {
-  constexpr int NQ = Tab<NB>::NQ, HP = NQ / 2;
-  double s[HP], d[HP];
-#pragma unroll
-  for (int q = 0; q < HP; ++q) {
-    s[q] = f[q] + f[NQ - 1 - q];
-    d[q] = f[q] - f[NQ - 1 - q];
-  }
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    if constexpr (DERIV) {
-      if (b == 0) {
-        out[b] = 0.0;
-        continue;
-      }
-    }
-    const bool even = DERIV ? (b & 1) : !(b & 1);
-    double acc = 0.0;
-#pragma unroll
-    for (int q = 0; q < HP; ++q) {
-      const double w = DERIV ? T.wD[b][q] : T.wV[b][q];
-      const double x = even ? s[q] : d[q];
-      acc = q == 0 ? w * x : fma(w, x, acc);
-    }
-    if constexpr (NQ & 1)
-      if (even) acc = fma(DERIV ? T.wD[b][HP] : T.wV[b][HP], f[HP], acc);
-    out[b] = acc;
-  }
-}
-
-// phi_b(x_q) at any q (compile-time indices)
-template <int NB>
-__device__ __forceinline__ double vq(const Tab<NB>& T, int b, int q) {
-  constexpr int NQ = Tab<NB>::NQ, H = Tab<NB>::H;
-  return q < H ? T.V[b][q] : ((b & 1) ? -T.V[b][NQ - 1 - q] : T.V[b][NQ - 1 - q]);
-}
-template <int NB>
-__device__ __forceinline__ double wvq(const Tab<NB>& T, int b, int q) {
-  constexpr int NQ = Tab<NB>::NQ, H = Tab<NB>::H;
-  return q < H ? T.wV[b][q] : ((b & 1) ? -T.wV[b][NQ - 1 - q] : T.wV[b][NQ - 1 - q]);
-}
-
-// both directions' fluxes of one state (Euler: one reciprocal)
-template <int FLUX>
-__device__ __forceinline__ void flux2(const double* w, double* fx, double* fy, double g) {
-  if constexpr (FLUX == RIDG_FLUX_BURGERS) {
-    fx[0] = 0.5 * w[0] * w[0];
-  } else {
-    const double ir = 1.0 / w[0], u = w[1] * ir, v = w[2] * ir;
-    const double p = (g - 1.0) * (w[3] - 0.5 * fma(w[1], u, w[2] * v)), h = w[3] + p;
-    fx[0] = w[1];
-    fx[1] = fma(w[1], u, p);
-    fx[2] = w[1] * v;
-    fx[3] = u * h;
-    fy[0] = w[2];
-    fy[1] = fx[2];
-    fy[2] = fma(w[2], v, p);
-    fy[3] = v * h;
-  }
-}
-template <int FLUX>
-__device__ __forceinline__ void flux1(const double* w, int dd, double* f, double g) {
-  if constexpr (FLUX == RIDG_FLUX_BURGERS) {
-    f[0] = 0.5 * w[0] * w[0];
-  } else {
-    const double ir = 1.0 / w[0], u = w[1] * ir, v = w[2] * ir;
-    const double p = (g - 1.0) * (w[3] - 0.5 * fma(w[1], u, w[2] * v));
-    const double un = dd == 0 ? u : v;
-    f[0] = dd == 0 ? w[1] : w[2];
-    f[1] = w[1] * un;
-    f[2] = w[2] * un;
-    if (dd == 0) f[1] += p; else f[2] += p;
-    f[3] = un * (w[3] + p);
-  }
-}
-
 // the cells left and right of region face f (dd * 12 + row * 4 + pos), -1 outside
 __device__ __forceinline__ void face_cells(int f, int& dd, int& cl, int& cr) {
   dd = f >= 12;
@@ -225,10 +114,8 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
     double* dst = B1 + ((c * NB + a) * NQ + y) * NQ;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) dst[q] = v[q];
-    double e = m[0], o = T.ep[1] * m[1];
-#pragma unroll
-    for (int b = 2; b < NB; ++b)
-      if (b & 1) o = fma(T.ep[b], m[b], o); else e = fma(T.ep[b], m[b], e);
+    double e, o;
+    traces<NB>(T, m, 1, e, o);
     Tr[((0 * C + c) * NB + a) * NQ + y] = e + o;
     Tr[((1 * C + c) * NB + a) * NQ + y] = e - o;
   }
@@ -236,10 +123,8 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
   for (int i = tid; i < C * NA * NB; i += NT) {
     const int c = i / (NA * NB), a = (i / NB) % NA, x = i % NB;
     const double* src = Ws + (c * NB + a) * THS + x;
-    double e = src[0], o = T.ep[1] * src[NB];
-#pragma unroll
-    for (int b = 2; b < NB; ++b)
-      if (b & 1) o = fma(T.ep[b], src[b * NB], o); else e = fma(T.ep[b], src[b * NB], e);
+    double e, o;
+    traces<NB>(T, src, NB, e, o);
     Tr[((2 * C + c) * NB + a) * NQ + x] = e + o;
     Tr[((3 * C + c) * NB + a) * NQ + x] = e - o;
   }

@@ -1,0 +1,149 @@
+// FP64 building blocks of the 2D nonlinear path's sum-factorised quadrature: transforms of one
+// line of modes or Gauss-point values held in registers, and the physical fluxes of a point.
+//
+// The FP64 pipe (2 FMA per clock and SM) bounds every kernel that uses them, so they spend
+// registers to save FP64 operations: the Gauss points are symmetric and phi_b is even or odd,
+// so the values at x_q and -x_q share their even and odd partial sums (NB = 3 modes to 4
+// points: 6 FMA instead of 12; 5 to 7: 20 instead of 35).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "k_nlflux.cuh"
+
+namespace ridg {
+namespace nl {
+
+// The residual's 1D rule (NQ = ceil((3M + 1) / 2) points).  Its lower half is kept, q < H, with
+// the centre point at H - 1 if NQ is odd.
+template <int NB>
+struct Rule {
+  static constexpr int NQ = (3 * (NB - 1) + 2) / 2, H = (NQ + 1) / 2;
+  double V[NB][H];     // phi_b(x_q)
+  double wV[NB][H];    // w_q phi_b(x_q)
+  double wD[NB][H];    // w_q phi_b'(x_q)
+  double ep[NB];       // phi_b(+1); phi_b(-1) = (-1)^b phi_b(+1)
+};
+// host (k_newton_mf.cu): the rule of NB = 2 .. 5
+template <int NB>
+Rule<NB> make_rule();
+
+// the traces at +1 (e + o) and -1 (e - o) of the polynomial with modes m[0], m[st], ...
+template <int NB>
+__device__ __forceinline__ void traces(const Rule<NB>& T, const double* m, int st, double& e,
+                                       double& o) {
+  e = m[0];
+  o = T.ep[1] * m[st];
+#pragma unroll
+  for (int b = 2; b < NB; ++b)
+    if (b & 1) o = fma(T.ep[b], m[b * st], o); else e = fma(T.ep[b], m[b * st], e);
+}
+
+// values at the NQ points of the polynomial with modes a
+template <int NB>
+__device__ __forceinline__ void interp(const Rule<NB>& T, const double (&a)[NB],
+                                       double (&v)[Rule<NB>::NQ]) {
+  constexpr int NQ = Rule<NB>::NQ;
+#pragma unroll
+  for (int q = 0; q < NQ / 2; ++q) {
+    double e = a[0];
+#pragma unroll
+    for (int b = 2; b < NB; b += 2) e = fma(T.V[b][q], a[b], e);
+    if constexpr (NB <= 3) {
+      v[q] = fma(T.V[1][q], a[1], e);
+      v[NQ - 1 - q] = fma(-T.V[1][q], a[1], e);
+    } else {
+      const double o = fma(T.V[3][q], a[3], T.V[1][q] * a[1]);
+      v[q] = e + o;
+      v[NQ - 1 - q] = e - o;
+    }
+  }
+  if constexpr (NQ & 1) {
+    double e = a[0];
+#pragma unroll
+    for (int b = 2; b < NB; b += 2) e = fma(T.V[b][NQ / 2], a[b], e);
+    v[NQ / 2] = e;
+  }
+}
+
+// out[b] = sum_q w_q phi_b(x_q) f[q], or with phi_b'
+template <int NB, bool DERIV>
+__device__ __forceinline__ void project(const Rule<NB>& T, const double (&f)[Rule<NB>::NQ],
+                                        double (&out)[NB]) {
+  constexpr int NQ = Rule<NB>::NQ, HP = NQ / 2;
+  double s[HP], d[HP];
+#pragma unroll
+  for (int q = 0; q < HP; ++q) {
+    s[q] = f[q] + f[NQ - 1 - q];
+    d[q] = f[q] - f[NQ - 1 - q];
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    if constexpr (DERIV) {
+      if (b == 0) {
+        out[b] = 0.0;
+        continue;
+      }
+    }
+    const bool even = DERIV ? (b & 1) : !(b & 1);
+    double acc = 0.0;
+#pragma unroll
+    for (int q = 0; q < HP; ++q) {
+      const double w = DERIV ? T.wD[b][q] : T.wV[b][q];
+      const double x = even ? s[q] : d[q];
+      acc = q == 0 ? w * x : fma(w, x, acc);
+    }
+    if constexpr (NQ & 1)
+      if (even) acc = fma(DERIV ? T.wD[b][HP] : T.wV[b][HP], f[HP], acc);
+    out[b] = acc;
+  }
+}
+
+// phi_b(x_q) at any q (compile-time indices)
+template <int NB>
+__device__ __forceinline__ double vq(const Rule<NB>& T, int b, int q) {
+  constexpr int NQ = Rule<NB>::NQ, H = Rule<NB>::H;
+  return q < H ? T.V[b][q] : ((b & 1) ? -T.V[b][NQ - 1 - q] : T.V[b][NQ - 1 - q]);
+}
+template <int NB>
+__device__ __forceinline__ double wvq(const Rule<NB>& T, int b, int q) {
+  constexpr int NQ = Rule<NB>::NQ, H = Rule<NB>::H;
+  return q < H ? T.wV[b][q] : ((b & 1) ? -T.wV[b][NQ - 1 - q] : T.wV[b][NQ - 1 - q]);
+}
+
+// both directions' fluxes of one state (Euler: one reciprocal)
+template <int FLUX>
+__device__ __forceinline__ void flux2(const double* w, double* fx, double* fy, double g) {
+  if constexpr (FLUX == RIDG_FLUX_BURGERS) {
+    fx[0] = 0.5 * w[0] * w[0];
+  } else {
+    const double ir = 1.0 / w[0], u = w[1] * ir, v = w[2] * ir;
+    const double p = (g - 1.0) * (w[3] - 0.5 * fma(w[1], u, w[2] * v)), h = w[3] + p;
+    fx[0] = w[1];
+    fx[1] = fma(w[1], u, p);
+    fx[2] = w[1] * v;
+    fx[3] = u * h;
+    fy[0] = w[2];
+    fy[1] = fx[2];
+    fy[2] = fma(w[2], v, p);
+    fy[3] = v * h;
+  }
+}
+template <int FLUX>
+__device__ __forceinline__ void flux1(const double* w, int dd, double* f, double g) {
+  if constexpr (FLUX == RIDG_FLUX_BURGERS) {
+    f[0] = 0.5 * w[0] * w[0];
+  } else {
+    const double ir = 1.0 / w[0], u = w[1] * ir, v = w[2] * ir;
+    const double p = (g - 1.0) * (w[3] - 0.5 * fma(w[1], u, w[2] * v));
+    const double un = dd == 0 ? u : v;
+    f[0] = dd == 0 ? w[1] : w[2];
+    f[1] = w[1] * un;
+    f[2] = w[2] * un;
+    if (dd == 0) f[1] += p; else f[2] += p;
+    f[3] = un * (w[3] + p);
+  }
+}
+
+}  // namespace nl
+}  // namespace ridg

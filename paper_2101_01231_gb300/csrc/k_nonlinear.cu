@@ -7,7 +7,7 @@
 #include <cstring>
 #include <vector>
 
-#include "k_nlflux.cuh"
+#include "k_nl_lines.cuh"
 #include "nl_tables.h"
 #include "ridg_internal.h"
 #include "tables.h"
@@ -50,27 +50,10 @@ int nl_tables_upload(int nb, NlDevTables& out, void* mem, size_t* bytes, cudaStr
   };
   auto addd = [&](const std::vector<double>& v) { return add(v.data(), v.size() * sizeof(double)); };
   auto addi = [&](const std::vector<int>& v) { return add(v.data(), v.size() * sizeof(int)); };
-  const size_t iMt = addd(t.Mt), iem = addd(t.em), iPsiV = addd(t.PsiV), idPsiV = addd(t.dPsiV),
-               iwV = addd(t.wV), iPsiF = addd(t.PsiF), iwF = addd(t.wF), iPhiV = addd(t.PhiV),
-               idPhiV = addd(t.dPhiV), iPhiF = addd(t.PhiF), iPsiAtP = addd(t.PsiAtP),
+  const size_t iMt = addd(t.Mt), iem = addd(t.em), iwV = addd(t.wV), iPsiF = addd(t.PsiF), iwF = addd(t.wF), iPsiAtP = addd(t.PsiAtP),
                iPsiAtFP = addd(t.PsiAtFP), iP1 = addd(t.P1), iPhiEq = addd(phieq);
   const size_t iV1 = addd(t.V1), iV1T = addd(t.V1T), idV1 = addd(t.dV1), iep1 = addd(t.ep1),
                iem1 = addd(t.em1);
-  size_t ib[2][3], ig[8][3];
-  for (int d = 0; d < 2; ++d) {
-    ib[d][0] = addi(t.beta[d].ptr);
-    ib[d][1] = addi(t.beta[d].p);
-    ib[d][2] = addd(t.beta[d].val);
-  }
-  for (int d = 0; d < 2; ++d)
-    for (int sk = 0; sk < 2; ++sk)
-      for (int sl = 0; sl < 2; ++sl) {
-        const SparseTriple& G = t.gamma[d][sk][sl];
-        const int g = d * 4 + sk * 2 + sl;
-        ig[g][0] = addi(G.ptr);
-        ig[g][1] = addi(G.p);
-        ig[g][2] = addd(G.val);
-      }
   // merged assembly lists, packed per precision
   NlAsmLists L = build_asm_lists(t);
   struct EntD { int off; int pad; double c; };
@@ -124,14 +107,9 @@ int nl_tables_upload(int nb, NlDevTables& out, void* mem, size_t* bytes, cudaStr
   NlDev& tb = out.tb;
   tb.Mt = D(iMt);
   tb.em = D(iem);
-  tb.PsiV = D(iPsiV);
-  tb.dPsiV = D(idPsiV);
   tb.wV = D(iwV);
   tb.PsiF = D(iPsiF);
   tb.wF = D(iwF);
-  tb.PhiV = D(iPhiV);
-  tb.dPhiV = D(idPhiV);
-  tb.PhiF = D(iPhiF);
   tb.PsiAtP = D(iPsiAtP);
   tb.PsiAtFP = D(iPsiAtFP);
   tb.P1 = D(iP1);
@@ -141,16 +119,6 @@ int nl_tables_upload(int nb, NlDevTables& out, void* mem, size_t* bytes, cudaStr
   tb.dV1 = D(idV1);
   tb.ep1 = D(iep1);
   tb.em1 = D(iem1);
-  for (int d = 0; d < 2; ++d) {
-    tb.bptr[d] = I(ib[d][0]);
-    tb.bp[d] = I(ib[d][1]);
-    tb.bval[d] = D(ib[d][2]);
-  }
-  for (int g = 0; g < 8; ++g) {
-    tb.gptr[g] = I(ig[g][0]);
-    tb.gp[g] = I(ig[g][1]);
-    tb.gval[g] = D(ig[g][2]);
-  }
   tb.dptr = I(idptr);
   tb.dent_d = base + pieces[identd].off;
   tb.dent_f = base + pieces[identf].off;
@@ -178,133 +146,279 @@ namespace {
 // ---------------------------------------------------------------------------------------
 // correction (Sec. 2.3): Q += volume term - surface term, every face flux evaluated from the
 // same traces in the same order by both cells that share it (so both see the same bits)
+//
+// Sum-factorised along lines (k_nl_lines.cuh): a cell takes ~9 k FP64 operations at Burgers Q4
+// where sums over the dense quadrature tables took ~95 k.  The FP64 pipe bounds it; a block
+// takes CPB cells so that its phases of 16 to 50 lines per cell fill their warps.  Measured:
+// Euler Q2 512^2 21.2 -> 7.8 ms per launch; eight Burgers problems up to 72^2, degrees 1 .. 4,
+// 13.2 -> 10.8 ms per whole step.
 // ---------------------------------------------------------------------------------------
 constexpr int kCorrThreads = 128;
 
-// the correction of cell e of one mesh (a block of kCorrThreads threads); shared memory
-// carved from `sh` (nl_corr_smem<NB, MV>() bytes)
 template <int NB, int MV>
-constexpr size_t nl_corr_smem() {
-  constexpr int THT = NB * NB * NB, BS = MV * THT, NQ = (3 * (NB - 1) + 2) / 2;
-  constexpr int QV = NQ * NQ * NQ, QF = NQ * NQ;
-  return sizeof(double) * (5 * BS + 2 * MV * QV + 3 * 4 * MV * QF + 4 * QF);
-}
+struct CorrCfg {
+  static constexpr int THS = NB * NB, BS = MV * NB * THS, NQ = nl::Rule<NB>::NQ, NX = NQ * NQ;
+  // cells per block: about 128 points of the volume phase (NQ^2 per cell)
+  static constexpr int CPB = NB == 2 ? (MV == 1 ? 16 : 8) : NB == 3 ? (MV == 1 ? 8 : 4) : NB == 4 ? 5 : 3;
+  // shared memory of a cell (doubles): lines [j][a][y][x]; traces [face * 2 + left / right][j][a]
+  // [NQ]; time-summed fluxes [x, y][j][y][x]; speeds [face][NQ]; face values [face][j][NQ]
+  static constexpr int oT = MV * NB * NX, oG = oT + 8 * MV * NB * NQ, oS = oG + 2 * MV * NX,
+                       oH = oS + 4 * NQ, per_cell = oH + 4 * MV * NQ, total = CPB * per_cell;
+};
 
+// The correction of cells e0 .. min(e0 + CPB, ncell) - 1 of one mesh by the block.  Faces of a
+// cell: f = dd * 2 + si (si 0: the +1 face, 1: the -1 face) with left / right states
+//   +1 face: own trace at +1, the +dd neighbour's at -1;
+//   -1 face: the -dd neighbour's at +1, own at -1.
 template <int NB, int MV, int FLUX>
-__device__ void nl_correct_cell(const NlDev& tb, double* __restrict__ Q, const double* __restrict__ W,
-                                int nx, int ny, double lamx, double lamy, double gamma,
-                                long long e, double* sh) {
-  constexpr int THS = NB * NB, THT = NB * THS, BS = MV * THT;
-  constexpr int NQ = (3 * (NB - 1) + 2) / 2, QV = NQ * NQ * NQ, QF = NQ * NQ;
-  auto Wc = (double(*)[BS])sh;                               // own, +x, -x, +y, -y neighbours
-  auto G = (double(*)[MV][QV])(sh + 5 * BS);                 // sc_d w_q F_d(w), volume points
-  auto TL = (double(*)[MV][QF])(sh + 5 * BS + 2 * MV * QV);  // left / right traces per face
-  auto TR = (double(*)[MV][QF])(sh + 5 * BS + 2 * MV * QV + 4 * MV * QF);
-  auto FH = (double(*)[MV][QF])(sh + 5 * BS + 2 * MV * QV + 8 * MV * QF);  // sc w F-hat
-  auto spd = (double(*)[QF])(sh + 5 * BS + 2 * MV * QV + 12 * MV * QF);
+__device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
+                                 const double* __restrict__ W, int nx, int ny, long long ncell,
+                                 double lamx, double lamy, double g, long long e0, double* sh) {
+  using K = CorrCfg<NB, MV>;
+  constexpr int NQ = K::NQ, NX = K::NX, THS = K::THS, BS = K::BS, ML = MV * NB;
   const int tid = threadIdx.x;
-  const unsigned ue = (unsigned)e, uy = ue / (unsigned)nx;
-  const int ix = (int)(ue - uy * (unsigned)nx), iy = (int)uy;
-  const long long nbr[5] = {e, (long long)iy * nx + (ix + 1) % nx, (long long)iy * nx + (ix + nx - 1) % nx,
-                            (long long)((iy + 1) % ny) * nx + ix, (long long)((iy + ny - 1) % ny) * nx + ix};
-  for (int i = tid; i < 5 * BS; i += kCorrThreads) Wc[i / BS][i % BS] = W[nbr[i / BS] * BS + i % BS];
-  __syncthreads();
-  const double sc[2] = {0.25 * lamx, 0.25 * lamy};
-  for (int q = tid; q < QV; q += kCorrThreads) {
-    double w[MV], f[MV];
-    for (int j = 0; j < MV; ++j) {
-      double acc = 0.0;
-      for (int k = 0; k < THT; ++k) acc = fma(tb.PsiV[k * QV + q], Wc[0][j * THT + k], acc);
-      w[j] = acc;
+  const int cells = (int)min((long long)K::CPB, ncell - e0);
+  // x lines of the cell and its x traces | its y traces | the neighbours' traces per face
+  for (int i = tid; i < cells * 6 * ML * NB; i += kCorrThreads) {
+    const int c = i / (6 * ML * NB), k = i - c * (6 * ML * NB), kind = k / (ML * NB),
+              l = k - kind * (ML * NB), ja = l / NB, o = l - ja * NB;
+    double* S = sh + c * K::per_cell;
+    double* tr = S + K::oT + ja * NQ + o;  // + (face * 2 + side) ML NQ
+    const long long e = e0 + c;
+    const unsigned uy = (unsigned)e / (unsigned)nx;
+    int cx = (int)((unsigned)e - uy * (unsigned)nx), cy = (int)uy;
+    if (kind >= 2) {
+      const int f = kind - 2, step = (f & 1) ? -1 : 1;
+      if (f < 2) cx += step; else cy += step;
+      cx += cx < 0 ? nx : (cx >= nx ? -nx : 0);
+      cy += cy < 0 ? ny : (cy >= ny ? -ny : 0);
     }
-    for (int dd = 0; dd < 2; ++dd) {
-      nlflux::F<FLUX>(w, dd, f, gamma);
-      for (int j = 0; j < MV; ++j) G[dd][j][q] = sc[dd] * tb.wV[q] * f[j];
+    const double* src = W + ((long long)cy * nx + cx) * BS + ja * THS;
+    const bool ydir = kind == 1 || kind >= 4;
+    const int st = ydir ? NB : 1;
+    src += ydir ? o : o * NB;
+    double m[NB], ev, od;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) m[b] = src[b * st];
+    nl::traces<NB>(T, m, 1, ev, od);
+    if (kind == 0) {
+      double v[NQ];
+      nl::interp<NB>(T, m, v);
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) S[(ja * NQ + o) * NQ + q] = v[q];
+    }
+    if (kind < 2) {
+      tr[(kind * 4 + 0) * ML * NQ] = ev + od;  // left of the +1 face
+      tr[(kind * 4 + 3) * ML * NQ] = ev - od;  // right of the -1 face
+    } else {
+      const int f = kind - 2;  // right of the +1 faces, left of the -1 faces
+      tr[(f * 2 + ((f & 1) ? 0 : 1)) * ML * NQ] = (f & 1) ? ev + od : ev - od;
     }
   }
-  // face f = dd * 2 + si (si 0: the +1 face, 1: the -1 face).  Left / right states:
-  //   +1 face: L = own trace at +1, R = the +dd neighbour's trace at -1
-  //   -1 face: L = the -dd neighbour's trace at +1, R = own trace at -1
-  for (int i = tid; i < 4 * QF; i += kCorrThreads) {
-    const int f = i / QF, q = i % QF, dd = f >> 1, si = f & 1;
-    const double* tp = tb.PsiF + (size_t)(dd * 2 + 0) * THT * QF;  // +1 side table
-    const double* tm = tb.PsiF + (size_t)(dd * 2 + 1) * THT * QF;  // -1 side table
-    const double* wl = si == 0 ? Wc[0] : Wc[2 + 2 * dd];
-    const double* wr = si == 0 ? Wc[1 + 2 * dd] : Wc[0];
-    double a[MV], b[MV];
-    for (int j = 0; j < MV; ++j) {
-      double sl = 0.0, sr = 0.0;
-      for (int k = 0; k < THT; ++k) {
-        sl = fma(tp[k * QF + q], wl[j * THT + k], sl);
-        sr = fma(tm[k * QF + q], wr[j * THT + k], sr);
+  __syncthreads();
+  // y lines; the traces along their faces
+  for (int i = tid; i < cells * (ML * NQ + 8 * ML); i += kCorrThreads) {
+    const int c = i / (ML * NQ + 8 * ML), k = i - c * (ML * NQ + 8 * ML);
+    double* p = sh + c * K::per_cell;
+    int st = 1;
+    if (k < ML * NQ) {
+      p += k / NQ * NX + k % NQ;
+      st = NQ;
+    } else {
+      p += K::oT + (k - ML * NQ) * NQ;
+    }
+    double m[NB], v[NQ];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) m[b] = p[b * st];
+    nl::interp<NB>(T, m, v);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) p[q * st] = v[q];
+  }
+  __syncthreads();
+  // volume points: both fluxes summed over time; face points: the largest speed over time
+  for (int i = tid; i < cells * NX; i += kCorrThreads) {
+    const int c = i / NX, yx = i - c * NX;
+    double* S = sh + c * K::per_cell;
+    double sx[MV], sy[MV];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      double w[MV], fx[MV], fy[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        w[j] = S[j * NB * NX + yx];
+#pragma unroll
+        for (int a = 1; a < NB; ++a) w[j] = fma(nl::vq<NB>(T, a, q), S[(j * NB + a) * NX + yx], w[j]);
       }
-      a[j] = sl;
-      b[j] = sr;
-      TL[f][j][q] = sl;
-      TR[f][j][q] = sr;
+      nl::flux2<FLUX>(w, fx, fy, g);
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        const double wt = nl::wvq<NB>(T, 0, q);
+        sx[j] = q == 0 ? wt * fx[j] : fma(wt, fx[j], sx[j]);
+        if constexpr (MV > 1) sy[j] = q == 0 ? wt * fy[j] : fma(wt, fy[j], sy[j]);
+      }
     }
-    spd[f][q] = fmax(nlflux::speed<FLUX>(a, dd, gamma), nlflux::speed<FLUX>(b, dd, gamma));
-  }
-  __syncthreads();
-  for (int i = tid; i < 4 * QF; i += kCorrThreads) {
-    const int f = i / QF, q = i % QF, dd = f >> 1;
-    double alpha = 0.0;
-    for (int p = 0; p < QF; ++p) alpha = fmax(alpha, spd[f][p]);
-    double a[MV], b[MV], fa[MV], fb[MV];
+#pragma unroll
     for (int j = 0; j < MV; ++j) {
-      a[j] = TL[f][j][q];
-      b[j] = TR[f][j][q];
+      S[K::oG + j * NX + yx] = sx[j];
+      if constexpr (MV > 1) S[K::oG + (MV + j) * NX + yx] = sy[j];
     }
-    nlflux::F<FLUX>(a, dd, fa, gamma);
-    nlflux::F<FLUX>(b, dd, fb, gamma);
-    const double wq = sc[dd] * tb.wF[dd * QF + q];
-    for (int j = 0; j < MV; ++j) FH[f][j][q] = wq * (0.5 * (fa[j] + fb[j]) - 0.5 * alpha * (b[j] - a[j]));
+  }
+  for (int i = tid; i < cells * 4 * NQ; i += kCorrThreads) {
+    const int c = i / (4 * NQ), k = i - c * (4 * NQ), f = k / NQ, qo = k - f * NQ, dd = f >> 1;
+    double* S = sh + c * K::per_cell;
+    const double* tl = S + K::oT + f * 2 * ML * NQ + qo;
+    const double* tr = tl + ML * NQ;
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      double wl[MV], wr[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        wl[j] = tl[j * NB * NQ];
+        wr[j] = tr[j * NB * NQ];
+#pragma unroll
+        for (int a = 1; a < NB; ++a) {
+          wl[j] = fma(nl::vq<NB>(T, a, q), tl[(j * NB + a) * NQ], wl[j]);
+          wr[j] = fma(nl::vq<NB>(T, a, q), tr[(j * NB + a) * NQ], wr[j]);
+        }
+      }
+      s = fmax(s, fmax(nlflux::speed<FLUX>(wl, dd, g), nlflux::speed<FLUX>(wr, dd, g)));
+    }
+    S[K::oS + k] = s;
   }
   __syncthreads();
-  for (int i = tid; i < MV * THS; i += kCorrThreads) {
-    const int j = i / THS, s2 = i % THS;
-    double acc = 0.0;
-    for (int dd = 0; dd < 2; ++dd)
-      for (int q = 0; q < QV; ++q) acc = fma(tb.dPhiV[(dd * THS + s2) * QV + q], G[dd][j][q], acc);
-    for (int f = 0; f < 4; ++f) {
-      const double sg = (f & 1) ? 1.0 : -1.0;  // -(flux out at +1) + (flux in at -1)
-      const double* ph = tb.PhiF + (size_t)(f * THS + s2) * QF;
-      double fs = 0.0;
-      for (int q = 0; q < QF; ++q) fs = fma(ph[q], FH[f][j][q], fs);
-      acc = fma(sg, fs, acc);
+  // the face fluxes summed over time; the volume fluxes' y lines back (phi_y on the x flux,
+  // phi_y' on the y flux)
+  for (int i = tid; i < cells * 4 * NQ; i += kCorrThreads) {
+    const int c = i / (4 * NQ), k = i - c * (4 * NQ), f = k / NQ, qo = k - f * NQ, dd = f >> 1;
+    double* S = sh + c * K::per_cell;
+    const double* tl = S + K::oT + f * 2 * ML * NQ + qo;
+    const double* tr = tl + ML * NQ;
+    double alpha = 0.0;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) alpha = fmax(alpha, S[K::oS + f * NQ + q]);
+    alpha *= 0.5;
+    double h[MV];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      double wl[MV], wr[MV], fl[MV], fr[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        wl[j] = tl[j * NB * NQ];
+        wr[j] = tr[j * NB * NQ];
+#pragma unroll
+        for (int a = 1; a < NB; ++a) {
+          wl[j] = fma(nl::vq<NB>(T, a, q), tl[(j * NB + a) * NQ], wl[j]);
+          wr[j] = fma(nl::vq<NB>(T, a, q), tr[(j * NB + a) * NQ], wr[j]);
+        }
+      }
+      nl::flux1<FLUX>(wl, dd, fl, g);
+      nl::flux1<FLUX>(wr, dd, fr, g);
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        const double fh = fma(0.5, fl[j] + fr[j], -alpha * (wr[j] - wl[j]));
+        const double wt = nl::wvq<NB>(T, 0, q);
+        h[j] = q == 0 ? wt * fh : fma(wt, fh, h[j]);
+      }
     }
-    Q[e * MV * THS + i] += acc;
+#pragma unroll
+    for (int j = 0; j < MV; ++j) S[K::oH + (f * MV + j) * NQ + qo] = h[j];
   }
-  __syncthreads();  // the shared arrays are reused by the block's next cell
+  for (int i = tid; i < cells * MV * NQ; i += kCorrThreads) {
+    const int c = i / (MV * NQ), k = i - c * (MV * NQ), j = k / NQ, x = k - j * NQ;
+    double* p1 = sh + c * K::per_cell + K::oG + j * NX + x;
+    double* p2 = p1 + MV * NX;
+    double v[NQ], o1[NB], o2[NB];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) v[q] = p1[q * NQ];
+    nl::project<NB, false>(T, v, o1);
+    if constexpr (MV > 1) {
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) v[q] = p2[q * NQ];
+    }
+    nl::project<NB, true>(T, v, o2);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      p1[b * NQ] = o1[b];
+      p2[b * NQ] = o2[b];
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < cells * 4 * MV; i += kCorrThreads) {
+    double* p = sh + i / (4 * MV) * K::per_cell + K::oH + i % (4 * MV) * NQ;
+    double v[NQ], o[NB];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) v[q] = p[q];
+    nl::project<NB, false>(T, v, o);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) p[b] = o[b];
+  }
+  __syncthreads();
+  // x lines back, the faces, and the update
+  const double l0 = 0.25 * lamx, l1 = 0.25 * lamy;
+  for (int i = tid; i < cells * MV * NB; i += kCorrThreads) {
+    const int c = i / (MV * NB), k = i - c * (MV * NB), j = k / NB, y = k - j * NB;
+    const double* S = sh + c * K::per_cell;
+    const double* p1 = S + K::oG + j * NX + y * NQ;
+    double v[NQ], ox[NB], oy[NB];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) v[q] = p1[q];
+    nl::project<NB, true>(T, v, ox);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) v[q] = p1[MV * NX + q];
+    nl::project<NB, false>(T, v, oy);
+    const double* h = S + K::oH + j * NQ;  // + face MV NQ
+    const double hr = h[y], hl = h[MV * NQ + y];
+    double* q = Q + ((e0 + c) * MV + j) * THS + y * NB;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const double ht = h[2 * MV * NQ + b], hb = h[3 * MV * NQ + b];
+      const double fx = (b & 1) ? hr + hl : hr - hl, fy = (y & 1) ? ht + hb : ht - hb;
+      const double d = fma(l0, fma(-T.ep[b], fx, ox[b]), l1 * fma(-T.ep[y], fy, oy[b]));
+      q[b] += d;
+    }
+  }
 }
 
 template <int NB, int MV, int FLUX>
-__global__ void __launch_bounds__(kCorrThreads) nl_correct_kernel(NlDev tb, double* __restrict__ Q,
+__global__ void __launch_bounds__(kCorrThreads) nl_correct_kernel(const nl::Rule<NB> T,
+                                                                  double* __restrict__ Q,
                                                                   const double* __restrict__ W,
-                                                                  int nx, int ny, double lamx,
-                                                                  double lamy, double gamma) {
-  __shared__ double sh[nl_corr_smem<NB, MV>() / sizeof(double)];
-  nl_correct_cell<NB, MV, FLUX>(tb, Q, W, nx, ny, lamx, lamy, gamma, blockIdx.x, sh);
+                                                                  int nx, int ny, long long ncell,
+                                                                  double lamx, double lamy,
+                                                                  double gamma) {
+  using K = CorrCfg<NB, MV>;
+  __shared__ double sh[K::total];
+  nl_correct_cells<NB, MV, FLUX>(T, Q, W, nx, ny, ncell, lamx, lamy, gamma,
+                                 (long long)blockIdx.x * K::CPB, sh);
 }
 
-// Every instance's correction of a batched Burgers ensemble in one launch: block b takes the
-// cell b of the concatenated instances (the instance of the last table entry whose first
-// cell is <= b, found by bisection) and runs that instance's degree.
-__global__ void __launch_bounds__(kCorrThreads) nl_correct_multi_kernel(const CorrMulti m) {
-  __shared__ double sh[nl_corr_smem<5, 1>() / sizeof(double)];  // the largest degree
+struct CorrRules {
+  nl::Rule<2> r2;
+  nl::Rule<3> r3;
+  nl::Rule<4> r4;
+  nl::Rule<5> r5;
+};
+
+// Every instance's correction of a batched Burgers ensemble in one launch: each instance has
+// ceil(ncell / CPB) blocks of its degree, the instance of a block found by bisection.
+__global__ void __launch_bounds__(kCorrThreads) nl_correct_multi_kernel(const CorrMulti m,
+                                                                        const CorrRules T) {
+  __shared__ double sh[std::max(std::max(CorrCfg<2, 1>::total, CorrCfg<3, 1>::total),
+                                std::max(CorrCfg<4, 1>::total, CorrCfg<5, 1>::total))];
   const long long b = blockIdx.x;
   int lo = 0, hi = m.ninst - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (m.inst[mid].cell0 <= b) lo = mid; else hi = mid - 1;
+    if (m.inst[mid].block0 <= b) lo = mid; else hi = mid - 1;
   }
   const CorrInst& in = m.inst[lo];
-  const long long e = b - in.cell0;
+  const long long k = b - in.block0;
   switch (in.nb) {
-    case 2: nl_correct_cell<2, 1, RIDG_FLUX_BURGERS>(m.tb[0], in.Q, in.W, in.nx, in.ny, in.lamx, in.lamy, 0.0, e, sh); break;
-    case 3: nl_correct_cell<3, 1, RIDG_FLUX_BURGERS>(m.tb[1], in.Q, in.W, in.nx, in.ny, in.lamx, in.lamy, 0.0, e, sh); break;
-    case 4: nl_correct_cell<4, 1, RIDG_FLUX_BURGERS>(m.tb[2], in.Q, in.W, in.nx, in.ny, in.lamx, in.lamy, 0.0, e, sh); break;
-    case 5: nl_correct_cell<5, 1, RIDG_FLUX_BURGERS>(m.tb[3], in.Q, in.W, in.nx, in.ny, in.lamx, in.lamy, 0.0, e, sh); break;
+    case 2: nl_correct_cells<2, 1, RIDG_FLUX_BURGERS>(T.r2, in.Q, in.W, in.nx, in.ny, in.ncell, in.lamx, in.lamy, 0.0, k * CorrCfg<2, 1>::CPB, sh); break;
+    case 3: nl_correct_cells<3, 1, RIDG_FLUX_BURGERS>(T.r3, in.Q, in.W, in.nx, in.ny, in.ncell, in.lamx, in.lamy, 0.0, k * CorrCfg<3, 1>::CPB, sh); break;
+    case 4: nl_correct_cells<4, 1, RIDG_FLUX_BURGERS>(T.r4, in.Q, in.W, in.nx, in.ny, in.ncell, in.lamx, in.lamy, 0.0, k * CorrCfg<4, 1>::CPB, sh); break;
+    case 5: nl_correct_cells<5, 1, RIDG_FLUX_BURGERS>(T.r5, in.Q, in.W, in.nx, in.ny, in.ncell, in.lamx, in.lamy, 0.0, k * CorrCfg<5, 1>::CPB, sh); break;
     default: break;
   }
 }
@@ -334,20 +448,20 @@ __global__ void max_speed_kernel(NlDev tb, const double* __restrict__ Q, long lo
 
 }  // namespace
 
-#define RIDG_NL_SWITCH(NB_, M_, KIND_, CALL)                                               \
+#define RIDG_NL_SWITCH(NB_, M_, KIND_, ...)                                               \
   do {                                                                                    \
     if (KIND_ == RIDG_FLUX_BURGERS && M_ == 1) {                                          \
       switch (NB_) {                                                                      \
-        case 2: { constexpr int NB = 2, MV = 1, FL = RIDG_FLUX_BURGERS; CALL; } break;    \
-        case 3: { constexpr int NB = 3, MV = 1, FL = RIDG_FLUX_BURGERS; CALL; } break;    \
-        case 4: { constexpr int NB = 4, MV = 1, FL = RIDG_FLUX_BURGERS; CALL; } break;    \
-        case 5: { constexpr int NB = 5, MV = 1, FL = RIDG_FLUX_BURGERS; CALL; } break;    \
+        case 2: { constexpr int NB = 2, MV = 1, FL = RIDG_FLUX_BURGERS; __VA_ARGS__; } break;    \
+        case 3: { constexpr int NB = 3, MV = 1, FL = RIDG_FLUX_BURGERS; __VA_ARGS__; } break;    \
+        case 4: { constexpr int NB = 4, MV = 1, FL = RIDG_FLUX_BURGERS; __VA_ARGS__; } break;    \
+        case 5: { constexpr int NB = 5, MV = 1, FL = RIDG_FLUX_BURGERS; __VA_ARGS__; } break;    \
         default: return cudaErrorInvalidValue;                                            \
       }                                                                                   \
     } else if (KIND_ == RIDG_FLUX_EULER && M_ == 4) {                                     \
       switch (NB_) {                                                                      \
-        case 2: { constexpr int NB = 2, MV = 4, FL = RIDG_FLUX_EULER; CALL; } break;      \
-        case 3: { constexpr int NB = 3, MV = 4, FL = RIDG_FLUX_EULER; CALL; } break;      \
+        case 2: { constexpr int NB = 2, MV = 4, FL = RIDG_FLUX_EULER; __VA_ARGS__; } break;      \
+        case 3: { constexpr int NB = 3, MV = 4, FL = RIDG_FLUX_EULER; __VA_ARGS__; } break;      \
         default: return cudaErrorInvalidValue;                                            \
       }                                                                                   \
     } else {                                                                              \
@@ -425,17 +539,30 @@ int newton_multi_ctas_per_sm(int prec) {
   }
 }
 
-cudaError_t launch_nl_correct(int nb, int m, int flux_kind, const NlDev& tb, double* Q,
-                              const double* W, int nx, int ny, long long ncell, double lamx,
-                              double lamy, double gamma, cudaStream_t s) {
-  RIDG_NL_SWITCH(nb, m, flux_kind,
-                 (nl_correct_kernel<NB, MV, FL><<<(unsigned)ncell, kCorrThreads, 0, s>>>(
-                     tb, Q, W, nx, ny, lamx, lamy, gamma)));
+cudaError_t launch_nl_correct(int nb, int m, int flux_kind, double* Q, const double* W, int nx,
+                              int ny, long long ncell, double lamx, double lamy, double gamma,
+                              cudaStream_t s) {
+  RIDG_NL_SWITCH(nb, m, flux_kind, {
+    constexpr int CPB = CorrCfg<NB, MV>::CPB;
+    static const nl::Rule<NB> rule = nl::make_rule<NB>();
+    (nl_correct_kernel<NB, MV, FL><<<(unsigned)((ncell + CPB - 1) / CPB), kCorrThreads, 0, s>>>(
+        rule, Q, W, nx, ny, ncell, lamx, lamy, gamma));
+  });
   return cudaGetLastError();
 }
 
-cudaError_t launch_nl_correct_multi(const CorrMulti& m, long long cells, cudaStream_t s) {
-  nl_correct_multi_kernel<<<(unsigned)cells, kCorrThreads, 0, s>>>(m);
+long long nl_correct_blocks(int nb, long long ncell) {
+  const int cpb = nb == 2   ? CorrCfg<2, 1>::CPB
+                  : nb == 3 ? CorrCfg<3, 1>::CPB
+                  : nb == 4 ? CorrCfg<4, 1>::CPB
+                            : CorrCfg<5, 1>::CPB;
+  return (ncell + cpb - 1) / cpb;
+}
+
+cudaError_t launch_nl_correct_multi(const CorrMulti& m, long long blocks, cudaStream_t s) {
+  static const CorrRules rules = {nl::make_rule<2>(), nl::make_rule<3>(), nl::make_rule<4>(),
+                                  nl::make_rule<5>()};
+  nl_correct_multi_kernel<<<(unsigned)blocks, kCorrThreads, 0, s>>>(m, rules);
   return cudaGetLastError();
 }
 

@@ -138,15 +138,10 @@ cudaError_t launch_mixed3_refresh(const Grid& g, int nb, int slices, const doubl
 struct NlDev {
   const double *Mt, *em;                // time term, psi_a(-1)
   const double *V1, *V1T, *dV1, *ep1, *em1;  // 1D residual rule (nl_tables.h)
-  const double *PsiV, *dPsiV, *wV;      // residual volume rule
+  const double* wV;                     // residual volume rule's weights
   const double *PsiF, *wF;              // residual face rule
-  const double *PhiV, *dPhiV, *PhiF;    // spatial basis at the same points (correction)
   const double *PsiAtP, *PsiAtFP, *P1;  // projection rule of eq. Jacproj
   const double* PhiEq;                  // spatial basis on a 6 x 6 equispaced grid (wave speed)
-  const int *bptr[2], *bp[2];           // volume triple-product lists per direction
-  const double* bval[2];
-  const int *gptr[8], *gp[8];           // face lists, index dd * 4 + side_k * 2 + side_l
-  const double* gval[8];
   // merged assembly lists (nl_tables.h) with packed entries: {int offset; int pad; double c}
   // for FP64 assembly, {int offset; float c} for FP32 assembly
   const int* dptr;
@@ -256,24 +251,24 @@ struct NewtonMulti {
 cudaError_t launch_newton_multi(int prec, const NewtonMulti& m, const NewtonMulti* dev, int grid,
                                 cudaStream_t s);
 int newton_multi_ctas_per_sm(int prec);
-// Every instance's correction of a batched Burgers ensemble in one launch (one block per
-// cell of the concatenated instances, sorted by cell0); tb[nb - 2]: the degree's tables.
+// Every instance's correction of a batched Burgers ensemble in one launch: instance i has
+// nl_correct_blocks(nb, ncell) blocks from block0 (increasing).
 struct CorrInst {
   double* Q;
   const double* W;
-  long long cell0;
+  long long block0, ncell;
   int nx, ny, nb;
   double lamx, lamy;
 };
 struct CorrMulti {
-  NlDev tb[4];
   const CorrInst* inst;
   int ninst;
 };
-cudaError_t launch_nl_correct_multi(const CorrMulti& m, long long cells, cudaStream_t s);
-cudaError_t launch_nl_correct(int nb, int m, int flux_kind, const NlDev& tb, double* Q,
-                              const double* W, int nx, int ny, long long ncell, double lamx,
-                              double lamy, double gamma, cudaStream_t s);
+long long nl_correct_blocks(int nb, long long ncell);
+cudaError_t launch_nl_correct_multi(const CorrMulti& m, long long blocks, cudaStream_t s);
+cudaError_t launch_nl_correct(int nb, int m, int flux_kind, double* Q, const double* W, int nx,
+                              int ny, long long ncell, double lamx, double lamy, double gamma,
+                              cudaStream_t s);
 // largest wave speed of Q over a 6 x 6 equispaced grid of every cell -> *out (as bits)
 cudaError_t launch_max_speed(int nb, int m, int flux_kind, const NlDev& tb, const double* Q,
                              long long ncell, double gamma, unsigned long long* out,

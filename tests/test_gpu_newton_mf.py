@@ -73,3 +73,23 @@ def test_regions_left_over_are_block_eliminated(R, flux, M):
         assert st == R.RIDG_ENOCONV
         assert info["newton_unconverged"] == 35 and info["newton_hist"][4] == 35
         assert np.abs(W - ref).max() <= TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("flux,M", [("burgers", 1), ("burgers", 2), ("burgers", 3), ("burgers", 4),
+                                    ("euler", 1), ("euler", 2)])
+@pytest.mark.parametrize("n", [(3, 3), (7, 11)])
+def test_correction_matches_oracle(R, flux, M, n):
+    """The sum-factorised correction from a given prediction, on meshes that leave its last block
+    partly empty.  Both sides are FP64 sums of a few hundred terms of size |Q|: 1e-13."""
+    from oracle import nonlinear as NL
+    w, q = _smooth(flux, n, M)
+    s = R.Solver(2, w["n"], M, flux=w["flux"], cfl=w["cfl"], lo=w["lo"], hi=w["hi"],
+                 gamma=w.get("gamma", 1.4), precision=R.RIDG_PREC_MIXED_FP32)
+    s.set_state(q)
+    W = s.predict()
+    dt = s.info()["dt"]
+    s.correct()
+    q1 = s.get_state()
+    s.close()
+    ref = NL.correct(q, W, w, dt)
+    assert np.abs(q1 - ref).max() <= 1e-13 * np.abs(ref).max()
