@@ -75,7 +75,9 @@ typedef struct {
 } ridg_flux;
 
 enum {
-  RIDG_PREC_FP64 = 0,        /* every step of the path in FP64                           */
+  RIDG_PREC_FP64 = 0,        /* every step of the path to FP64 accuracy (2D Newton: each
+                                linear system by FP32 iterations refined against its FP64
+                                residual down to round-off, or FP64 block elimination)    */
   RIDG_PREC_MIXED_BF16 = 1,  /* linear prediction as a sliced BF16 tensor-core contraction
                                 with FP32 accumulation recombined into double-float pairs
                                 (split-operand refinement); in the step the contraction

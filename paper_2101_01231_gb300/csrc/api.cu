@@ -339,6 +339,7 @@ cudaError_t enqueue_newton_mf(const ridg_t* h, ridg::NewtonArgs& a, int* list, c
   f.lam[0] = a.lam[0];
   f.lam[1] = a.lam[1];
   f.gamma = a.gamma;
+  f.fp64 = newton_prec(h) == ridg::kNewtonF64;
   f.max_iters = a.max_iters;
   f.tol = a.tol;
   f.stats = a.stats;
@@ -373,7 +374,7 @@ int enqueue_newton(ridg_t* h) {
   a.counter = h->nl_words;
   a.stats = h->nl_words + 1;
   a.iters_total = (unsigned long long*)(h->nl_words + 6);
-  if (h->nl_list) RIDG_CUDA(h, enqueue_newton_mf(h, a, h->nl_list, h->stream));
+  RIDG_CUDA(h, enqueue_newton_mf(h, a, h->nl_list, h->stream));
   RIDG_CUDA(h, ridg::launch_newton(h->nb, h->m, h->flux.kind, newton_prec(h), a, h->nl_grid,
                                    h->stream));
   return RIDG_OK;
@@ -649,9 +650,8 @@ int ridg_create(const ridg_mesh* mesh, int order, const ridg_flux* flux, double 
     const size_t scratch = h->nl_scratch_cta * (size_t)h->nl_grid_max;
     h->nl_scratch = h->nl_grid_max > 0 ? dev_alloc(h, scratch) : nullptr;
     h->nl_words = (int*)dev_alloc(h, 24 * sizeof(int));
-    const bool mixed = newton_prec(h) != ridg::kNewtonF64;
-    if (mixed) h->nl_list = (int*)dev_alloc(h, ((size_t)h->ncell + 1) * sizeof(int));
-    if (!tb_mem || !h->nl_scratch || !h->nl_words || (mixed && !h->nl_list)) {
+    h->nl_list = (int*)dev_alloc(h, ((size_t)h->ncell + 1) * sizeof(int));
+    if (!tb_mem || !h->nl_scratch || !h->nl_words || !h->nl_list) {
       dev_free(h, tb_mem);
       ridg_destroy(h);
       return RIDG_ENOMEM;
@@ -1183,7 +1183,7 @@ struct NlGroup {
   std::vector<ridg::NlInst> host;      // the table, refreshed before every batch launch
   ridg::NlInst* table = nullptr;       // device copy
   int* counter = nullptr;              // region counter of the group's launch
-  int* list = nullptr;                 // mixed: as ridg_handle::nl_list, over the group's regions
+  int* list = nullptr;                 // as ridg_handle::nl_list, over the group's regions
   long long regions = 0;
   size_t scratch_off = 0;              // the degree's block storage in the batch's
 };
@@ -1283,10 +1283,8 @@ ridg::NewtonArgs group_args(ridg_batch_t* b, const NlGroup& g) {
   a.iters_total = (unsigned long long*)(h->nl_words + 6);
   a.inst = g.table;
   a.ninst = (int)g.idx.size();
-  if (g.list) {
-    a.list_count = g.list;
-    a.list = g.list + 1;
-  }
+  a.list_count = g.list;
+  a.list = g.list + 1;
   return a;
 }
 
@@ -1294,7 +1292,7 @@ ridg::NewtonArgs group_args(ridg_batch_t* b, const NlGroup& g) {
 int enqueue_newton_group(ridg_batch_t* b, const NlGroup& g) {
   ridg_t* h = b->inst[g.idx[0]];
   ridg::NewtonArgs a = group_args(b, g);
-  if (g.list) RIDG_CUDA(h, enqueue_newton_mf(h, a, g.list, b->stream));
+  RIDG_CUDA(h, enqueue_newton_mf(h, a, g.list, b->stream));
   RIDG_CUDA(h, ridg::launch_newton(h->nb, h->m, h->flux.kind, newton_prec(h), a, h->nl_grid,
                                    b->stream));
   return RIDG_OK;
@@ -1325,7 +1323,6 @@ int enqueue_batch_multi(ridg_batch_t* b) {
   ridg_t* h0 = b->inst[0];
   const int grid = ridg::newton_multi_ctas_per_sm(newton_prec(h0)) * sm_count();
   for (const NlGroup& g : b->groups) {
-    if (!g.list) continue;
     ridg_t* h = b->inst[g.idx[0]];
     ridg::NewtonArgs a = group_args(b, g);
     RIDG_CUDA(h, enqueue_newton_mf(h, a, g.list, b->stream));
@@ -1416,13 +1413,10 @@ int ridg_batch_create(int count, const ridg_mesh* meshes, const int* orders, con
       g.host.resize(g.idx.size());
       g.table = (ridg::NlInst*)dev_alloc(b->inst[0], g.idx.size() * sizeof(ridg::NlInst));
       g.counter = (int*)dev_alloc(b->inst[0], 4 * sizeof(int));
-      const bool mixed = newton_prec(b->inst[0]) != ridg::kNewtonF64;
-      if (mixed) {
-        size_t regions = 0;
-        for (int i : g.idx) regions += (size_t)b->inst[i]->ncell;
-        g.list = (int*)dev_alloc(b->inst[0], (regions + 1) * sizeof(int));
-      }
-      if (!g.table || !g.counter || (mixed && !g.list)) {
+      size_t regions = 0;
+      for (int i : g.idx) regions += (size_t)b->inst[i]->ncell;
+      g.list = (int*)dev_alloc(b->inst[0], (regions + 1) * sizeof(int));
+      if (!g.table || !g.counter || !g.list) {
         ridg_batch_destroy(b);
         return RIDG_ENOMEM;
       }

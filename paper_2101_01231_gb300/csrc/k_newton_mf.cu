@@ -8,12 +8,12 @@
 namespace ridg {
 namespace nl {
 
-template <int NB>
-Rule<NB> make_rule() {
-  Rule<NB> T{};
+template <int NB, int NP>
+Rule<NB, NP> make_rule() {
+  Rule<NB, NP> T{};
   std::vector<double> x, w, v(NB), dv(NB);
-  gauss_legendre(Rule<NB>::NQ, x, w);
-  for (int q = 0; q < Rule<NB>::H; ++q) {
+  gauss_legendre(NP, x, w);
+  for (int q = 0; q < Rule<NB, NP>::H; ++q) {
     phi_values(NB, x[q], v.data(), dv.data());
     for (int b = 0; b < NB; ++b) {
       T.V[b][q] = v[b];
@@ -24,10 +24,12 @@ Rule<NB> make_rule() {
   phi_values(NB, 1.0, T.ep, nullptr);
   return T;
 }
-template Rule<2> make_rule<2>();
-template Rule<3> make_rule<3>();
-template Rule<4> make_rule<4>();
-template Rule<5> make_rule<5>();
+template Rule<2, 2> make_rule<2, 2>();
+template Rule<3, 4> make_rule<3, 4>();
+template Rule<4, 5> make_rule<4, 5>();
+template Rule<5, 7> make_rule<5, 7>();
+template Rule<2, 3> make_rule<2, 3>();
+template Rule<3, 5> make_rule<3, 5>();
 
 }  // namespace nl
 
@@ -90,18 +92,25 @@ Tab<NB> make_tab() {
   return T;
 }
 
-template <int NB, int MV, int FLUX>
-cudaError_t launch_one(const NewtonMfArgs& a, cudaStream_t s) {
-  using K = Cfg<NB, MV>;
+template <int NB, int MV, int FLUX, bool F64>
+cudaError_t launch_prec(const NewtonMfArgs& a, cudaStream_t s) {
+  using K = Cfg<NB, MV, F64>;
   static_assert(K::bytes <= 232448, "shared memory above the per-CTA limit");
   static const Tab<NB> tab = make_tab<NB>();
-  auto kern = a.ninst > 0 ? newton_mf_kernel<NB, MV, FLUX, true> : newton_mf_kernel<NB, MV, FLUX, false>;
+  static const Rule<NB, K::NP> jrule = make_rule<NB, K::NP>();
+  auto kern = a.ninst > 0 ? newton_mf_kernel<NB, MV, FLUX, F64, true>
+                          : newton_mf_kernel<NB, MV, FLUX, F64, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::bytes);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(a.list_count, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)a.ncell, K::NT, K::bytes, s>>>(a, tab);
+  kern<<<(unsigned)a.ncell, K::NT, K::bytes, s>>>(a, tab, jrule);
   return cudaGetLastError();
+}
+
+template <int NB, int MV, int FLUX>
+cudaError_t launch_one(const NewtonMfArgs& a, cudaStream_t s) {
+  return a.fp64 ? launch_prec<NB, MV, FLUX, true>(a, s) : launch_prec<NB, MV, FLUX, false>(a, s);
 }
 
 }  // namespace

@@ -1,9 +1,11 @@
-// Matrix-free Newton prediction for a nonlinear flux in 2D (Sec. 3): the mixed precisions'
-// first solver, one CTA per region.
+// Matrix-free Newton prediction for a nonlinear flux in 2D (Sec. 3): the first solver of every
+// precision, one CTA per region.
 //
 // The region system of eq. pred_full_system is solved by the same outer iteration as in
-// k_newton.cuh -- FP64 residual by quadrature, FP64 iterate, linear solves in FP32, stop when
-// ||dW||_inf <= tol max(1, ||W||_inf) -- but no Jacobian is stored and nothing is factorised:
+// k_newton.cuh -- FP64 residual by quadrature, FP64 iterate, stop when ||dW||_inf <=
+// tol max(1, ||W||_inf); the mixed precisions solve the linear systems in FP32, the FP64 form
+// refines those solutions against the linear system's FP64 residual down to round-off -- but
+// no Jacobian is stored and nothing is factorised:
 //  * the linearised residual is applied in FP32 on the nodal basis of the NB^3 Gauss points
 //    of every cell, where a product with F'(w) is pointwise and a derivative is one NB x NB
 //    matrix per line (the integrals int d Psi_k Psi_l F'(w) by NB points per dimension);
@@ -20,7 +22,7 @@
 // multiplications), one flux evaluation per point for both directions and one per face.
 // Measured against the block elimination alone (one step, tensor-core / FP32 solves): Euler
 // Q2 160^2 214 -> 16.3 ms, Euler Q1 67 x 90 7.7 -> 1.1 ms, eight Burgers problems of up to
-// 72^2 at degrees 1 .. 4 228 -> 13.2 ms.
+// 72^2 at degrees 1 .. 4 228 -> 13.2 ms; FP64, Burgers Q2 45 x 33 31.7 -> 0.65 ms.
 //
 // The initial iterate is Q^n extended constant in time, so the first residual is evaluated
 // with one time mode and one time point.
@@ -54,10 +56,10 @@ struct Tab : nl::Rule<NB> {
   float L[2][NB];      // [side][n] w_n / 2 E: trace of node values
 };
 
-template <int NB, int MV>
+template <int NB, int MV, bool F64 = false>
 struct Cfg {
   static constexpr int THS = NB * NB, THT = NB * THS, BS = MV * THT, C = 9 * MV;
-  static constexpr int NQ = Tab<NB>::NQ;
+  static constexpr int NQ = residual_points(NB);
   static constexpr int COL = 9 * THS;               // columns (cell, y, x) of the region
   static constexpr int NT = (COL + 31) / 32 * 32, NW = NT / 32;
   static constexpr int VT = NB * MV;                // values per column
@@ -66,16 +68,22 @@ struct Cfg {
   static_assert(FL <= NT, "one thread per face line");
   // CTAs per SM that the registers are held to (168 / 128 / 96 a thread at Euler, Burgers Q4,
   // Burgers Q2 and Q3; unbounded they are 127 to 254 and one CTA fewer fits)
-  static constexpr int MINB = MV == 4 ? (NB == 2 ? 5 : 4) : (NB == 2 ? 8 : NB == 3 ? 6 : NB == 4 ? 4 : 2);
+  static constexpr int MINB = F64 && MV == 4 ? 2 : MV == 4 ? (NB == 2 ? 5 : 4) : (NB == 2 ? 8 : NB == 3 ? 6 : NB == 4 ? 4 : 2);
   // FP64 arena: B1, B2 (line buffers), face fluxes; the face traces share B2
   static constexpr int nB = C * NB * NQ * NQ, nTr = 4 * C * NB * NQ, nH = 24 * MV * NB * NQ;
   static constexpr int nB2 = nB > nTr ? nB : nTr;
-  static constexpr int nArena64 = nB + nB2 + nH;
+  // FP64 linear solves: the rule of the Jacobian (2M + 1 points of the quasi-quadrature-free
+  // form; Burgers: exact with the residual's), the lines of two fields and the face fluxes
+  static constexpr int NP = MV == 1 ? NQ : 2 * NB - 1;
+  static constexpr int jB = C * NB * NP * NP, jTr = 4 * C * NB * NP, jH = 24 * MV * NB * NP;
+  static constexpr int nLin = 2 * (jB > jTr ? jB : jTr) + jH;
+  static constexpr int nRes = nB + nB2 + nH, nArena64 = F64 && nLin > nRes ? nLin : nRes;
   // FP32 arena: the vector, its fluxes, the face fluxes
   static constexpr int nP = VT * COL, nF = 24 * VT * NB;
   static constexpr int nArena32 = (1 + NG) * nP + nF;
   static constexpr size_t arena = nArena64 * 8 > nArena32 * 4 ? nArena64 * 8 : nArena32 * 4;
-  static constexpr size_t oR = 8 * 9 * BS, oQ = 2 * oR, oRed = oQ + 8 * C * THS, oArena = (oRed + 4 * 2 * 4 * NW + 15) / 16 * 16;
+  static constexpr size_t oR = 8 * 9 * BS, oZ = 2 * oR, oD = oZ + (F64 ? oR : 0),
+                          oQ = oD + (F64 ? oR : 0), oRed = oQ + 8 * C * THS, oArena = (oRed + 4 * 2 * 4 * NW + 15) / 16 * 16;
   static constexpr size_t bytes = oArena + arena;
 };
 
@@ -110,12 +118,12 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
     double m[NB], v[NQ];
 #pragma unroll
     for (int b = 0; b < NB; ++b) m[b] = src[b];
-    interp<NB>(T, m, v);
+    interp(T, m, v);
     double* dst = B1 + ((c * NB + a) * NQ + y) * NQ;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) dst[q] = v[q];
     double e, o;
-    traces<NB>(T, m, 1, e, o);
+    traces(T, m, 1, e, o);
     Tr[((0 * C + c) * NB + a) * NQ + y] = e + o;
     Tr[((1 * C + c) * NB + a) * NQ + y] = e - o;
   }
@@ -124,7 +132,7 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
     const int c = i / (NA * NB), a = (i / NB) % NA, x = i % NB;
     const double* src = Ws + (c * NB + a) * THS + x;
     double e, o;
-    traces<NB>(T, src, NB, e, o);
+    traces(T, src, NB, e, o);
     Tr[((2 * C + c) * NB + a) * NQ + x] = e + o;
     Tr[((3 * C + c) * NB + a) * NQ + x] = e - o;
   }
@@ -137,7 +145,7 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
     double m[NB], v[NQ];
 #pragma unroll
     for (int b = 0; b < NB; ++b) m[b] = p[b * NQ];
-    interp<NB>(T, m, v);
+    interp(T, m, v);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) p[q * NQ] = v[q];
   }
@@ -146,7 +154,7 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
     double m[NB], v[NQ];
 #pragma unroll
     for (int b = 0; b < NB; ++b) m[b] = p[b];
-    interp<NB>(T, m, v);
+    interp(T, m, v);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) p[q] = v[q];
   }
@@ -198,8 +206,8 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
         wr[j] = mr[j][0];
 #pragma unroll
         for (int a = 1; a < NA; ++a) {
-          wl[j] = fma(vq<NB>(T, a, q), ml[j][a], wl[j]);
-          wr[j] = fma(vq<NB>(T, a, q), mr[j][a], wr[j]);
+          wl[j] = fma(vq(T, a, q), ml[j][a], wl[j]);
+          wr[j] = fma(vq(T, a, q), mr[j][a], wr[j]);
         }
       }
       if (cl >= 0) flux1<FLUX>(wl, dd, fl, g);
@@ -213,7 +221,7 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
           acc[j][0] = 2.0 * fh;
         } else {
 #pragma unroll
-          for (int a = 0; a < NA; ++a) acc[j][a] = fma(wvq<NB>(T, a, q), fh, acc[j][a]);
+          for (int a = 0; a < NA; ++a) acc[j][a] = fma(wvq(T, a, q), fh, acc[j][a]);
         }
       }
     }
@@ -242,10 +250,10 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
       double m[NB], v[NQ];
 #pragma unroll
       for (int a = 0; a < NB; ++a) m[a] = p1[a * NX];
-      interp<NB>(T, m, v);
+      interp(T, m, v);
 #pragma unroll
       for (int q = 0; q < NQ; ++q) v[q] = 0.5 * v[q] * v[q];
-      project<NB, false>(T, v, m);
+      project<false>(T, v, m);
 #pragma unroll
       for (int a = 0; a < NB; ++a) p1[a * NX] = m[a];
     } else {
@@ -264,15 +272,15 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
         for (int j = 0; j < MV; ++j) {
           w[j] = m[j][0];
 #pragma unroll
-          for (int a = 1; a < NB; ++a) w[j] = fma(vq<NB>(T, a, q), m[j][a], w[j]);
+          for (int a = 1; a < NB; ++a) w[j] = fma(vq(T, a, q), m[j][a], w[j]);
         }
         flux2<FLUX>(w, fx, fy, g);
 #pragma unroll
         for (int j = 0; j < MV; ++j)
 #pragma unroll
           for (int a = 0; a < NB; ++a) {
-            ax[j][a] = fma(wvq<NB>(T, a, q), fx[j], ax[j][a]);
-            ay[j][a] = fma(wvq<NB>(T, a, q), fy[j], ay[j][a]);
+            ax[j][a] = fma(wvq(T, a, q), fx[j], ax[j][a]);
+            ay[j][a] = fma(wvq(T, a, q), fy[j], ay[j][a]);
           }
       }
 #pragma unroll
@@ -293,12 +301,12 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
     double f[NQ], o1[NB], o2[NB];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) f[q] = p1[q * NQ];
-    project<NB, false>(T, f, o1);
+    project<false>(T, f, o1);
     if constexpr (K::NG == 2) {
 #pragma unroll
       for (int q = 0; q < NQ; ++q) f[q] = p2[q * NQ];
     }
-    project<NB, true>(T, f, o2);
+    project<true>(T, f, o2);
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       p1[b * NQ] = o1[b];
@@ -310,7 +318,7 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
     double f[NQ], o[NB];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) f[q] = p[q];
-    project<NB, false>(T, f, o);
+    project<false>(T, f, o);
 #pragma unroll
     for (int b = 0; b < NB; ++b) p[b] = o[b];
   }
@@ -331,10 +339,10 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
     double f[NQ], ox[NB], oy[NB];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) f[q] = p1[q];
-    project<NB, true>(T, f, ox);
+    project<true>(T, f, ox);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) f[q] = p2[q];
-    project<NB, false>(T, f, oy);
+    project<false>(T, f, oy);
     const double* hx = Hf + (((ry * 4 + rx) * MV + j) * NB + a) * NQ;         // left face
     const double* hy = Hf + (((12 + rx * 4 + ry) * MV + j) * NB + a) * NQ;    // lower face
     const double hl = hx[y], hr = hx[MV * NB * NQ + y];
@@ -354,6 +362,220 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
         acc = fma((a & 1) ? T.ep[a] : -T.ep[a], Qs[c * THS + y * NB + b], acc);
       }
       out[b] = acc;
+    }
+  }
+  __syncthreads();
+}
+
+// ---------------------------------------------------------------------------------------
+// Rs -= J z in FP64: the linearised residual at W (the sums of `residual` with F'(w) z for the
+// fluxes), by the rule T of the Jacobian.  Euler: 2M + 1 points per dimension, on which the
+// quasi-quadrature-free Jacobian's projection onto degree 2M is interpolation and its triple
+// products are exact -- the same matrix as the block elimination's.
+// ---------------------------------------------------------------------------------------
+template <int NB, int MV, int FLUX, int NP>
+__device__ void linear_update(const Rule<NB, NP>& T, const double (&Mt)[NB][NB], const double* Ws,
+                              const double* Zs, double* Rs, const double* alpha, double* arena,
+                              const double* lam, double g) {
+  using K = Cfg<NB, MV, true>;
+  constexpr int C = K::C, NT = K::NT, THS = K::THS, NX = NP * NP;
+  const int tid = threadIdx.x;
+  double* B0 = arena;                                      // lines of w, then the x flux
+  double* B1 = B0 + (K::jB > K::jTr ? K::jB : K::jTr);     // lines of z, then the y flux
+  double* Hf = B1 + (K::jB > K::jTr ? K::jB : K::jTr);     // [face][j][a][NP]
+  // face traces of both fields, [dd][side][c][a][NP] in B0 (w) and B1 (z)
+  for (int i = tid; i < 4 * C * NB * NB; i += NT) {
+    const int fd = i / (C * NB * NB), k = i - fd * (C * NB * NB), ca = k / NB, o = k - ca * NB;
+    const int dd = fd & 1;
+    const double* src = (fd & 2 ? Zs : Ws) + ca * THS + (dd ? o : o * NB);
+    double* tr = (fd & 2 ? B1 : B0) + (dd * 2 * C * NB + ca) * NP + o;
+    double e, od;
+    traces(T, src, dd ? NB : 1, e, od);
+    tr[0] = e + od;
+    tr[C * NB * NP] = e - od;
+  }
+  __syncthreads();
+  for (int i = tid; i < 8 * C * NB; i += NT) {
+    double* p = (i < 4 * C * NB ? B0 + i * NP : B1 + (i - 4 * C * NB) * NP);
+    double m[NB], v[NP];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) m[b] = p[b];
+    interp(T, m, v);
+#pragma unroll
+    for (int q = 0; q < NP; ++q) p[q] = v[q];
+  }
+  __syncthreads();
+  for (int i = tid; i < 24 * NP; i += NT) {
+    const int f = i / NP, qo = i - f * NP;
+    int dd, cl, cr;
+    face_cells(f, dd, cl, cr);
+    const int tl = (dd * 2 * C + (cl < 0 ? cr : cl) * MV) * NB * NP + qo;
+    const int tr = ((dd * 2 + 1) * C + (cr < 0 ? cl : cr) * MV) * NB * NP + qo;
+    const double al = 0.5 * alpha[f];
+    double acc[MV][NB];
+#pragma unroll
+    for (int j = 0; j < MV; ++j)
+#pragma unroll
+      for (int a = 0; a < NB; ++a) acc[j][a] = 0.0;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      double wl[MV], wr[MV], zl[MV], zr[MV], fl[MV], fr[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        wl[j] = B0[tl + j * NB * NP];
+        wr[j] = B0[tr + j * NB * NP];
+        zl[j] = B1[tl + j * NB * NP];
+        zr[j] = B1[tr + j * NB * NP];
+#pragma unroll
+        for (int a = 1; a < NB; ++a) {
+          const double v = vq(T, a, q);
+          const int at = (j * NB + a) * NP;
+          wl[j] = fma(v, B0[tl + at], wl[j]);
+          wr[j] = fma(v, B0[tr + at], wr[j]);
+          zl[j] = fma(v, B1[tl + at], zl[j]);
+          zr[j] = fma(v, B1[tr + at], zr[j]);
+        }
+      }
+      if (cl >= 0) dflux1<FLUX>(wl, zl, dd, fl, g);
+      if (cr >= 0) dflux1<FLUX>(wr, zr, dd, fr, g);
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        const double fh = cl < 0 ? fr[j] : cr < 0 ? fl[j]
+                          : fma(0.5, fl[j] + fr[j], -al * (zr[j] - zl[j]));
+#pragma unroll
+        for (int a = 0; a < NB; ++a) acc[j][a] = fma(wvq(T, a, q), fh, acc[j][a]);
+      }
+    }
+    double* h = Hf + f * MV * NB * NP + qo;
+#pragma unroll
+    for (int j = 0; j < MV; ++j)
+#pragma unroll
+      for (int a = 0; a < NB; ++a) h[(j * NB + a) * NP] = acc[j][a];
+  }
+  __syncthreads();
+  // volume: x lines, y lines of both fields
+  for (int i = tid; i < 2 * C * NB * NB; i += NT) {
+    const bool z = i >= C * NB * NB;
+    const int k = z ? i - C * NB * NB : i, ca = k / NB, y = k - ca * NB;
+    const double* src = (z ? Zs : Ws) + ca * THS + y * NB;
+    double* dst = (z ? B1 : B0) + (ca * NP + y) * NP;
+    double m[NB], v[NP];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) m[b] = src[b];
+    interp(T, m, v);
+#pragma unroll
+    for (int q = 0; q < NP; ++q) dst[q] = v[q];
+  }
+  __syncthreads();
+  for (int i = tid; i < 2 * C * NB * NP; i += NT) {
+    const bool z = i >= C * NB * NP;
+    const int k = z ? i - C * NB * NP : i, ca = k / NP;
+    double* p = (z ? B1 : B0) + ca * NX + (k - ca * NP);
+    double m[NB], v[NP];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) m[b] = p[b * NP];
+    interp(T, m, v);
+#pragma unroll
+    for (int q = 0; q < NP; ++q) p[q * NP] = v[q];
+  }
+  __syncthreads();
+  for (int i = tid; i < 9 * NX; i += NT) {
+    const int r = i / NX, at = r * MV * NB * NX + (i - r * NX);
+    double* p0 = B0 + at;
+    double* p1 = B1 + at;
+    double ax[MV][NB], ay[MV][NB];
+#pragma unroll
+    for (int j = 0; j < MV; ++j)
+#pragma unroll
+      for (int a = 0; a < NB; ++a) ax[j][a] = ay[j][a] = 0.0;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      double w[MV], z[MV], fx[MV], fy[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        w[j] = p0[j * NB * NX];
+        z[j] = p1[j * NB * NX];
+#pragma unroll
+        for (int a = 1; a < NB; ++a) {
+          const double v = vq(T, a, q);
+          w[j] = fma(v, p0[(j * NB + a) * NX], w[j]);
+          z[j] = fma(v, p1[(j * NB + a) * NX], z[j]);
+        }
+      }
+      dflux2<FLUX>(w, z, fx, fy, g);
+#pragma unroll
+      for (int j = 0; j < MV; ++j)
+#pragma unroll
+        for (int a = 0; a < NB; ++a) {
+          ax[j][a] = fma(wvq(T, a, q), fx[j], ax[j][a]);
+          if constexpr (MV > 1) ay[j][a] = fma(wvq(T, a, q), fy[j], ay[j][a]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < MV; ++j)
+#pragma unroll
+      for (int a = 0; a < NB; ++a) {
+        p0[(j * NB + a) * NX] = ax[j][a];
+        if constexpr (MV > 1) p1[(j * NB + a) * NX] = ay[j][a];
+      }
+  }
+  __syncthreads();
+  for (int i = tid; i < C * NB * NP; i += NT) {
+    const int ca = i / NP;
+    double* p0 = B0 + ca * NX + (i - ca * NP);
+    double* p1 = B1 + ca * NX + (i - ca * NP);
+    double f[NP], o1[NB], o2[NB];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) f[q] = p0[q * NP];
+    project<false>(T, f, o1);
+    if constexpr (MV > 1) {
+#pragma unroll
+      for (int q = 0; q < NP; ++q) f[q] = p1[q * NP];
+    }
+    project<true>(T, f, o2);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      p0[b * NP] = o1[b];
+      p1[b * NP] = o2[b];
+    }
+  }
+  for (int i = tid; i < 24 * MV * NB; i += NT) {
+    double* p = Hf + i * NP;
+    double f[NP], o[NB];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) f[q] = p[q];
+    project<false>(T, f, o);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) p[b] = o[b];
+  }
+  __syncthreads();
+  const double l0 = 0.25 * lam[0], l1 = 0.25 * lam[1];
+  for (int i = tid; i < C * NB * NB; i += NT) {
+    const int c = i / (NB * NB), a = (i / NB) % NB, y = i % NB;
+    const int r = c / MV, j = c - r * MV, ry = r / 3, rx = r - 3 * ry;
+    double* out = Rs + (c * NB + a) * THS + y * NB;
+    const double* p0 = B0 + ((c * NB + a) * NP + y) * NP;
+    const double* p1 = B1 + ((c * NB + a) * NP + y) * NP;
+    double f[NP], ox[NB], oy[NB];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) f[q] = p0[q];
+    project<true>(T, f, ox);
+#pragma unroll
+    for (int q = 0; q < NP; ++q) f[q] = p1[q];
+    project<false>(T, f, oy);
+    const double* hx = Hf + (((ry * 4 + rx) * MV + j) * NB + a) * NP;
+    const double* hy = Hf + (((12 + rx * 4 + ry) * MV + j) * NB + a) * NP;
+    const double hl = hx[y], hr = hx[MV * NB * NP + y], ey = T.ep[y];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const double hb = hy[b], ht = hy[MV * NB * NP + b];
+      const double fx = (b & 1) ? hr + hl : hr - hl, fy = (y & 1) ? ht + hb : ht - hb;
+      double acc = l0 * fma(T.ep[b], fx, -ox[b]);
+      acc = fma(l1, fma(ey, fy, -oy[b]), acc);
+      const double* z = Zs + c * K::THT + y * NB + b;
+#pragma unroll
+      for (int e = 0; e < NB; ++e) acc = fma(Mt[a][e], z[e * THS], acc);
+      out[b] -= acc;
     }
   }
   __syncthreads();
@@ -584,17 +806,217 @@ __device__ __forceinline__ void apply(const Tab<NB>& T, const Rows<NB>& R, const
   }
 }
 
-constexpr int kMaxSolves = 7;   // linear solves of a region before it is left to the list
+constexpr int kMaxSolves = 7;   // linear solves of a region (mixed) before it is left to the list
+constexpr int kMaxRefine = 5;   // FP32 solves per Newton iteration (FP64) before that
 constexpr int kMaxInner = 24;   // BiCGStab iterations per solve
 
-template <int NB, int MV, int FLUX, bool BATCH>
-__global__ void __launch_bounds__((Cfg<NB, MV>::NT), (Cfg<NB, MV>::MINB)) newton_mf_kernel(const NewtonMfArgs a,
-                                                                      const Tab<NB> T) {
+// The linearisation point at W: F' at the thread's nodes and at both sides of its face line.
+template <int NB, int MV>
+__device__ __forceinline__ void linearise(const Tab<NB>& T, const double* Ws, const Rows<NB>& R,
+                                          Lin<NB, MV>& S, float* P, float g1) {
   using K = Cfg<NB, MV>;
+  constexpr int VT = K::VT, COL = K::COL;
+  const int tid = threadIdx.x;
+  to_nodes<NB, MV>(T, Ws, 1.0, P);
+  if (tid < COL) {
+    float m[VT], w[VT];
+#pragma unroll
+    for (int tj = 0; tj < VT; ++tj) m[tj] = P[tj * COL + tid];
+#pragma unroll
+    for (int t = 0; t < NB; ++t)
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        float s = 0.f;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) s = fmaf(T.N[b][t], m[b * MV + j], s);
+        w[t * MV + j] = s;
+      }
+#pragma unroll
+    for (int tj = 0; tj < VT; ++tj) P[tj * COL + tid] = w[tj];
+#pragma unroll
+    for (int t = 0; t < NB; ++t) {
+      if constexpr (MV == 1) S.w[t] = w[t];
+      else S.w[t] = prim_of(w + t * MV, g1);
+    }
+  }
+  __syncthreads();
+  if (tid < K::FL) {
+    const int st = R.dd ? NB : 1;
+    // outside the region the inner trace stands in (its flux is not used)
+    const int bl = R.bl < 0 ? R.br : R.bl, br = R.br < 0 ? R.bl : R.br;
+#pragma unroll
+    for (int t = 0; t < NB; ++t) {
+      float l[MV], r[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        const float* p = P + (t * MV + j) * COL;
+        l[j] = r[j] = 0.f;
+#pragma unroll
+        for (int n = 0; n < NB; ++n) {
+          l[j] = fmaf(T.L[R.bl < 0][n], p[bl + n * st], l[j]);
+          r[j] = fmaf(T.L[R.br < 0 ? 0 : 1][n], p[br + n * st], r[j]);
+        }
+      }
+      if constexpr (MV == 1) {
+        S.wl[t] = l[0];
+        S.wr[t] = r[0];
+      } else {
+        S.wl[t] = prim_of(l, g1);
+        S.wr[t] = prim_of(r, g1);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// J z = scale Rs by BiCGStab in FP32 to a relative residual of about atol / |Rs| within
+// [rmin, rmax]; the modes of z are left in P (all threads may read them) and the relative
+// residual reached in `ratio`.  False if it stalled.
+template <int NB, int MV, int FLUX>
+__device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
+                                         const Lin<NB, MV>& S, const double* Rs, double scale,
+                                         float atol, float rmin, float rmax, float* P, float* G,
+                                         float* Fh, float* red, int& buf, float g1,
+                                         float& ratio) {
+  using K = Cfg<NB, MV>;
+  constexpr int VT = K::VT, COL = K::COL, NW = K::NW;
+  const int tid = threadIdx.x;
+  // right-hand side: node values of (time operator)^-1 R, scaled
+  to_nodes<NB, MV>(T, Rs, scale, P);
+  float r[VT], rh[VT], p[VT], v[VT], t[VT], x[VT];
+  float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < VT; ++k) r[k] = p[k] = v[k] = t[k] = x[k] = 0.f;
+  if (tid < COL) {
+    float m[VT];
+#pragma unroll
+    for (int tj = 0; tj < VT; ++tj) m[tj] = P[tj * COL + tid];
+#pragma unroll
+    for (int n = 0; n < NB; ++n)
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        float s = 0.f;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) s = fmaf(T.TN[n][b], m[b * MV + j], s);
+        r[n * MV + j] = s;
+      }
+  }
+#pragma unroll
+  for (int k = 0; k < VT; ++k) {
+    rh[k] = p[k] = r[k];
+    s4[0] = fmaf(r[k], r[k], s4[0]);
+  }
+  {
+    float s1[1] = {s4[0]};
+    reduce<NW, 1, false>(s1, red, buf);
+    s4[0] = s1[0];
+  }
+  const float bb = s4[0];
+  const float bmean = sqrtf(bb / (9 * K::BS)) / (float)scale;
+  const float tol = fminf(rmax, fmaxf(rmin, atol / bmean));
+  const float stop = tol * tol * bb;
+  float rho = bb, rr = bb;
+#pragma unroll 1
+  for (int k = 0; k < kMaxInner && rr > stop; ++k) {
+    apply<NB, MV, FLUX>(T, R, S, p, v, P, G, Fh, g1);
+    float s1[1] = {0.f};
+    if (tid < COL)
+#pragma unroll
+      for (int q = 0; q < VT; ++q) s1[0] = fmaf(rh[q], v[q], s1[0]);
+    reduce<NW, 1, false>(s1, red, buf);
+    const float al = rho / s1[0];
+#pragma unroll
+    for (int q = 0; q < VT; ++q) r[q] = fmaf(-al, v[q], r[q]);  // s of the method
+    apply<NB, MV, FLUX>(T, R, S, r, t, P, G, Fh, g1);
+    s4[0] = s4[1] = s4[2] = s4[3] = 0.f;
+    if (tid < COL)
+#pragma unroll
+      for (int q = 0; q < VT; ++q) {
+        s4[0] = fmaf(t[q], r[q], s4[0]);
+        s4[1] = fmaf(t[q], t[q], s4[1]);
+        s4[2] = fmaf(rh[q], t[q], s4[2]);
+        s4[3] = fmaf(r[q], r[q], s4[3]);
+      }
+    reduce<NW, 4, false>(s4, red, buf);
+    const float om = s4[1] > 0.f ? s4[0] / s4[1] : 0.f;
+#pragma unroll
+    for (int q = 0; q < VT; ++q) {
+      x[q] = fmaf(al, p[q], fmaf(om, r[q], x[q]));
+      r[q] = fmaf(-om, t[q], r[q]);
+    }
+    rr = fmaxf(0.f, s4[3] - om * s4[0]);
+    const float rho1 = -om * s4[2];  // <rh, r>, as <rh, s> = 0
+    const float be = rho1 / rho * (al / om);
+    rho = rho1;
+#pragma unroll
+    for (int q = 0; q < VT; ++q) p[q] = fmaf(be, fmaf(-om, v[q], p[q]), r[q]);
+    if (!(fabsf(al) < 1e30f) || !(rr < 1e30f)) return false;
+    // (a vanished residual leaves be undefined)
+    if (rr > stop && !(fabsf(be) < 1e30f)) return false;
+  }
+  if (rr > 1e-2f * bb) return false;
+  ratio = bb > 0.f ? sqrtf(rr / bb) : 0.f;
+  // the modes of x
+  __syncthreads();
+  if (tid < COL) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        float s = 0.f;
+#pragma unroll
+        for (int n = 0; n < NB; ++n) s = fmaf(T.M[b][n], x[n * MV + j], s);
+        P[(b * MV + j) * COL + tid] = s;
+      }
+  }
+  __syncthreads();
+  lines<NB, MV, false>(T, P, true);
+  __syncthreads();
+  lines<NB, MV, false>(T, P, false);
+  __syncthreads();
+  return true;
+}
+
+// the largest |Rs| (3e38 if one is not finite), as a power of two in ex; false if unusable
+template <int NB, int MV>
+__device__ __forceinline__ bool rhs_scale(const double* Rs, float* red, int& buf, float& rmax,
+                                          int& ex) {
+  using K = Cfg<NB, MV>;
+  float m[1] = {0.f};
+  for (int i = threadIdx.x; i < 9 * K::BS; i += K::NT) {
+    const double x = fabs(Rs[i]);
+    m[0] = x <= 1e30 ? fmaxf(m[0], (float)x) : 3e38f;  // (a NaN compares false)
+  }
+  reduce<K::NW, 1, true>(m, red, buf);
+  rmax = m[0];
+  ex = rmax > 1e-30f ? ilogbf(rmax) : -100;
+  return rmax <= 1e30f;
+}
+
+// index in P of the modal entry i of a region field ([cell][variable][time][y, x])
+template <int NB, int MV>
+__device__ __forceinline__ int p_index(int i) {
+  using K = Cfg<NB, MV>;
+  const int c = i / K::THT, m = i - c * K::THT, a = m / K::THS, s = m - a * K::THS;
+  const int r = c / MV, j = c - r * MV;
+  return (a * MV + j) * K::COL + r * K::THS + s;
+}
+
+// F64 = false (the mixed precisions): chord iteration -- one FP32 solve per FP64 residual, the
+// linearisation renewed where it no longer contracts well.  F64 = true: Newton with every
+// linear system solved to FP64 accuracy, by FP32 solves refined against its FP64 residual, so
+// that the iterates are the block elimination's to round-off.
+template <int NB, int MV, int FLUX, bool F64, bool BATCH>
+__global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MINB))
+    newton_mf_kernel(const NewtonMfArgs a, const Tab<NB> T,
+                     const Rule<NB, Cfg<NB, MV, F64>::NP> TJ) {
+  using K = Cfg<NB, MV, F64>;
   constexpr int VT = K::VT, COL = K::COL, NT = K::NT, NW = K::NW, THS = K::THS, BS = K::BS;
   extern __shared__ __align__(16) unsigned char smem[];
   double* Ws = (double*)smem;
   double* Rs = (double*)(smem + K::oR);
+  double* Zs = (double*)(smem + K::oZ);  // F64: the last FP32 solve's result
+  double* Ds = (double*)(smem + K::oD);  // F64: the Newton update
   double* Qs = (double*)(smem + K::oQ);
   __shared__ double alpha[24];
   float* red = (float*)(smem + K::oRed);
@@ -631,6 +1053,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV>::NT), (Cfg<NB, MV>::MINB)) newton
   }
   const unsigned ue = (unsigned)e, uy = ue / (unsigned)nx;
   const int ix = (int)(ue - uy * (unsigned)nx), iy = (int)uy;
+  float wmax[1] = {0.f};
   for (int i = tid; i < 9 * MV * THS; i += NT) {
     const int r = i / (MV * THS), rem = i - r * (MV * THS);
     int cx = ix + r % 3 - 1, cy = iy + r / 3 - 1;
@@ -638,13 +1061,16 @@ __global__ void __launch_bounds__((Cfg<NB, MV>::NT), (Cfg<NB, MV>::MINB)) newton
     cy += cy < 0 ? ny : (cy >= ny ? -ny : 0);
     const double q = Qg[((long long)cy * nx + cx) * (MV * THS) + rem];
     Qs[i] = q;
+    wmax[0] = fmaxf(wmax[0], (float)fabs(q));
     const int j = rem / THS, s = rem - j * THS;
     double* w = Ws + (r * MV + j) * K::THT + s;  // Q^n extended constant in time
     w[0] = q;
 #pragma unroll
     for (int t = 1; t < NB; ++t) w[t * THS] = 0.0;
   }
-  __syncthreads();
+  int buf = 0;
+  reduce<NW, 1, true>(wmax, red, buf);
+  float wnorm = wmax[0];
 
   // thread constants
   Rows<NB> R;
@@ -671,211 +1097,90 @@ __global__ void __launch_bounds__((Cfg<NB, MV>::NT), (Cfg<NB, MV>::MINB)) newton
     const int st = R.dd ? 1 : NB;
     R.bl = cl < 0 ? -1 : cl * THS + o * st;
     R.br = cr < 0 ? -1 : cr * THS + o * st;
-    R.al = 0.f;
   }
   Lin<NB, MV> S;
   const float g1 = (float)(a.gamma - 1.0);
-  int buf = 0, it = 0;
+  int it = 0;
   bool conv = false, lin = true;
   double dprev = 0.0;
-  float bprev = 0.f, wnorm = 1.f;
+  float bprev = 0.f;
+  const int solves = F64 ? a.max_iters : kMaxSolves;
 #pragma unroll 1
-  for (int solve = 0; solve < kMaxSolves; ++solve) {
+  for (int solve = 0; solve < solves; ++solve) {
     if (solve == 0)
       residual<NB, MV, FLUX, true>(T, Ws, Qs, Rs, alpha, arena, lam, a.gamma);
     else
       residual<NB, MV, FLUX, false>(T, Ws, Qs, Rs, alpha, arena, lam, a.gamma);
     // scale of the right-hand side (a power of two, so that its squares stay normal in FP32)
-    float m1[1] = {0.f};
-    for (int i = tid; i < 9 * BS; i += NT) {
-      const double x = fabs(Rs[i]);
-      m1[0] = x <= 1e30 ? fmaxf(m1[0], (float)x) : 3e38f;  // (a NaN compares false)
-    }
-    reduce<NW, 1, true>(m1, red, buf);
-    const float rmax = m1[0];
-    if (!(rmax <= 1e30f)) break;
-    const int ex = rmax > 1e-30f ? ilogbf(rmax) : -100;
-    const double scale = scalbn(1.0, -ex), unscale = scalbn(1.0, ex);
-    // a new linearisation where the last one no longer contracts by 3e3 per solve
-    if (solve > 0 && rmax > 3e-4f * bprev && it < a.max_iters) lin = true;
+    float rmax;
+    int ex;
+    if (!rhs_scale<NB, MV>(Rs, red, buf, rmax, ex)) break;
+    // mixed: a new linearisation where the last one no longer contracts by 3e3 per solve
+    if (F64 || (solve > 0 && rmax > 3e-4f * bprev && it < a.max_iters)) lin = true;
     bprev = rmax;
     if (lin) {
-      to_nodes<NB, MV>(T, Ws, 1.0, P);
-      float w[VT];
-      if (tid < COL) {
-        float m[VT];
-#pragma unroll
-        for (int tj = 0; tj < VT; ++tj) m[tj] = P[tj * COL + tid];
-#pragma unroll
-        for (int t = 0; t < NB; ++t)
-#pragma unroll
-          for (int j = 0; j < MV; ++j) {
-            float s = 0.f;
-#pragma unroll
-            for (int b = 0; b < NB; ++b) s = fmaf(T.N[b][t], m[b * MV + j], s);
-            w[t * MV + j] = s;
-          }
-#pragma unroll
-        for (int tj = 0; tj < VT; ++tj) P[tj * COL + tid] = w[tj];
-#pragma unroll
-        for (int t = 0; t < NB; ++t) {
-          if constexpr (MV == 1) S.w[t] = w[t];
-          else S.w[t] = prim_of(w + t * MV, g1);
-        }
-      }
-      __syncthreads();
-      if (tid < K::FL) {
-        const int st = R.dd ? NB : 1;
-        // outside the region the inner trace stands in (its flux is not used)
-        const int bl = R.bl < 0 ? R.br : R.bl, br = R.br < 0 ? R.bl : R.br;
-#pragma unroll
-        for (int t = 0; t < NB; ++t) {
-          float l[MV], r[MV];
-#pragma unroll
-          for (int j = 0; j < MV; ++j) {
-            const float* p = P + (t * MV + j) * COL;
-            l[j] = r[j] = 0.f;
-#pragma unroll
-            for (int n = 0; n < NB; ++n) {
-              l[j] = fmaf(T.L[R.bl < 0][n], p[bl + n * st], l[j]);
-              r[j] = fmaf(T.L[R.br < 0 ? 0 : 1][n], p[br + n * st], r[j]);
-            }
-          }
-          if constexpr (MV == 1) {
-            S.wl[t] = l[0];
-            S.wr[t] = r[0];
-          } else {
-            S.wl[t] = prim_of(l, g1);
-            S.wr[t] = prim_of(r, g1);
-          }
-        }
-        R.al = 0.5f * (float)alpha[tid / NB];
-      }
-      __syncthreads();
-      lin = false;
+      linearise<NB, MV>(T, Ws, R, S, P, g1);
+      R.al = 0.5f * (float)alpha[tid < K::FL ? tid / NB : 0];
+      lin = F64;
       ++it;
     }
-    // right-hand side: node values of (time operator)^-1 R, scaled
-    to_nodes<NB, MV>(T, Rs, scale, P);
-    float r[VT], rh[VT], p[VT], v[VT], t[VT], x[VT];
-    float s4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int k = 0; k < VT; ++k) r[k] = p[k] = v[k] = t[k] = x[k] = 0.f;
-    if (tid < COL) {
-      float m[VT];
-#pragma unroll
-      for (int tj = 0; tj < VT; ++tj) m[tj] = P[tj * COL + tid];
-#pragma unroll
-      for (int n = 0; n < NB; ++n)
-#pragma unroll
-        for (int j = 0; j < MV; ++j) {
-          float s = 0.f;
-#pragma unroll
-          for (int b = 0; b < NB; ++b) s = fmaf(T.TN[n][b], m[b * MV + j], s);
-          r[n * MV + j] = s;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < VT; ++k) {
-      rh[k] = p[k] = r[k];
-      s4[0] = fmaf(r[k], r[k], s4[0]);
-    }
-    {
-      float s1[1] = {s4[0]};
-      reduce<NW, 1, false>(s1, red, buf);
-      s4[0] = s1[0];
-    }
-    const float bb = s4[0];
-    // relative accuracy: 1e-4 in the first solve (whose result the nonlinearity limits), then
-    // down to an absolute ~1e-15 of the iterate, at most 1e-5 (FP32)
-    const float bmean = sqrtf(bb / (9 * BS)) * (float)unscale;
-    const float tol = solve == 0 ? 1e-4f : fminf(1e-2f, fmaxf(1e-5f, 1e-15f * wnorm / bmean));
-    const float stop = tol * tol * bb;
-    float rho = bb, rr = bb;
-    bool ok = true;
-    int k = 0;
+    float mx[2] = {0.f, 0.f}, ratio;
+    if constexpr (!F64) {
+      // relative accuracy: 1e-4 in the first solve (whose result the nonlinearity limits), then
+      // down to an absolute ~1e-15 of the iterate, at most 1e-5 (FP32)
+      const float rmin = solve == 0 ? 1e-4f : 1e-5f, rtop = solve == 0 ? 1e-4f : 1e-2f;
+      if (!bicgstab<NB, MV, FLUX>(T, R, S, Rs, scalbn(1.0, -ex), 1e-15f * wnorm, rmin, rtop, P, G,
+                                  Fh, red, buf, g1, ratio))
+        break;
+      const double unscale = scalbn(1.0, ex);
+      for (int i = tid; i < 9 * BS; i += NT) {
+        const double d = unscale * (double)P[p_index<NB, MV>(i)];
+        const double w = Ws[i] - d;
+        Ws[i] = w;
+        // (rounded up, so that the FP32 comparison below is never the looser one)
+        mx[0] = isfinite(d) ? fmaxf(mx[0], __double2float_ru(fabs(d))) : 3e38f;
+        mx[1] = isfinite(w) ? fmaxf(mx[1], __double2float_rd(fabs(w))) : 3e38f;
+      }
+    } else {
+      bool ok = true;
 #pragma unroll 1
-    for (; k < kMaxInner && rr > stop; ++k) {
-      apply<NB, MV, FLUX>(T, R, S, p, v, P, G, Fh, g1);
-      float s1[1] = {0.f};
-      if (tid < COL)
-#pragma unroll
-        for (int q = 0; q < VT; ++q) s1[0] = fmaf(rh[q], v[q], s1[0]);
-      reduce<NW, 1, false>(s1, red, buf);
-      const float al = rho / s1[0];
-#pragma unroll
-      for (int q = 0; q < VT; ++q) r[q] = fmaf(-al, v[q], r[q]);  // s of the method
-      apply<NB, MV, FLUX>(T, R, S, r, t, P, G, Fh, g1);
-      s4[0] = s4[1] = s4[2] = s4[3] = 0.f;
-      if (tid < COL)
-#pragma unroll
-        for (int q = 0; q < VT; ++q) {
-          s4[0] = fmaf(t[q], r[q], s4[0]);
-          s4[1] = fmaf(t[q], t[q], s4[1]);
-          s4[2] = fmaf(rh[q], t[q], s4[2]);
-          s4[3] = fmaf(r[q], r[q], s4[3]);
+      for (int ref = 0;; ++ref) {
+        if (ref > 0 && !rhs_scale<NB, MV>(Rs, red, buf, rmax, ex)) ok = false;
+        ok = ok && ref < kMaxRefine &&
+             bicgstab<NB, MV, FLUX>(T, R, S, Rs, scalbn(1.0, -ex), 1e-17f * wnorm, 3e-6f, 1e-3f,
+                                    P, G, Fh, red, buf, g1, ratio);
+        if (!ok) break;
+        const double unscale = scalbn(1.0, ex);
+        float zm[1] = {0.f};
+        for (int i = tid; i < 9 * BS; i += NT) {
+          const double z = unscale * (double)P[p_index<NB, MV>(i)];
+          Zs[i] = z;
+          Ds[i] = ref == 0 ? z : Ds[i] + z;
+          zm[0] = isfinite(z) ? fmaxf(zm[0], (float)fabs(z)) : 3e38f;
         }
-      reduce<NW, 4, false>(s4, red, buf);
-      const float om = s4[1] > 0.f ? s4[0] / s4[1] : 0.f;
-#pragma unroll
-      for (int q = 0; q < VT; ++q) {
-        x[q] = fmaf(al, p[q], fmaf(om, r[q], x[q]));
-        r[q] = fmaf(-om, t[q], r[q]);
+        reduce<NW, 1, true>(zm, red, buf);
+        if (!(zm[0] < 1e30f)) ok = false;
+        // what is left of the linear system is below the iterate's round-off
+        if (!ok || zm[0] * fmaxf(ratio, 1e-6f) <= 5e-17f * wnorm) break;
+        linear_update<NB, MV, FLUX>(TJ, T.Mt, Ws, Zs, Rs, alpha, arena, lam, a.gamma);
       }
-      rr = fmaxf(0.f, s4[3] - om * s4[0]);
-      const float rho1 = -om * s4[2];  // <rh, r>, <rh, s> = 0
-      const float be = rho1 / rho * (al / om);
-      rho = rho1;
-#pragma unroll
-      for (int q = 0; q < VT; ++q) p[q] = fmaf(be, fmaf(-om, v[q], p[q]), r[q]);
-      if (!(fabsf(al) < 1e30f) || !(rr < 1e30f)) {
-        ok = false;
-        break;
+      if (!ok) break;
+      for (int i = tid; i < 9 * BS; i += NT) {
+        const double d = Ds[i], w = Ws[i] - d;
+        Ws[i] = w;
+        mx[0] = isfinite(d) ? fmaxf(mx[0], __double2float_ru(fabs(d))) : 3e38f;
+        mx[1] = isfinite(w) ? fmaxf(mx[1], __double2float_rd(fabs(w))) : 3e38f;
       }
-      if (rr > stop && !(fabsf(be) < 1e30f)) {  // (a vanished residual leaves be undefined)
-        ok = false;
-        break;
-      }
-    }
-    if (!ok || rr > 1e-2f * bb) break;  // stalled
-    // the update in modes
-    __syncthreads();
-    if (tid < COL) {
-#pragma unroll
-      for (int b = 0; b < NB; ++b)
-#pragma unroll
-        for (int j = 0; j < MV; ++j) {
-          float s = 0.f;
-#pragma unroll
-          for (int n = 0; n < NB; ++n) s = fmaf(T.M[b][n], x[n * MV + j], s);
-          P[(b * MV + j) * COL + tid] = s;
-        }
-    }
-    __syncthreads();
-    lines<NB, MV, false>(T, P, true);
-    __syncthreads();
-    lines<NB, MV, false>(T, P, false);
-    __syncthreads();
-    float mx[2] = {0.f, 0.f};
-    for (int i = tid; i < 9 * BS; i += NT) {
-      const int c = i / K::THT, m = i - c * K::THT, aa = m / THS, s = m - aa * THS;
-      const int rg = c / MV, j = c - rg * MV;
-      const double d = unscale * (double)P[(aa * MV + j) * COL + rg * THS + s];
-      const double w = Ws[i] - d;
-      Ws[i] = w;
-      // (rounded up, so that the FP32 comparison below is never the looser one)
-      mx[0] = isfinite(d) ? fmaxf(mx[0], __double2float_ru(fabs(d))) : 3e38f;
-      mx[1] = isfinite(w) ? fmaxf(mx[1], __double2float_rd(fabs(w))) : 3e38f;
     }
     reduce<NW, 2, true>(mx, red, buf);
     if (!(mx[0] < 1e30f) || !(mx[1] < 1e30f)) break;
     const double dn = mx[0], wn = mx[1];
-    wnorm = fmaxf(1.f, mx[1]);
+    wnorm = mx[1];
     if (dn <= a.tol * fmax(1.0, wn)) {
       conv = true;
       break;
     }
-    if (solve > 0 && dn > 0.1 * dprev) break;
+    if (!F64 && solve > 0 && dn > 0.1 * dprev) break;
     dprev = dn;
   }
   if (conv) {

@@ -14,23 +14,26 @@
 namespace ridg {
 namespace nl {
 
-// The residual's 1D rule (NQ = ceil((3M + 1) / 2) points).  Its lower half is kept, q < H, with
-// the centre point at H - 1 if NQ is odd.
-template <int NB>
+// The residual's points per dimension, ceil((3M + 1) / 2).
+constexpr int residual_points(int nb) { return (3 * (nb - 1) + 2) / 2; }
+
+// An NP-point Gauss rule for NB modes.  Its lower half is kept, q < H, with the centre point
+// at H - 1 if NP is odd.
+template <int NB, int NP = residual_points(NB)>
 struct Rule {
-  static constexpr int NQ = (3 * (NB - 1) + 2) / 2, H = (NQ + 1) / 2;
+  static constexpr int NQ = NP, H = (NQ + 1) / 2;
   double V[NB][H];     // phi_b(x_q)
   double wV[NB][H];    // w_q phi_b(x_q)
   double wD[NB][H];    // w_q phi_b'(x_q)
   double ep[NB];       // phi_b(+1); phi_b(-1) = (-1)^b phi_b(+1)
 };
-// host (k_newton_mf.cu): the rule of NB = 2 .. 5
-template <int NB>
-Rule<NB> make_rule();
+// host (k_newton_mf.cu): NB = 2 .. 5 with NP = residual_points(NB) or 2 NB - 1
+template <int NB, int NP = residual_points(NB)>
+Rule<NB, NP> make_rule();
 
 // the traces at +1 (e + o) and -1 (e - o) of the polynomial with modes m[0], m[st], ...
-template <int NB>
-__device__ __forceinline__ void traces(const Rule<NB>& T, const double* m, int st, double& e,
+template <int NB, int NQ>
+__device__ __forceinline__ void traces(const Rule<NB, NQ>& T, const double* m, int st, double& e,
                                        double& o) {
   e = m[0];
   o = T.ep[1] * m[st];
@@ -40,10 +43,9 @@ __device__ __forceinline__ void traces(const Rule<NB>& T, const double* m, int s
 }
 
 // values at the NQ points of the polynomial with modes a
-template <int NB>
-__device__ __forceinline__ void interp(const Rule<NB>& T, const double (&a)[NB],
-                                       double (&v)[Rule<NB>::NQ]) {
-  constexpr int NQ = Rule<NB>::NQ;
+template <int NB, int NQ>
+__device__ __forceinline__ void interp(const Rule<NB, NQ>& T, const double (&a)[NB],
+                                       double (&v)[NQ]) {
 #pragma unroll
   for (int q = 0; q < NQ / 2; ++q) {
     double e = a[0];
@@ -67,10 +69,10 @@ __device__ __forceinline__ void interp(const Rule<NB>& T, const double (&a)[NB],
 }
 
 // out[b] = sum_q w_q phi_b(x_q) f[q], or with phi_b'
-template <int NB, bool DERIV>
-__device__ __forceinline__ void project(const Rule<NB>& T, const double (&f)[Rule<NB>::NQ],
+template <bool DERIV, int NB, int NQ>
+__device__ __forceinline__ void project(const Rule<NB, NQ>& T, const double (&f)[NQ],
                                         double (&out)[NB]) {
-  constexpr int NQ = Rule<NB>::NQ, HP = NQ / 2;
+  constexpr int HP = NQ / 2;
   double s[HP], d[HP];
 #pragma unroll
   for (int q = 0; q < HP; ++q) {
@@ -99,15 +101,15 @@ __device__ __forceinline__ void project(const Rule<NB>& T, const double (&f)[Rul
   }
 }
 
-// phi_b(x_q) at any q (compile-time indices)
-template <int NB>
-__device__ __forceinline__ double vq(const Rule<NB>& T, int b, int q) {
-  constexpr int NQ = Rule<NB>::NQ, H = Rule<NB>::H;
+// phi_b(x_q), and w_q phi_b(x_q), at any q (compile-time indices)
+template <int NB, int NQ>
+__device__ __forceinline__ double vq(const Rule<NB, NQ>& T, int b, int q) {
+  constexpr int H = (NQ + 1) / 2;
   return q < H ? T.V[b][q] : ((b & 1) ? -T.V[b][NQ - 1 - q] : T.V[b][NQ - 1 - q]);
 }
-template <int NB>
-__device__ __forceinline__ double wvq(const Rule<NB>& T, int b, int q) {
-  constexpr int NQ = Rule<NB>::NQ, H = Rule<NB>::H;
+template <int NB, int NQ>
+__device__ __forceinline__ double wvq(const Rule<NB, NQ>& T, int b, int q) {
+  constexpr int H = (NQ + 1) / 2;
   return q < H ? T.wV[b][q] : ((b & 1) ? -T.wV[b][NQ - 1 - q] : T.wV[b][NQ - 1 - q]);
 }
 
@@ -142,6 +144,40 @@ __device__ __forceinline__ void flux1(const double* w, int dd, double* f, double
     f[2] = w[2] * un;
     if (dd == 0) f[1] += p; else f[2] += p;
     f[3] = un * (w[3] + p);
+  }
+}
+
+// F'(w) z of both directions, or of one (Euler: of the state's primitives)
+template <int FLUX>
+__device__ __forceinline__ void dflux2(const double* w, const double* z, double* fx, double* fy,
+                                       double g) {
+  if constexpr (FLUX == RIDG_FLUX_BURGERS) {
+    fx[0] = w[0] * z[0];
+  } else {
+    const double ir = 1.0 / w[0], u = w[1] * ir, v = w[2] * ir, k = 0.5 * fma(u, u, v * v);
+    const double H = (w[3] + (g - 1.0) * fma(-w[0], k, w[3])) * ir;
+    const double dp = (g - 1.0) * (fma(k, z[0], z[3]) - fma(u, z[1], v * z[2]));
+    const double a = fma(-u, z[0], z[1]), b = fma(-v, z[0], z[2]), h = z[3] + dp;
+    fx[0] = z[1];
+    fx[1] = fma(u, z[1] + a, dp);
+    fx[2] = fma(v, a, u * z[2]);
+    fx[3] = fma(H, a, u * h);
+    fy[0] = z[2];
+    fy[1] = fma(u, b, v * z[1]);
+    fy[2] = fma(v, z[2] + b, dp);
+    fy[3] = fma(H, b, v * h);
+  }
+}
+template <int FLUX>
+__device__ __forceinline__ void dflux1(const double* w, const double* z, int dd, double* f,
+                                       double g) {
+  if constexpr (FLUX == RIDG_FLUX_BURGERS) {
+    f[0] = w[0] * z[0];
+  } else {
+    double fx[4], fy[4];
+    dflux2<FLUX>(w, z, fx, fy, g);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) f[j] = dd ? fy[j] : fx[j];
   }
 }
 

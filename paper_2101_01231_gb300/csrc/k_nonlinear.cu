@@ -200,10 +200,10 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
     double m[NB], ev, od;
 #pragma unroll
     for (int b = 0; b < NB; ++b) m[b] = src[b * st];
-    nl::traces<NB>(T, m, 1, ev, od);
+    nl::traces(T, m, 1, ev, od);
     if (kind == 0) {
       double v[NQ];
-      nl::interp<NB>(T, m, v);
+      nl::interp(T, m, v);
 #pragma unroll
       for (int q = 0; q < NQ; ++q) S[(ja * NQ + o) * NQ + q] = v[q];
     }
@@ -230,7 +230,7 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
     double m[NB], v[NQ];
 #pragma unroll
     for (int b = 0; b < NB; ++b) m[b] = p[b * st];
-    nl::interp<NB>(T, m, v);
+    nl::interp(T, m, v);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) p[q * st] = v[q];
   }
@@ -247,12 +247,12 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
       for (int j = 0; j < MV; ++j) {
         w[j] = S[j * NB * NX + yx];
 #pragma unroll
-        for (int a = 1; a < NB; ++a) w[j] = fma(nl::vq<NB>(T, a, q), S[(j * NB + a) * NX + yx], w[j]);
+        for (int a = 1; a < NB; ++a) w[j] = fma(nl::vq(T, a, q), S[(j * NB + a) * NX + yx], w[j]);
       }
       nl::flux2<FLUX>(w, fx, fy, g);
 #pragma unroll
       for (int j = 0; j < MV; ++j) {
-        const double wt = nl::wvq<NB>(T, 0, q);
+        const double wt = nl::wvq(T, 0, q);
         sx[j] = q == 0 ? wt * fx[j] : fma(wt, fx[j], sx[j]);
         if constexpr (MV > 1) sy[j] = q == 0 ? wt * fy[j] : fma(wt, fy[j], sy[j]);
       }
@@ -278,8 +278,8 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
         wr[j] = tr[j * NB * NQ];
 #pragma unroll
         for (int a = 1; a < NB; ++a) {
-          wl[j] = fma(nl::vq<NB>(T, a, q), tl[(j * NB + a) * NQ], wl[j]);
-          wr[j] = fma(nl::vq<NB>(T, a, q), tr[(j * NB + a) * NQ], wr[j]);
+          wl[j] = fma(nl::vq(T, a, q), tl[(j * NB + a) * NQ], wl[j]);
+          wr[j] = fma(nl::vq(T, a, q), tr[(j * NB + a) * NQ], wr[j]);
         }
       }
       s = fmax(s, fmax(nlflux::speed<FLUX>(wl, dd, g), nlflux::speed<FLUX>(wr, dd, g)));
@@ -308,8 +308,8 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
         wr[j] = tr[j * NB * NQ];
 #pragma unroll
         for (int a = 1; a < NB; ++a) {
-          wl[j] = fma(nl::vq<NB>(T, a, q), tl[(j * NB + a) * NQ], wl[j]);
-          wr[j] = fma(nl::vq<NB>(T, a, q), tr[(j * NB + a) * NQ], wr[j]);
+          wl[j] = fma(nl::vq(T, a, q), tl[(j * NB + a) * NQ], wl[j]);
+          wr[j] = fma(nl::vq(T, a, q), tr[(j * NB + a) * NQ], wr[j]);
         }
       }
       nl::flux1<FLUX>(wl, dd, fl, g);
@@ -317,7 +317,7 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
 #pragma unroll
       for (int j = 0; j < MV; ++j) {
         const double fh = fma(0.5, fl[j] + fr[j], -alpha * (wr[j] - wl[j]));
-        const double wt = nl::wvq<NB>(T, 0, q);
+        const double wt = nl::wvq(T, 0, q);
         h[j] = q == 0 ? wt * fh : fma(wt, fh, h[j]);
       }
     }
@@ -331,12 +331,12 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
     double v[NQ], o1[NB], o2[NB];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) v[q] = p1[q * NQ];
-    nl::project<NB, false>(T, v, o1);
+    nl::project<false>(T, v, o1);
     if constexpr (MV > 1) {
 #pragma unroll
       for (int q = 0; q < NQ; ++q) v[q] = p2[q * NQ];
     }
-    nl::project<NB, true>(T, v, o2);
+    nl::project<true>(T, v, o2);
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       p1[b * NQ] = o1[b];
@@ -349,7 +349,7 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
     double v[NQ], o[NB];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) v[q] = p[q];
-    nl::project<NB, false>(T, v, o);
+    nl::project<false>(T, v, o);
 #pragma unroll
     for (int b = 0; b < NB; ++b) p[b] = o[b];
   }
@@ -363,10 +363,10 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
     double v[NQ], ox[NB], oy[NB];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) v[q] = p1[q];
-    nl::project<NB, true>(T, v, ox);
+    nl::project<true>(T, v, ox);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) v[q] = p1[MV * NX + q];
-    nl::project<NB, false>(T, v, oy);
+    nl::project<false>(T, v, oy);
     const double* h = S + K::oH + j * NQ;  // + face MV NQ
     const double hr = h[y], hl = h[MV * NQ + y];
     double* q = Q + ((e0 + c) * MV + j) * THS + y * NB;

@@ -218,7 +218,7 @@ struct NewtonArgs {
   const int* list;
   const int* list_count;
 };
-// The matrix-free Newton prediction (k_newton_mf.cuh), the mixed precisions' first solver: it
+// The matrix-free Newton prediction (k_newton_mf.cuh), the first solver of every precision: it
 // solves every region it can and lists the others for launch_newton.
 struct NewtonMfArgs {
   const double* Q;
@@ -227,6 +227,7 @@ struct NewtonMfArgs {
   long long ncell;     // regions (batched launch: of all instances)
   double lam[2];
   double gamma;
+  bool fp64;           // plain Newton with linear solves to FP64 accuracy; else FP32 solves
   int max_iters;       // linearisations per region
   double tol;
   int* stats;          // as in NewtonArgs
@@ -339,8 +340,8 @@ struct ridg_handle {
   int nl_grid_max = 0;    // CTAs the block storage is allocated for
   int tune_gemm3_slots = 0;   // 3D GEMM plane-operand ring depth (0: as many as fit)
   int tune_corr3_block = 128; // 3D correction block size
-  int* nl_list = nullptr; // mixed precisions: [0] count, [1..] the regions that the matrix-free
-                          // solver leaves to the block elimination
+  int* nl_list = nullptr; // 2D: [0] count, [1..] the regions that the matrix-free solver leaves
+                          // to the block elimination
   bool nl_scratch_shared = false;  // block storage owned by the batch
   int* nl_words = nullptr;  // [0] work counter, [1..3] Newton statistics, [4..5] max speed
                             // bits, [6..7] total Newton iterations, [8..23] iteration histogram

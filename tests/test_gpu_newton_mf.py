@@ -62,6 +62,28 @@ def test_matrix_free_matches_fp64(R, flux, M, n):
         assert np.abs(W - ref).max() <= TOL * np.abs(ref).max()
 
 
+@pytest.mark.parametrize("flux,M", [("burgers", 1), ("burgers", 2), ("burgers", 3), ("burgers", 4),
+                                    ("euler", 1), ("euler", 2)])
+@pytest.mark.parametrize("scale", [1.0, 1e-3])
+def test_fp64_newton_path_is_the_block_eliminations(R, flux, M, scale):
+    """FP64: with a tolerance that no iterate meets, every region goes to the block elimination
+    and stops at the cap; the matrix-free Newton's own iterates, stopped by the default
+    tolerance, count the same iterations as the oracle and agree to round-off (the linear
+    systems are solved to FP64 accuracy whatever the state's scale)."""
+    from oracle import nonlinear as NL
+    w, q = _smooth(flux, (4, 5), M)
+    if flux == "burgers":
+        q = scale * q
+    W, info, st = _predict(R, w, q, R.RIDG_PREC_FP64)
+    direct, dinfo, dst = _predict(R, w, q, R.RIDG_PREC_FP64, newton_tol=1e-30)
+    assert st == R.RIDG_OK and dst == R.RIDG_ENOCONV and dinfo["newton_hist"][4] == 20
+    assert np.abs(W - direct).max() <= 1e-12 * np.abs(direct).max()
+    cells = np.arange(20)[:: 1 if M < 3 else 7]
+    _, it, conv = NL.newton_predict(q, w, info["dt"], cells=cells, return_iters=True, chunk=4)
+    assert conv.all()
+    assert info["newton_iters_max"] >= it.max() and info["newton_hist"][it.max()] >= 1
+
+
 @pytest.mark.parametrize("flux,M", [("burgers", 2), ("burgers", 4), ("euler", 2)])
 def test_regions_left_over_are_block_eliminated(R, flux, M):
     # a tolerance below round-off: no region converges, every one goes through the list to the
