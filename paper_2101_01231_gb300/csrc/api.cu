@@ -321,6 +321,9 @@ int enqueue_newton3(ridg_t* h) {
   a.counter = h->nl_words;
   a.stats = h->nl_words + 1;
   a.iters_total = (unsigned long long*)(h->nl_words + 6);
+  a.list_count = h->nl_list;
+  a.list = h->nl_list + 1;
+  RIDG_CUDA(h, ridg::launch_newton3_mf(newton_prec(h) != ridg::kNewtonF64, a, h->stream));
   RIDG_CUDA(h, ridg::launch_newton3(h->nb, newton_prec(h) != ridg::kNewtonF64, a, h->nl_grid,
                                     h->stream));
   return RIDG_OK;
@@ -384,8 +387,7 @@ int enqueue_nl_correct(ridg_t* h) {
   if (h->dim == 3) {
     double lam[3];
     for (int d = 0; d < 3; ++d) lam[d] = h->dt / h->h[d];
-    RIDG_CUDA(h, ridg::launch_nl3_correct(h->nb, h->nl3, h->Q, h->W, h->n, h->ncell, lam,
-                                          h->stream));
+    RIDG_CUDA(h, ridg::launch_nl3_correct(h->nb, h->Q, h->W, h->n, h->ncell, lam, h->stream));
     return RIDG_OK;
   }
   RIDG_CUDA(h, ridg::launch_nl_correct(h->nb, h->m, h->flux.kind, h->Q, h->W, h->n[0],
@@ -626,7 +628,8 @@ int ridg_create(const ridg_mesh* mesh, int order, const ridg_flux* flux, double 
     h->nl_scratch_cta = ridg::newton3_scratch_per_cta(h->nb, newton_prec(h) != ridg::kNewtonF64);
     h->nl_scratch = h->nl_grid > 0 ? dev_alloc(h, h->nl_scratch_cta * (size_t)h->nl_grid) : nullptr;
     h->nl_words = (int*)dev_alloc(h, 24 * sizeof(int));
-    if (!h->nl3_mem || !h->nl_scratch || !h->nl_words) {
+    h->nl_list = (int*)dev_alloc(h, ((size_t)h->ncell + 1) * sizeof(int));
+    if (!h->nl3_mem || !h->nl_scratch || !h->nl_words || !h->nl_list) {
       ridg_destroy(h);
       return RIDG_ENOMEM;
     }

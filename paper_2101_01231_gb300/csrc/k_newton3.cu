@@ -1,7 +1,8 @@
 // The 3D nonlinear prediction (Sec. 2.2, eq. pred_full_system; Newton of Sec. 3) for
 // Burgers' flux F_d(q) = q^2 / 2, and its correction (Sec. 2.3).
 //
-// One persistent CTA per SM takes regions (3 x 3 x 3 cells, 27 theta_T unknowns each) from
+// The matrix-free solver of k_newton3_mf.cu goes first and lists the regions it could not
+// solve; one persistent CTA per SM takes those (3 x 3 x 3 cells, 27 theta_T unknowns each) from
 // an atomic counter.  Per Newton iteration, in FP64: the iterate's values at the residual's
 // Gauss points (volume and the six faces of every region cell), the Rusanov face fluxes
 // (speeds frozen at the initial iterate, Q^n extended in time; interior traces on the
@@ -133,11 +134,14 @@ __global__ void __launch_bounds__(kT3, 1) newton3_kernel(const Newton3Args a) {
   const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
   const double lam8[3] = {a.lam[0] / 8.0, a.lam[1] / 8.0, a.lam[2] / 8.0};
   for (;;) {
-    if (tid == 0) misc[0] = atomicAdd(a.counter, 1);
+    if (tid == 0) {
+      const int k = atomicAdd(a.counter, 1);
+      misc[0] = k < *a.list_count ? a.list[k] : -1;
+    }
     __syncthreads();
     const long long e = misc[0];
     __syncthreads();
-    if (e >= a.ncell) break;
+    if (e < 0) break;
     const int ix = (int)(e % nx), iy = (int)((e / nx) % ny), iz = (int)(e / ((long long)nx * ny));
     for (int i = tid; i < D::NR * THS; i += kT3) {
       const int r = i / THS, s = i % THS;
@@ -397,72 +401,100 @@ __global__ void __launch_bounds__(kT3, 1) newton3_kernel(const Newton3Args a) {
 }
 
 // ---------------------------------------------------------------------------------------
-// the correction: one thread per cell; every face flux is computed by both of its cells
-// from the same traces in the same order (the same bits: the mass telescopes exactly)
+// the correction at degree 1: one thread per node (z, y, x) of a cell, where the residual's
+// two-point rule makes the node values sums and differences of modes (k_newton3_mf.cu).  Every
+// face flux is computed by both of its cells from the same traces in the same order (the same
+// bits).  One thread per cell over the dense tables took ~15 k FP64 operations in a row; eight
+// threads with ~300 each keep small meshes from being latency-bound.
 // ---------------------------------------------------------------------------------------
-template <int NB>
-__global__ void __launch_bounds__(128) nl3_correct_kernel(const Nl3Dev tb, double* __restrict__ Q,
+// both time nodes of the trace on the face (D, side s = +-sqrt 3) at the tangential node whose
+// bits are in `node`: the normal's pair of modes, then sums / differences
+template <int D>
+__device__ __forceinline__ void node_trace(const double* w, double s, int node, double (&v)[2]) {
+  constexpr int st = 1 << D, e1 = D == 0 ? 2 : 1, e2 = D == 2 ? 2 : 4;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const double* m = w + 8 * a;
+    const double c00 = fma(s, m[st], m[0]), c01 = fma(s, m[e1 + st], m[e1]),
+                 c10 = fma(s, m[e2 + st], m[e2]), c11 = fma(s, m[e1 + e2 + st], m[e1 + e2]);
+    const double r0 = (node & e1) ? c00 + c01 : c00 - c01, r1 = (node & e1) ? c10 + c11 : c10 - c11;
+    v[a] = (node & e2) ? r0 + r1 : r0 - r1;
+  }
+  const double m0 = v[0];
+  v[0] = m0 - v[1];
+  v[1] = m0 + v[1];
+}
+
+// the face's flux summed over time (weights 1, halved), at the thread's tangential node; the
+// speed is the largest over the face's nodes (the lanes that differ in the tangential bits)
+template <int D>
+__device__ __forceinline__ double node_face(const double* wl, const double* wr, int node) {
+  const double s3 = 1.7320508075688772935;
+  double l[2], r[2];
+  node_trace<D>(wl, s3, node, l);
+  node_trace<D>(wr, -s3, node, r);
+  double al = fmax(fmax(fabs(l[0]), fabs(l[1])), fmax(fabs(r[0]), fabs(r[1])));
+  constexpr int e1 = D == 0 ? 2 : 1, e2 = D == 2 ? 2 : 4;
+  al = fmax(al, __shfl_xor_sync(0xffffffffu, al, e1));
+  al = fmax(al, __shfl_xor_sync(0xffffffffu, al, e2));
+  double f = 0.0;
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+    f += 0.25 * (l[t] * l[t] + r[t] * r[t]) - 0.5 * al * (r[t] - l[t]);
+  return 0.5 * f;
+}
+
+__global__ void __launch_bounds__(128) nl3_correct_kernel(double* __restrict__ Q,
                                                           const double* __restrict__ W, int nx,
                                                           int ny, int nz, long long ncell,
                                                           double lx, double ly, double lz) {
-  using D = D3<NB>;
-  constexpr int THT = D::THT, THS = D::THS;
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= ncell) return;
-  const int ix = (int)(e % nx), iy = (int)((e / nx) % ny), iz = (int)(e / ((long long)nx * ny));
-  const double lam8[3] = {lx / 8.0, ly / 8.0, lz / 8.0};
-  const double* We = W + e * THT;
-  double dq[THS];
-  for (int s = 0; s < THS; ++s) dq[s] = 0.0;
-  // volume: sum_d lam_d / 8 sum_q w_q d_d Phi_s(q) F(w(q))
-  for (int qv = 0; qv < D::QV; ++qv) {
-    const int q[4] = {qv % D::NQ, (qv / D::NQ) % D::NQ, (qv / (D::NQ * D::NQ)) % D::NQ,
-                      qv / (D::NQ * D::NQ * D::NQ)};
-    const double wq = tb.w1[q[0]] * tb.w1[q[1]] * tb.w1[q[2]] * tb.w1[q[3]];
-    const double w = eval_volume<NB>(tb, We, qv);
-    const double f = 0.5 * w * w * wq;
-    for (int s = 0; s < THS; ++s) {
-      const int b[3] = {s % NB, (s / NB) % NB, s / (NB * NB)};
-      for (int d = 0; d < 3; ++d) {
-        double g = lam8[d];
-        for (int e2 = 0; e2 < 3; ++e2) g *= (e2 == d ? tb.dV1 : tb.V1)[b[e2] * D::NQ + q[1 + e2]];
-        dq[s] += g * f;
-      }
-    }
+  const double s3 = 1.7320508075688772935;
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long e = min(i >> 3, ncell - 1);  // (all lanes take part in the shuffles)
+  const int node = (int)i & 7;
+  const unsigned u = (unsigned)e, uz = u / (unsigned)(nx * ny), ur = u - uz * (unsigned)(nx * ny);
+  const int iy = (int)(ur / (unsigned)nx), ix = (int)ur - iy * nx, iz = (int)uz;
+  const double* We = W + e * 16;
+  // volume: F at the node's two times, its partners along the directions by shuffle
+  double m[2], g;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const double* c = We + 8 * a;
+    double r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r[k] = (node & 1) ? c[2 * k] + c[2 * k + 1] : c[2 * k] - c[2 * k + 1];
+    const double y0 = (node & 2) ? r[0] + r[1] : r[0] - r[1], y1 = (node & 2) ? r[2] + r[3] : r[2] - r[3];
+    m[a] = (node & 4) ? y0 + y1 : y0 - y1;
   }
-  // faces: the flux at i + 1/2 from (w_i at +1, w_{i+1} at -1), at i - 1/2 from (w_{i-1} at +1,
-  // w_i at -1); Rusanov with the face's largest speed
+  const double w0 = m[0] - m[1], w1 = m[0] + m[1];
+  g = 0.25 * (w0 * w0 + w1 * w1);
+  const double lam[3] = {lx, ly, lz};
+  double dq = 0.0;
+#pragma unroll
   for (int d = 0; d < 3; ++d) {
-    for (int side = -1; side <= 1; side += 2) {
-      int c[3] = {ix, iy, iz};
-      const int nn[3] = {nx, ny, nz};
-      c[d] = (c[d] + side + nn[d]) % nn[d];
-      const long long en = ((long long)c[2] * ny + c[1]) * nx + c[0];
-      const double* WL = side > 0 ? We : W + en * THT;
-      const double* WR = side > 0 ? W + en * THT : We;
-      double wl[D::QF], wr[D::QF];
-      double al = 0.0;
-      for (int qf = 0; qf < D::QF; ++qf) {
-        wl[qf] = eval_face<NB>(tb, WL, d, +1, qf);
-        wr[qf] = eval_face<NB>(tb, WR, d, -1, qf);
-        al = fmax(al, fmax(fabs(wl[qf]), fabs(wr[qf])));
-      }
-      const int e1 = d == 0 ? 1 : 0, e2 = d == 2 ? 1 : 2;
-      for (int qf = 0; qf < D::QF; ++qf) {
-        const int qt = qf % D::NQ, q1 = (qf / D::NQ) % D::NQ, q2 = qf / (D::NQ * D::NQ);
-        const double fh = 0.5 * (0.5 * wl[qf] * wl[qf] + 0.5 * wr[qf] * wr[qf]) -
-                          0.5 * al * (wr[qf] - wl[qf]);
-        const double wq = tb.w1[qt] * tb.w1[q1] * tb.w1[q2] * fh;
-        for (int s = 0; s < THS; ++s) {
-          const int b[3] = {s % NB, (s / NB) % NB, s / (NB * NB)};
-          const double phi = (side > 0 ? tb.ep : tb.em)[b[d]] * tb.V1[b[e1] * D::NQ + q1] *
-                             tb.V1[b[e2] * D::NQ + q2];
-          dq[s] -= side * lam8[d] * phi * wq;
-        }
-      }
-    }
+    const int n = d == 0 ? nx : d == 1 ? ny : nz, c = d == 0 ? ix : d == 1 ? iy : iz;
+    const long long st = d == 0 ? 1 : d == 1 ? nx : (long long)nx * ny;
+    const double* Wr = We + 16 * st * (c + 1 == n ? 1 - n : 1);
+    const double* Wl = We - 16 * st * (c == 0 ? 1 - n : 1);
+    const double fr = d == 0 ? node_face<0>(We, Wr, node) : d == 1 ? node_face<1>(We, Wr, node)
+                                                                   : node_face<2>(We, Wr, node);
+    const double fl = d == 0 ? node_face<0>(Wl, We, node) : d == 1 ? node_face<1>(Wl, We, node)
+                                                                   : node_face<2>(Wl, We, node);
+    const bool up = node >> d & 1;
+    const double gs = g + __shfl_xor_sync(0xffffffffu, g, 1 << d);
+    // + D F - E(+1) F_{i+1/2} + E(-1) F_{i-1/2}
+    double v = (up ? s3 : -s3) * gs;
+    v = fma(up ? -1.0 - s3 : s3 - 1.0, fr, v);
+    v = fma(up ? 1.0 - s3 : 1.0 + s3, fl, v);
+    dq = fma(lam[d], v, dq);
   }
-  for (int s = 0; s < THS; ++s) Q[e * THS + s] += dq[s];
+  // to modes
+#pragma unroll
+  for (int b = 1; b < 8; b <<= 1) {
+    const double o = __shfl_xor_sync(0xffffffffu, dq, b);
+    dq = 0.5 * ((node & b) ? dq - o : dq + o);
+  }
+  if ((i >> 3) < ncell) Q[e * 8 + node] += dq;
 }
 
 template <int NB>
@@ -527,11 +559,11 @@ cudaError_t launch_newton3(int nb, bool fp32, const Newton3Args& a, int grid, cu
   return cudaGetLastError();
 }
 
-cudaError_t launch_nl3_correct(int nb, const Nl3Dev& tb, double* Q, const double* W, const int* n,
-                               long long ncell, const double* lam, cudaStream_t s) {
+cudaError_t launch_nl3_correct(int nb, double* Q, const double* W, const int* n, long long ncell,
+                               const double* lam, cudaStream_t s) {
   if (nb != 2) return cudaErrorInvalidValue;
-  nl3_correct_kernel<2><<<(unsigned)((ncell + 127) / 128), 128, 0, s>>>(
-      tb, Q, W, n[0], n[1], n[2], ncell, lam[0], lam[1], lam[2]);
+  nl3_correct_kernel<<<(unsigned)((8 * ncell + 127) / 128), 128, 0, s>>>(
+      Q, W, n[0], n[1], n[2], ncell, lam[0], lam[1], lam[2]);
   return cudaGetLastError();
 }
 

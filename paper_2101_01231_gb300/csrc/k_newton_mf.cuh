@@ -581,31 +581,6 @@ __device__ void linear_update(const Rule<NB, NP>& T, const double (&Mt)[NB][NB],
   __syncthreads();
 }
 
-// ---- block reductions: NV sums (or maxima), one barrier; buf alternates between calls -------
-template <int NW, int NV, bool MAX>
-__device__ __forceinline__ void reduce(float (&v)[NV], float* red, int& buf) {
-  static_assert(NV <= 4, "four slots per warp");
-#pragma unroll
-  for (int k = 0; k < NV; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float t = __shfl_xor_sync(0xffffffffu, v[k], o);
-      v[k] = MAX ? fmaxf(v[k], t) : v[k] + t;
-    }
-  float* p = red + buf * 4 * NW;
-  buf ^= 1;
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) p[(threadIdx.x >> 5) * 4 + k] = v[k];
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    v[k] = p[k];
-#pragma unroll
-    for (int w = 1; w < NW; ++w) v[k] = MAX ? fmaxf(v[k], p[w * 4 + k]) : v[k] + p[w * 4 + k];
-  }
-}
-
 // (F' v) for primitives (u, v, H) and both directions, or one
 struct Prim {
   float u, v, H;
@@ -1077,7 +1052,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
   {
     const int c = tid < COL ? tid : 0, r = c / THS, s = c - r * THS, y = s / NB, x = s - y * NB;
     const int ry = r / 3, rx = r - 3 * ry;
-    const float l0 = (float)lam[0], l1 = (float)lam[1];
+    const float l0 = keep((float)lam[0]), l1 = keep((float)lam[1]);
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
       R.dx[n] = -l0 * T.D[x][n];
@@ -1099,7 +1074,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
     R.br = cr < 0 ? -1 : cr * THS + o * st;
   }
   Lin<NB, MV> S;
-  const float g1 = (float)(a.gamma - 1.0);
+  const float g1 = keep((float)(a.gamma - 1.0));
   int it = 0;
   bool conv = false, lin = true;
   double dprev = 0.0;
@@ -1120,7 +1095,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
     bprev = rmax;
     if (lin) {
       linearise<NB, MV>(T, Ws, R, S, P, g1);
-      R.al = 0.5f * (float)alpha[tid < K::FL ? tid / NB : 0];
+      R.al = keep(0.5f * (float)alpha[tid < K::FL ? tid / NB : 0]);
       lin = F64;
       ++it;
     }

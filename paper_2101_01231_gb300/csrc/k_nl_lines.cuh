@@ -181,5 +181,38 @@ __device__ __forceinline__ void dflux1(const double* w, const double* z, int dd,
   }
 }
 
+// An FP32 value made from FP64 ones that is kept, not recomputed: where registers run short the
+// compiler otherwise repeats the conversion (an FP64-pipe instruction) at every use.
+__device__ __forceinline__ float keep(float x) {
+  asm volatile("" : "+f"(x));
+  return x;
+}
+
+// Block reduction of NV sums (or maxima) over NW warps, one barrier; red holds 8 NW floats, and
+// buf alternates between calls so that the next one needs no barrier before it.
+template <int NW, int NV, bool MAX>
+__device__ __forceinline__ void reduce(float (&v)[NV], float* red, int& buf) {
+  static_assert(NV <= 4, "four slots per warp");
+#pragma unroll
+  for (int k = 0; k < NV; ++k)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float t = __shfl_xor_sync(0xffffffffu, v[k], o);
+      v[k] = MAX ? fmaxf(v[k], t) : v[k] + t;
+    }
+  float* p = red + buf * 4 * NW;
+  buf ^= 1;
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) p[(threadIdx.x >> 5) * 4 + k] = v[k];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    v[k] = p[k];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) v[k] = MAX ? fmaxf(v[k], p[w * 4 + k]) : v[k] + p[w * 4 + k];
+  }
+}
+
 }  // namespace nl
 }  // namespace ridg

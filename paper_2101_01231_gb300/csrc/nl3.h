@@ -39,14 +39,19 @@ struct Newton3Args {
   int* counter;          // region counter (zeroed by the launcher)
   int* stats;            // as the 2D kernel: [0] unconverged, [1] max iters, [2] flags, [7..22]
   unsigned long long* iters_total;
+  int* list;             // regions that the matrix-free solver leaves to the dense LU
+  int* list_count;       // their number
 };
 bool newton3_supported(int nb);
+// The matrix-free solver (k_newton3_mf.cu, degree 1): solves every region it can (fp32: each
+// Newton system to FP32 accuracy, else to FP64's) and lists the others for launch_newton3.
+cudaError_t launch_newton3_mf(bool fp32, const Newton3Args& a, cudaStream_t s);
 size_t newton3_scratch_per_cta(int nb, bool fp32);
-// one persistent CTA per SM; fp32: the region Jacobian factorised in FP32 (the residual,
+// the listed regions, one persistent CTA per SM; fp32: the region Jacobian factorised in FP32 (the residual,
 // the iterate and the stopping test stay FP64)
 cudaError_t launch_newton3(int nb, bool fp32, const Newton3Args& a, int grid, cudaStream_t s);
-cudaError_t launch_nl3_correct(int nb, const Nl3Dev& tb, double* Q, const double* W, const int* n,
-                               long long ncell, const double* lam, cudaStream_t s);
+cudaError_t launch_nl3_correct(int nb, double* Q, const double* W, const int* n, long long ncell,
+                               const double* lam, cudaStream_t s);
 // largest |q| over a 6 x 6 x 6 equispaced grid of every cell -> *out (as bits)
 cudaError_t launch_max_speed3(int nb, const double* Q, long long ncell, unsigned long long* out,
                               cudaStream_t s);

@@ -340,8 +340,8 @@ struct ridg_handle {
   int nl_grid_max = 0;    // CTAs the block storage is allocated for
   int tune_gemm3_slots = 0;   // 3D GEMM plane-operand ring depth (0: as many as fit)
   int tune_corr3_block = 128; // 3D correction block size
-  int* nl_list = nullptr; // 2D: [0] count, [1..] the regions that the matrix-free solver leaves
-                          // to the block elimination
+  int* nl_list = nullptr; // [0] count, [1..] the regions that the matrix-free solver leaves to the
+                          // block elimination (3D: the dense LU)
   bool nl_scratch_shared = false;  // block storage owned by the batch
   int* nl_words = nullptr;  // [0] work counter, [1..3] Newton statistics, [4..5] max speed
                             // bits, [6..7] total Newton iterations, [8..23] iteration histogram

@@ -90,3 +90,32 @@ def test_3d_nonlinear_rejects_unsupported(R):
         R.Solver(3, (4, 4, 4), 1, flux="euler")          # Euler is 2D
     with pytest.raises(R.RidgError):
         R.Solver(3, (4, 4, 4), 1, flux="burgers", precision=R.RIDG_PREC_MIXED_TF32)
+
+
+@pytest.mark.parametrize("n", [(3, 3, 3), (7, 3, 5)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_3d_matrix_free_against_the_dense_solves(R, n, prec):
+    """Every region wraps onto itself at three cells per direction.  With a tolerance that no
+    iterate meets, every region goes through the list to the dense LU and stops at its cap;
+    the matrix-free solver's predictions agree with those (FP64: round-off; FP32 solves: the
+    Newton tolerance), and the correction with the oracle's from the same prediction."""
+    w = _w(n)
+    q = _state(w)
+    p = {"fp64": R.RIDG_PREC_FP64, "fp32": R.RIDG_PREC_MIXED_FP32}[prec]
+    out = []
+    for tol in (0.0, 1e-30):
+        s = R.Solver(3, n, 1, flux="burgers", cfl=w["cfl"], precision=p, newton_max_iters=8,
+                     newton_tol=tol)
+        s.set_state(q)
+        dt = s.info()["dt"]
+        W = s.predict()
+        info = s.info()
+        cells = int(np.prod(n))
+        assert sum(info["newton_hist"]) == cells
+        assert info["newton_unconverged"] == (cells if tol else 0)
+        s.correct()
+        q1 = s.get_state()
+        assert _rel(q1, NL.correct(q, W, w, dt)) < 1e-13
+        out.append(W)
+        s.close()
+    assert _rel(out[0], out[1]) < (1e-12 if prec == "fp64" else 1e-10)
