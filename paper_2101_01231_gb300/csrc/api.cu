@@ -434,14 +434,14 @@ int enqueue_correct_after_mean(ridg_t* h) {
   return RIDG_OK;
 }
 
-// Small 1D FP64 meshes run a whole sequence of steps in one launch.
+// 1D FP64: several steps per launch.
 bool use_run1d(const ridg_t* h) {
-  return is_linear(h) && h->opt.precision == RIDG_PREC_FP64 && ridg::run1d_fits(grid_of(h), h->nb);
+  return is_linear(h) && h->opt.precision == RIDG_PREC_FP64 && h->dim == 1;
 }
 
 int enqueue_run1d(ridg_t* h, int n) {
   const CorrParams cp = corr_params(h);
-  RIDG_CUDA(h, ridg::launch_run1d_fp64(grid_of(h), h->nb, h->Q, h->P, n, cp, h->stream));
+  RIDG_CUDA(h, ridg::launch_run1d_fp64(grid_of(h), h->nb, h->Q, h->Wbar, h->P, n, cp, h->stream));
   return RIDG_OK;
 }
 

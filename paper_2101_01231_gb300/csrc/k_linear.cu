@@ -17,6 +17,10 @@
 // flux and the cell averages are conserved to round-off of the final additions.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
+#include <utility>
+
 #include "ridg_internal.h"
 
 namespace ridg {
@@ -236,77 +240,144 @@ __global__ void __launch_bounds__(128) correct_modes_kernel(double* __restrict__
   Q[e * THS + s] = Q[e * THS + s] + dq;
 }
 
-// A whole run of n steps of a small 1D mesh in one CTA: the state and the time means stay in
-// shared memory, each step is the prediction (the same sums as predict_fp64_kernel) and the
-// correction (the same sums as correct_linear_kernel<1, NB>) separated by barriers.  Removes
-// the two launches per step that bound tiny meshes.
+// 1D: k steps of a chunk of C cells per block and launch (temporal blocking).  With upwind face
+// values a step reads two cells upstream (the time mean of the upstream neighbour reads one
+// more), so a block that starts from 2k more cells upstream computes its own cells' k steps
+// alone, each step on two cells fewer; blocks recompute each other's cells instead of
+// exchanging them.  The sums are those of predict_fp64_kernel and correct_linear_kernel in the
+// same order (the face value of the side that the velocity does not come from, multiplied by
+// zero there, is left out), so the states are theirs bit for bit.
+//
+// A step costs ~0.8 us of dependent FP64 operations and barriers whatever its cells, a launch
+// ~1.7 us, and the FP64 pipe (2 FMA per clock and SM) adds the work of C + k cells on average;
+// run1d_plan weighs the three.  Measured per step, against the whole run in one CTA (or, above
+// 96 KB of state, one launch per kernel and step): 64 cells Q3 2.13 -> 1.14 us, 600 cells Q7 35.8
+// -> 2.0, 1000 cells Q4 27.7 -> 1.6, 100000 cells Q3 37.4 -> 17.6.  Splitting the sums into two
+// halves for a shorter chain gained nothing (1.21 us at 64 cells).
+//
+// One thread per (cell, mode); local cell u counts downstream, own cells are u >= 2k.
 template <int NB>
-__global__ void __launch_bounds__(256) run1d_fp64_kernel(double* __restrict__ Q,
-                                                         const double* __restrict__ P, int n,
-                                                         int nsteps, CorrParams cp, int lo, int nr) {
-  const int K = nr * NB;     // the upwind cells lo .. lo + nr - 1 of the region
+__global__ void __launch_bounds__(768) run1d_chunk_kernel(const double* __restrict__ Qin,
+                                                           double* __restrict__ Qout,
+                                                           const double* __restrict__ P, int n,
+                                                           int k, int C, CorrParams cp, int dir,
+                                                           int nr) {
   extern __shared__ double sm1[];
-  double* sP = sm1;          // NB x K (the time-mean rows)
-  double* sQ = sP + NB * K;  // n x NB
-  double* sW = sQ + n * NB;  // n x NB
-  for (int i = threadIdx.x; i < NB * K; i += blockDim.x) sP[i] = P[i];
-  for (int i = threadIdx.x; i < n * NB; i += blockDim.x) sQ[i] = Q[i];
-  __syncthreads();
-  for (int step = 0; step < nsteps; ++step) {
-    for (int i = threadIdx.x; i < n * NB; i += blockDim.x) {
-      const int c = i / NB, k = i % NB;
-      double acc = 0.0;
-      for (int r = 0; r < nr; ++r) {
-        const double* q = sQ + wrap(c + lo + r, n) * NB;
-        const double* p = sP + k * K + r * NB;
+  const int U = C + 2 * k;
+  double* sQ = sm1;           // U x NB
+  double* sW = sQ + U * NB;   // time means
+  double* sF = sW + U * NB;   // value of the cell's downstream face
+  const int tid = threadIdx.x, u = tid / NB, a = tid - u * NB;
+  const bool act = u < U;
+  // flow coordinate of the cell (periodic), its global cell
+  int f = (int)((blockIdx.x * (long long)C + u - 2 * k) % n);
+  f += f < 0 ? n : 0;
+  const long long g = (long long)(dir > 0 ? f : n - 1 - f) * NB + a;
+  double q = act ? Qin[g] : 0.0;
+  double pr[2 * NB];  // this mode's row of the time-mean operator
 #pragma unroll
-        for (int s2 = 0; s2 < NB; ++s2) acc = fma(p[s2], q[s2], acc);
+  for (int i = 0; i < 2 * NB; ++i) pr[i] = i < nr * NB ? P[(size_t)a * nr * NB + i] : 0.0;
+  const double nu = cp.nu[0], ep = cp.ep[a], em = cp.em[a];
+  double tc[NB];  // the downstream face's trace
+#pragma unroll
+  for (int b = 0; b < NB; ++b) tc[b] = dir > 0 ? cp.ep[b] : cp.em[b];
+  const double nf = dir > 0 ? cp.nup[0] : cp.num[0];
+  double d[NB];  // row a of D, zero where a <= b or a + b is even
+#pragma unroll
+  for (int b = 0; b < NB; ++b) d[b] = a > b && ((a + b) & 1) ? cp.D[a * kMaxNB + b] : 0.0;
+  if (act) sQ[tid] = q;
+  __syncthreads();
+  // the region's cells lo + 0, lo + 1: upstream and own for a > 0, own and upstream for a < 0
+  const int r0 = nr == 2 ? (dir > 0 ? -NB : 0) : 0, r1 = dir > 0 ? 0 : -NB;
+  for (int j = 1; j <= k; ++j) {
+    if (act && u >= 2 * j - 1) {
+      const double* x = sQ + u * NB;
+      double acc = 0.0;
+#pragma unroll
+      for (int s2 = 0; s2 < NB; ++s2) acc = fma(pr[s2], x[r0 + s2], acc);
+      if (nr == 2) {
+#pragma unroll
+        for (int s2 = 0; s2 < NB; ++s2) acc = fma(pr[NB + s2], x[r1 + s2], acc);
       }
-      sW[i] = acc;
+      sW[tid] = acc;
     }
     __syncthreads();
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-      const double* w = sW + c * NB;
-      double dq[NB];
+    double v = 0.0;
+    if (act && u >= 2 * j) {
+      const double* w = sW + u * NB;
+      double acc = 0.0;
 #pragma unroll
-      for (int a = 0; a < NB; ++a) {
-        double acc = 0.0;
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-          if (a > b && ((a + b) & 1)) acc = fma(cp.D[a * kMaxNB + b], w[b], acc);
-        dq[a] = fma(cp.nu[0], acc, 0.0);
-      }
-      double trp, trm, nbt;
-      face_trace<1, NB>(w, 0, cp.ep, &trp);
-      face_trace<1, NB>(w, 0, cp.em, &trm);
-      face_trace<1, NB>(sW + wrap(c + 1, n) * NB, 0, cp.em, &nbt);
-      const double fp = face_value(trp, nbt, cp.nup[0], cp.num[0]);
-      face_trace<1, NB>(sW + wrap(c - 1, n) * NB, 0, cp.ep, &nbt);
-      const double fm = face_value(nbt, trm, cp.nup[0], cp.num[0]);
-#pragma unroll
-      for (int a = 0; a < NB; ++a) {
-        double v = dq[a];
-        v = fma(-cp.ep[a], fp, v);
-        v = fma(cp.em[a], fm, v);
-        sQ[c * NB + a] = sQ[c * NB + a] + v;
-      }
+      for (int b = 0; b < NB; ++b)
+        if (d[b] != 0.0) acc = fma(d[b], w[b], acc);
+      v = fma(nu, acc, 0.0);
+    }
+    if (tid < U && tid >= 2 * j - 1) {
+      double t;
+      face_trace<1, NB>(sW + tid * NB, 0, tc, &t);
+      sF[tid] = nf * t;
+    }
+    __syncthreads();
+    if (act && u >= 2 * j) {
+      const double fp = sF[dir > 0 ? u : u - 1], fm = sF[dir > 0 ? u - 1 : u];
+      v = fma(-ep, fp, v);
+      v = fma(em, fm, v);
+      q = q + v;
+      sQ[tid] = q;
     }
     __syncthreads();
   }
-  for (int i = threadIdx.x; i < n * NB; i += blockDim.x) Q[i] = sQ[i];
+  if (act && u >= 2 * k && blockIdx.x * (long long)C + u - 2 * k < n) Qout[g] = q;
+}
+
+struct Run1dPlan {
+  int C, k;
+};
+// cells per block and steps per launch: the least of  max(chain, FP64 work) + launch / k  per
+// step, in clocks (fitted to a sweep over C and k at 16 to 20000 cells, degrees 1 to 7; its
+// choices are within 10% of the sweep's best)
+Run1dPlan run1d_plan(long long n, int nb, int nsteps, int sms) {
+  const double f = nb * (2.0 * nb + 2.0) + nb * (0.25 * nb + 4.0);  // FP64 operations per cell
+  Run1dPlan best = {1, 1};
+  double cost = 1e300;
+  for (int C : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64})
+    for (int k = 1; k <= 16 && k <= nsteps; ++k) {
+      if ((C + 2 * k) * nb > 768) break;
+      const double blocks = std::ceil((double)n / C);
+      const double work = std::ceil(blocks / std::max(1, sms)) * (C + k) * f / 2.0;
+      const double c = std::max(1200.0 + 60.0 * nb, 700.0 + 1.5 * work) + (3000.0 + 100.0 * nb * nb) / k;
+      if (c < cost) {
+        cost = c;
+        best = {C, k};
+      }
+    }
+  return best;
 }
 
 template <int NB>
-cudaError_t run1d_dispatch(const Grid& g, double* Q, const double* P, int nsteps,
+cudaError_t run1d_dispatch(const Grid& g, double* Q, double* Q2, const double* P, int nsteps,
                            const CorrParams& cp, cudaStream_t s) {
-  const size_t smem = (size_t)(NB * g.box.n * NB + 2 * g.ncell * NB) * sizeof(double);
-  auto kern = run1d_fp64_kernel<NB>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+  int dev = 0, sms = 1;
+  if (cudaGetDevice(&dev) == cudaSuccess)
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const Run1dPlan pl = run1d_plan(g.ncell, NB, nsteps, sms);
+  // an even number of launches leaves the state in Q (a single one is copied back)
+  int launches = (nsteps + pl.k - 1) / pl.k;
+  if ((launches & 1) && launches < nsteps) ++launches;
+  const int dir = g.box.lo[0] < 0 ? 1 : (g.box.cnt[0] > 1 ? -1 : 1);
+  const unsigned blocks = (unsigned)((g.ncell + pl.C - 1) / pl.C);
+  double *in = Q, *out = Q2;
+  for (int l = 0; l < launches; ++l) {
+    const int k = nsteps / launches + (l < nsteps % launches);
+    const int U = pl.C + 2 * k, threads = (U * NB + 31) / 32 * 32;
+    const size_t smem = (size_t)U * (2 * NB + 1) * sizeof(double);
+    run1d_chunk_kernel<NB><<<blocks, threads, smem, s>>>(in, out, P, (int)g.ncell, k, pl.C, cp, dir,
+                                                         g.box.cnt[0]);
+    std::swap(in, out);
   }
-  kern<<<1, 256, smem, s>>>(Q, P, (int)g.ncell, nsteps, cp, g.box.lo[0], g.box.cnt[0]);
-  return cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess && in != Q)
+    e = cudaMemcpyAsync(Q, in, (size_t)g.ncell * NB * sizeof(double), cudaMemcpyDeviceToDevice, s);
+  return e;
 }
 
 template <int DIM, int NB>
@@ -390,28 +461,22 @@ cudaError_t launch_predict_fp64(const Grid& g, int nb, const double* Q, const do
   return cudaErrorInvalidValue;
 }
 
-bool run1d_fits(const Grid& g, int nb) {
-  return g.dim == 1 && nb >= 1 && nb <= kMaxNB && g.ncell <= kRun1dMaxCells &&
-         g.box.n >= 1 && g.box.n <= 2 &&
-         (size_t)(g.box.n * nb * nb + 2 * g.ncell * nb) * sizeof(double) <= 96 * 1024;
-}
-
-cudaError_t launch_run1d_fp64(const Grid& g, int nb, double* Q, const double* P, int nsteps,
-                              const CorrParams& cp, cudaStream_t s) {
-  if (!run1d_fits(g, nb)) return cudaErrorInvalidValue;
+cudaError_t launch_run1d_fp64(const Grid& g, int nb, double* Q, double* Q2, const double* P,
+                              int nsteps, const CorrParams& cp, cudaStream_t s) {
+  if (g.dim != 1 || g.box.n < 1 || g.box.n > 2) return cudaErrorInvalidValue;
   switch (nb) {
-    case 1: return run1d_dispatch<1>(g, Q, P, nsteps, cp, s);
-    case 2: return run1d_dispatch<2>(g, Q, P, nsteps, cp, s);
-    case 3: return run1d_dispatch<3>(g, Q, P, nsteps, cp, s);
-    case 4: return run1d_dispatch<4>(g, Q, P, nsteps, cp, s);
-    case 5: return run1d_dispatch<5>(g, Q, P, nsteps, cp, s);
-    case 6: return run1d_dispatch<6>(g, Q, P, nsteps, cp, s);
-    case 7: return run1d_dispatch<7>(g, Q, P, nsteps, cp, s);
-    case 8: return run1d_dispatch<8>(g, Q, P, nsteps, cp, s);
-    case 9: return run1d_dispatch<9>(g, Q, P, nsteps, cp, s);
-    case 10: return run1d_dispatch<10>(g, Q, P, nsteps, cp, s);
-    case 11: return run1d_dispatch<11>(g, Q, P, nsteps, cp, s);
-    case 12: return run1d_dispatch<12>(g, Q, P, nsteps, cp, s);
+    case 1: return run1d_dispatch<1>(g, Q, Q2, P, nsteps, cp, s);
+    case 2: return run1d_dispatch<2>(g, Q, Q2, P, nsteps, cp, s);
+    case 3: return run1d_dispatch<3>(g, Q, Q2, P, nsteps, cp, s);
+    case 4: return run1d_dispatch<4>(g, Q, Q2, P, nsteps, cp, s);
+    case 5: return run1d_dispatch<5>(g, Q, Q2, P, nsteps, cp, s);
+    case 6: return run1d_dispatch<6>(g, Q, Q2, P, nsteps, cp, s);
+    case 7: return run1d_dispatch<7>(g, Q, Q2, P, nsteps, cp, s);
+    case 8: return run1d_dispatch<8>(g, Q, Q2, P, nsteps, cp, s);
+    case 9: return run1d_dispatch<9>(g, Q, Q2, P, nsteps, cp, s);
+    case 10: return run1d_dispatch<10>(g, Q, Q2, P, nsteps, cp, s);
+    case 11: return run1d_dispatch<11>(g, Q, Q2, P, nsteps, cp, s);
+    case 12: return run1d_dispatch<12>(g, Q, Q2, P, nsteps, cp, s);
     default: return cudaErrorInvalidValue;
   }
 }
