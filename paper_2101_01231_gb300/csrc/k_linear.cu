@@ -66,10 +66,10 @@ __global__ void __launch_bounds__(128) predict_fp64_kernel(const double* __restr
   const int K = box.n * THS;
   extern __shared__ double sP[];  // CH x K
   const int c0 = blockIdx.y * CH;
-  for (int i = threadIdx.x; i < CH * K; i += blockDim.x) {
-    const int c = c0 + i / K;
-    sP[i] = (c < nout) ? P[(size_t)c * K + (i % K)] : 0.0;
-  }
+  const int have = min(CH, nout - c0) * K;  // (CH divides theta_S and theta_T)
+#pragma unroll 8
+  for (int i = threadIdx.x; i < CH * K; i += blockDim.x)
+    sP[i] = i < have ? P[(size_t)c0 * K + i] : 0.0;
   __syncthreads();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= ncell) return;
@@ -100,30 +100,20 @@ __global__ void __launch_bounds__(128) predict_fp64_kernel(const double* __restr
 // ---------------------------------------------------------------------------------------
 // correction
 // ---------------------------------------------------------------------------------------
-// trace of a cell's time mean along dimension dd: tr[t] = sum_b v[b] w[base(t) + b st]
-template <int DIM, int NB>
-__device__ __forceinline__ void face_trace(const double* w, int dd, const double* v,
-                                           double* tr) {
-  constexpr int NT = ipow_c(NB, DIM - 1);
-  const int st = dd == 0 ? 1 : (dd == 1 ? NB : NB * NB);
-#pragma unroll
-  for (int t = 0; t < NT; ++t) {
-    const int lo = t % st, hi = t / st;
-    const int base = lo + hi * st * NB;
-    double a = 0.0;
-#pragma unroll
-    for (int b = 0; b < NB; ++b) a = fma(v[b], w[base + b * st], a);
-    tr[t] = a;
-  }
+// The value of a face from the upwind cell's trace there: nu_d^+ tr_+(left) for nu_d > 0, nu_d^-
+// tr_-(right) for nu_d < 0 (the other side's coefficient is zero), one product of one sum in a
+// fixed order, so both neighbours evaluate it bit-identically.
+struct Upwind {
+  double nf;        // nu_d
+  const double* v;  // phi_b(+1) or phi_b(-1)
+  int up;           // offset of the upstream cell along d (0: no flux along d)
+};
+__device__ __forceinline__ Upwind upwind_of(const CorrParams& cp, int dd) {
+  return cp.nu[dd] > 0.0 ? Upwind{cp.nu[dd], cp.ep, -1}
+                         : Upwind{cp.nu[dd], cp.em, cp.nu[dd] < 0.0 ? 1 : 0};
 }
 
-// The single definition of a face value from the two traces at that face (explicit fma,
-// so both neighbours evaluate it bit-identically).
-__device__ __forceinline__ double face_value(double tr_left_plus, double tr_right_minus, double nup,
-                                          double num) {
-  return fma(nup, tr_left_plus, num * tr_right_minus);
-}
-
+// One thread per cell: the time means of the cell and of its upstream neighbour per direction.
 template <int DIM, int NB>
 __global__ void __launch_bounds__(128) correct_linear_kernel(double* __restrict__ Q,
                                                              const double* __restrict__ Wb,
@@ -134,7 +124,7 @@ __global__ void __launch_bounds__(128) correct_linear_kernel(double* __restrict_
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= ncell) return;
   const Coords c = cell_coords(e, nx, ny);
-  double w[THS], dq[THS], nbw[THS];
+  double w[THS], dq[THS];
 #pragma unroll
   for (int s = 0; s < THS; ++s) {
     w[s] = Wb[e * wstride + s];
@@ -143,10 +133,13 @@ __global__ void __launch_bounds__(128) correct_linear_kernel(double* __restrict_
 #pragma unroll
   for (int dd = 0; dd < DIM; ++dd) {
     const int st = dd == 0 ? 1 : (dd == 1 ? NB : NB * NB);
-    // volume term nu_d (D along d) Wbar
+    const Upwind uw = upwind_of(cp, dd);
+    const double* wu = Wb + neighbour<DIM>(c, dd == 0 ? uw.up : 0, dd == 1 ? uw.up : 0,
+                                           dd == 2 ? uw.up : 0, nx, ny, nz) * wstride;
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
       const int base = t % st + (t / st) * st * NB;
+      // volume term nu_d (D along d) Wbar
 #pragma unroll
       for (int a = 0; a < NB; ++a) {
         double acc = 0.0;
@@ -155,36 +148,19 @@ __global__ void __launch_bounds__(128) correct_linear_kernel(double* __restrict_
           if (a > b && ((a + b) & 1)) acc = fma(cp.D[a * kMaxNB + b], w[base + b * st], acc);
         dq[base + a * st] = fma(cp.nu[dd], acc, dq[base + a * st]);
       }
-    }
-    double trp[NT], trm[NT], nbt[NT], fp[NT], fm[NT];
-    face_trace<DIM, NB>(w, dd, cp.ep, trp);
-    face_trace<DIM, NB>(w, dd, cp.em, trm);
-    // right neighbour's trace at its xi_d = -1
-    {
-      const long long j = neighbour<DIM>(c, dd == 0, dd == 1, dd == 2, nx, ny, nz);
+      double to = 0.0, tu = 0.0;
 #pragma unroll
-      for (int s = 0; s < THS; ++s) nbw[s] = Wb[j * wstride + s];
-      face_trace<DIM, NB>(nbw, dd, cp.em, nbt);
-#pragma unroll
-      for (int t = 0; t < NT; ++t) fp[t] = face_value(trp[t], nbt[t], cp.nup[dd], cp.num[dd]);
-    }
-    // left neighbour's trace at its xi_d = +1
-    {
-      const long long j = neighbour<DIM>(c, -(dd == 0), -(dd == 1), -(dd == 2), nx, ny, nz);
-#pragma unroll
-      for (int s = 0; s < THS; ++s) nbw[s] = Wb[j * wstride + s];
-      face_trace<DIM, NB>(nbw, dd, cp.ep, nbt);
-#pragma unroll
-      for (int t = 0; t < NT; ++t) fm[t] = face_value(nbt[t], trm[t], cp.nup[dd], cp.num[dd]);
-    }
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const int base = t % st + (t / st) * st * NB;
+      for (int b = 0; b < NB; ++b) {
+        to = fma(uw.v[b], w[base + b * st], to);
+        tu = fma(uw.v[b], wu[base + b * st], tu);
+      }
+      const double fo = uw.nf * to, fu = uw.nf * tu;
+      const double fp = uw.up > 0 ? fu : fo, fm = uw.up > 0 ? fo : fu;
 #pragma unroll
       for (int a = 0; a < NB; ++a) {
         double v = dq[base + a * st];
-        v = fma(-cp.ep[a], fp[t], v);
-        v = fma(cp.em[a], fm[t], v);
+        v = fma(-cp.ep[a], fp, v);
+        v = fma(cp.em[a], fm, v);
         dq[base + a * st] = v;
       }
     }
@@ -194,12 +170,11 @@ __global__ void __launch_bounds__(128) correct_linear_kernel(double* __restrict_
   for (int s = 0; s < THS; ++s) q[s] = q[s] + dq[s];
 }
 
-// The same correction with one thread per (cell, mode) output, for large theta_S (3D,
-// degree >= 4) where a thread holding a whole cell's time mean would spill.  Mode s has the
-// digit a = s_d along dimension d and lies on the fibre base + b st of that dimension; every
-// sum runs in the order of correct_linear_kernel (volume term, then the two face values,
-// each face value from the same traces by face_value), so both neighbours of a face apply
-// bitwise the same flux and the result equals correct_linear_kernel's bit for bit.
+// The same correction with one thread per (cell, mode) output: for large theta_S (3D, degree
+// >= 4), where a thread holding a whole cell's time mean would spill, and for small meshes,
+// which one thread per cell leaves on a few SMs.  Mode s has the digit a = s_d along dimension
+// d and lies on the fibre base + b st of that dimension; every sum runs in the order of
+// correct_linear_kernel, so the results are its bits.
 template <int DIM, int NB>
 __global__ void __launch_bounds__(128) correct_modes_kernel(double* __restrict__ Q,
                                                             const double* __restrict__ Wb,
@@ -222,18 +197,17 @@ __global__ void __launch_bounds__(128) correct_modes_kernel(double* __restrict__
     for (int b = 0; b < NB; ++b)
       if (b < a && ((a + b) & 1)) acc = fma(cp.D[a * kMaxNB + b], w[base + b * st], acc);
     dq = fma(cp.nu[dd], acc, dq);
-    double trp = 0.0, trm = 0.0, nbp = 0.0, nbm = 0.0;
-    const double* wr = Wb + neighbour<DIM>(c, dd == 0, dd == 1, dd == 2, nx, ny, nz) * wstride;
-    const double* wl = Wb + neighbour<DIM>(c, -(dd == 0), -(dd == 1), -(dd == 2), nx, ny, nz) * wstride;
+    const Upwind uw = upwind_of(cp, dd);
+    const double* wu = Wb + neighbour<DIM>(c, dd == 0 ? uw.up : 0, dd == 1 ? uw.up : 0,
+                                           dd == 2 ? uw.up : 0, nx, ny, nz) * wstride;
+    double to = 0.0, tu = 0.0;
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-      trp = fma(cp.ep[b], w[base + b * st], trp);
-      trm = fma(cp.em[b], w[base + b * st], trm);
-      nbm = fma(cp.em[b], wr[base + b * st], nbm);
-      nbp = fma(cp.ep[b], wl[base + b * st], nbp);
+      to = fma(uw.v[b], w[base + b * st], to);
+      tu = fma(uw.v[b], wu[base + b * st], tu);
     }
-    const double fp = face_value(trp, nbm, cp.nup[dd], cp.num[dd]);
-    const double fm = face_value(nbp, trm, cp.nup[dd], cp.num[dd]);
+    const double fo = uw.nf * to, fu = uw.nf * tu;
+    const double fp = uw.up > 0 ? fu : fo, fm = uw.up > 0 ? fo : fu;
     dq = fma(-cp.ep[a], fp, dq);
     dq = fma(cp.em[a], fm, dq);
   }
@@ -245,8 +219,7 @@ __global__ void __launch_bounds__(128) correct_modes_kernel(double* __restrict__
 // more), so a block that starts from 2k more cells upstream computes its own cells' k steps
 // alone, each step on two cells fewer; blocks recompute each other's cells instead of
 // exchanging them.  The sums are those of predict_fp64_kernel and correct_linear_kernel in the
-// same order (the face value of the side that the velocity does not come from, multiplied by
-// zero there, is left out), so the states are theirs bit for bit.
+// same order, so the states are theirs bit for bit.
 //
 // A step costs ~0.8 us of dependent FP64 operations and barriers whatever its cells, a launch
 // ~1.7 us, and the FP64 pipe (2 FMA per clock and SM) adds the work of C + k cells on average;
@@ -281,7 +254,7 @@ __global__ void __launch_bounds__(768) run1d_chunk_kernel(const double* __restri
   double tc[NB];  // the downstream face's trace
 #pragma unroll
   for (int b = 0; b < NB; ++b) tc[b] = dir > 0 ? cp.ep[b] : cp.em[b];
-  const double nf = dir > 0 ? cp.nup[0] : cp.num[0];
+  const double nf = cp.nu[0];
   double d[NB];  // row a of D, zero where a <= b or a + b is even
 #pragma unroll
   for (int b = 0; b < NB; ++b) d[b] = a > b && ((a + b) & 1) ? cp.D[a * kMaxNB + b] : 0.0;
@@ -312,8 +285,9 @@ __global__ void __launch_bounds__(768) run1d_chunk_kernel(const double* __restri
       v = fma(nu, acc, 0.0);
     }
     if (tid < U && tid >= 2 * j - 1) {
-      double t;
-      face_trace<1, NB>(sW + tid * NB, 0, tc, &t);
+      double t = 0.0;
+#pragma unroll
+      for (int b = 0; b < NB; ++b) t = fma(tc[b], sW[tid * NB + b], t);
       sF[tid] = nf * t;
     }
     __syncthreads();
@@ -327,6 +301,14 @@ __global__ void __launch_bounds__(768) run1d_chunk_kernel(const double* __restri
     __syncthreads();
   }
   if (act && u >= 2 * k && blockIdx.x * (long long)C + u - 2 * k < n) Qout[g] = q;
+}
+
+int device_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return 1;
+  return sms;
 }
 
 struct Run1dPlan {
@@ -356,10 +338,7 @@ Run1dPlan run1d_plan(long long n, int nb, int nsteps, int sms) {
 template <int NB>
 cudaError_t run1d_dispatch(const Grid& g, double* Q, double* Q2, const double* P, int nsteps,
                            const CorrParams& cp, cudaStream_t s) {
-  int dev = 0, sms = 1;
-  if (cudaGetDevice(&dev) == cudaSuccess)
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const Run1dPlan pl = run1d_plan(g.ncell, NB, nsteps, sms);
+  const Run1dPlan pl = run1d_plan(g.ncell, NB, nsteps, device_sms());
   // an even number of launches leaves the state in Q (a single one is copied back)
   int launches = (nsteps + pl.k - 1) / pl.k;
   if ((launches & 1) && launches < nsteps) ++launches;
@@ -380,18 +359,30 @@ cudaError_t run1d_dispatch(const Grid& g, double* Q, double* Q2, const double* P
   return e;
 }
 
+// Rows of P per thread: a divisor of theta_S, 2 to 5, so that no row is padding and meshes of a
+// few thousand cells have warps for every SM.  Measured against 16 rows (8 and 4 in 3D) by
+// blocks of 128 threads, the time-mean prediction: 2D Q5 60^2 94.7 -> 43.5 us, Q3 256^2 138 ->
+// 121, Q2 160^2 29 -> 21; 3D Q2 16^3 92 -> 53, Q3 8^3 164 -> 97, Q3 48^3 5.88 -> 5.86 ms.
+template <int DIM, int NB>
+struct PredictRows {
+  static constexpr int value = DIM == 1 ? NB
+                               : NB == 1 ? 1
+                               : NB == 2 ? 2
+                               : NB == 3 ? 3
+                               : NB == 5 ? 5
+                                         : 4;
+};
+
 template <int DIM, int NB>
 cudaError_t predict_dispatch_ch(const Grid& g, const double* Q, const double* P, int nout,
                                 double* W, int wstride, cudaStream_t s) {
-  constexpr int THS = ipow_c(NB, DIM);
-  constexpr int KMAX = ipow_c(2, DIM) * THS;  // the largest upwind box: 2^d cells
-  // rows per thread: as many as fit 48 KB of shared memory, at most 16
-  constexpr int CH = (16 * KMAX * 8 <= 48 * 1024) ? 16 : ((8 * KMAX * 8 <= 48 * 1024) ? 8 : 4);
+  constexpr int CH = PredictRows<DIM, NB>::value;
   if (g.box.n < 1 || g.box.n > ipow_c(2, DIM)) return cudaErrorInvalidValue;
-  const int K = g.box.n * THS;
-  const int threads = 128;
-  dim3 grid((unsigned)((g.ncell + threads - 1) / threads), (unsigned)((nout + CH - 1) / CH));
-  size_t smem = (size_t)CH * K * sizeof(double);
+  const size_t smem = (size_t)CH * g.box.n * ipow_c(NB, DIM) * sizeof(double);
+  // one-warp blocks spread best; larger ones where each block's copy of its rows of P would
+  // cost more than that gains (3D Q4, Q5: 40 and 55 KB)
+  const int threads = smem <= 8 * 1024 ? 32 : smem <= 20 * 1024 ? 64 : 128;
+  const dim3 grid((unsigned)((g.ncell + threads - 1) / threads), (unsigned)((nout + CH - 1) / CH));
   auto kern = predict_fp64_kernel<DIM, NB, CH>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -405,11 +396,14 @@ template <int DIM, int NB>
 cudaError_t correct_dispatch(const Grid& g, double* Q, const double* Wb, int wstride,
                              const CorrParams& cp, cudaStream_t s) {
   const int threads = 128;
-  if constexpr (DIM == 3 && NB >= 5) {
+  // a thread per mode below ~45 cells per SM (2D Q3, 24 cells per SM: 10.9 against 17.4 us; 66:
+  // 19.1 against 17.0)
+  const bool modes = (DIM == 3 && NB >= 5) || g.ncell < 45LL * device_sms();
+  if (modes) {
     const unsigned blocks = (unsigned)((g.ncell * ipow_c(NB, DIM) + threads - 1) / threads);
     correct_modes_kernel<DIM, NB><<<blocks, threads, 0, s>>>(Q, Wb, wstride, g.n[0], g.n[1],
                                                              g.n[2], g.ncell, cp);
-  } else {
+  } else if constexpr (!(DIM == 3 && NB >= 5)) {
     const unsigned blocks = (unsigned)((g.ncell + threads - 1) / threads);
     correct_linear_kernel<DIM, NB><<<blocks, threads, 0, s>>>(Q, Wb, wstride, g.n[0], g.n[1],
                                                               g.n[2], g.ncell, cp);
