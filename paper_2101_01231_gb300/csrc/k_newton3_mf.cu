@@ -27,7 +27,7 @@ namespace {
 
 constexpr int kCols = 216, kNT = 224, kNW = kNT / 32;
 constexpr int kFaceLines = 432;  // 3 directions x 9 rows x 4 faces x 4 tangential nodes
-constexpr int kMaxRefine3 = 5, kMaxInner3 = 24;
+constexpr int kMaxRefine3 = 8, kMaxInner3 = 32;
 constexpr double kS3 = 1.7320508075688772935;
 
 // the two face lines of a thread: first nodes left / right of the face (-1 outside the
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kNT, 4) newton3_mf_kernel(const Newton3Args a)
       const float bb = m1[0], bmean = sqrtf(bb / (2 * kCols)) * (float)unscale;
       const float tol = fminf(F64 ? 1e-3f : 1e-2f, fmaxf(F64 ? 3e-6f : 1e-6f, (F64 ? 1e-17f : 1e-15f) * wnorm / bmean));
       const float stop = tol * tol * bb;
-      float rho = bb, rr = bb;
+      float rho = bb, rr = bb, hh = bb;
       auto apply = [&](const float (&in)[2], float (&out)[2]) {
         float s[2];
         spatial<float, true>(Cf, L, Sf, in, s, P, Fh);
@@ -277,17 +277,23 @@ __global__ void __launch_bounds__(kNT, 4) newton3_mf_kernel(const Newton3Args a)
           rv[i] -= om * t[i];
         }
         rr = fmaxf(0.f, s4[3] - om * s4[0]);
-        const float rho1 = -om * s4[2], be = rho1 / rho * (al / om);
-        rho = rho1;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) p[i] = rv[i] + be * (p[i] - om * v[i]);
-        // (a vanished residual leaves be undefined)
-        if (!(fabsf(al) < 1e30f) || !(rr < 1e30f) || (rr > stop && !(fabsf(be) < 1e30f))) {
+        if (!(fabsf(al) < 1e30f) || !(rr < 1e30f)) {
           ok = false;
           break;
         }
+        const float rho1 = -om * s4[2];
+        if (rho1 * rho1 <= 1e-5f * rr * hh) {  // about to stall: start anew (k_newton_mf.cuh)
+          rh[0] = p[0] = rv[0];
+          rh[1] = p[1] = rv[1];
+          rho = hh = rr;
+          continue;
+        }
+        const float be = rho1 / rho * (al / om);
+        rho = rho1;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) p[i] = rv[i] + be * (p[i] - om * v[i]);
       }
-      if (!ok || rr > 1e-2f * bb) {
+      if (!ok || rr > 0.1f * bb) {
         ok = false;
         break;
       }

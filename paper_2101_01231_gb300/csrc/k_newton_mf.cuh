@@ -782,8 +782,8 @@ __device__ __forceinline__ void apply(const Tab<NB>& T, const Rows<NB>& R, const
 }
 
 constexpr int kMaxSolves = 7;   // linear solves of a region (mixed) before it is left to the list
-constexpr int kMaxRefine = 5;   // FP32 solves per Newton iteration (FP64) before that
-constexpr int kMaxInner = 24;   // BiCGStab iterations per solve
+constexpr int kMaxRefine = 8;   // FP32 solves per Newton iteration (FP64) before that
+constexpr int kMaxInner = 32;   // BiCGStab iterations per solve
 
 // The linearisation point at W: F' at the thread's nodes and at both sides of its face line.
 template <int NB, int MV>
@@ -890,7 +890,7 @@ __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
   const float bmean = sqrtf(bb / (9 * K::BS)) / (float)scale;
   const float tol = fminf(rmax, fmaxf(rmin, atol / bmean));
   const float stop = tol * tol * bb;
-  float rho = bb, rr = bb;
+  float rho = bb, rr = bb, hh = bb;  // <rh, r>, |r|^2, |rh|^2
 #pragma unroll 1
   for (int k = 0; k < kMaxInner && rr > stop; ++k) {
     apply<NB, MV, FLUX>(T, R, S, p, v, P, G, Fh, g1);
@@ -920,16 +920,24 @@ __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
       r[q] = fmaf(-om, t[q], r[q]);
     }
     rr = fmaxf(0.f, s4[3] - om * s4[0]);
+    if (!(fabsf(al) < 1e30f) || !(rr < 1e30f)) return false;
     const float rho1 = -om * s4[2];  // <rh, r>, as <rh, s> = 0
+    if (rho1 * rho1 <= 1e-5f * rr * hh) {
+      // r is all but orthogonal to the shadow vector, and the method about to stall (a few
+      // regions in ten thousand, mostly with right-hand sides of round-off size): start anew
+      // from r
+#pragma unroll
+      for (int q = 0; q < VT; ++q) rh[q] = p[q] = r[q];
+      rho = hh = rr;
+      continue;
+    }
     const float be = rho1 / rho * (al / om);
     rho = rho1;
 #pragma unroll
     for (int q = 0; q < VT; ++q) p[q] = fmaf(be, fmaf(-om, v[q], p[q]), r[q]);
-    if (!(fabsf(al) < 1e30f) || !(rr < 1e30f)) return false;
-    // (a vanished residual leaves be undefined)
-    if (rr > stop && !(fabsf(be) < 1e30f)) return false;
   }
-  if (rr > 1e-2f * bb) return false;
+  // (what a slow solve leaves is the next one's right-hand side)
+  if (rr > 0.1f * bb) return false;
   ratio = bb > 0.f ? sqrtf(rr / bb) : 0.f;
   // the modes of x
   __syncthreads();
