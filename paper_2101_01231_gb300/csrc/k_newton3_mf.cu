@@ -259,7 +259,18 @@ __global__ void __launch_bounds__(kNT, 4) newton3_mf_kernel(const Newton3Args a)
         if (!col) out[0] = out[1] = 0.f;
       };
 #pragma unroll 1
-      for (int k = 0; k < kMaxInner3 && rr > stop; ++k) {
+      for (int k = 0; k < 2 * kMaxInner3 && rr > stop; ++k) {
+        if (k == kMaxInner3) {  // stalled: again with another shadow vector (k_newton_mf.cuh)
+          if (rr <= 0.1f * bb) break;
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            p[i] = rv[i];
+            rh[i] = (tid & 1) ? 0.f : rv[i];
+          }
+          m1[0] = rh[0] * rv[0] + rh[1] * rv[1];
+          nl::reduce<kNW, 1, false>(m1, red, buf);
+          rho = hh = m1[0];
+        }
         apply(p, v);
         m1[0] = rh[0] * v[0] + rh[1] * v[1];
         nl::reduce<kNW, 1, false>(m1, red, buf);

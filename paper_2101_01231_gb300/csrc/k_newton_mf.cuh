@@ -66,9 +66,9 @@ struct Cfg {
   static constexpr int FL = 24 * NB;                // face lines: 24 faces, NB lines each
   static constexpr int NG = MV == 1 ? 1 : 2;        // Burgers: one flux for both directions
   static_assert(FL <= NT, "one thread per face line");
-  // CTAs per SM that the registers are held to (168 / 128 / 96 a thread at Euler, Burgers Q4,
-  // Burgers Q2 and Q3; unbounded they are 127 to 254 and one CTA fewer fits)
-  static constexpr int MINB = F64 && MV == 4 ? 2 : MV == 4 ? (NB == 2 ? 5 : 4) : (NB == 2 ? 8 : NB == 3 ? 6 : NB == 4 ? 4 : 2);
+  // CTAs per SM that the registers are held to: the best of a sweep (Euler Q2: 3 and 2 leave no
+  // spills, 4.53 against 5.02 ms at 96^2 with 4; Burgers Q3: 6, 2.26 against 2.37 ms with 4)
+  static constexpr int MINB = MV == 4 ? (NB == 2 ? 5 : F64 ? 2 : 3) : (NB == 2 ? 9 : NB == 3 ? 5 : NB == 4 ? 6 : 2);
   // FP64 arena: B1, B2 (line buffers), face fluxes; the face traces share B2
   static constexpr int nB = C * NB * NQ * NQ, nTr = 4 * C * NB * NQ, nH = 24 * MV * NB * NQ;
   static constexpr int nB2 = nB > nTr ? nB : nTr;
@@ -645,7 +645,7 @@ __device__ __forceinline__ void lines(const Tab<NB>& T, float* P, bool ydir) {
 
 // modal FP64 field src (scaled) to FP32 values at the (y, x) nodes, time still modal
 template <int NB, int MV>
-__device__ __forceinline__ void to_nodes(const Tab<NB>& T, const double* src, double scale,
+__device__ __forceinline__ void to_nodes(const Tab<NB>& T, const double* src, float scale,
                                          float* P) {
   using K = Cfg<NB, MV>;
   for (int i = threadIdx.x; i < K::VT * 9 * NB; i += K::NT) {
@@ -654,7 +654,7 @@ __device__ __forceinline__ void to_nodes(const Tab<NB>& T, const double* src, do
     const double* s = src + ((r * MV + j) * NB + a) * K::THS + y * NB;
     float in[NB];
 #pragma unroll
-    for (int b = 0; b < NB; ++b) in[b] = (float)(s[b] * scale);
+    for (int b = 0; b < NB; ++b) in[b] = (float)s[b] * scale;
     float* p = P + tj * K::COL + r * K::THS + y * NB;
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
@@ -792,7 +792,7 @@ __device__ __forceinline__ void linearise(const Tab<NB>& T, const double* Ws, co
   using K = Cfg<NB, MV>;
   constexpr int VT = K::VT, COL = K::COL;
   const int tid = threadIdx.x;
-  to_nodes<NB, MV>(T, Ws, 1.0, P);
+  to_nodes<NB, MV>(T, Ws, 1.f, P);
   if (tid < COL) {
     float m[VT], w[VT];
 #pragma unroll
@@ -849,7 +849,7 @@ __device__ __forceinline__ void linearise(const Tab<NB>& T, const double* Ws, co
 // residual reached in `ratio`.  False if it stalled.
 template <int NB, int MV, int FLUX>
 __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
-                                         const Lin<NB, MV>& S, const double* Rs, double scale,
+                                         const Lin<NB, MV>& S, const double* Rs, float scale,
                                          float atol, float rmin, float rmax, float* P, float* G,
                                          float* Fh, float* red, int& buf, float g1,
                                          float& ratio) {
@@ -887,14 +887,28 @@ __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
     s4[0] = s1[0];
   }
   const float bb = s4[0];
-  const float bmean = sqrtf(bb / (9 * K::BS)) / (float)scale;
+  const float bmean = sqrtf(bb / (9 * K::BS)) / scale;
   const float tol = fminf(rmax, fmaxf(rmin, atol / bmean));
   const float stop = tol * tol * bb;
   float rho = bb, rr = bb, hh = bb;  // <rh, r>, |r|^2, |rh|^2
 #pragma unroll 1
-  for (int k = 0; k < kMaxInner && rr > stop; ++k) {
-    apply<NB, MV, FLUX>(T, R, S, p, v, P, G, Fh, g1);
+  for (int k = 0; k < 2 * kMaxInner && rr > stop; ++k) {
     float s1[1] = {0.f};
+    if (k == kMaxInner) {
+      if (rr <= 0.1f * bb) break;
+      // stalled (a few regions in ten thousand, with right-hand sides of round-off size): again
+      // from r with another shadow vector, every second column of r
+#pragma unroll
+      for (int q = 0; q < VT; ++q) {
+        p[q] = r[q];
+        rh[q] = (tid & 1) ? 0.f : r[q];
+        s1[0] = fmaf(rh[q], r[q], s1[0]);
+      }
+      reduce<NW, 1, false>(s1, red, buf);
+      rho = hh = s1[0];
+      s1[0] = 0.f;
+    }
+    apply<NB, MV, FLUX>(T, R, S, p, v, P, G, Fh, g1);
     if (tid < COL)
 #pragma unroll
       for (int q = 0; q < VT; ++q) s1[0] = fmaf(rh[q], v[q], s1[0]);
@@ -923,8 +937,7 @@ __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
     if (!(fabsf(al) < 1e30f) || !(rr < 1e30f)) return false;
     const float rho1 = -om * s4[2];  // <rh, r>, as <rh, s> = 0
     if (rho1 * rho1 <= 1e-5f * rr * hh) {
-      // r is all but orthogonal to the shadow vector, and the method about to stall (a few
-      // regions in ten thousand, mostly with right-hand sides of round-off size): start anew
+      // r is all but orthogonal to the shadow vector, and the method about to stall: start anew
       // from r
 #pragma unroll
       for (int q = 0; q < VT; ++q) rh[q] = p[q] = r[q];
@@ -960,18 +973,33 @@ __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
   return true;
 }
 
-// the largest |Rs| (3e38 if one is not finite), as a power of two in ex; false if unusable
+// The largest |x| of a thread's FP64 values by their high words (positive doubles order like
+// their bits; no FP64 operation): a lower bound to 2^-20, infinite if one is not finite.
+struct MaxAbs {
+  int hi = 0;
+  __device__ __forceinline__ void add(double x) { hi = max(hi, __double2hiint(x) & 0x7fffffff); }
+};
+
+// the block's largest |x| of MaxAbs values, rounded down; 3e38 if not finite or above 1e30
+template <int NW>
+__device__ __forceinline__ float block_max(MaxAbs m, float* red, int& buf) {
+  float v[1] = {__int_as_float(m.hi)};  // (an order of the bits, NaN patterns aside)
+  // high words up to 0x7f7fffff are finite FP32 patterns; larger ones (|x| >= 2^1016) are cut
+  v[0] = m.hi < 0x7f000000 ? v[0] : __int_as_float(0x7f000000);
+  nl::reduce<NW, 1, true>(v, red, buf);
+  const int hi = __float_as_int(v[0]);
+  const double d = __hiloint2double(hi, 0);
+  return hi < 0x46293e59 ? __double2float_rd(d) : 3e38f;  // 0x46293e59: 1e30
+}
+
+// the largest |Rs| and its exponent ex; false if unusable
 template <int NB, int MV>
 __device__ __forceinline__ bool rhs_scale(const double* Rs, float* red, int& buf, float& rmax,
                                           int& ex) {
   using K = Cfg<NB, MV>;
-  float m[1] = {0.f};
-  for (int i = threadIdx.x; i < 9 * K::BS; i += K::NT) {
-    const double x = fabs(Rs[i]);
-    m[0] = x <= 1e30 ? fmaxf(m[0], (float)x) : 3e38f;  // (a NaN compares false)
-  }
-  reduce<K::NW, 1, true>(m, red, buf);
-  rmax = m[0];
+  MaxAbs m;
+  for (int i = threadIdx.x; i < 9 * K::BS; i += K::NT) m.add(Rs[i]);
+  rmax = block_max<K::NW>(m, red, buf);
   ex = rmax > 1e-30f ? ilogbf(rmax) : -100;
   return rmax <= 1e30f;
 }
@@ -1036,7 +1064,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
   }
   const unsigned ue = (unsigned)e, uy = ue / (unsigned)nx;
   const int ix = (int)(ue - uy * (unsigned)nx), iy = (int)uy;
-  float wmax[1] = {0.f};
+  MaxAbs wmax;
   for (int i = tid; i < 9 * MV * THS; i += NT) {
     const int r = i / (MV * THS), rem = i - r * (MV * THS);
     int cx = ix + r % 3 - 1, cy = iy + r / 3 - 1;
@@ -1044,7 +1072,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
     cy += cy < 0 ? ny : (cy >= ny ? -ny : 0);
     const double q = Qg[((long long)cy * nx + cx) * (MV * THS) + rem];
     Qs[i] = q;
-    wmax[0] = fmaxf(wmax[0], (float)fabs(q));
+    wmax.add(q);
     const int j = rem / THS, s = rem - j * THS;
     double* w = Ws + (r * MV + j) * K::THT + s;  // Q^n extended constant in time
     w[0] = q;
@@ -1052,8 +1080,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
     for (int t = 1; t < NB; ++t) w[t * THS] = 0.0;
   }
   int buf = 0;
-  reduce<NW, 1, true>(wmax, red, buf);
-  float wnorm = wmax[0];
+  float wnorm = block_max<NW>(wmax, red, buf);
 
   // thread constants
   Rows<NB> R;
@@ -1085,8 +1112,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
   const float g1 = keep((float)(a.gamma - 1.0));
   int it = 0;
   bool conv = false, lin = true;
-  double dprev = 0.0;
-  float bprev = 0.f;
+  float dprev = 0.f, bprev = 0.f;
   const int solves = F64 ? a.max_iters : kMaxSolves;
 #pragma unroll 1
   for (int solve = 0; solve < solves; ++solve) {
@@ -1107,63 +1133,72 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
       lin = F64;
       ++it;
     }
-    float mx[2] = {0.f, 0.f}, ratio;
+    // the update: its largest entry, rounded up so that the test below is never looser than
+    // with FP64 maxima (the FP32 modes in P, unscaled by a power of two, are exact; FP64 ones are
+    // known from their high words), and the iterate's, rounded down
+    float ratio, dn;
+    MaxAbs wm;
     if constexpr (!F64) {
       // relative accuracy: 1e-4 in the first solve (whose result the nonlinearity limits), then
       // down to an absolute ~1e-15 of the iterate, at most 1e-5 (FP32)
       const float rmin = solve == 0 ? 1e-4f : 1e-5f, rtop = solve == 0 ? 1e-4f : 1e-2f;
-      if (!bicgstab<NB, MV, FLUX>(T, R, S, Rs, scalbn(1.0, -ex), 1e-15f * wnorm, rmin, rtop, P, G,
+      if (!bicgstab<NB, MV, FLUX>(T, R, S, Rs, scalbnf(1.f, -ex), 1e-15f * wnorm, rmin, rtop, P, G,
                                   Fh, red, buf, g1, ratio))
         break;
       const double unscale = scalbn(1.0, ex);
+      float zm[1] = {0.f};
       for (int i = tid; i < 9 * BS; i += NT) {
-        const double d = unscale * (double)P[p_index<NB, MV>(i)];
-        const double w = Ws[i] - d;
+        const float z = P[p_index<NB, MV>(i)];
+        const double w = fma(-unscale, (double)z, Ws[i]);
         Ws[i] = w;
-        // (rounded up, so that the FP32 comparison below is never the looser one)
-        mx[0] = isfinite(d) ? fmaxf(mx[0], __double2float_ru(fabs(d))) : 3e38f;
-        mx[1] = isfinite(w) ? fmaxf(mx[1], __double2float_rd(fabs(w))) : 3e38f;
+        zm[0] = fabsf(z) <= 1e30f ? fmaxf(zm[0], fabsf(z)) : 3e38f;  // (a NaN compares false)
+        wm.add(w);
       }
+      reduce<NW, 1, true>(zm, red, buf);
+      dn = zm[0] <= 1e30f ? scalbnf(zm[0], ex) : 3e38f;
     } else {
       bool ok = true;
 #pragma unroll 1
       for (int ref = 0;; ++ref) {
         if (ref > 0 && !rhs_scale<NB, MV>(Rs, red, buf, rmax, ex)) ok = false;
         ok = ok && ref < kMaxRefine &&
-             bicgstab<NB, MV, FLUX>(T, R, S, Rs, scalbn(1.0, -ex), 1e-17f * wnorm, 3e-6f, 1e-3f,
+             bicgstab<NB, MV, FLUX>(T, R, S, Rs, scalbnf(1.f, -ex), 1e-17f * wnorm, 3e-6f, 1e-3f,
                                     P, G, Fh, red, buf, g1, ratio);
         if (!ok) break;
         const double unscale = scalbn(1.0, ex);
         float zm[1] = {0.f};
         for (int i = tid; i < 9 * BS; i += NT) {
-          const double z = unscale * (double)P[p_index<NB, MV>(i)];
+          const float zf = P[p_index<NB, MV>(i)];
+          const double z = unscale * (double)zf;
           Zs[i] = z;
           Ds[i] = ref == 0 ? z : Ds[i] + z;
-          zm[0] = isfinite(z) ? fmaxf(zm[0], (float)fabs(z)) : 3e38f;
+          zm[0] = fabsf(zf) <= 1e30f ? fmaxf(zm[0], fabsf(zf)) : 3e38f;
         }
         reduce<NW, 1, true>(zm, red, buf);
-        if (!(zm[0] < 1e30f)) ok = false;
+        if (!(zm[0] <= 1e30f)) ok = false;
         // what is left of the linear system is below the iterate's round-off
-        if (!ok || zm[0] * fmaxf(ratio, 1e-6f) <= 5e-17f * wnorm) break;
+        if (!ok || scalbnf(zm[0], ex) * fmaxf(ratio, 1e-6f) <= 5e-17f * wnorm) break;
         linear_update<NB, MV, FLUX>(TJ, T.Mt, Ws, Zs, Rs, alpha, arena, lam, a.gamma);
       }
       if (!ok) break;
+      MaxAbs dm;
       for (int i = tid; i < 9 * BS; i += NT) {
         const double d = Ds[i], w = Ws[i] - d;
         Ws[i] = w;
-        mx[0] = isfinite(d) ? fmaxf(mx[0], __double2float_ru(fabs(d))) : 3e38f;
-        mx[1] = isfinite(w) ? fmaxf(mx[1], __double2float_rd(fabs(w))) : 3e38f;
+        dm.add(d);
+        wm.add(w);
       }
+      ++dm.hi;  // rounded up
+      dn = block_max<NW>(dm, red, buf) * 1.0000002f;
     }
-    reduce<NW, 2, true>(mx, red, buf);
-    if (!(mx[0] < 1e30f) || !(mx[1] < 1e30f)) break;
-    const double dn = mx[0], wn = mx[1];
-    wnorm = mx[1];
-    if (dn <= a.tol * fmax(1.0, wn)) {
+    const float wn = block_max<NW>(wm, red, buf);
+    if (!(dn < 1e30f) || !(wn < 1e30f)) break;
+    wnorm = wn;
+    if ((double)dn <= a.tol * fmax(1.0, (double)wn)) {
       conv = true;
       break;
     }
-    if (!F64 && solve > 0 && dn > 0.1 * dprev) break;
+    if (!F64 && solve > 0 && dn > 0.1f * dprev) break;
     dprev = dn;
   }
   if (conv) {
