@@ -478,94 +478,128 @@ __device__ __forceinline__ double f2d_scaled(float f, int k) {
   return __hiloint2double((int)hiw, (int)low);
 }
 
-// One thread per cell: dQ = V + the upwind face terms of both directions, summed in
-// registers (every mode index a compile-time constant); the block's state rows are read and
-// written coalesced through shared memory; then the cell's digit rows, group by group.
-template <int NB, int S>
+// The part of the correction that a thread does: modes [8 G0, 8 G1) of its cell, dQ = V + the
+// upwind face terms of both directions, summed in registers (every mode index a compile-time
+// constant), then the cell's new coefficients (in q) and their digit rows.
+template <int NB, int S, int G0, int G1>
+__device__ __forceinline__ bool correct_groups(double* q, const float2* __restrict__ Y, long long e,
+                                               int ix, int iy, int nx, int ny, long long ncell,
+                                               const CorrParams& cp, int sgnx, int sgny, int kfin,
+                                               int snext, uint4* __restrict__ planes, bool f16,
+                                               unsigned long long& mymax) {
+  constexpr int THS = NB * NB;
+  constexpr int M0 = 8 * G0, M1 = 8 * G1 < THS ? 8 * G1 : THS;
+  DF dq[M1 - M0];
+#pragma unroll
+  for (int j = M0; j < M1; ++j) {
+    const float2 y = Y[(long long)j * ncell + e];  // volume term V
+    dq[j - M0] = DF{y.x, y.y};
+  }
+#pragma unroll
+  for (int dd = 0; dd < 2; ++dd) {
+    const int sg = dd == 0 ? sgnx : sgny;
+    if (sg == 0) continue;
+    const int st = dd == 0 ? 1 : NB;
+    int rx = ix, ry = iy, lx = ix, ly = iy;
+    if (dd == 0) {
+      if (sg > 0) lx = ix == 0 ? nx - 1 : ix - 1; else rx = ix + 1 == nx ? 0 : ix + 1;
+    } else {
+      if (sg > 0) ly = iy == 0 ? ny - 1 : iy - 1; else ry = iy + 1 == ny ? 0 : iy + 1;
+    }
+    const long long jr = (long long)ry * nx + rx, jl = (long long)ly * nx + lx;
+    const float2* u = Y + (long long)(THS + dd * NB) * ncell;
+    // line t of modes t NB + a (x) or t + a NB (y): those with a mode of this thread's
+    float2 fa[NB], fb[NB];
+#pragma unroll
+    for (int t = 0; t < NB; ++t)
+      if (dd == 1 || ((t + 1) * NB > M0 && t * NB < M1)) {
+        fa[t] = u[t * ncell + jr];
+        fb[t] = u[t * ncell + jl];
+      }
+#pragma unroll
+    for (int t = 0; t < NB; ++t) {
+      if (dd == 0 && ((t + 1) * NB <= M0 || t * NB >= M1)) continue;
+      const int base = dd == 0 ? t * NB : t;
+      const DF fr = DF{fa[t].x, fa[t].y}, fl = DF{fb[t].x, fb[t].y};
+      const DF w_even = df_add(fl, df_neg(fr));  // -F(i+1/2) + F(i-1/2)
+      const DF w_odd = df_neg(df_add(fl, fr));   // -F(i+1/2) - F(i-1/2)
+#pragma unroll
+      for (int a2 = 0; a2 < NB; ++a2) {
+        const int m = base + a2 * st;
+        if (m < M0 || m >= M1) continue;
+        const DF w = (a2 & 1) ? w_odd : w_even;
+        const DF c = (a2 == 0) ? w : df_mul_const(cp.eph[a2], cp.epl[a2], w);
+        dq[m - M0] = df_add(dq[m - M0], c);
+      }
+    }
+  }
+  bool fits = true;
+#pragma unroll
+  for (int pg = G0; pg < G1; ++pg) {
+    double qn[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int sm = pg * 8 + j;
+      if (sm < THS) {
+        double v = q[sm];
+        v = v + f2d_scaled(dq[sm - M0].h, kfin);
+        v = v + f2d_scaled(dq[sm - M0].l, kfin);
+        q[sm] = v;
+        qn[j] = v;
+        const unsigned long long ab = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFULL;
+        mymax = ab > mymax ? ab : mymax;
+      } else {
+        qn[j] = 0.0;
+      }
+    }
+    fits &= write_group_digits<NB, S>(qn, pg, ix, iy, nx, ny, snext, planes, f16);
+  }
+  return fits;
+}
+
+// SPLIT: two threads per cell, each a group of 8 modes (the halves of a block, so that a warp
+// has one), where a cell has two full groups (Q3): one thread per cell leaves 13 warps per SM
+// at 256^2, each with 16 modes' digits in a row.  (Groups without a mode are zero in the planes
+// from their creation.)
+template <int NB, int S, bool SPLIT>
 __global__ void __launch_bounds__(128) mixed_correct_kernel(
     double* __restrict__ Q, const float2* __restrict__ Y, int nx, int ny, CorrParams cp, int gmax,
     int sgnx, int sgny, int* __restrict__ exps, unsigned long long* __restrict__ maxbits,
     uint4* __restrict__ planes, int* status) {
   constexpr int THS = NB * NB;
-  constexpr int P = ((THS + 15) / 16) * 2;
-  constexpr int BT = 128;
+  static_assert(!SPLIT || NB == 4, "two full groups of modes");
+  constexpr int BT = 128, CELLS = SPLIT ? BT / 2 : BT;
   constexpr int PITCH = THS + 1;  // odd pitch: conflict-free row access
-  __shared__ double sq[BT * PITCH];
+  __shared__ double sq[CELLS * PITCH];
   __shared__ unsigned long long shmax[4];
   const long long ncell = (long long)nx * ny;
-  const long long e0 = (long long)blockIdx.x * BT;
-  const int nblk = (int)min((long long)BT, ncell - e0);
+  const long long e0 = (long long)blockIdx.x * CELLS;
+  const int nblk = (int)min((long long)CELLS, ncell - e0);
   const int ys = exps[1];                                  // exponent of Y
   const int snext = exponent_above(maxbits[0]) + 1;        // exponent for the new digits
   // coalesced load of the block's state rows
   for (int i = threadIdx.x; i < nblk * THS; i += BT) sq[(i / THS) * PITCH + i % THS] = Q[e0 * THS + i];
   __syncthreads();
-  const long long e = e0 + threadIdx.x;
+  const int c = threadIdx.x % CELLS;
+  const long long e = e0 + c;
   unsigned long long mymax = 0;
   bool fits = true;
-  if (threadIdx.x < nblk) {
+  if (c < nblk) {
     const unsigned ue = (unsigned)e, uy = ue / (unsigned)nx;
     const int ix = (int)(ue - uy * (unsigned)nx), iy = (int)uy;
-    DF dq[THS];
-#pragma unroll
-    for (int j = 0; j < THS; ++j) {
-      const float2 y = Y[(long long)j * ncell + e];  // volume term V
-      dq[j] = DF{y.x, y.y};
-    }
-#pragma unroll
-    for (int dd = 0; dd < 2; ++dd) {
-      const int sg = dd == 0 ? sgnx : sgny;
-      if (sg == 0) continue;
-      const int st = dd == 0 ? 1 : NB;
-      int rx = ix, ry = iy, lx = ix, ly = iy;
-      if (dd == 0) {
-        if (sg > 0) lx = ix == 0 ? nx - 1 : ix - 1; else rx = ix + 1 == nx ? 0 : ix + 1;
-      } else {
-        if (sg > 0) ly = iy == 0 ? ny - 1 : iy - 1; else ry = iy + 1 == ny ? 0 : iy + 1;
-      }
-      const long long jr = (long long)ry * nx + rx, jl = (long long)ly * nx + lx;
-      const float2* u = Y + (long long)(THS + dd * NB) * ncell;
-      float2 fa[NB], fb[NB];
-#pragma unroll
-      for (int t = 0; t < NB; ++t) {
-        fa[t] = u[t * ncell + jr];
-        fb[t] = u[t * ncell + jl];
-      }
-#pragma unroll
-      for (int t = 0; t < NB; ++t) {
-        const int base = dd == 0 ? t * NB : t;
-        const DF fr = DF{fa[t].x, fa[t].y}, fl = DF{fb[t].x, fb[t].y};
-        const DF w_even = df_add(fl, df_neg(fr));  // -F(i+1/2) + F(i-1/2)
-        const DF w_odd = df_neg(df_add(fl, fr));   // -F(i+1/2) - F(i-1/2)
-#pragma unroll
-        for (int a2 = 0; a2 < NB; ++a2) {
-          const DF w = (a2 & 1) ? w_odd : w_even;
-          const DF c = (a2 == 0) ? w : df_mul_const(cp.eph[a2], cp.epl[a2], w);
-          dq[base + a2 * st] = df_add(dq[base + a2 * st], c);
-        }
-      }
-    }
     const int kfin = ys + gmax - 16;
-    double* q = sq + threadIdx.x * PITCH;
-#pragma unroll
-    for (int pg = 0; pg < P; ++pg) {
-      double qn[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int sm = pg * 8 + j;
-        if (sm < THS) {
-          double v = q[sm];
-          v = v + f2d_scaled(dq[sm].h, kfin);
-          v = v + f2d_scaled(dq[sm].l, kfin);
-          q[sm] = v;
-          qn[j] = v;
-          const unsigned long long ab = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFULL;
-          mymax = ab > mymax ? ab : mymax;
-        } else {
-          qn[j] = 0.0;
-        }
-      }
-      fits &= write_group_digits<NB, S>(qn, pg, ix, iy, nx, ny, snext, planes, exps[2] != 0);
+    const bool f16 = exps[2] != 0;
+    double* q = sq + c * PITCH;
+    if constexpr (SPLIT) {
+      if (threadIdx.x < CELLS)
+        fits = correct_groups<NB, S, 0, 1>(q, Y, e, ix, iy, nx, ny, ncell, cp, sgnx, sgny, kfin,
+                                           snext, planes, f16, mymax);
+      else
+        fits = correct_groups<NB, S, 1, 2>(q, Y, e, ix, iy, nx, ny, ncell, cp, sgnx, sgny, kfin,
+                                           snext, planes, f16, mymax);
+    } else {
+      fits = correct_groups<NB, S, 0, (THS + 7) / 8>(q, Y, e, ix, iy, nx, ny, ncell, cp, sgnx, sgny,
+                                                     kfin, snext, planes, f16, mymax);
     }
   }
   if (!fits) atomicOr(status, kStatusRange);
@@ -741,10 +775,19 @@ template <int NB, int S>
 static cudaError_t launch_correct_t(const Grid& g, double* Q, const void* Y, int gmax,
                                     const CorrParams& cp, int sgnx, int sgny, MixedState& ms,
                                     cudaStream_t s) {
-  const unsigned blocks = (unsigned)((g.ncell + 127) / 128);  // one thread per cell
-  mixed_correct_kernel<NB, S><<<blocks, 128, 0, s>>>(Q, (const float2*)Y, g.n[0], g.n[1], cp, gmax,
-                                                     sgnx, sgny, ms.exps, ms.maxbits,
-                                                     (uint4*)ms.planes, ms.status);
+  // two threads per cell up to 512 cells per SM: beyond, one per cell fills the SMs and reads
+  // the y faces' values once (step at 256^2 28.8 -> 27.7 us with two; 320^2 37.0 -> 38.0, 512^2
+  // 93.6 -> 97.6)
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const bool split = NB == 4 && g.ncell <= 512LL * sms;
+  const unsigned blocks = (unsigned)((g.ncell * (split ? 2 : 1) + 127) / 128);
+  auto kern = mixed_correct_kernel<NB, S, false>;
+  if constexpr (NB == 4)
+    if (split) kern = mixed_correct_kernel<NB, S, true>;
+  kern<<<blocks, 128, 0, s>>>(Q, (const float2*)Y, g.n[0], g.n[1], cp, gmax, sgnx, sgny, ms.exps,
+                              ms.maxbits, (uint4*)ms.planes, ms.status);
   return cudaGetLastError();
 }
 
