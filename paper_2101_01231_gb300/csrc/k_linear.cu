@@ -21,6 +21,7 @@
 #include <cmath>
 #include <utility>
 
+#include "k_pdl.cuh"
 #include "ridg_internal.h"
 
 namespace ridg {
@@ -57,7 +58,7 @@ __device__ __forceinline__ long long neighbour(const Coords& c, int ox, int oy, 
 // prediction: each thread owns one cell and CH consecutive output rows of P
 // ---------------------------------------------------------------------------------------
 template <int DIM, int NB, int CH>
-__global__ void __launch_bounds__(128) predict_fp64_kernel(const double* __restrict__ Q,
+__global__ void __launch_bounds__(128) predict_fp64_kernel(const double* Q,
                                                            const double* __restrict__ P, int nout,
                                                            double* __restrict__ W, int wstride,
                                                            int nx, int ny, int nz, long long ncell,
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(128) predict_fp64_kernel(const double* __restr
 #pragma unroll 8
   for (int i = threadIdx.x; i < CH * K; i += blockDim.x)
     sP[i] = i < have ? P[(size_t)c0 * K + i] : 0.0;
+  grid_wait();
   __syncthreads();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= ncell) return;
@@ -86,7 +88,7 @@ __global__ void __launch_bounds__(128) predict_fp64_kernel(const double* __restr
     const double* p = sP + r * THS;
 #pragma unroll
     for (int s = 0; s < THS; ++s) {
-      const double x = __ldg(q + s);
+      const double x = q[s];
 #pragma unroll
       for (int j = 0; j < CH; ++j) acc[j] = fma(p[j * K + s], x, acc[j]);
     }
@@ -115,13 +117,13 @@ __device__ __forceinline__ Upwind upwind_of(const CorrParams& cp, int dd) {
 
 // One thread per cell: the time means of the cell and of its upstream neighbour per direction.
 template <int DIM, int NB>
-__global__ void __launch_bounds__(128) correct_linear_kernel(double* __restrict__ Q,
-                                                             const double* __restrict__ Wb,
+__global__ void __launch_bounds__(128) correct_linear_kernel(double* Q, const double* Wb,
                                                              int wstride, int nx, int ny, int nz,
                                                              long long ncell, CorrParams cp) {
   constexpr int THS = ipow_c(NB, DIM);
   constexpr int NT = ipow_c(NB, DIM - 1);
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  grid_wait();
   if (e >= ncell) return;
   const Coords c = cell_coords(e, nx, ny);
   double w[THS], dq[THS];
@@ -176,12 +178,12 @@ __global__ void __launch_bounds__(128) correct_linear_kernel(double* __restrict_
 // d and lies on the fibre base + b st of that dimension; every sum runs in the order of
 // correct_linear_kernel, so the results are its bits.
 template <int DIM, int NB>
-__global__ void __launch_bounds__(128) correct_modes_kernel(double* __restrict__ Q,
-                                                            const double* __restrict__ Wb,
+__global__ void __launch_bounds__(128) correct_modes_kernel(double* Q, const double* Wb,
                                                             int wstride, int nx, int ny, int nz,
                                                             long long ncell, CorrParams cp) {
   constexpr int THS = ipow_c(NB, DIM);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  grid_wait();
   if (i >= ncell * THS) return;
   const long long e = i / THS;
   const int s = (int)(i - e * THS);
@@ -230,8 +232,7 @@ __global__ void __launch_bounds__(128) correct_modes_kernel(double* __restrict__
 //
 // One thread per (cell, mode); local cell u counts downstream, own cells are u >= 2k.
 template <int NB>
-__global__ void __launch_bounds__(768) run1d_chunk_kernel(const double* __restrict__ Qin,
-                                                           double* __restrict__ Qout,
+__global__ void __launch_bounds__(768) run1d_chunk_kernel(const double* Qin, double* Qout,
                                                            const double* __restrict__ P, int n,
                                                            int k, int C, CorrParams cp, int dir,
                                                            int nr) {
@@ -246,7 +247,6 @@ __global__ void __launch_bounds__(768) run1d_chunk_kernel(const double* __restri
   int f = (int)((blockIdx.x * (long long)C + u - 2 * k) % n);
   f += f < 0 ? n : 0;
   const long long g = (long long)(dir > 0 ? f : n - 1 - f) * NB + a;
-  double q = act ? Qin[g] : 0.0;
   double pr[2 * NB];  // this mode's row of the time-mean operator
 #pragma unroll
   for (int i = 0; i < 2 * NB; ++i) pr[i] = i < nr * NB ? P[(size_t)a * nr * NB + i] : 0.0;
@@ -258,6 +258,8 @@ __global__ void __launch_bounds__(768) run1d_chunk_kernel(const double* __restri
   double d[NB];  // row a of D, zero where a <= b or a + b is even
 #pragma unroll
   for (int b = 0; b < NB; ++b) d[b] = a > b && ((a + b) & 1) ? cp.D[a * kMaxNB + b] : 0.0;
+  grid_wait();
+  double q = act ? Qin[g] : 0.0;
   if (act) sQ[tid] = q;
   __syncthreads();
   // the region's cells lo + 0, lo + 1: upstream and own for a > 0, own and upstream for a < 0
@@ -349,12 +351,13 @@ cudaError_t run1d_dispatch(const Grid& g, double* Q, double* Q2, const double* P
     const int k = nsteps / launches + (l < nsteps % launches);
     const int U = pl.C + 2 * k, threads = (U * NB + 31) / 32 * 32;
     const size_t smem = (size_t)U * (2 * NB + 1) * sizeof(double);
-    run1d_chunk_kernel<NB><<<blocks, threads, smem, s>>>(in, out, P, (int)g.ncell, k, pl.C, cp, dir,
-                                                         g.box.cnt[0]);
+    const cudaError_t e = launch_dependent(run1d_chunk_kernel<NB>, blocks, threads, smem, s, in, out, P,
+                                           (int)g.ncell, k, pl.C, cp, dir, g.box.cnt[0]);
+    if (e != cudaSuccess) return e;
     std::swap(in, out);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && in != Q)
+  cudaError_t e = cudaSuccess;
+  if (in != Q)
     e = cudaMemcpyAsync(Q, in, (size_t)g.ncell * NB * sizeof(double), cudaMemcpyDeviceToDevice, s);
   return e;
 }
@@ -388,8 +391,8 @@ cudaError_t predict_dispatch_ch(const Grid& g, const double* Q, const double* P,
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  kern<<<grid, threads, smem, s>>>(Q, P, nout, W, wstride, g.n[0], g.n[1], g.n[2], g.ncell, g.box);
-  return cudaGetLastError();
+  return launch_dependent(kern, grid, threads, smem, s, Q, P, nout, W, wstride, g.n[0], g.n[1],
+                          g.n[2], g.ncell, g.box);
 }
 
 template <int DIM, int NB>
@@ -401,14 +404,14 @@ cudaError_t correct_dispatch(const Grid& g, double* Q, const double* Wb, int wst
   const bool modes = (DIM == 3 && NB >= 5) || g.ncell < 45LL * device_sms();
   if (modes) {
     const unsigned blocks = (unsigned)((g.ncell * ipow_c(NB, DIM) + threads - 1) / threads);
-    correct_modes_kernel<DIM, NB><<<blocks, threads, 0, s>>>(Q, Wb, wstride, g.n[0], g.n[1],
-                                                             g.n[2], g.ncell, cp);
+    return launch_dependent(correct_modes_kernel<DIM, NB>, blocks, threads, 0, s, Q, Wb, wstride,
+                            g.n[0], g.n[1], g.n[2], g.ncell, cp);
   } else if constexpr (!(DIM == 3 && NB >= 5)) {
     const unsigned blocks = (unsigned)((g.ncell + threads - 1) / threads);
-    correct_linear_kernel<DIM, NB><<<blocks, threads, 0, s>>>(Q, Wb, wstride, g.n[0], g.n[1],
-                                                              g.n[2], g.ncell, cp);
+    return launch_dependent(correct_linear_kernel<DIM, NB>, blocks, threads, 0, s, Q, Wb, wstride,
+                            g.n[0], g.n[1], g.n[2], g.ncell, cp);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
