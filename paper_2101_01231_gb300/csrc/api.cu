@@ -829,10 +829,14 @@ int ridg_predict(ridg_t* h, double* w_out, int on_device) {
                                    h->stream));
     }
     return read_newton_stats(h);
-  } else if (is_mixed_linear(h) && h->dim == 2) {
+  }
+  // straight into the caller's device buffer; what a following ridg_correct needs, the time
+  // means, is kept (copying all of W out took 73 MB read and written at 61 x 50 x 37 Q2 for 24)
+  double* const W = w_out && on_device ? w_out : h->W;
+  if (is_mixed_linear(h) && h->dim == 2) {
     int rc = ensure_digits(h);
     if (rc) return rc;
-    RIDG_CUDA(h, ridg::launch_mixed_gemm(g, h->nb, h->mixed_pred, h->ms, h->W, h->thT, 1, false,
+    RIDG_CUDA(h, ridg::launch_mixed_gemm(g, h->nb, h->mixed_pred, h->ms, W, h->thT, 1, false,
                                          h->stream));
   } else if (is_mixed_linear(h) && h->dim == 3) {
     // P's theta_T rows on the tensor cores in blocks (without the step's exponent
@@ -847,25 +851,24 @@ int ridg_predict(ridg_t* h, double* w_out, int on_device) {
     for (int r0 = 0, c = 0; r0 < h->thT; r0 += h->mixed3_pred_rows, ++c) {
       const ridg::MixedOp& op = h->mixed3_pred[c];
       if (op.nout <= 32) {
-        RIDG_CUDA(h, ridg::launch_mixed3_predict(g, h->nb, op, h->ms, h->W, h->thT, r0,
+        RIDG_CUDA(h, ridg::launch_mixed3_predict(g, h->nb, op, h->ms, W, h->thT, r0,
                                                  h->tune_gemm3_slots, h->stream));
       } else {
         RIDG_CUDA(h, ridg::launch_mixed3_gemm(g, h->nb, op, h->ms, h->Y, h->tune_gemm3_slots,
                                               h->stream, false));
         RIDG_CUDA(h, ridg::launch_mixed3_to_w(g, op.nout, r0, h->thT, h->Y, op.gmax, h->ms,
-                                              h->W, h->stream));
+                                              W, h->stream));
       }
     }
   } else {
-    RIDG_CUDA(h, ridg::launch_predict_fp64(g, h->nb, h->Q, h->P, h->thT, h->W, h->thT, h->stream));
+    RIDG_CUDA(h, ridg::launch_predict_fp64(g, h->nb, h->Q, h->P, h->thT, W, h->thT, h->stream));
   }
+  RIDG_CUDA(h, ridg::launch_time_means(W, h->thT, h->Wbar, h->thS, h->ncell, h->stream));
   h->have_pred = true;
-  if (w_out) {
-    const size_t bytes = (size_t)h->ncell * h->m * h->thT * sizeof(double);
-    RIDG_CUDA(h, cudaMemcpyAsync(w_out, h->W, bytes,
-                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                                 h->stream));
-    if (!on_device) RIDG_CUDA(h, cudaStreamSynchronize(h->stream));
+  if (w_out && !on_device) {
+    const size_t bytes = (size_t)h->ncell * h->thT * sizeof(double);
+    RIDG_CUDA(h, cudaMemcpyAsync(w_out, W, bytes, cudaMemcpyDeviceToHost, h->stream));
+    RIDG_CUDA(h, cudaStreamSynchronize(h->stream));
   }
   return RIDG_OK;
 }
@@ -878,7 +881,7 @@ int ridg_correct(ridg_t* h) {
     if (rc) return rc;
   } else {
     CorrParams cp = corr_params(h);
-    RIDG_CUDA(h, ridg::launch_correct_linear(grid_of(h), h->nb, h->Q, h->W, h->thT, cp, h->stream));
+    RIDG_CUDA(h, ridg::launch_correct_linear(grid_of(h), h->nb, h->Q, h->Wbar, h->thS, cp, h->stream));
   }
   h->ms.valid = false;
   h->have_pred = false;

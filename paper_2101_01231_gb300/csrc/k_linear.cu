@@ -216,6 +216,14 @@ __global__ void __launch_bounds__(128) correct_modes_kernel(double* Q, const dou
   Q[e * THS + s] = Q[e * THS + s] + dq;
 }
 
+// Wb[e * thS + s] = W[e * thT + s], s < thS: the time means of a prediction, a warp per cell
+__global__ void __launch_bounds__(256) time_means_kernel(const double* __restrict__ W, int thT,
+                                                         double* __restrict__ Wb, int thS,
+                                                         long long ncell) {
+  for (long long e = blockIdx.x * 8LL + (threadIdx.x >> 5); e < ncell; e += gridDim.x * 8LL)
+    for (int s = threadIdx.x & 31; s < thS; s += 32) Wb[e * thS + s] = W[e * thT + s];
+}
+
 // 1D: k steps of a chunk of C cells per block and launch (temporal blocking).  With upwind face
 // values a step reads two cells upstream (the time mean of the upstream neighbour reads one
 // more), so a block that starts from 2k more cells upstream computes its own cells' k steps
@@ -456,6 +464,13 @@ cudaError_t launch_predict_fp64(const Grid& g, int nb, const double* Q, const do
     }
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_time_means(const double* W, int thT, double* Wb, int thS, long long ncell,
+                              cudaStream_t s) {
+  const unsigned blocks = (unsigned)std::min<long long>((ncell + 7) / 8, 8LL * device_sms());
+  time_means_kernel<<<blocks, 256, 0, s>>>(W, thT, Wb, thS, ncell);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_run1d_fp64(const Grid& g, int nb, double* Q, double* Q2, const double* P,

@@ -44,6 +44,9 @@ struct Grid {
 // X_e stacks the Q of the box's cells around e, x fastest)
 cudaError_t launch_predict_fp64(const Grid& g, int nb, const double* Q, const double* P, int nout,
                                 double* W, int wstride, cudaStream_t s);
+// the time means (the first thS of a cell's thT entries) of a prediction W
+cudaError_t launch_time_means(const double* W, int thT, double* Wb, int thS, long long ncell,
+                              cudaStream_t s);
 // 1D: a run of nsteps FP64 steps (prediction of the time means with the operator's first
 // theta_S rows, then the correction), several steps per launch; Q2: room for another state
 cudaError_t launch_run1d_fp64(const Grid& g, int nb, double* Q, double* Q2, const double* P,
@@ -309,7 +312,8 @@ struct ridg_handle {
   // device buffers
   double* Q = nullptr;      // state, canonical layout
   double* W = nullptr;      // last full prediction (cells * m * theta_T)
-  double* Wbar = nullptr;   // time-mean prediction used by the step (cells * m * theta_S)
+  double* Wbar = nullptr;   // time-mean prediction that the correction reads (cells * m * theta_S);
+                            // 1D steps: the other state of a pair
   double* P = nullptr;      // linear operator, theta_T x K (time-mean rows first)
   double* red = nullptr;    // reduction partials
   int* status = nullptr;    // device status word(s)
