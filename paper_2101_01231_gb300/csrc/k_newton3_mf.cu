@@ -14,7 +14,7 @@
 // The dense LU costs 54 MFLOP per region and iteration and moves its trailing matrix through
 // L2 for each of 432 columns; here a region takes ~0.1 M FP64 operations per iteration, and
 // the FP64 pipe and the barriers of the ~10 applications per solve bound it.  Measured, one
-// step of 10 x 11 x 9 cells in FP64 (with the nodal correction of k_newton3.cu): 585 -> 1.04 ms,
+// step of 10 x 11 x 9 cells in FP64 (with the nodal correction of k_newton3.cu): 585 -> 0.97 ms,
 // of it 0.83 ms this kernel (2.35 ms before the FP32 copies were kept from being reconverted).
 #include <cuda_runtime.h>
 

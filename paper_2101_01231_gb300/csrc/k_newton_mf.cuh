@@ -20,9 +20,10 @@
 // the outer iteration cannot do without; those are evaluated by sum factorisation along lines
 // held in registers, with the even / odd symmetry of the Gauss points (about half the
 // multiplications), one flux evaluation per point for both directions and one per face.
-// Measured against the block elimination alone (one step, tensor-core / FP32 solves): Euler
-// Q2 160^2 214 -> 16.3 ms, Euler Q1 67 x 90 7.7 -> 1.1 ms, eight Burgers problems of up to
-// 72^2 at degrees 1 .. 4 228 -> 13.2 ms; FP64, Burgers Q2 45 x 33 31.7 -> 0.65 ms.
+// Measured against the block elimination alone (one step with its correction, tensor-core /
+// FP32 solves): Euler Q2 160^2 214 -> 12.6 ms (the residuals' FP64 operations alone: 8.8 ms),
+// Euler Q1 67 x 90 7.7 -> 0.91 ms, eight Burgers problems of up to 72^2 at degrees 1 .. 4
+// 227 -> 10.0 ms; FP64, Burgers Q2 45 x 33 31.7 -> 0.55 ms.
 //
 // The initial iterate is Q^n extended constant in time, so the first residual is evaluated
 // with one time mode and one time point.
@@ -93,6 +94,23 @@ __device__ __forceinline__ void face_cells(int f, int& dd, int& cl, int& cr) {
   const int k = f - 12 * dd, row = k >> 2, pos = k & 3;
   cl = pos > 0 ? (dd ? (pos - 1) * 3 + row : row * 3 + pos - 1) : -1;
   cr = pos < 3 ? (dd ? pos * 3 + row : row * 3 + pos) : -1;
+}
+
+// body(line, time point, whether it counts) for LINES time lines of two points, a lane pair per
+// line; whole warps take part (lanes past the end repeat the last line and must not write)
+template <int LINES, int NT, class F>
+__device__ __forceinline__ void time_pairs(F body) {
+  for (int i0 = threadIdx.x & ~31; i0 < 2 * LINES; i0 += NT) {
+    const int i = i0 + (threadIdx.x & 31), line = i >> 1;
+    body(line < LINES ? line : LINES - 1, i & 1, line < LINES);
+  }
+}
+
+// mode q of the two-point line whose values the lane pair holds (q: this lane's point)
+__device__ __forceinline__ double pair_mode(const nl::Rule<2>& T, double f, int q) {
+  const double o = __shfl_xor_sync(0xffffffffu, f, 1);
+  const double so = __hiloint2double(__double2hiint(o) ^ (q << 31), __double2loint(o));  // -+o
+  return (q ? -T.wV[1][0] : T.wV[0][0]) * (f + so);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -179,7 +197,37 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
     }
     __syncthreads();
   }
+  // Degree 1: the 36 volume and 48 face time lines fill little over half of two warps, whose
+  // idle lanes cost the FP64 pipe as much as busy ones; a lane pair shares a line, one of its two
+  // time points each, and exchanges the fluxes (Euler 67 x 90, four steps: 3.79 -> 3.65 ms).
+  constexpr bool PAIR = NB == 2 && !FIRST;
   // time lines of the face points: both traces, the face flux, projected onto the time modes
+  if constexpr (PAIR) {
+    time_pairs<24 * NQ, NT>([&](int f_qo, int q, bool act) {
+      const int f = f_qo / NQ, qo = f_qo - f * NQ;
+      int dd, cl, cr;
+      face_cells(f, dd, cl, cr);
+      const double* tl = Tr + (dd * 2 * C + (cl < 0 ? cr : cl) * MV) * NB * NQ + qo;
+      const double* tr = Tr + ((dd * 2 + 1) * C + (cr < 0 ? cl : cr) * MV) * NB * NQ + qo;
+      const double al = 0.5 * alpha[f], v1 = q ? -T.V[1][0] : T.V[1][0];
+      double wl[MV], wr[MV], fl[MV], fr[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        wl[j] = fma(v1, tl[(j * NB + 1) * NQ], tl[j * NB * NQ]);
+        wr[j] = fma(v1, tr[(j * NB + 1) * NQ], tr[j * NB * NQ]);
+      }
+      if (cl >= 0) flux1<FLUX>(wl, dd, fl, g);
+      if (cr >= 0) flux1<FLUX>(wr, dd, fr, g);
+      double* h = Hf + (f * MV * NB + q) * NQ + qo;
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        const double fh = cl < 0 ? fr[j] : cr < 0 ? fl[j]
+                          : fma(0.5, fl[j] + fr[j], -al * (wr[j] - wl[j]));
+        const double m = pair_mode(T, fh, q);
+        if (act) h[j * NB * NQ] = m;
+      }
+    });
+  } else
   for (int i = tid; i < 24 * NQ; i += NT) {
     const int f = i / NQ, qo = i - f * NQ;
     int dd, cl, cr;
@@ -232,6 +280,31 @@ __device__ void residual(const Tab<NB>& T, const double* Ws, const double* Qs, d
   }
   __syncthreads();  // the traces (in B2) are consumed
   // time lines of the volume points: values, both fluxes, projected onto the time modes
+  if constexpr (PAIR) {
+    time_pairs<9 * NX, NT>([&](int i, int q, bool act) {
+      const int r = i / NX, yx = i - r * NX;
+      double* p1 = B1 + r * MV * NB * NX + yx;
+      double* p2 = B2 + r * MV * NB * NX + yx;
+      const double v1 = q ? -T.V[1][0] : T.V[1][0];
+      double w[MV], fx[MV], fy[MV];
+#pragma unroll
+      for (int j = 0; j < MV; ++j) w[j] = fma(v1, p1[(j * NB + 1) * NX], p1[j * NB * NX]);
+      flux2<FLUX>(w, fx, fy, g);
+#pragma unroll
+      for (int j = 0; j < MV; ++j) {
+        fx[j] = pair_mode(T, fx[j], q);
+        if constexpr (K::NG == 2) fy[j] = pair_mode(T, fy[j], q);
+      }
+      __syncwarp();  // p1 is read by both lanes of a line
+      if (act) {
+#pragma unroll
+        for (int j = 0; j < MV; ++j) {
+          p1[(j * NB + q) * NX] = fx[j];
+          if constexpr (K::NG == 2) p2[(j * NB + q) * NX] = fy[j];
+        }
+      }
+    });
+  } else
   for (int i = tid; i < 9 * NX; i += NT) {
     const int r = i / NX, yx = i - r * NX;
     double* p1 = B1 + r * MV * NB * NX + yx;
