@@ -196,8 +196,9 @@ int ridg_predict(ridg_t* h, double* w_out, int on_device);
 int ridg_correct(ridg_t* h);
 
 /* n >= 1 full steps (prediction + correction), enqueued on the handle's stream; the
- * sequence is captured once into a CUDA graph per (n, dt) and replayed.  Returns after
- * enqueueing; ridg_sync waits.                                                          */
+ * sequence is captured once into a CUDA graph per (n, dt) and replayed (nonlinear flux: from
+ * the second call with that n and dt on, if n is small).  Returns after enqueueing; ridg_sync
+ * waits.                                                                                */
 int ridg_step(ridg_t* h, int n);
 
 /* Wait for all work of the handle; reports a device-side status (ENOCONV / ETIMEOUT).  */
@@ -250,9 +251,9 @@ typedef struct {
   double predict_ms;     /* average device time of the prediction kernel per step           */
   double correct_ms;     /* average device time of the correction kernel per step           */
   double step_ms;        /* average device time of one whole step                            */
-  int launches_per_step; /* prediction and correction launches per step (a mixed-precision
-                            Newton prediction, the iterative kernel and the block
-                            elimination of what it leaves, counts as one)                    */
+  int launches_per_step; /* prediction and correction launches per step (a Newton
+                            prediction, the iterative kernel and the block elimination
+                            of what it leaves, counts as one)                         */
 } ridg_profile_t;
 
 /* Run n steps (the same arithmetic as ridg_step) as individual launches bracketed by CUDA
@@ -309,9 +310,9 @@ int ridg_batch_step(ridg_batch_t* b, int n);
  * launch -- every degree's regions, highest degree first, each CTA moving to the next
  * degree's queue as one runs out -- and every instance's correction in one more launch;
  * 0: one Newton launch per degree and one correction per instance) and the prediction and
- * correction launches of one step.  In the mixed precisions each Newton launch is the block
- * elimination of the regions that the iterative solver, one more launch per degree ahead of
- * it, left; those are not counted.  Burgers batches default to 1 unless the autotuner recorded otherwise.     */
+ * correction launches of one step.  Each Newton launch is the block elimination of the regions
+ * that the iterative solver, one more launch per degree ahead of it, left; those are not
+ * counted.  Burgers batches default to 1 unless the autotuner recorded otherwise.         */
 int ridg_batch_schedule(ridg_batch_t* b, int* schedule, int* launches_per_step);
 /* Time one step in each schedule from the instances' current states (restored afterwards,
  * graphs dropped) and keep the faster; the choice goes into the autotuner's cache (and to

@@ -112,6 +112,22 @@ void drop_graphs(ridg_t* h) {
   for (auto& kv : h->graph_defs) cudaGraphDestroy(kv.second);
   h->graphs.clear();
   h->graph_defs.clear();
+  h->counts_run.clear();
+}
+
+// Nonlinear flux: whether the n steps of a call are launched one by one instead of as a captured
+// graph, the first time that n comes up after a change of dt (which drops the graphs; every
+// ridg_set_state takes a new dt).  Capturing and instantiating cost more than the few launches of
+// a Newton step, and only a replay earns them back (ridg_set_state, one step, ridg_get_state in
+// 3D, Burgers Q1 on 10 x 11 x 9 cells: 1014 -> 972 us).  A linear step's kernels are as short as
+// their launches and its dt stays: a graph from the start.  So are calls of more launches than
+// the stream takes without blocking the caller (about a thousand; half of it is left free).  A
+// capturing stream goes the graph's way, which refuses it before anything of the step is recorded.
+bool run_direct(std::set<int>& counts_run, int n, size_t launches_per_step, cudaStream_t s) {
+  if (n > 512 / (int)launches_per_step) return false;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;
+  return counts_run.insert(n).second;
 }
 
 CorrParams corr_params(const ridg_t* h) {
@@ -897,15 +913,22 @@ int ridg_step(ridg_t* h, int n) {
   if (rc0) return rc0;
   if (!is_linear(h))  // Newton statistics of this call's steps (read by ridg_sync)
     RIDG_CUDA(h, clear_newton_stats(h));
+  auto enqueue = [&] {
+    if (use_run1d(h)) return enqueue_run1d(h, n);
+    int rc = RIDG_OK;
+    for (int i = 0; i < n && rc == RIDG_OK; ++i) rc = enqueue_step(h);
+    return rc;
+  };
   auto it = h->graphs.find(n);
-  if (it == h->graphs.end()) {
+  const bool direct = !is_linear(h) && it == h->graphs.end() &&
+                      run_direct(h->counts_run, n, 8, h->stream);
+  if (direct) {
+    const int rc = enqueue();
+    if (rc != RIDG_OK) return rc;
+  } else if (it == h->graphs.end()) {
     cudaGraph_t graph = nullptr;
     RIDG_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    int rc = RIDG_OK;
-    if (use_run1d(h))
-      rc = enqueue_run1d(h, n);
-    else
-      for (int i = 0; i < n && rc == RIDG_OK; ++i) rc = enqueue_step(h);
+    const int rc = enqueue();
     cudaError_t ce = cudaStreamEndCapture(h->stream, &graph);
     if (rc != RIDG_OK) {
       if (graph) cudaGraphDestroy(graph);
@@ -922,7 +945,7 @@ int ridg_step(ridg_t* h, int n) {
     h->graph_defs[n] = graph;
     it = h->graphs.find(n);
   }
-  RIDG_CUDA(h, cudaGraphLaunch(it->second, h->stream));
+  if (!direct) RIDG_CUDA(h, cudaGraphLaunch(it->second, h->stream));
   h->have_pred = false;
   h->t += n * h->dt;
   h->steps += n;
@@ -1201,6 +1224,7 @@ struct ridg_batch {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   std::map<int, cudaGraphExec_t> graphs;
+  std::set<int> counts_run;  // step counts that have run (run_direct)
   std::map<int, cudaGraph_t> defs;
   std::vector<unsigned long long> gens;  // operator generation of each instance at capture
   // nonlinear flux: one Newton launch over every degree's regions and one correction launch
@@ -1479,7 +1503,7 @@ int ridg_batch_get_state(ridg_batch_t* b, int i, double* q, int on_device) {
   return h ? ridg_get_state(h, q, on_device) : RIDG_EINVAL;
 }
 
-int ridg_batch_step(ridg_batch_t* b, int n) {
+static int batch_step(ridg_batch_t* b, int n, bool may_direct) {
   if (!b || n < 1) return RIDG_EINVAL;
   for (ridg_t* h : b->inst) {
     if (!(h->dt > 0)) return set_err(h, RIDG_ESTATE, "no dt yet: call ridg_set_state first");
@@ -1493,6 +1517,7 @@ int ridg_batch_step(ridg_batch_t* b, int n) {
     for (auto& kv : b->defs) cudaGraphDestroy(kv.second);
     b->graphs.clear();
     b->defs.clear();
+    b->counts_run.clear();
     b->gens.clear();
     for (ridg_t* h : b->inst) b->gens.push_back(h->gen);
   }
@@ -1502,11 +1527,7 @@ int ridg_batch_step(ridg_batch_t* b, int n) {
     if (!rc && b->schedule == 1 && b->corr_table) rc = upload_batch_multi(b);
     if (rc) return rc;
   }
-  auto it = b->graphs.find(n);
-  if (it == b->graphs.end()) {
-    cudaGraph_t graph = nullptr;
-    if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
-      return RIDG_ECUDA;
+  auto enqueue = [&] {
     int rc = RIDG_OK;
     for (int i = 0; i < n && rc == RIDG_OK; ++i) {
       if (b->groups.empty()) {
@@ -1532,6 +1553,20 @@ int ridg_batch_step(ridg_batch_t* b, int n) {
         }
       }
     }
+    return rc;
+  };
+  auto it = b->graphs.find(n);
+  const bool direct = may_direct && !b->groups.empty() && it == b->graphs.end() &&
+                      run_direct(b->counts_run, n, 8 * b->groups.size() + b->inst.size(),
+                                 b->stream);
+  if (direct) {
+    const int rc = enqueue();
+    if (rc != RIDG_OK) return rc;
+  } else if (it == b->graphs.end()) {
+    cudaGraph_t graph = nullptr;
+    if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+      return RIDG_ECUDA;
+    const int rc = enqueue();
     cudaError_t ce = cudaStreamEndCapture(b->stream, &graph);
     if (rc != RIDG_OK || ce != cudaSuccess) {
       if (graph) cudaGraphDestroy(graph);
@@ -1546,13 +1581,15 @@ int ridg_batch_step(ridg_batch_t* b, int n) {
     b->defs[n] = graph;
     it = b->graphs.find(n);
   }
-  if (cudaGraphLaunch(it->second, b->stream) != cudaSuccess) return RIDG_ECUDA;
+  if (!direct && cudaGraphLaunch(it->second, b->stream) != cudaSuccess) return RIDG_ECUDA;
   for (ridg_t* h : b->inst) {
     h->t += n * h->dt;
     h->steps += n;
   }
   return RIDG_OK;
 }
+
+int ridg_batch_step(ridg_batch_t* b, int n) { return batch_step(b, n, true); }
 
 int ridg_batch_schedule(ridg_batch_t* b, int* schedule, int* launches_per_step) {
   if (!b) return RIDG_EINVAL;
@@ -1608,7 +1645,7 @@ int ridg_batch_autotune(ridg_batch_t* b, const char* cache_path) {
       for (int rep = 0; rep < 2 && !rc; ++rep) {  // the first run captures the graph
         restore();
         cudaEventRecord(e0, b->stream);
-        rc = ridg_batch_step(b, 1);
+        rc = batch_step(b, 1, false);
         cudaEventRecord(e1, b->stream);
         if (!rc && cudaEventSynchronize(e1) != cudaSuccess) rc = RIDG_ECUDA;
         float ms = 0.f;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <map>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -330,6 +331,7 @@ struct ridg_handle {
   std::vector<double> P_host;
   // graphs: key = number of steps
   std::map<int, cudaGraphExec_t> graphs;
+  std::set<int> counts_run;  // step counts that have run since the graphs were dropped
   std::map<int, cudaGraph_t> graph_defs;
   // nonlinear flux: tables, elimination plan, per-CTA block storage of the Newton kernel
   ridg::NlDevTables nl;

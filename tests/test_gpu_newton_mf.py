@@ -115,3 +115,24 @@ def test_correction_matches_oracle(R, flux, M, n):
     s.close()
     ref = NL.correct(q, W, w, dt)
     assert np.abs(q1 - ref).max() <= 1e-13 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("flux,M", [("burgers", 2), ("euler", 1)])
+def test_first_call_of_a_step_count_equals_its_replay(R, flux, M):
+    """The steps of a call are launched one by one the first time and replayed as a graph from
+    the second: the same kernels in the same order, so the same bits."""
+    w, q = _smooth(flux, (6, 5), M)
+    s = R.Solver(2, w["n"], M, flux=flux, cfl=w["cfl"], lo=w["lo"], hi=w["hi"],
+                 gamma=w.get("gamma", 1.4))
+    s.set_state(q)
+    for _ in range(3):                  # direct, captured, replayed
+        s.step(2)
+    assert s.sync() == R.RIDG_OK
+    t = R.Solver(2, w["n"], M, flux=flux, cfl=w["cfl"], lo=w["lo"], hi=w["hi"],
+                 gamma=w.get("gamma", 1.4))
+    t.set_state(q)
+    t.step(6)
+    assert t.sync() == R.RIDG_OK
+    np.testing.assert_array_equal(s.get_state(), t.get_state())
+    s.close()
+    t.close()
