@@ -251,9 +251,9 @@ def adv1d_section(R, I, reps):
 
 def ensemble_section(R, I, steps, cpu_cells, rank=0, ws=1):
     """The batched Burgers ensemble (64 instances, N ~ U{64..512}, Q1-Q4, seeded Fourier data)
-    advanced by ridg_batch_step: one captured graph per step holding one persistent Newton
-    launch per degree over all the instances of that degree, then the corrections; TF32
-    block updates with the FP64 residual.  Warm-up on the same ensemble capped at 64 x 64
+    advanced by ridg_batch_step: one captured graph per step holding one matrix-free Newton
+    launch per degree over all the instances of that degree, the block elimination (TF32) of
+    the regions that it leaves over, and the corrections.  Warm-up on the same ensemble capped at 64 x 64
     (the same kernels), then `steps` full-size steps timed with CUDA events on the batch's
     stream; the oracle's Newton prediction on a sample of cells per degree, extrapolated."""
     import torch
@@ -305,8 +305,7 @@ def ensemble_section(R, I, steps, cpu_cells, rank=0, ws=1):
     R.ridg_batch_destroy(b)
     ms = max_over_ranks(float(np.mean(times)), ws, "cuda")
     dof = sum(int(np.prod(w["n"])) * (w["M"] + 1) ** 2 for w in ens_all)
-    # algorithmic work of the block eliminations: 118 b^3 flop per factorisation, b = theta_T
-    flops = sum(118.0 * (w["M"] + 1) ** 9 * inf["newton_iters_total"] for w, inf in zip(ens, infos))
+    flops = sum(2.0 * region_fp64_ops(w["M"], 1) * int(np.prod(w["n"])) for w in ens)
     ach = flops / (ms * 1e-3) / 1e12  # per GPU: this rank's instances over the step time
     out = {"workload": "burgers_ensemble_64", "instances": len(ens_all),
            "scaling": "strong: the 64 instances round-robin over the ranks",
@@ -315,17 +314,18 @@ def ensemble_section(R, I, steps, cpu_cells, rank=0, ws=1):
                                 for m in (1, 2, 3, 4)},
            "precision": "mixed_tf32", "steps": steps, "ms_per_step": ms,
            "value": dof / (ms * 1e-3), "unit": "element-DOF updates/s",
-           "schedule": ("the whole ensemble's Newton prediction in one launch (every degree's "
-                        "regions, highest degree first) + every instance's correction in one"
+           "schedule": ("one matrix-free Newton launch per degree, one launch for the regions "
+                        "left over, one for every instance's correction"
                         if sched["schedule"] == 1 else
-                        "one Newton launch per degree + one correction per instance"),
+                        "two Newton launches per degree + one correction per instance"),
            "launches_per_step": sched["launches_per_step"],
            "newton_unconverged": sum(inf["newton_unconverged"] for inf in infos),
            "status": [int(x) for x in status],
-           "roofline": {"bound": "alu", "kernel": "newton_kernel (all degrees)",
-                        "achieved": ach, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-                        "frac": ach / FP32_PEAK_TFLOPS, "traffic": None,
-                        "peak_source": "nominal: FMA pipes x 2 flop x 2.07 GHz"}}
+           "newton_iters_total": sum(inf["newton_iters_total"] for inf in infos),
+           "roofline": {"bound": "alu", "kernel": "newton_mf_kernel (FP64 residuals, all degrees)",
+                        "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
+                        "frac": ach / FP64_PEAK_TFLOPS, "traffic": None,
+                        "peak_source": "nominal: FP64 FMA pipes x 2 flop x 2.07 GHz"}}
     out["accuracy"] = ensemble_accuracy(R, I, R.RIDG_PREC_MIXED_TF32)
     # the oracle: per-cell Newton prediction time per degree (a 32 x 32 copy of the first
     # instance of each degree), extrapolated to the ensemble's cells
@@ -473,20 +473,43 @@ def paper_bump_section(R, I, dim):
 # ---------------------------------------------------------------------------------------
 NL_WORKLOAD = "euler2d_n512_q2"
 AUTOTUNE = [1]  # set from --autotune
-FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12   # FP32 FMA pipes x 2 flop x max SM clock
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12     # FP64 FMA: 2 per clock per SM
+
+
+def residual_fp64_ops(M, m, first=False):
+    """FP64-pipe operations of one sum-factorised residual of a 2D region (9 cells, 24 faces),
+    with the even / odd symmetry of the Gauss points; first: at the initial iterate, whose
+    time-constant fields need one time mode and one time point."""
+    nb, nq = M + 1, (3 * M + 2) // 2
+    line = nq // 2 * (nb + 2) + nq % 2 * ((nb + 1) // 2)   # nb modes <-> nq points
+    nt, qt, t = (1, 1, 0) if first else (nb, nq, line)
+    ng, fx, fc = (1, 2, 10) if m == 1 else (2, 30, 40)     # fluxes per point: volume, face
+    vol = 9 * m * (nt * nb * line * 3 + nt * nq * line * 3 + nq * nq * t * (1 + ng)) \
+        + 9 * nq * nq * qt * fx
+    face = 36 * m * nt * line + 24 * nq * (3 * m * t + qt * fc) + 24 * m * nt * line
+    time_term = 0 if first else 9 * m * nb ** 3 * (nb + 5)
+    return vol + face + time_term
+
+
+def region_fp64_ops(M, m, iters=None):
+    """FP64 operations of one region's Newton solve: the residuals of its iterates.  The mixed
+    forms take three (the initial iterate's and two more); iters: of an FP64 solve."""
+    full = 2 if iters is None else max(iters - 1, 0)
+    return residual_fp64_ops(M, m, first=True) + full * residual_fp64_ops(M, m)
 
 
 def newton_section(R, I, steps, cpu_cells):
     """The Newton prediction + correction of the 2D Euler vortex (512 x 512, Q2, m = 4): at full
-    size the TF32 tensor-core block updates and the FP32 solves (both with the FP64 residual),
-    FP64 solves on a 128 x 128 mesh of the same problem, and the oracle on a sample of cells
-    (extrapolated per step)."""
+    size in the TF32 and FP32 precisions (matrix-free FP32 solves, FP64 residual; the two differ
+    only in the solver of the regions that those leave over), FP64 solves on a 128 x 128 mesh of
+    the same problem, and the oracle on a sample of cells (extrapolated per step).  Roofline:
+    the FP64 operations of the residuals against the FP64 pipe."""
     from oracle import nonlinear as ONL
     out = {"workload": NL_WORKLOAD}
-    for tag, mesh, prec, peak in (("mixed_tf32", None, R.RIDG_PREC_MIXED_TF32, FP32_PEAK_TFLOPS),
-                                  ("mixed_fp32", None, R.RIDG_PREC_MIXED_FP32, FP32_PEAK_TFLOPS),
-                                  ("fp64_128x128", (128, 128), R.RIDG_PREC_FP64, FP64_PEAK_TFLOPS)):
+    peak = FP64_PEAK_TFLOPS
+    for tag, mesh, prec in (("mixed_tf32", None, R.RIDG_PREC_MIXED_TF32),
+                            ("mixed_fp32", None, R.RIDG_PREC_MIXED_FP32),
+                            ("fp64_128x128", (128, 128), R.RIDG_PREC_FP64)):
         w = I.workload(NL_WORKLOAD, **({"n": mesh} if mesh else {}))
         s = R.Solver(2, w["n"], w["M"], flux="euler", cfl=w["cfl"], lo=w["lo"], hi=w["hi"],
                      gamma=w["gamma"], precision=prec)
@@ -500,30 +523,20 @@ def newton_section(R, I, steps, cpu_cells):
         grid = s.tuning()["newton_grid"]
         s.close()
         cells = int(np.prod(w["n"]))
-        bs = 4 * (w["M"] + 1) ** 3               # unknowns of one region cell (m theta_T)
         iters = info["newton_iters_total"] / steps
-        # algorithmic work of the block elimination (3 x 3 region, corners - edges - centre):
-        # 9 block LUs (2/3 b^3), 17 block solves and 39 block updates (2 b^3 each) = 118 b^3
-        flops = 118.0 * bs ** 3 * iters
+        flops = 2.0 * cells * region_fp64_ops(w["M"], 4, None if tag.startswith("mixed")
+                                              else iters / cells)
         ach = flops / (p["predict_ms"] * 1e-3) / 1e12
         r = {"mesh": list(w["n"]), "ms_per_step": p["step_ms"], "predict_ms": p["predict_ms"],
              "correct_ms": p["correct_ms"],
              "value": cells * 4 * (w["M"] + 1) ** 2 / (p["step_ms"] * 1e-3),
              "unit": "element-DOF updates/s", "newton_iters_per_cell": iters / cells,
              "newton_iters_max": info["newton_iters_max"], "newton_grid_ctas": grid,
-             "roofline": {"bound": "alu", "kernel": "newton_kernel", "achieved": ach, "peak": peak,
-                          "unit": "TFLOP/s", "frac": ach / peak,
-                          "traffic": (_recorded_traffic("newton_" + tag[6:], info["newton_iters_total"] / steps)
+             "roofline": {"bound": "alu", "kernel": "newton_mf_kernel (FP64 residuals)",
+                          "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+                          "traffic": (_recorded_traffic("newton_" + tag[6:], iters)
                                       if tag.startswith("mixed") else None),
-                          "peak_source": "nominal: FMA pipes x 2 flop x 2.07 GHz"}}
-        if tag == "mixed_tf32":
-            # the 56 block products alone (2 b^3 flop each: 112 of the 118 b^3) on the TF32
-            # tensor cores: TF32 peak = the measured BF16 peak x the nominal TF32 / BF16 ratio
-            tf32_peak = _peaks()[1] * 0.5
-            upd = 112.0 * bs ** 3 * iters / (p["predict_ms"] * 1e-3) / 1e12
-            r["tensor"] = {"kernel": "newton_kernel (block updates)", "achieved": upd,
-                           "peak": tf32_peak, "unit": "TFLOP/s", "frac": upd / tf32_peak,
-                           "peak_source": "measured BF16 x nominal TF32/BF16 (1/2)"}
+                          "peak_source": "nominal: FP64 FMA pipes x 2 flop x 2.07 GHz"}}
         out[tag] = r
     out["accuracy"] = newton_accuracy(R, I)
     # the oracle: Newton prediction of a sample of cells and the correction of the whole
@@ -548,9 +561,9 @@ def newton_section(R, I, steps, cpu_cells):
 
 def newton3d_section(R, I, cpu=True):
     """The 3D nonlinear prediction (3D Burgers, degree 1, smooth seeded data): one step at 32^3
-    with FP32 region solves (FP64 residual and update) and at 12^3 in FP64, each with the
-    rate of its dense per-region LU (2/3 n^3 flop per factorisation, n = 27 theta_T = 432)
-    against the FP32 / FP64 pipe, and the oracle's per-region time on the host."""
+    with FP32 region solves (FP64 residual and update) and at 12^3 in FP64, each with the FP64
+    operations of its residuals (one per Newton iteration: 216 columns and 432 face lines of
+    two time nodes) against the FP64 pipe, and the oracle's per-region time on the host."""
     import torch
     from oracle import linear as OL
     from oracle import nonlinear as ONL
@@ -561,9 +574,10 @@ def newton3d_section(R, I, cpu=True):
                              * np.sin(2 * np.pi * z) + 0.05 * np.cos(2 * np.pi * (x + z)))
         return w, np.ascontiguousarray(I.project_tensor(f, w, 2)[:, 0, :])
 
-    out = {"workload": "burgers3d Q1, smooth data (sines)", "solver": "dense per-region LU"}
-    for tag, n, prec, peak in (("mixed_fp32", 32, R.RIDG_PREC_MIXED_FP32, FP32_PEAK_TFLOPS),
-                               ("fp64", 12, R.RIDG_PREC_FP64, FP64_PEAK_TFLOPS)):
+    out = {"workload": "burgers3d Q1, smooth data (sines)", "solver": "matrix-free BiCGStab"}
+    peak = FP64_PEAK_TFLOPS
+    for tag, n, prec in (("mixed_fp32", 32, R.RIDG_PREC_MIXED_FP32),
+                         ("fp64", 12, R.RIDG_PREC_FP64)):
         w, q = data(n)
         s = R.Solver(3, w["n"], 1, flux="burgers", cfl=w["cfl"], precision=prec,
                      newton_max_iters=8)
@@ -574,16 +588,16 @@ def newton3d_section(R, I, cpu=True):
         info = s.info()
         s.close()
         cells = n ** 3
-        flops = 2.0 / 3.0 * 432.0 ** 3 * info["newton_iters_total"]
+        flops = 2.0 * (216 * 2 * 14 + 432 * 2 * 12) * info["newton_iters_total"]
         ach = flops / (p["predict_ms"] * 1e-3) / 1e12
         out[tag] = {"mesh": [n] * 3, "ms_per_step": p["step_ms"], "predict_ms": p["predict_ms"],
                     "correct_ms": p["correct_ms"], "value": cells * 8 / (p["step_ms"] * 1e-3),
                     "unit": "element-DOF updates/s",
                     "newton_iters_per_cell": info["newton_iters_total"] / cells,
-                    "roofline": {"bound": "alu", "kernel": "newton3_kernel (LU flops)",
+                    "roofline": {"bound": "alu", "kernel": "newton3_mf_kernel (FP64 residuals)",
                                  "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                                  "frac": ach / peak, "traffic": None,
-                                 "peak_source": "nominal: FMA pipes x 2 flop x 2.07 GHz"}}
+                                 "peak_source": "nominal: FP64 FMA pipes x 2 flop x 2.07 GHz"}}
     if cpu:
         w, q = data(12)
         dt, _ = OL.time_step(w, ONL.max_speed(q, w))
