@@ -751,6 +751,17 @@ static bool pinned_host(const void* p) {
   }
   return a.type == cudaMemoryTypeHost && a.devicePointer == p;
 }
+// Memory of the current device, which its kernels may write (a peer's, which a copy reaches, only
+// where access is enabled).
+static bool own_device_memory(const void* p) {
+  cudaPointerAttributes a;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
 int ridg_set_state(ridg_t* h, const double* q, int on_device) {
@@ -848,7 +859,7 @@ int ridg_predict(ridg_t* h, double* w_out, int on_device) {
   }
   // straight into the caller's device buffer; what a following ridg_correct needs, the time
   // means, is kept (copying all of W out took 73 MB read and written at 61 x 50 x 37 Q2 for 24)
-  double* const W = w_out && on_device ? w_out : h->W;
+  double* const W = w_out && on_device && own_device_memory(w_out) ? w_out : h->W;
   if (is_mixed_linear(h) && h->dim == 2) {
     int rc = ensure_digits(h);
     if (rc) return rc;
@@ -881,10 +892,12 @@ int ridg_predict(ridg_t* h, double* w_out, int on_device) {
   }
   RIDG_CUDA(h, ridg::launch_time_means(W, h->thT, h->Wbar, h->thS, h->ncell, h->stream));
   h->have_pred = true;
-  if (w_out && !on_device) {
+  if (w_out && W != w_out) {
     const size_t bytes = (size_t)h->ncell * h->thT * sizeof(double);
-    RIDG_CUDA(h, cudaMemcpyAsync(w_out, W, bytes, cudaMemcpyDeviceToHost, h->stream));
-    RIDG_CUDA(h, cudaStreamSynchronize(h->stream));
+    RIDG_CUDA(h, cudaMemcpyAsync(w_out, W, bytes,
+                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                 h->stream));
+    if (!on_device) RIDG_CUDA(h, cudaStreamSynchronize(h->stream));
   }
   return RIDG_OK;
 }
