@@ -28,7 +28,7 @@
 // The initial iterate is Q^n extended constant in time, so the first residual is evaluated
 // with one time mode and one time point.
 //
-// A region that does not converge quickly (contraction below 10x per solve, BiCGStab
+// A region that does not converge quickly (mixed: contraction below 10x per solve; BiCGStab
 // stalled, a non-finite value) is put on a list; the block elimination of k_newton.cuh then
 // solves the listed regions from the start, with its own iteration cap and statistics.
 #pragma once
@@ -1184,7 +1184,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
   Lin<NB, MV> S;
   const float g1 = keep((float)(a.gamma - 1.0));
   int it = 0;
-  bool conv = false, lin = true;
+  bool conv = false, capped = false, lin = true;
   float dprev = 0.f, bprev = 0.f;
   const int solves = F64 ? a.max_iters : kMaxSolves;
 #pragma unroll 1
@@ -1273,10 +1273,14 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
     }
     if (!F64 && solve > 0 && dn > 0.1f * dprev) break;
     dprev = dn;
+    // the FP64 iterates are the block elimination's to round-off, also at the cap (a tolerance
+    // below round-off, where the two differ, stays the block elimination's to decide)
+    capped = F64 && solve + 1 == solves && (double)dn > 1e-12 * fmax(1.0, (double)wn);
   }
-  if (conv) {
+  if (conv || capped) {
     for (int i = tid; i < BS; i += NT) Wg[e * BS + i] = Ws[4 * BS + i];
     if (tid == 0) {
+      if (!conv) atomicAdd(&stats[0], 1);
       atomicMax(&stats[1], it);
       atomicAdd(&stats[7 + (it < 15 ? it : 15)], 1);
       atomicAdd(itot, (unsigned long long)it);

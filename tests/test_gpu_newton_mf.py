@@ -136,3 +136,29 @@ def test_first_call_of_a_step_count_equals_its_replay(R, flux, M):
     np.testing.assert_array_equal(s.get_state(), t.get_state())
     s.close()
     t.close()
+
+
+@pytest.mark.parametrize("flux,M,dim", [("burgers", 2, 2), ("euler", 1, 2), ("burgers", 1, 3)])
+def test_fp64_regions_at_the_cap_keep_newtons_iterate(R, flux, M, dim):
+    """FP64 regions stopped by the iteration cap are kept as the matrix-free solver leaves them:
+    the oracle's iterate after as many steps (tolerance as the converged parity), all counted
+    as unconverged."""
+    from oracle import nonlinear as NL
+    if dim == 2:
+        w, q = _smooth(flux, (3, 4), M)
+    else:
+        w = dict(flux=flux, dim=3, n=(3, 3, 4), M=M, lo=(0.0,) * 3, hi=(1.0,) * 3, cfl=0.3)
+        f = lambda x, y, z: 0.3 + 0.1 * np.sin(2 * np.pi * x) * np.cos(2 * np.pi * (y - z))
+        q = np.ascontiguousarray(I.project_tensor(f, w, 2)[:, 0, :])
+    s = R.Solver(dim, w["n"], M, flux=flux, cfl=w["cfl"], lo=w["lo"], hi=w["hi"],
+                 gamma=w.get("gamma", 1.4), newton_max_iters=2)
+    s.set_state(q)
+    dt = s.info()["dt"]
+    cells = int(np.prod(w["n"]))
+    Wd = s.predict()
+    assert s.last_status == R.RIDG_ENOCONV
+    info = s.info()
+    s.close()
+    ref = NL.newton_predict(q, w, dt, max_iters=2)
+    assert info["newton_unconverged"] == cells and info["newton_iters_max"] == 2
+    assert np.abs(Wd - ref).max() <= 1e-12 * np.abs(ref).max()
