@@ -769,8 +769,9 @@ int ridg_set_state(ridg_t* h, const double* q, int on_device) {
   const size_t bytes = (size_t)h->ncell * h->m * h->thS * sizeof(double);
   const long long count = (long long)(bytes / sizeof(double));
   RIDG_CUDA(h, cudaMemsetAsync(h->status, 0, sizeof(int), h->stream));
-  if (!on_device && pinned_host(q) && aligned16(q) && aligned16(h->Q)) {
-    // pinned host memory: the SMs read it over C2C, copy and finite check in one pass
+  if (aligned16(q) && aligned16(h->Q) && (on_device ? own_device_memory(q) : pinned_host(q))) {
+    // pinned host memory (the SMs read it over C2C) or this device's: copy and finite check in
+    // one pass
     RIDG_CUDA(h, ridg::launch_ingest(q, h->Q, count, h->status, h->stream));
   } else {
     RIDG_CUDA(h, cudaMemcpyAsync(h->Q, q, bytes,

@@ -4,6 +4,8 @@
 // partials in block order, so results are run-to-run deterministic.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "k_tcgen05.cuh"
 #include "ridg_internal.h"
 
@@ -98,7 +100,9 @@ __global__ void bounded_wait_probe_kernel(int* status) {
 // set_state from a pinned host buffer: the SMs read it over the coherent C2C link themselves
 // (16-byte loads, four in flight per thread per iteration), write the device state and raise
 // *flag on a value that is not finite -- the copy and the finite check in one pass (measured
-// on GB300: 61 us against 73 us for a copy-engine copy followed by the check, 256^2 Q3).
+// on GB300: 61 us against 73 us for a copy-engine copy followed by the check, 256^2 Q3).  Also
+// from this device's own memory, where it saves the check's second pass over the state
+// (set_state and prediction at 61 x 50 x 37 Q2: 215 -> 201 us, with the wider state maximum).
 __global__ void __launch_bounds__(256) ingest_kernel(const double* __restrict__ src,
                                                      double* __restrict__ dst, long long n,
                                                      int* __restrict__ flag) {
@@ -148,12 +152,13 @@ cudaError_t launch_l2_partials(const double* Q, const double* X, long long ncell
   return cudaGetLastError();
 }
 
-cudaError_t launch_ingest(const double* host, double* dev, long long count, int* flag,
+cudaError_t launch_ingest(const double* src, double* dev, long long count, int* flag,
                           cudaStream_t s) {
   int d = 0, sms = 0;
   cudaGetDevice(&d);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
-  ingest_kernel<<<sms * 4, 256, 0, s>>>(host, dev, count, flag);
+  const long long b = (count / 2 + 255) / 256;
+  ingest_kernel<<<(unsigned)std::max(1LL, std::min(b, 4LL * sms)), 256, 0, s>>>(src, dev, count, flag);
   return cudaGetLastError();
 }
 

@@ -764,7 +764,8 @@ template <int NB, int S>
 static cudaError_t launch_refresh_t(const Grid& g, const double* Q, MixedState& ms, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(ms.maxbits, 0, 2 * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  state_max_kernel<<<256, 256, 0, s>>>(Q, g.ncell * NB * NB, ms.maxbits);
+  const long long count = g.ncell * NB * NB;
+  state_max_kernel<<<state_max_blocks(count), 256, 0, s>>>(Q, count, ms.maxbits);
   const unsigned blocks = (unsigned)((g.ncell + 127) / 128);
   state_digits_kernel<NB, S><<<blocks, 128, 0, s>>>(Q, g.n[0], g.n[1], ms.maxbits, ms.exps,
                                                     (uint4*)ms.planes, ms.status);
