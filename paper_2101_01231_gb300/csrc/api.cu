@@ -1,5 +1,6 @@
 // C ABI of the RIDG library (include/ridg.h): handle lifecycle, state transfer, the
 // prediction / correction / step entry points, diagnostics and the batched ensemble.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -751,16 +752,33 @@ static bool pinned_host(const void* p) {
   }
   return a.type == cudaMemoryTypeHost && a.devicePointer == p;
 }
-// Memory of the current device, which its kernels may write (a peer's, which a copy reaches, only
-// where access is enabled).
-static bool own_device_memory(const void* p) {
+// Whether a kernel may read or write `bytes` of doubles at p where a copy did before: memory of the
+// current device (a peer's, which a copy reaches, only where access is enabled), on a double's
+// boundary (a copy takes any address, a kernel's store faults) and inside one allocation (a copy
+// past its end is refused, a kernel's store is not).  Anything else stays with the copy.
+static bool own_device_memory(const void* p, size_t bytes) {
+  using RangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const RangeFn range = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault,
+                                         &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      fn = nullptr;
+    return (RangeFn)fn;
+  }();
+  if (((uintptr_t)p & 7) || !range) return false;
   cudaPointerAttributes a;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return a.type == cudaMemoryTypeDevice && a.device == dev;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  return a.type == cudaMemoryTypeDevice && a.device == dev &&
+         range(&base, &size, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS &&
+         (size_t)((uintptr_t)p - base) <= size && bytes <= size - (size_t)((uintptr_t)p - base);
 }
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
@@ -769,7 +787,7 @@ int ridg_set_state(ridg_t* h, const double* q, int on_device) {
   const size_t bytes = (size_t)h->ncell * h->m * h->thS * sizeof(double);
   const long long count = (long long)(bytes / sizeof(double));
   RIDG_CUDA(h, cudaMemsetAsync(h->status, 0, sizeof(int), h->stream));
-  if (aligned16(q) && aligned16(h->Q) && (on_device ? own_device_memory(q) : pinned_host(q))) {
+  if (aligned16(q) && aligned16(h->Q) && (on_device ? own_device_memory(q, bytes) : pinned_host(q))) {
     // pinned host memory (the SMs read it over C2C) or this device's: copy and finite check in
     // one pass
     RIDG_CUDA(h, ridg::launch_ingest(q, h->Q, count, h->status, h->stream));
@@ -860,7 +878,8 @@ int ridg_predict(ridg_t* h, double* w_out, int on_device) {
   }
   // straight into the caller's device buffer; what a following ridg_correct needs, the time
   // means, is kept (copying all of W out took 73 MB read and written at 61 x 50 x 37 Q2 for 24)
-  double* const W = w_out && on_device && own_device_memory(w_out) ? w_out : h->W;
+  const size_t wbytes = (size_t)h->ncell * h->thT * sizeof(double);
+  double* const W = w_out && on_device && own_device_memory(w_out, wbytes) ? w_out : h->W;
   if (is_mixed_linear(h) && h->dim == 2) {
     int rc = ensure_digits(h);
     if (rc) return rc;
@@ -894,8 +913,7 @@ int ridg_predict(ridg_t* h, double* w_out, int on_device) {
   RIDG_CUDA(h, ridg::launch_time_means(W, h->thT, h->Wbar, h->thS, h->ncell, h->stream));
   h->have_pred = true;
   if (w_out && W != w_out) {
-    const size_t bytes = (size_t)h->ncell * h->thT * sizeof(double);
-    RIDG_CUDA(h, cudaMemcpyAsync(w_out, W, bytes,
+    RIDG_CUDA(h, cudaMemcpyAsync(w_out, W, wbytes,
                                  on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                                  h->stream));
     if (!on_device) RIDG_CUDA(h, cudaStreamSynchronize(h->stream));
