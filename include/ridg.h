@@ -107,7 +107,9 @@ typedef struct {
   int precision;          /* RIDG_PREC_*                                                */
   int slices;             /* digit slices per operand for MIXED_BF16 / MIXED_FP16, 2..7
                              (0 = default 6)                                                */
-  int newton_max_iters;   /* 0 = default 4                                              */
+  int newton_max_iters;   /* 0 = default 4.  Caps the linearisations of a region; FP64: one
+                             solve each, MIXED_FP32: up to 3 more solves against the FP64
+                             residual reuse one, MIXED_TF32: up to 8                       */
   double newton_tol;      /* <= 0 = default 1e-10: stop when ||dW||_inf <= tol max(1,||W||_inf) */
   void* stream;           /* cudaStream_t (not the legacy default stream) or NULL       */
   ridg_alloc_fn alloc;    /* optional device allocator (default cudaMalloc)             */

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdint>
@@ -361,6 +362,8 @@ cudaError_t enqueue_newton_mf(const ridg_t* h, ridg::NewtonArgs& a, int* list, c
   f.gamma = a.gamma;
   f.fp64 = newton_prec(h) == ridg::kNewtonF64;
   f.max_iters = a.max_iters;
+  const int sweeps = newton_prec(h) == ridg::kNewtonTF32 ? ridg::kSweepsTf32 : ridg::kSweepsFp32;
+  f.max_solves = (int)std::min((long long)a.max_iters * (1 + sweeps), (long long)INT_MAX);
   f.tol = a.tol;
   f.stats = a.stats;
   f.iters_total = a.iters_total;

@@ -1625,9 +1625,8 @@ __device__ void newton_regions(const NewtonArgs& a, unsigned char* smem, uint32_
     // FP64 form: Newton (a new Jacobian every iteration).  FP32 form: after a factorisation,
     // refinement sweeps reuse it with the FP64 residual while each contracts the update by
     // at least 10x (at most kSweeps per factorisation); max_iters caps the factorisations.
-    // (TF32 block updates leave a coarser factorisation: more sweeps before a refactorisation)
     constexpr bool CHORD = sizeof(T) == 4;
-    constexpr int kSweeps = TC ? 8 : 3;
+    constexpr int kSweeps = TC ? kSweepsTf32 : kSweepsFp32;
     int it = 0, sweeps = 0;
     bool conv = false, bad = false, refactor = true;
     double dprev = 0.0;

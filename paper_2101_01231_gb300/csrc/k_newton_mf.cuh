@@ -854,7 +854,10 @@ __device__ __forceinline__ void apply(const Tab<NB>& T, const Rows<NB>& R, const
   }
 }
 
-constexpr int kMaxSolves = 7;   // linear solves of a region (mixed) before it is left to the list
+// Linear solves of a region (mixed) before it is left to the list; no more than the block
+// elimination makes at the caller's cap (1 + kSweepsFp32 per factorisation, which is fewer at a
+// cap of one), so that a region stopped by the cap there is not reported as converged here.
+constexpr int kMaxSolves = 7;
 constexpr int kMaxRefine = 8;   // FP32 solves per Newton iteration (FP64) before that
 constexpr int kMaxInner = 32;   // BiCGStab iterations per solve
 
@@ -1186,7 +1189,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
   int it = 0;
   bool conv = false, capped = false, lin = true;
   float dprev = 0.f, bprev = 0.f;
-  const int solves = F64 ? a.max_iters : kMaxSolves;
+  const int solves = F64 ? a.max_iters : min(kMaxSolves, a.max_solves);
 #pragma unroll 1
   for (int solve = 0; solve < solves; ++solve) {
     if (solve == 0)

@@ -220,6 +220,9 @@ struct NewtonArgs {
   const int* list;
   const int* list_count;
 };
+// Mixed precisions: solves that reuse a factorisation of the block elimination, at most (TF32
+// block updates leave a coarser factorisation: more sweeps before a refactorisation).
+constexpr int kSweepsFp32 = 3, kSweepsTf32 = 8;
 // The matrix-free Newton prediction (k_newton_mf.cuh), the first solver of every precision: it
 // solves every region it can and lists the others for launch_newton.
 struct NewtonMfArgs {
@@ -231,6 +234,8 @@ struct NewtonMfArgs {
   double gamma;
   bool fp64;           // plain Newton with linear solves to FP64 accuracy; else FP32 solves
   int max_iters;       // linearisations per region
+  int max_solves;      // mixed precisions: linear solves per region, at most those that the block
+                       // elimination would make at this cap
   double tol;
   int* stats;          // as in NewtonArgs
   unsigned long long* iters_total;
