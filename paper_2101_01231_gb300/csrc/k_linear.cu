@@ -359,7 +359,7 @@ cudaError_t run1d_dispatch(const Grid& g, double* Q, double* Q2, const double* P
     const int k = nsteps / launches + (l < nsteps % launches);
     const int U = pl.C + 2 * k, threads = (U * NB + 31) / 32 * 32;
     const size_t smem = (size_t)U * (2 * NB + 1) * sizeof(double);
-    const cudaError_t e = launch_dependent(run1d_chunk_kernel<NB>, blocks, threads, smem, s, in, out, P,
+    const cudaError_t e = launch_dependent(true, run1d_chunk_kernel<NB>, blocks, threads, smem, s, in, out, P,
                                            (int)g.ncell, k, pl.C, cp, dir, g.box.cnt[0]);
     if (e != cudaSuccess) return e;
     std::swap(in, out);
@@ -384,6 +384,14 @@ struct PredictRows {
                                          : 4;
 };
 
+// The correction's form: a thread per mode below ~45 cells per SM (2D Q3, 24 cells per SM: 10.9
+// against 17.4 us; 66: 19.1 against 17.0), and where a cell's time means do not fit a thread.
+bool correct_by_modes(int dim, int nb, long long ncell) {
+  return (dim == 3 && nb >= 5) || ncell < 45LL * device_sms();
+}
+constexpr int kCorrectThreads = 128;
+long long correct_mode_blocks(long long modes) { return (modes + kCorrectThreads - 1) / kCorrectThreads; }
+
 template <int DIM, int NB>
 cudaError_t predict_dispatch_ch(const Grid& g, const double* Q, const double* P, int nout,
                                 double* W, int wstride, cudaStream_t s) {
@@ -399,25 +407,32 @@ cudaError_t predict_dispatch_ch(const Grid& g, const double* Q, const double* P,
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  return launch_dependent(kern, grid, threads, smem, s, Q, P, nout, W, wstride, g.n[0], g.n[1],
-                          g.n[2], g.ncell, g.box);
+  // Launched early, the blocks go to the SMs with room beside the correction of the step before.
+  // Where that correction has a block per 128 modes and they no longer all run at once, these are
+  // the few SMs that ran out first: a prediction that does not fill the chip then piles up there
+  // (3D Q4 12^3 778 against 417 us a step, Q3 16^3 424 against 262, 2D Q5 82^2 156 against 97;
+  // up to 8 blocks per SM, 2D Q5 60^2, 3D Q2 14^3, it saves 6 to 8%).
+  const int sms = device_sms();
+  const long long resident = std::min({32LL, 2048LL / threads, 232448LL / (long long)(smem + 1024)});
+  const bool early = !correct_by_modes(DIM, NB, g.ncell) ||
+                     correct_mode_blocks(g.ncell * ipow_c(NB, DIM)) <= 8LL * sms ||
+                     10LL * grid.x * grid.y >= 9 * resident * sms;
+  return launch_dependent(early, kern, grid, threads, smem, s, Q, P, nout, W, wstride, g.n[0],
+                          g.n[1], g.n[2], g.ncell, g.box);
 }
 
 template <int DIM, int NB>
 cudaError_t correct_dispatch(const Grid& g, double* Q, const double* Wb, int wstride,
                              const CorrParams& cp, cudaStream_t s) {
-  const int threads = 128;
-  // a thread per mode below ~45 cells per SM (2D Q3, 24 cells per SM: 10.9 against 17.4 us; 66:
-  // 19.1 against 17.0)
-  const bool modes = (DIM == 3 && NB >= 5) || g.ncell < 45LL * device_sms();
-  if (modes) {
-    const unsigned blocks = (unsigned)((g.ncell * ipow_c(NB, DIM) + threads - 1) / threads);
-    return launch_dependent(correct_modes_kernel<DIM, NB>, blocks, threads, 0, s, Q, Wb, wstride,
-                            g.n[0], g.n[1], g.n[2], g.ncell, cp);
+  const int threads = kCorrectThreads;
+  if (correct_by_modes(DIM, NB, g.ncell)) {
+    const unsigned blocks = (unsigned)correct_mode_blocks(g.ncell * ipow_c(NB, DIM));
+    return launch_dependent(true, correct_modes_kernel<DIM, NB>, blocks, threads, 0, s, Q, Wb,
+                            wstride, g.n[0], g.n[1], g.n[2], g.ncell, cp);
   } else if constexpr (!(DIM == 3 && NB >= 5)) {
     const unsigned blocks = (unsigned)((g.ncell + threads - 1) / threads);
-    return launch_dependent(correct_linear_kernel<DIM, NB>, blocks, threads, 0, s, Q, Wb, wstride,
-                            g.n[0], g.n[1], g.n[2], g.ncell, cp);
+    return launch_dependent(true, correct_linear_kernel<DIM, NB>, blocks, threads, 0, s, Q, Wb,
+                            wstride, g.n[0], g.n[1], g.n[2], g.ncell, cp);
   }
   return cudaErrorInvalidValue;
 }

@@ -4,7 +4,8 @@
 // tail.  Every such kernel calls grid_wait() in every thread before it reads or writes anything
 // that an earlier kernel touches: it returns when the kernel before it has completed and its
 // writes are visible.  grid_wait() also lets the next kernel start its own prologue; as that
-// happens only after the wait, at most two neighbours in a chain overlap.
+// happens only after the wait, at most two neighbours in a chain overlap.  Without `early` the
+// launch waits for the kernel before it as any other.
 //
 // Pointers to what earlier kernels write carry no __restrict__ in such a kernel: with it the
 // compiler may take the data for unchanging and load them ahead of the wait.
@@ -22,7 +23,7 @@ __device__ __forceinline__ void grid_wait() {
 }
 
 template <typename... Params, typename... Args>
-cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem,
+cudaError_t launch_dependent(bool early, void (*kern)(Params...), dim3 grid, dim3 block, size_t smem,
                              cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t c = {};
   c.gridDim = grid;
@@ -33,7 +34,7 @@ cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, siz
   a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   a.val.programmaticStreamSerializationAllowed = 1;
   c.attrs = &a;
-  c.numAttrs = 1;
+  c.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&c, kern, Params(std::forward<Args>(args))...);
 }
 
