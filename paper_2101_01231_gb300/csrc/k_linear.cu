@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(128) predict_fp64_kernel(const double* Q,
   const int K = box.n * THS;
   extern __shared__ double sP[];  // CH x K
   const int c0 = blockIdx.y * CH;
-  const int have = min(CH, nout - c0) * K;  // (CH divides theta_S and theta_T)
+  const int have = min(CH, nout - c0) * K;  // (the last rows may be padding)
 #pragma unroll 8
   for (int i = threadIdx.x; i < CH * K; i += blockDim.x)
     sP[i] = i < have ? P[(size_t)c0 * K + i] : 0.0;
@@ -370,10 +370,11 @@ cudaError_t run1d_dispatch(const Grid& g, double* Q, double* Q2, const double* P
   return e;
 }
 
-// Rows of P per thread: a divisor of theta_S, 2 to 5, so that no row is padding and meshes of a
-// few thousand cells have warps for every SM.  Measured against 16 rows (8 and 4 in 3D) by
-// blocks of 128 threads, the time-mean prediction: 2D Q5 60^2 94.7 -> 43.5 us, Q3 256^2 138 ->
-// 121, Q2 160^2 29 -> 21; 3D Q2 16^3 92 -> 53, Q3 8^3 164 -> 97, Q3 48^3 5.88 -> 5.86 ms.
+// Rows of P per thread in 2D and 3D: up to 5 and a divisor of theta_S (4 of 3D Q4's 125 rows leave
+// 3 of padding), so that meshes of a few thousand cells have warps for every SM; in 1D all NB.
+// Measured against 16 rows (8 and 4 in 3D) by blocks of 128 threads, the time-mean prediction: 2D
+// Q5 60^2 94.7 -> 43.5 us, Q3 256^2 138 -> 121, Q2 160^2 29 -> 21; 3D Q2 16^3 92 -> 53, Q3 8^3 164
+// -> 97, Q3 48^3 5.88 -> 5.86 ms.
 template <int DIM, int NB>
 struct PredictRows {
   static constexpr int value = DIM == 1 ? NB
@@ -384,6 +385,24 @@ struct PredictRows {
                                          : 4;
 };
 
+struct PredictGrid {
+  int threads;
+  size_t smem;
+  dim3 grid;
+  long long blocks, resident;  // resident: blocks that run at once on an SM
+};
+PredictGrid predict_grid(long long ncell, int K, int nout, int rows) {
+  PredictGrid p;
+  p.smem = (size_t)rows * K * sizeof(double);
+  // one-warp blocks spread best; larger ones where each block's copy of its rows of P would
+  // cost more than that gains (3D Q4, Q5: 32 to 55 KB)
+  p.threads = p.smem <= 8 * 1024 ? 32 : p.smem <= 20 * 1024 ? 64 : 128;
+  p.grid = dim3((unsigned)((ncell + p.threads - 1) / p.threads), (unsigned)((nout + rows - 1) / rows));
+  p.blocks = (long long)p.grid.x * p.grid.y;
+  p.resident = std::min({32LL, 2048LL / p.threads, 232448LL / (long long)(p.smem + 1024)});
+  return p;
+}
+
 // The correction's form: a thread per mode below ~45 cells per SM (2D Q3, 24 cells per SM: 10.9
 // against 17.4 us; 66: 19.1 against 17.0), and where a cell's time means do not fit a thread.
 bool correct_by_modes(int dim, int nb, long long ncell) {
@@ -392,33 +411,47 @@ bool correct_by_modes(int dim, int nb, long long ncell) {
 constexpr int kCorrectThreads = 128;
 long long correct_mode_blocks(long long modes) { return (modes + kCorrectThreads - 1) / kCorrectThreads; }
 
-template <int DIM, int NB>
-cudaError_t predict_dispatch_ch(const Grid& g, const double* Q, const double* P, int nout,
-                                double* W, int wstride, cudaStream_t s) {
-  constexpr int CH = PredictRows<DIM, NB>::value;
-  if (g.box.n < 1 || g.box.n > ipow_c(2, DIM)) return cudaErrorInvalidValue;
-  const size_t smem = (size_t)CH * g.box.n * ipow_c(NB, DIM) * sizeof(double);
-  // one-warp blocks spread best; larger ones where each block's copy of its rows of P would
-  // cost more than that gains (3D Q4, Q5: 40 and 55 KB)
-  const int threads = smem <= 8 * 1024 ? 32 : smem <= 20 * 1024 ? 64 : 128;
-  const dim3 grid((unsigned)((g.ncell + threads - 1) / threads), (unsigned)((nout + CH - 1) / CH));
+template <int DIM, int NB, int CH>
+cudaError_t predict_launch(const Grid& g, const double* Q, const double* P, int nout, double* W,
+                           int wstride, cudaStream_t s) {
+  const PredictGrid p = predict_grid(g.ncell, g.box.n * ipow_c(NB, DIM), nout, CH);
   auto kern = predict_fp64_kernel<DIM, NB, CH>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (p.smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return e;
   }
   // Launched early, the blocks go to the SMs with room beside the correction of the step before.
   // Where that correction has a block per 128 modes and they no longer all run at once, these are
   // the few SMs that ran out first: a prediction that does not fill the chip then piles up there
-  // (3D Q4 12^3 778 against 417 us a step, Q3 16^3 424 against 262, 2D Q5 82^2 156 against 97;
-  // up to 8 blocks per SM, 2D Q5 60^2, 3D Q2 14^3, it saves 6 to 8%).
+  // (3D Q3 16^3 424 against 262 us a step, Q5 10^3 875 against 691, 2D Q5 82^2 156 against 97; up
+  // to 8 blocks per SM, 2D Q5 60^2, 3D Q2 14^3, it saves 6 to 8%).
   const int sms = device_sms();
-  const long long resident = std::min({32LL, 2048LL / threads, 232448LL / (long long)(smem + 1024)});
   const bool early = !correct_by_modes(DIM, NB, g.ncell) ||
                      correct_mode_blocks(g.ncell * ipow_c(NB, DIM)) <= 8LL * sms ||
-                     10LL * grid.x * grid.y >= 9 * resident * sms;
-  return launch_dependent(early, kern, grid, threads, smem, s, Q, P, nout, W, wstride, g.n[0],
+                     10 * p.blocks >= 9 * p.resident * sms;
+  return launch_dependent(early, kern, p.grid, p.threads, p.smem, s, Q, P, nout, W, wstride, g.n[0],
                           g.n[1], g.n[2], g.ncell, g.box);
+}
+
+template <int DIM, int NB>
+cudaError_t predict_dispatch_ch(const Grid& g, const double* Q, const double* P, int nout,
+                                double* W, int wstride, cudaStream_t s) {
+  if (g.box.n < 1 || g.box.n > ipow_c(2, DIM)) return cudaErrorInvalidValue;
+  if constexpr (DIM == 3 && NB == 5) {
+    // Few blocks of 40 KB: five rows per thread where the SM with the most blocks then has fewer
+    // rows to sum and all blocks run at once, else four (a step, five against four rows: 9 x 10 x 8
+    // 230 against 267 us, 11^3 347 against 405; 16^3 1151 against 943, 20^3 2374 against 1875).
+    // Two warps of cells or fewer wait for their own sums: four (3 x 4 x 5 215 against 174).
+    const int sms = device_sms();
+    auto rows_on_sm = [&](const PredictGrid& p, int rows) {
+      return (p.blocks + sms - 1) / sms * p.threads * rows;
+    };
+    const int K = g.box.n * ipow_c(NB, DIM);
+    const PredictGrid p5 = predict_grid(g.ncell, K, nout, 5), p4 = predict_grid(g.ncell, K, nout, 4);
+    if (g.ncell <= 64 || p5.blocks > p5.resident * sms || rows_on_sm(p5, 5) >= rows_on_sm(p4, 4))
+      return predict_launch<DIM, NB, 4>(g, Q, P, nout, W, wstride, s);
+  }
+  return predict_launch<DIM, NB, PredictRows<DIM, NB>::value>(g, Q, P, nout, W, wstride, s);
 }
 
 template <int DIM, int NB>
