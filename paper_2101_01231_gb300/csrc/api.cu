@@ -171,6 +171,7 @@ CorrParams corr_params(const ridg_t* h) {
 // exponent words of the mixed path: [2] = 1 for FP16 digit operands (read by the kernels)
 cudaError_t init_exps(ridg_t* h) {
   static const int zero[4] = {0, 0, 0, 0}, one[4] = {0, 0, 1, 0};
+  h->ms.f16 = digits_f16(h);
   return cudaMemcpyAsync(h->ms.exps, digits_f16(h) ? one : zero, 4 * sizeof(int),
                          cudaMemcpyHostToDevice, h->stream);
 }

@@ -561,8 +561,10 @@ __device__ __forceinline__ bool correct_groups(double* q, const float2* __restri
 // has one), where a cell has two full groups (Q3): one thread per cell leaves 13 warps per SM
 // at 256^2, each with 16 modes' digits in a row.  (Groups without a mode are zero in the planes
 // from their creation.)
-template <int NB, int S, bool SPLIT>
-__global__ void __launch_bounds__(128) mixed_correct_kernel(
+// Seven blocks per SM at Q3 where the compiler would take more registers (4 slices, 512^2: 83 -> 76
+// us a step; 7 slices 114 -> 95; 5 slices keep seven by themselves, and lose 3% to the bound).
+template <int NB, int S, bool SPLIT, int FMT>
+__global__ void __launch_bounds__(128, (NB == 4 && !SPLIT && S != 5 ? 7 : 0)) mixed_correct_kernel(
     double* __restrict__ Q, const float2* __restrict__ Y, int nx, int ny, CorrParams cp, int gmax,
     int sgnx, int sgny, int* __restrict__ exps, unsigned long long* __restrict__ maxbits,
     uint4* __restrict__ planes, int* status) {
@@ -588,7 +590,7 @@ __global__ void __launch_bounds__(128) mixed_correct_kernel(
     const unsigned ue = (unsigned)e, uy = ue / (unsigned)nx;
     const int ix = (int)(ue - uy * (unsigned)nx), iy = (int)uy;
     const int kfin = ys + gmax - 16;
-    const bool f16 = exps[2] != 0;
+    const bool f16 = digits_fp16<FMT>(exps);
     double* q = sq + c * PITCH;
     if constexpr (SPLIT) {
       if (threadIdx.x < CELLS)
@@ -784,9 +786,12 @@ static cudaError_t launch_correct_t(const Grid& g, double* Q, const void* Y, int
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const bool split = NB == 4 && g.ncell <= 512LL * sms;
   const unsigned blocks = (unsigned)((g.ncell * (split ? 2 : 1) + 127) / 128);
-  auto kern = mixed_correct_kernel<NB, S, false>;
+  auto kern = ms.f16 ? mixed_correct_kernel<NB, S, false, kFp16Digits>
+                     : mixed_correct_kernel<NB, S, false, kBf16Digits>;
   if constexpr (NB == 4)
-    if (split) kern = mixed_correct_kernel<NB, S, true>;
+    if (split)
+      kern = ms.f16 ? mixed_correct_kernel<NB, S, true, kFp16Digits>
+                    : mixed_correct_kernel<NB, S, true, kBf16Digits>;
   kern<<<blocks, 128, 0, s>>>(Q, (const float2*)Y, g.n[0], g.n[1], cp, gmax, sgnx, sgny, ms.exps,
                               ms.maxbits, (uint4*)ms.planes, ms.status);
   return cudaGetLastError();

@@ -369,7 +369,7 @@ __device__ __forceinline__ void dfu_acc(DFU& a, DFU x) {
 // F(i - 1/2) - F(i + 1/2))], s_a = (-1)^a = phi_a(-1) / phi_a(+1), in double-float; then
 // Q += dQ in FP64, the new state's digit rows (and ghost copies) and the running maximum.
 // Degrees up to 2: a mode has at most one volume-term source per direction.
-template <int NB, int S, int BT>
+template <int NB, int S, int BT, int FMT>
 __global__ void __launch_bounds__(BT) mixed3_correct_kernel(
     double* __restrict__ Q, const float2* __restrict__ Y, int nx, int ny, int nz, CorrParams cp,
     int gmax, int* __restrict__ exps, unsigned long long* __restrict__ maxbits,
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(BT) mixed3_correct_kernel(
         }
       }
       uint4 rows[S];
-      fits &= make_digit_rows<S>(qn, snext, rows, exps[2] != 0);
+      fits &= make_digit_rows<S>(qn, snext, rows, digits_fp16<FMT>(exps));
 #pragma unroll
       for (int a = 0; a < S; ++a) {
         uint4* base = planes + (long long)(a * P + pg) * plane;
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(BT) mixed3_correct_kernel(
 // double-float.  Then the block updates its cells' state rows together (Q += dQ in FP64,
 // read and written coalesced), and each thread writes its cell's digit rows (and ghost
 // copies) and the running maximum, as in the kernel above.
-template <int NB, int S, int BT>
+template <int NB, int S, int BT, int FMT>
 __global__ void __launch_bounds__(BT) mixed3_fcorrect_kernel(
     double* __restrict__ Q, const float2* __restrict__ Y, int nx, int ny, int nz, CorrParams cp,
     int gmax, int* __restrict__ exps, unsigned long long* __restrict__ maxbits,
@@ -688,7 +688,7 @@ __global__ void __launch_bounds__(BT) mixed3_fcorrect_kernel(
 #pragma unroll
       for (int j = 0; j < 8; ++j) qn[j] = pg * 8 + j < THS ? q[pg * 8 + j] : 0.0;
       uint4 rows[S];
-      fits &= make_digit_rows<S>(qn, snext, rows, exps[2] != 0);
+      fits &= make_digit_rows<S>(qn, snext, rows, digits_fp16<FMT>(exps));
 #pragma unroll
       for (int a = 0; a < S; ++a) planes[(long long)(a * P + pg) * plane + own] = rows[a];
       if (ghost) {
@@ -916,6 +916,16 @@ cudaError_t launch_mixed3_predict(const Grid& g, int nb, const MixedOp& op, Mixe
   }
 }
 
+template <int NB, int S, int FMT>
+static auto correct3_kernel(bool fused, int block) {
+  return fused ? (block == 64    ? mixed3_fcorrect_kernel<NB, S, 64, FMT>
+                  : block == 128 ? mixed3_fcorrect_kernel<NB, S, 128, FMT>
+                                 : mixed3_fcorrect_kernel<NB, S, 256, FMT>)
+               : (block == 64    ? mixed3_correct_kernel<NB, S, 64, FMT>
+                  : block == 128 ? mixed3_correct_kernel<NB, S, 128, FMT>
+                                 : mixed3_correct_kernel<NB, S, 256, FMT>);
+}
+
 template <int NB, int S>
 static cudaError_t launch_correct3_t(const Grid& g, double* Q, const void* Y, int gmax,
                                      const CorrParams& cp, MixedState& ms, int block, bool fused,
@@ -927,12 +937,20 @@ static cudaError_t launch_correct3_t(const Grid& g, double* Q, const void* Y, in
   // (the fused form keeps its rows at an odd pitch)
   constexpr int THS = NB * NB * NB;
   const size_t smem = (size_t)block * (fused ? (THS | 1) : THS) * sizeof(float2);
-  auto kern = fused ? (block == 64    ? mixed3_fcorrect_kernel<NB, S, 64>
-                       : block == 128 ? mixed3_fcorrect_kernel<NB, S, 128>
-                                      : mixed3_fcorrect_kernel<NB, S, 256>)
-                    : (block == 64    ? mixed3_correct_kernel<NB, S, 64>
-                       : block == 128 ? mixed3_correct_kernel<NB, S, 128>
-                                      : mixed3_correct_kernel<NB, S, 256>);
+  constexpr bool kAny = NB == 3 && S <= 3;
+  auto kern = correct3_kernel<NB, S, kAny ? kAnyFormat : kBf16Digits>(fused, block);
+  if constexpr (!kAny)
+    if (ms.f16) kern = correct3_kernel<NB, S, kFp16Digits>(fused, block);
+  if constexpr (NB == 3 && S == 6) {
+    // Six slices at Q2: the form that reads the flag takes 79 registers against 89, a sixth block
+    // per SM, which gains while the state, the outputs and the planes stay in L2 (61 x 50 x 37, 92
+    // MB of 129: a step 123 against 131 us) and loses beyond (56^3, 143 MB: 177 against 163).
+    int dev = 0, l2 = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+    constexpr long long cell_bytes = 16LL * THS + 16LL * S * (((THS + 15) / 16) * 2);
+    if (g.ncell * cell_bytes <= l2) kern = correct3_kernel<NB, S, kAnyFormat>(fused, block);
+  }
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

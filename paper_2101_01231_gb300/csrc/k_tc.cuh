@@ -167,6 +167,16 @@ __device__ __forceinline__ bool value_digits(double x, int s, float (&d)[S]) {
   return fits;
 }
 
+// The digits' format as a correction kernel's constant: computing both and selecting one, with a
+// flag read at run time, costs instructions and registers (3D Q2, 6 slices, 64^3: 250 -> 222 us a
+// step; Q1, 96^3, 274 -> 270).  kAnyFormat reads the flag: 3D Q2 up to 3 slices, where it is the
+// one that schedules as well or better (80^3, 3 slices: 249 against 253 us).
+enum DigitFormat : int { kBf16Digits = 0, kFp16Digits = 1, kAnyFormat = 2 };
+template <int FMT>
+__device__ __forceinline__ bool digits_fp16(const int* exps) {
+  return FMT == kAnyFormat ? exps[2] != 0 : FMT == kFp16Digits;
+}
+
 // S balanced base-256 digits of 8 consecutive coefficients, packed as BF16 (their FP32 values'
 // upper halves) or, f16, FP16 -- exact either way: one 16 B row per digit.  Returns false if a
 // value does not fit below 2^s.  (A byte permutation and an addition per digit and one

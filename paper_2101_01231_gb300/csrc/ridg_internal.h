@@ -71,6 +71,7 @@ struct MixedState {
   alignas(64) unsigned char map_pred[128];  // the same for the full prediction
   int* exps = nullptr;                    // [0] exponent of the planes, [1] of the outputs,
                                           // [2] 1 if the digits are FP16 (else BF16)
+  bool f16 = false;                       // the same for the host
   unsigned long long* maxbits = nullptr;  // [0] max |Q| of the current state, [1] accumulator
   int* status = nullptr;                  // shared status word
   bool valid = false;                     // planes describe the current state
