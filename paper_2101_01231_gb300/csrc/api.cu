@@ -456,8 +456,9 @@ int enqueue_correct_after_mean(ridg_t* h) {
 }
 
 // 1D FP64: several steps per launch.
-bool use_run1d(const ridg_t* h) {
-  return is_linear(h) && h->opt.precision == RIDG_PREC_FP64 && h->dim == 1;
+bool use_run1d(const ridg_t* h, int n) {
+  return is_linear(h) && h->opt.precision == RIDG_PREC_FP64 && h->dim == 1 &&
+         ridg::run1d_pays(grid_of(h), h->nb, n);
 }
 
 int enqueue_run1d(ridg_t* h, int n) {
@@ -950,7 +951,7 @@ int ridg_step(ridg_t* h, int n) {
   if (!is_linear(h))  // Newton statistics of this call's steps (read by ridg_sync)
     RIDG_CUDA(h, clear_newton_stats(h));
   auto enqueue = [&] {
-    if (use_run1d(h)) return enqueue_run1d(h, n);
+    if (use_run1d(h, n)) return enqueue_run1d(h, n);
     int rc = RIDG_OK;
     for (int i = 0; i < n && rc == RIDG_OK; ++i) rc = enqueue_step(h);
     return rc;

@@ -224,6 +224,10 @@ __global__ void __launch_bounds__(256) time_means_kernel(const double* __restric
     for (int s = threadIdx.x & 31; s < thS; s += 32) Wb[e * thS + s] = W[e * thT + s];
 }
 
+// FP64 operations of a 1D step per cell
+double run1d_ops(int nb) { return nb * (2.0 * nb + 2.0) + nb * (0.25 * nb + 4.0); }
+constexpr int kRun1dThreads = 768;
+
 // 1D: k steps of a chunk of C cells per block and launch (temporal blocking).  With upwind face
 // values a step reads two cells upstream (the time mean of the upstream neighbour reads one
 // more), so a block that starts from 2k more cells upstream computes its own cells' k steps
@@ -238,9 +242,11 @@ __global__ void __launch_bounds__(256) time_means_kernel(const double* __restric
 // -> 2.0, 1000 cells Q4 27.7 -> 1.6, 100000 cells Q3 37.4 -> 17.6.  Splitting the sums into two
 // halves for a shorter chain gained nothing (1.21 us at 64 cells).
 //
+// A mesh of one block keeps its state in place (every read is ahead of the first barrier).
+//
 // One thread per (cell, mode); local cell u counts downstream, own cells are u >= 2k.
 template <int NB>
-__global__ void __launch_bounds__(768) run1d_chunk_kernel(const double* Qin, double* Qout,
+__global__ void __launch_bounds__(kRun1dThreads) run1d_chunk_kernel(const double* Qin, double* Qout,
                                                            const double* __restrict__ P, int n,
                                                            int k, int C, CorrParams cp, int dir,
                                                            int nr) {
@@ -322,39 +328,48 @@ int device_sms() {
 }
 
 struct Run1dPlan {
-  int C, k;
+  int C, launches;
 };
-// cells per block and steps per launch: the least of  max(chain, FP64 work) + launch / k  per
+// Cells per block and steps k per launch: the least of  max(chain, FP64 work) + launch / k  per
 // step, in clocks (fitted to a sweep over C and k at 16 to 20000 cells, degrees 1 to 7; its
-// choices are within 10% of the sweep's best)
+// choices are within 10% of the sweep's best).  Several blocks alternate between two states: an
+// even number of launches, or a copy back; one block (C = n) keeps one state, which a few steps of
+// a small mesh gain by (16 cells Q2, one step: 27.9 -> 25.6 us a call).
 Run1dPlan run1d_plan(long long n, int nb, int nsteps, int sms) {
-  const double f = nb * (2.0 * nb + 2.0) + nb * (0.25 * nb + 4.0);  // FP64 operations per cell
-  Run1dPlan best = {1, 1};
+  const double chain = 1200.0 + 60.0 * nb, launch = 3000.0 + 100.0 * nb * nb;
+  auto step = [&](long long C, int k) {
+    const double blocks = std::ceil((double)n / C);
+    const double work = std::ceil(blocks / std::max(1, sms)) * (C + k) * run1d_ops(nb) / 2.0;
+    return std::max(chain, 700.0 + 1.5 * work);
+  };
+  int C = 1, k = 1;
   double cost = 1e300;
-  for (int C : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64})
-    for (int k = 1; k <= 16 && k <= nsteps; ++k) {
-      if ((C + 2 * k) * nb > 768) break;
-      const double blocks = std::ceil((double)n / C);
-      const double work = std::ceil(blocks / std::max(1, sms)) * (C + k) * f / 2.0;
-      const double c = std::max(1200.0 + 60.0 * nb, 700.0 + 1.5 * work) + (3000.0 + 100.0 * nb * nb) / k;
-      if (c < cost) {
-        cost = c;
-        best = {C, k};
+  for (int c : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64})
+    for (int q = 1; q <= 16 && q <= nsteps && (c + 2 * q) * nb <= kRun1dThreads; ++q) {
+      const double t = step(c, q) + launch / q;
+      if (t < cost) {
+        cost = t;
+        C = c;
+        k = q;
       }
     }
-  return best;
+  int launches = (nsteps + k - 1) / k;
+  const bool copy = (launches & 1) && launches == nsteps;
+  if ((launches & 1) && !copy) ++launches;
+  if (nsteps <= 16 && (n + 2 * nsteps) * nb <= kRun1dThreads &&
+      nsteps * step(n, nsteps) + launch < nsteps * step(C, k) + launches * launch + (copy ? 4000.0 : 0.0))
+    return {(int)n, 1};
+  return {C, launches};
 }
 
 template <int NB>
 cudaError_t run1d_dispatch(const Grid& g, double* Q, double* Q2, const double* P, int nsteps,
                            const CorrParams& cp, cudaStream_t s) {
   const Run1dPlan pl = run1d_plan(g.ncell, NB, nsteps, device_sms());
-  // an even number of launches leaves the state in Q (a single one is copied back)
-  int launches = (nsteps + pl.k - 1) / pl.k;
-  if ((launches & 1) && launches < nsteps) ++launches;
+  const int launches = pl.launches;
   const int dir = g.box.lo[0] < 0 ? 1 : (g.box.cnt[0] > 1 ? -1 : 1);
   const unsigned blocks = (unsigned)((g.ncell + pl.C - 1) / pl.C);
-  double *in = Q, *out = Q2;
+  double *in = Q, *out = pl.C < g.ncell ? Q2 : Q;
   for (int l = 0; l < launches; ++l) {
     const int k = nsteps / launches + (l < nsteps % launches);
     const int U = pl.C + 2 * k, threads = (U * NB + 31) / 32 * 32;
@@ -409,7 +424,29 @@ bool correct_by_modes(int dim, int nb, long long ncell) {
   return (dim == 3 && nb >= 5) || ncell < 45LL * device_sms();
 }
 constexpr int kCorrectThreads = 128;
-long long correct_mode_blocks(long long modes) { return (modes + kCorrectThreads - 1) / kCorrectThreads; }
+long long correct_blocks(bool modes, long long ncell, int ths) {
+  return (ncell * (modes ? ths : 1) + kCorrectThreads - 1) / kCorrectThreads;
+}
+
+// Whether at most half of the correction's blocks that an SM can hold run on it.
+template <int DIM, int NB>
+bool correct_leaves_room(long long ncell) {
+  auto resident = [](auto kern) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kCorrectThreads, 0) != cudaSuccess) n = 0;
+    return n;
+  };
+  const bool modes = correct_by_modes(DIM, NB, ncell);
+  long long room = 0;
+  if (modes) {
+    static const int n = resident(correct_modes_kernel<DIM, NB>);
+    room = n;
+  } else if constexpr (!(DIM == 3 && NB >= 5)) {
+    static const int n = resident(correct_linear_kernel<DIM, NB>);
+    room = n;
+  }
+  return 2 * correct_blocks(modes, ncell, ipow_c(NB, DIM)) <= room * device_sms();
+}
 
 template <int DIM, int NB, int CH>
 cudaError_t predict_launch(const Grid& g, const double* Q, const double* P, int nout, double* W,
@@ -421,14 +458,12 @@ cudaError_t predict_launch(const Grid& g, const double* Q, const double* P, int 
     if (e != cudaSuccess) return e;
   }
   // Launched early, the blocks go to the SMs with room beside the correction of the step before.
-  // Where that correction has a block per 128 modes and they no longer all run at once, these are
-  // the few SMs that ran out first: a prediction that does not fill the chip then piles up there
-  // (3D Q3 16^3 424 against 262 us a step, Q5 10^3 875 against 691, 2D Q5 82^2 156 against 97; up
-  // to 8 blocks per SM, 2D Q5 60^2, 3D Q2 14^3, it saves 6 to 8%).
+  // Where that correction fills more than half of the chip, these are the few SMs that ran out
+  // first, and a prediction that does not fill the chip by itself piles up there (3D Q3 16^3 424
+  // against 262 us a step, Q5 10^3 875 against 691, 2D Q5 82^2 156 against 97, 1D Q11 100000 cells
+  // 108 against 84; with room, 2D Q5 60^2, 3D Q2 14^3, it saves 6 to 8%).
   const int sms = device_sms();
-  const bool early = !correct_by_modes(DIM, NB, g.ncell) ||
-                     correct_mode_blocks(g.ncell * ipow_c(NB, DIM)) <= 8LL * sms ||
-                     10 * p.blocks >= 9 * p.resident * sms;
+  const bool early = correct_leaves_room<DIM, NB>(g.ncell) || 10 * p.blocks >= 9 * p.resident * sms;
   return launch_dependent(early, kern, p.grid, p.threads, p.smem, s, Q, P, nout, W, wstride, g.n[0],
                           g.n[1], g.n[2], g.ncell, g.box);
 }
@@ -459,11 +494,11 @@ cudaError_t correct_dispatch(const Grid& g, double* Q, const double* Wb, int wst
                              const CorrParams& cp, cudaStream_t s) {
   const int threads = kCorrectThreads;
   if (correct_by_modes(DIM, NB, g.ncell)) {
-    const unsigned blocks = (unsigned)correct_mode_blocks(g.ncell * ipow_c(NB, DIM));
+    const unsigned blocks = (unsigned)correct_blocks(true, g.ncell, ipow_c(NB, DIM));
     return launch_dependent(true, correct_modes_kernel<DIM, NB>, blocks, threads, 0, s, Q, Wb,
                             wstride, g.n[0], g.n[1], g.n[2], g.ncell, cp);
   } else if constexpr (!(DIM == 3 && NB >= 5)) {
-    const unsigned blocks = (unsigned)((g.ncell + threads - 1) / threads);
+    const unsigned blocks = (unsigned)correct_blocks(false, g.ncell, 1);
     return launch_dependent(true, correct_linear_kernel<DIM, NB>, blocks, threads, 0, s, Q, Wb,
                             wstride, g.n[0], g.n[1], g.n[2], g.ncell, cp);
   }
@@ -519,6 +554,12 @@ cudaError_t launch_time_means(const double* W, int thT, double* Wb, int thS, lon
   const unsigned blocks = (unsigned)std::min<long long>((ncell + 7) / 8, 8LL * device_sms());
   time_means_kernel<<<blocks, 256, 0, s>>>(W, thT, Wb, thS, ncell);
   return cudaGetLastError();
+}
+
+bool run1d_pays(const Grid& g, int nb, int nsteps) {
+  if (nb == 1 && nsteps == 1) return g.ncell + 2 <= kRun1dThreads || g.ncell >= 100000;
+  const double most = std::max(std::min(2000.0 * nb, 9000.0), 1250.0 * nb);
+  return nb <= 2 || (double)g.ncell * run1d_ops(nb) / (2.0 * device_sms()) < most;
 }
 
 cudaError_t launch_run1d_fp64(const Grid& g, int nb, double* Q, double* Q2, const double* P,

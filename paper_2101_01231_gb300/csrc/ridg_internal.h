@@ -49,7 +49,17 @@ cudaError_t launch_predict_fp64(const Grid& g, int nb, const double* Q, const do
 cudaError_t launch_time_means(const double* W, int thT, double* Wb, int thS, long long ncell,
                               cudaStream_t s);
 // 1D: a run of nsteps FP64 steps (prediction of the time means with the operator's first
-// theta_S rows, then the correction), several steps per launch; Q2: room for another state
+// theta_S rows, then the correction), several steps per launch; Q2: room for another state.
+// run1d_pays: whether it beats the two kernels of a step.  Recomputed halos and registers make a
+// chunk's FP64 operations ~1.7 times as dear, which pays where a step's launches cost more than
+// its operations: up to 9000 clocks of them per SM, fewer at degree 2, more from degree 8 on, whose
+// kernels take longer to start (at degrees 0 and 1, where the two kernels' passes over the state
+// bound a step, always).  Chunks against the two kernels per step: 5000 cells Q7 7.4 against 10.7
+// us, 10000 Q9 13.0 against 13.7, Q11 17.4 against 19.6, 20000 Q7 15.6 against 13.5, 50000 Q3 9.1
+// against 9.1, Q2 8.2 against 6.8, 100000 Q11 166 against 84, 1e6 Q6 627 against 274, Q1 61 against
+// 66.  A single step at degree 0 is two launches either way, the copy back the longer one below
+// 100000 cells (5000: 31.4 against 27.6 us a call).
+bool run1d_pays(const Grid& g, int nb, int nsteps);
 cudaError_t launch_run1d_fp64(const Grid& g, int nb, double* Q, double* Q2, const double* P,
                               int nsteps, const CorrParams& cp, cudaStream_t s);
 // Q[e] += correction from the time means Wbar (stride wstride) of e and its face neighbours
