@@ -943,13 +943,8 @@ int ridg_correct(ridg_t* h) {
   return RIDG_OK;
 }
 
-int ridg_step(ridg_t* h, int n) {
-  if (check_handle(h) || n < 1) return RIDG_EINVAL;
-  if (!(h->dt > 0)) return set_err(h, RIDG_ESTATE, "no dt yet: call ridg_set_state first");
-  int rc0 = ensure_digits(h);
-  if (rc0) return rc0;
-  if (!is_linear(h))  // Newton statistics of this call's steps (read by ridg_sync)
-    RIDG_CUDA(h, clear_newton_stats(h));
+// n steps as one graph (or, nonlinear flux, launched one by one the first time)
+static int step_graph(ridg_t* h, int n) {
   auto enqueue = [&] {
     if (use_run1d(h, n)) return enqueue_run1d(h, n);
     int rc = RIDG_OK;
@@ -983,12 +978,33 @@ int ridg_step(ridg_t* h, int n) {
     it = h->graphs.find(n);
   }
   if (!direct) RIDG_CUDA(h, cudaGraphLaunch(it->second, h->stream));
+  return RIDG_OK;
+}
+
+// 1D steps of one graph: a captured launch covers up to 16, and the nodes of a long run would hold
+// device memory (a million steps of 64 cells: 62500 nodes, 580 MB, 0.28 s of capture).
+constexpr int kRun1dGraphSteps = 8192;
+
+int ridg_step(ridg_t* h, int n) {
+  if (check_handle(h) || n < 1) return RIDG_EINVAL;
+  if (!(h->dt > 0)) return set_err(h, RIDG_ESTATE, "no dt yet: call ridg_set_state first");
+  int rc0 = ensure_digits(h);
+  if (rc0) return rc0;
+  if (!is_linear(h))  // Newton statistics of this call's steps (read by ridg_sync)
+    RIDG_CUDA(h, clear_newton_stats(h));
+  int left = n;
+  while (left > kRun1dGraphSteps && use_run1d(h, left)) {
+    const int rc = step_graph(h, kRun1dGraphSteps);
+    if (rc != RIDG_OK) return rc;
+    left -= kRun1dGraphSteps;
+  }
+  const int rc = step_graph(h, left);
+  if (rc != RIDG_OK) return rc;
   h->have_pred = false;
   h->t += n * h->dt;
   h->steps += n;
   return RIDG_OK;
 }
-
 
 int ridg_sync(ridg_t* h) {
   if (check_handle(h)) return RIDG_EINVAL;

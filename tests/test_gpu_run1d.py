@@ -56,3 +56,26 @@ def test_runs_are_no_slower_than_their_kernels(n, M):
     s.close()
     # (chunks took 1.5 times as long at 100000 cells Q11, twice at 300000 Q6)
     assert min(times) <= 1.1 * apart, (min(times), apart)
+
+
+def test_long_runs_replay_one_graph():
+    """A run of many steps takes the states of short ones and no device memory for its launches."""
+    import torch
+    q0 = np.random.default_rng(7).standard_normal((16, 3))
+    s, t = _solver(16, 2), _solver(16, 2)
+    for x in (s, t):
+        x.set_state(q0)
+        x.step(100)
+        x.sync()
+    s.step(40000)                       # 4 x 8192 and a rest
+    for _ in range(400):
+        t.step(100)
+    assert s.info()["steps"] == t.info()["steps"] == 40100
+    assert s.info()["t"] == 100 * s.info()["dt"] + 40000 * s.info()["dt"]
+    np.testing.assert_array_equal(s.get_state(), t.get_state())
+    free = torch.cuda.mem_get_info()[0]
+    s.step(400000)
+    s.sync()
+    assert free - torch.cuda.mem_get_info()[0] < 64 << 20      # (one graph: 230 MB)
+    s.close()
+    t.close()
