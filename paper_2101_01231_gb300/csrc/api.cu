@@ -881,10 +881,13 @@ int ridg_predict(ridg_t* h, double* w_out, int on_device) {
     }
     return read_newton_stats(h);
   }
-  // straight into the caller's device buffer; what a following ridg_correct needs, the time
-  // means, is kept (copying all of W out took 73 MB read and written at 61 x 50 x 37 Q2 for 24)
+  // From 4 MB on straight into the caller's device buffer; what a following ridg_correct needs, the
+  // time means, is kept (copying all of W out took 73 MB read and written at 61 x 50 x 37 Q2 for
+  // 24: the call 149 -> 130 us; below 4 MB the copy is a launch as the time means are, and 1 to 3
+  // us the shorter one: 2D Q1 60 x 50, mixed, 39 against 36 us).
   const size_t wbytes = (size_t)h->ncell * h->thT * sizeof(double);
-  double* const W = w_out && on_device && own_device_memory(w_out, wbytes) ? w_out : h->W;
+  double* const W = w_out && on_device && wbytes >= (size_t)4 << 20 && own_device_memory(w_out, wbytes)
+                        ? w_out : h->W;
   if (is_mixed_linear(h) && h->dim == 2) {
     int rc = ensure_digits(h);
     if (rc) return rc;
@@ -915,7 +918,9 @@ int ridg_predict(ridg_t* h, double* w_out, int on_device) {
   } else {
     RIDG_CUDA(h, ridg::launch_predict_fp64(g, h->nb, h->Q, h->P, h->thT, W, h->thT, h->stream));
   }
-  RIDG_CUDA(h, ridg::launch_time_means(W, h->thT, h->Wbar, h->thS, h->ncell, h->stream));
+  h->pred_means = W != h->W;
+  if (h->pred_means)
+    RIDG_CUDA(h, ridg::launch_time_means(W, h->thT, h->Wbar, h->thS, h->ncell, h->stream));
   h->have_pred = true;
   if (w_out && W != w_out) {
     RIDG_CUDA(h, cudaMemcpyAsync(w_out, W, wbytes,
@@ -934,7 +939,8 @@ int ridg_correct(ridg_t* h) {
     if (rc) return rc;
   } else {
     CorrParams cp = corr_params(h);
-    RIDG_CUDA(h, ridg::launch_correct_linear(grid_of(h), h->nb, h->Q, h->Wbar, h->thS, cp, h->stream));
+    RIDG_CUDA(h, ridg::launch_correct_linear(grid_of(h), h->nb, h->Q, h->pred_means ? h->Wbar : h->W,
+                                             h->pred_means ? h->thS : h->thT, cp, h->stream));
   }
   h->ms.valid = false;
   h->have_pred = false;

@@ -328,7 +328,9 @@ struct ridg_handle {
   bool dt_fixed = false, have_pred = false;
   // device buffers
   double* Q = nullptr;      // state, canonical layout
-  double* W = nullptr;      // last full prediction (cells * m * theta_T)
+  double* W = nullptr;      // last full prediction (cells * m * theta_T), unless it went straight
+                            // into the caller's buffer (pred_means)
+  bool pred_means = false;  // linear: the last prediction's time means are in Wbar, not in W
   double* Wbar = nullptr;   // time-mean prediction that the correction reads (cells * m * theta_S);
                             // 1D steps: the other state of a pair
   double* P = nullptr;      // linear operator, theta_T x K (time-mean rows first)

@@ -51,3 +51,27 @@ def test_any_device_address_gives_the_host_bits(dim, n, M, prec, offset):
     s.correct()
     np.testing.assert_array_equal(s.get_state(), q1)
     s.close()
+
+
+def test_a_prediction_that_stays_is_one_kernel():
+    """Without a buffer of the caller's a linear prediction is its kernel alone (the correction reads
+    it in place); at degree 0 in 1D that is the step's prediction kernel."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2101_01231_gb300 import ridg as R
+    s = R.Solver(1, (1000000,), 0, vel=(0.7,), cfl=0.2)
+    s.set_state(np.random.default_rng(1).standard_normal((s.cells, 1)))
+    s.profile_step(2)
+    kernel = min(s.profile_step(5)["predict_ms"] for _ in range(3))
+    times = []
+    for _ in range(8):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record(s.stream)
+        R.ridg_predict(s.h)
+        b.record(s.stream)
+        b.synchronize()
+        times.append(a.elapsed_time(b))
+    s.close()
+    # (with a pass over the prediction for its time means: twice as long)
+    assert min(times) <= 1.4 * kernel, (min(times), kernel)
