@@ -113,10 +113,13 @@ __device__ __forceinline__ double wvq(const Rule<NB, NQ>& T, int b, int q) {
   return q < H ? T.wV[b][q] : ((b & 1) ? -T.wV[b][NQ - 1 - q] : T.wV[b][NQ - 1 - q]);
 }
 
-// 1 / x to about one unit in the last place: the hardware's approximation (20 bits) and two
-// Newton-Raphson steps r += r (1 - x r), four FP64 operations where the correctly rounded
-// division takes about three times as many on the same pipe.  (0 and non-finite x give NaN,
-// which the solvers treat as the infinities of a division: the region or state is refused.)
+// 1 / x by Newton-Raphson, r += r (1 - x r), two steps from the hardware's approximation (relative
+// error 2^-20): 2^-80 ahead of the last rounding, so the correctly rounded value but where 1 / x
+// lies that close to the middle of two (one x in some 10^8, and x = 1 - 2^-53), there its
+// neighbour.  Four FP64 operations, where the division takes about three times as many on the
+// same pipe (Euler Q2, 160^2, a step 12.6 ms; with __drcp_rn 12.9).  For 2^-1022 <= |x| <= 2^1022:
+// 0, subnormal and non-finite x give NaN, larger finite ones 0.  The solver refuses such a density
+// (a NaN, or an iterate above 1e30), and its region is block-eliminated, with divisions.
 __device__ __forceinline__ double reciprocal(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -124,13 +127,30 @@ __device__ __forceinline__ double reciprocal(double x) {
   return fma(r, fma(-x, r, 1.0), r);
 }
 
-// both directions' fluxes of one state (Euler: one reciprocal)
-template <int FLUX>
+// u = w1 / rho, v = w2 / rho.  ANY: also for densities outside the reciprocal's range, by divisions
+// (the correction, whose states go to no other solver).
+template <bool ANY>
+__device__ __forceinline__ void velocity(const double* w, double& u, double& v) {
+  const double ir = reciprocal(w[0]);
+  u = w[1] * ir;
+  v = w[2] * ir;
+  if constexpr (ANY) {
+    const unsigned hi = (unsigned)__double2hiint(w[0]) & 0x7fffffffu;
+    if (hi - 0x00100000u >= 0x7fd00000u - 0x00100000u) {
+      u = w[1] / w[0];
+      v = w[2] / w[0];
+    }
+  }
+}
+
+// both directions' fluxes of one state (Euler: one reciprocal), or one's
+template <int FLUX, bool ANY = false>
 __device__ __forceinline__ void flux2(const double* w, double* fx, double* fy, double g) {
   if constexpr (FLUX == RIDG_FLUX_BURGERS) {
     fx[0] = 0.5 * w[0] * w[0];
   } else {
-    const double ir = reciprocal(w[0]), u = w[1] * ir, v = w[2] * ir;
+    double u, v;
+    velocity<ANY>(w, u, v);
     const double p = (g - 1.0) * (w[3] - 0.5 * fma(w[1], u, w[2] * v)), h = w[3] + p;
     fx[0] = w[1];
     fx[1] = fma(w[1], u, p);
@@ -142,12 +162,13 @@ __device__ __forceinline__ void flux2(const double* w, double* fx, double* fy, d
     fy[3] = v * h;
   }
 }
-template <int FLUX>
+template <int FLUX, bool ANY = false>
 __device__ __forceinline__ void flux1(const double* w, int dd, double* f, double g) {
   if constexpr (FLUX == RIDG_FLUX_BURGERS) {
     f[0] = 0.5 * w[0] * w[0];
   } else {
-    const double ir = reciprocal(w[0]), u = w[1] * ir, v = w[2] * ir;
+    double u, v;
+    velocity<ANY>(w, u, v);
     const double p = (g - 1.0) * (w[3] - 0.5 * fma(w[1], u, w[2] * v));
     const double un = dd == 0 ? u : v;
     f[0] = dd == 0 ? w[1] : w[2];

@@ -249,7 +249,7 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
 #pragma unroll
         for (int a = 1; a < NB; ++a) w[j] = fma(nl::vq(T, a, q), S[(j * NB + a) * NX + yx], w[j]);
       }
-      nl::flux2<FLUX>(w, fx, fy, g);
+      nl::flux2<FLUX, true>(w, fx, fy, g);
 #pragma unroll
       for (int j = 0; j < MV; ++j) {
         const double wt = nl::wvq(T, 0, q);
@@ -312,8 +312,8 @@ __device__ void nl_correct_cells(const nl::Rule<NB>& T, double* __restrict__ Q,
           wr[j] = fma(nl::vq(T, a, q), tr[(j * NB + a) * NQ], wr[j]);
         }
       }
-      nl::flux1<FLUX>(wl, dd, fl, g);
-      nl::flux1<FLUX>(wr, dd, fr, g);
+      nl::flux1<FLUX, true>(wl, dd, fl, g);
+      nl::flux1<FLUX, true>(wr, dd, fr, g);
 #pragma unroll
       for (int j = 0; j < MV; ++j) {
         const double fh = fma(0.5, fl[j] + fr[j], -alpha * (wr[j] - wl[j]));
