@@ -175,7 +175,12 @@ __global__ void __launch_bounds__(kNT, 4) newton3_mf_kernel(const Newton3Args a)
   int buf = 0, it = 0;
   float m1[1] = {(float)fabs(q)};
   nl::reduce<kNW, 1, true>(m1, red, buf);
-  float wnorm = m1[0];
+  double wnorm = m1[0];  // the iterate's largest entry (below FP32's range by its high word)
+  if (wnorm < 1e-30) {
+    nl::MaxAbs m;
+    m.add(q);
+    wnorm = __hiloint2double(nl::block_max_hi<kNW>(m, red, buf), 0);
+  }
   // Rusanov speeds of the initial iterate: the largest trace of both sides over the face
   if (col) Pd[tid] = q;
   if (tid < 108) alpha[tid] = 0.0;
@@ -228,14 +233,17 @@ __global__ void __launch_bounds__(kNT, 4) newton3_mf_kernel(const Newton3Args a)
     x[0] = x[1] = 0.0;
 #pragma unroll 1
     for (int ref = 0;; ++ref) {
-      const double ra = fmax(fabs(R[0]), fabs(R[1]));
-      m1[0] = !col ? 0.f : ra <= 1e30 ? (float)ra : 3e38f;
-      if (col && !(fabs(R[0]) <= 1e30 && fabs(R[1]) <= 1e30)) m1[0] = 3e38f;
-      nl::reduce<kNW, 1, true>(m1, red, buf);
-      ok = m1[0] <= 1e30f && ref < kMaxRefine3;
+      nl::MaxAbs rm;
+      if (col) {
+        rm.add(R[0]);
+        rm.add(R[1]);
+      }
+      const int rhi = nl::block_max_hi<kNW>(rm, red, buf);
+      ok = rhi < nl::kHi1e30 && ref < kMaxRefine3;
       if (!ok) break;
-      const int ex = m1[0] > 1e-30f ? ilogbf(m1[0]) : -100;
-      const double scale = scalbn(1.0, -ex), unscale = scalbn(1.0, ex);
+      const int ex = nl::exponent_of(rhi);
+      const double scale = nl::pow2(-ex), unscale = nl::pow2(ex);
+      const float wrel = (float)(wnorm * scale);  // wnorm on the right-hand side's scale
       // BiCGStab
       float rv[2], rh[2], p[2], v[2], t[2], xf[2] = {0.f, 0.f};
       {
@@ -247,8 +255,8 @@ __global__ void __launch_bounds__(kNT, 4) newton3_mf_kernel(const Newton3Args a)
       rh[1] = p[1] = rv[1];
       m1[0] = rv[0] * rv[0] + rv[1] * rv[1];
       nl::reduce<kNW, 1, false>(m1, red, buf);
-      const float bb = m1[0], bmean = sqrtf(bb / (2 * kCols)) * (float)unscale;
-      const float tol = fminf(F64 ? 1e-3f : 1e-2f, fmaxf(F64 ? 3e-6f : 1e-6f, (F64 ? 1e-17f : 1e-15f) * wnorm / bmean));
+      const float bb = m1[0], bmean = sqrtf(bb / (2 * kCols));
+      const float tol = fminf(F64 ? 1e-3f : 1e-2f, fmaxf(F64 ? 3e-6f : 1e-6f, (F64 ? 1e-17f : 1e-15f) * wrel / bmean));
       const float stop = tol * tol * bb;
       float rho = bb, rr = bb, hh = bb;
       auto apply = [&](const float (&in)[2], float (&out)[2]) {
@@ -313,10 +321,10 @@ __global__ void __launch_bounds__(kNT, 4) newton3_mf_kernel(const Newton3Args a)
       x[0] += z[0];
       x[1] += z[1];
       if (!F64) break;
-      m1[0] = (float)fmax(fabs(z[0]), fabs(z[1]));
+      m1[0] = fmaxf(fabsf(xf[0]), fabsf(xf[1]));
       nl::reduce<kNW, 1, true>(m1, red, buf);
       // what is left of the linear system is below the iterate's round-off
-      if (m1[0] * fmaxf(ratio, 1e-6f) <= 5e-17f * wnorm) break;
+      if (m1[0] * fmaxf(ratio, 1e-6f) <= 5e-17f * wrel) break;
       double Jz[2];
       spatial<double, true>(C, L, S, z, Jz, Pd, Fd);
       R[0] -= Jz[0] + T00 * z[0] + T01 * z[1];
@@ -341,6 +349,14 @@ __global__ void __launch_bounds__(kNT, 4) newton3_mf_kernel(const Newton3Args a)
     nl::reduce<kNW, 2, true>(mx, red, buf);
     if (!(mx[0] < 1e30f) || !(mx[1] < 1e30f)) break;
     wnorm = mx[1];
+    if (wnorm < 1e-30) {
+      nl::MaxAbs m;
+      if (col) {
+        m.add(wm[0]);
+        m.add(wm[1]);
+      }
+      wnorm = __hiloint2double(nl::block_max_hi<kNW>(m, red, buf), 0);
+    }
     if ((double)mx[0] <= a.tol * fmax(1.0, (double)mx[1])) {
       conv = true;
     } else {

@@ -716,18 +716,20 @@ __device__ __forceinline__ void lines(const Tab<NB>& T, float* P, bool ydir) {
   }
 }
 
-// modal FP64 field src (scaled) to FP32 values at the (y, x) nodes, time still modal
-template <int NB, int MV>
-__device__ __forceinline__ void to_nodes(const Tab<NB>& T, const double* src, float scale,
-                                         float* P) {
+// modal FP64 field src 2^-ex to FP32 values at the x nodes, y and time still modal; TINY: scaled in
+// FP64, where FP32 would lose the small values
+template <int NB, int MV, bool TINY>
+__device__ __forceinline__ void x_nodes(const Tab<NB>& T, const double* src, int ex, float* P) {
   using K = Cfg<NB, MV>;
+  const float sf = TINY ? 1.f : scalbnf(1.f, -ex);
+  const double sd = TINY ? pow2(-ex) : 1.0;
   for (int i = threadIdx.x; i < K::VT * 9 * NB; i += K::NT) {
     const int tj = i / (9 * NB), ro = i - tj * 9 * NB, r = ro / NB, y = ro - r * NB;
     const int a = tj / MV, j = tj - a * MV;
     const double* s = src + ((r * MV + j) * NB + a) * K::THS + y * NB;
     float in[NB];
 #pragma unroll
-    for (int b = 0; b < NB; ++b) in[b] = (float)s[b] * scale;
+    for (int b = 0; b < NB; ++b) in[b] = TINY ? (float)(s[b] * sd) : (float)s[b] * sf;
     float* p = P + tj * K::COL + r * K::THS + y * NB;
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
@@ -737,6 +739,12 @@ __device__ __forceinline__ void to_nodes(const Tab<NB>& T, const double* src, fl
       p[n] = v;
     }
   }
+}
+
+// the same at the (y, x) nodes
+template <int NB, int MV>
+__device__ __forceinline__ void to_nodes(const Tab<NB>& T, const double* src, int ex, float* P) {
+  if (ex >= -100) x_nodes<NB, MV, false>(T, src, ex, P); else x_nodes<NB, MV, true>(T, src, ex, P);
   __syncthreads();
   lines<NB, MV, true>(T, P, true);
   __syncthreads();
@@ -868,7 +876,7 @@ __device__ __forceinline__ void linearise(const Tab<NB>& T, const double* Ws, co
   using K = Cfg<NB, MV>;
   constexpr int VT = K::VT, COL = K::COL;
   const int tid = threadIdx.x;
-  to_nodes<NB, MV>(T, Ws, 1.f, P);
+  to_nodes<NB, MV>(T, Ws, 0, P);
   if (tid < COL) {
     float m[VT], w[VT];
 #pragma unroll
@@ -920,12 +928,12 @@ __device__ __forceinline__ void linearise(const Tab<NB>& T, const double* Ws, co
   __syncthreads();
 }
 
-// J z = scale Rs by BiCGStab in FP32 to a relative residual of about atol / |Rs| within
+// J z = 2^-ex Rs by BiCGStab in FP32 to a relative residual of about atol / |2^-ex Rs| within
 // [rmin, rmax]; the modes of z are left in P (all threads may read them) and the relative
 // residual reached in `ratio`.  False if it stalled.
 template <int NB, int MV, int FLUX>
 __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
-                                         const Lin<NB, MV>& S, const double* Rs, float scale,
+                                         const Lin<NB, MV>& S, const double* Rs, int ex,
                                          float atol, float rmin, float rmax, float* P, float* G,
                                          float* Fh, float* red, int& buf, float g1,
                                          float& ratio) {
@@ -933,7 +941,7 @@ __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
   constexpr int VT = K::VT, COL = K::COL, NW = K::NW;
   const int tid = threadIdx.x;
   // right-hand side: node values of (time operator)^-1 R, scaled
-  to_nodes<NB, MV>(T, Rs, scale, P);
+  to_nodes<NB, MV>(T, Rs, ex, P);
   float r[VT], rh[VT], p[VT], v[VT], t[VT], x[VT];
   float s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -963,7 +971,7 @@ __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
     s4[0] = s1[0];
   }
   const float bb = s4[0];
-  const float bmean = sqrtf(bb / (9 * K::BS)) / scale;
+  const float bmean = sqrtf(bb / (9 * K::BS));
   const float tol = fminf(rmax, fmaxf(rmin, atol / bmean));
   const float stop = tol * tol * bb;
   float rho = bb, rr = bb, hh = bb;  // <rh, r>, |r|^2, |rh|^2
@@ -1049,23 +1057,13 @@ __device__ __forceinline__ bool bicgstab(const Tab<NB>& T, const Rows<NB>& R,
   return true;
 }
 
-// The largest |x| of a thread's FP64 values by their high words (positive doubles order like
-// their bits; no FP64 operation): a lower bound to 2^-20, infinite if one is not finite.
-struct MaxAbs {
-  int hi = 0;
-  __device__ __forceinline__ void add(double x) { hi = max(hi, __double2hiint(x) & 0x7fffffff); }
-};
-
-// the block's largest |x| of MaxAbs values, rounded down; 3e38 if not finite or above 1e30
+// a block's largest |x| by its high word, rounded down; 3e38 if not finite or above 1e30
+__device__ __forceinline__ float max_of_hi(int hi) {
+  return hi < kHi1e30 ? __double2float_rd(__hiloint2double(hi, 0)) : 3e38f;
+}
 template <int NW>
 __device__ __forceinline__ float block_max(MaxAbs m, float* red, int& buf) {
-  float v[1] = {__int_as_float(m.hi)};  // (an order of the bits, NaN patterns aside)
-  // high words up to 0x7f7fffff are finite FP32 patterns; larger ones (|x| >= 2^1016) are cut
-  v[0] = m.hi < 0x7f000000 ? v[0] : __int_as_float(0x7f000000);
-  nl::reduce<NW, 1, true>(v, red, buf);
-  const int hi = __float_as_int(v[0]);
-  const double d = __hiloint2double(hi, 0);
-  return hi < 0x46293e59 ? __double2float_rd(d) : 3e38f;  // 0x46293e59: 1e30
+  return max_of_hi(block_max_hi<NW>(m, red, buf));
 }
 
 // the largest |Rs| and its exponent ex; false if unusable
@@ -1075,9 +1073,10 @@ __device__ __forceinline__ bool rhs_scale(const double* Rs, float* red, int& buf
   using K = Cfg<NB, MV>;
   MaxAbs m;
   for (int i = threadIdx.x; i < 9 * K::BS; i += K::NT) m.add(Rs[i]);
-  rmax = block_max<K::NW>(m, red, buf);
-  ex = rmax > 1e-30f ? ilogbf(rmax) : -100;
-  return rmax <= 1e30f;
+  const int hi = block_max_hi<K::NW>(m, red, buf);
+  rmax = max_of_hi(hi);
+  ex = exponent_of(hi);
+  return hi < kHi1e30;
 }
 
 // index in P of the modal entry i of a region field ([cell][variable][time][y, x])
@@ -1156,7 +1155,11 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
     for (int t = 1; t < NB; ++t) w[t * THS] = 0.0;
   }
   int buf = 0;
-  float wnorm = block_max<NW>(wmax, red, buf);
+  int whi = block_max_hi<NW>(wmax, red, buf);  // the iterate's largest entry, by its high word
+  auto on_scale_of = [&](int ex) {             // and on a right-hand side's scale
+    return ex >= -100 ? max_of_hi(whi) * scalbnf(1.f, -ex)
+                      : (float)(__hiloint2double(whi, 0) * pow2(-ex));
+  };
 
   // thread constants
   Rows<NB> R;
@@ -1196,10 +1199,11 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
       residual<NB, MV, FLUX, true>(T, Ws, Qs, Rs, alpha, arena, lam, a.gamma);
     else
       residual<NB, MV, FLUX, false>(T, Ws, Qs, Rs, alpha, arena, lam, a.gamma);
-    // scale of the right-hand side (a power of two, so that its squares stay normal in FP32)
+    // exponent of the right-hand side (scaled by it, its squares stay normal in FP32)
     float rmax;
     int ex;
     if (!rhs_scale<NB, MV>(Rs, red, buf, rmax, ex)) break;
+    float wrel = on_scale_of(ex);
     // mixed: a new linearisation where the last one no longer contracts by 3e3 per solve
     if (F64 || (solve > 0 && rmax > 3e-4f * bprev && it < a.max_iters)) lin = true;
     bprev = rmax;
@@ -1218,10 +1222,10 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
       // relative accuracy: 1e-4 in the first solve (whose result the nonlinearity limits), then
       // down to an absolute ~1e-15 of the iterate, at most 1e-5 (FP32)
       const float rmin = solve == 0 ? 1e-4f : 1e-5f, rtop = solve == 0 ? 1e-4f : 1e-2f;
-      if (!bicgstab<NB, MV, FLUX>(T, R, S, Rs, scalbnf(1.f, -ex), 1e-15f * wnorm, rmin, rtop, P, G,
-                                  Fh, red, buf, g1, ratio))
+      if (!bicgstab<NB, MV, FLUX>(T, R, S, Rs, ex, 1e-15f * wrel, rmin, rtop, P, G, Fh, red, buf,
+                                  g1, ratio))
         break;
-      const double unscale = scalbn(1.0, ex);
+      const double unscale = pow2(ex);
       float zm[1] = {0.f};
       for (int i = tid; i < 9 * BS; i += NT) {
         const float z = P[p_index<NB, MV>(i)];
@@ -1236,12 +1240,15 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
       bool ok = true;
 #pragma unroll 1
       for (int ref = 0;; ++ref) {
-        if (ref > 0 && !rhs_scale<NB, MV>(Rs, red, buf, rmax, ex)) ok = false;
+        if (ref > 0) {
+          if (!rhs_scale<NB, MV>(Rs, red, buf, rmax, ex)) ok = false;
+          wrel = on_scale_of(ex);
+        }
         ok = ok && ref < kMaxRefine &&
-             bicgstab<NB, MV, FLUX>(T, R, S, Rs, scalbnf(1.f, -ex), 1e-17f * wnorm, 3e-6f, 1e-3f,
-                                    P, G, Fh, red, buf, g1, ratio);
+             bicgstab<NB, MV, FLUX>(T, R, S, Rs, ex, 1e-17f * wrel, 3e-6f, 1e-3f, P, G, Fh, red,
+                                    buf, g1, ratio);
         if (!ok) break;
-        const double unscale = scalbn(1.0, ex);
+        const double unscale = pow2(ex);
         float zm[1] = {0.f};
         for (int i = tid; i < 9 * BS; i += NT) {
           const float zf = P[p_index<NB, MV>(i)];
@@ -1253,7 +1260,7 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
         reduce<NW, 1, true>(zm, red, buf);
         if (!(zm[0] <= 1e30f)) ok = false;
         // what is left of the linear system is below the iterate's round-off
-        if (!ok || scalbnf(zm[0], ex) * fmaxf(ratio, 1e-6f) <= 5e-17f * wnorm) break;
+        if (!ok || zm[0] * fmaxf(ratio, 1e-6f) <= 5e-17f * wrel) break;
         linear_update<NB, MV, FLUX>(TJ, T.Mt, Ws, Zs, Rs, alpha, arena, lam, a.gamma);
       }
       if (!ok) break;
@@ -1267,9 +1274,9 @@ __global__ void __launch_bounds__((Cfg<NB, MV, F64>::NT), (Cfg<NB, MV, F64>::MIN
       ++dm.hi;  // rounded up
       dn = block_max<NW>(dm, red, buf) * 1.0000002f;
     }
-    const float wn = block_max<NW>(wm, red, buf);
+    whi = block_max_hi<NW>(wm, red, buf);
+    const float wn = max_of_hi(whi);
     if (!(dn < 1e30f) || !(wn < 1e30f)) break;
-    wnorm = wn;
     if ((double)dn <= a.tol * fmax(1.0, (double)wn)) {
       conv = true;
       break;

@@ -246,5 +246,28 @@ __device__ __forceinline__ void reduce(float (&v)[NV], float* red, int& buf) {
   }
 }
 
+// The largest |x| of a thread's FP64 values by their high words (positive doubles order like
+// their bits; no FP64 operation): a lower bound to 2^-20, infinite if one is not finite.
+struct MaxAbs {
+  int hi = 0;
+  __device__ __forceinline__ void add(double x) { hi = max(hi, __double2hiint(x) & 0x7fffffff); }
+};
+
+// the block's largest high word (as FP32 patterns, which order like integers up to 0x7f7fffff;
+// larger ones, |x| >= 2^1008 or not finite, are cut)
+template <int NW>
+__device__ __forceinline__ int block_max_hi(MaxAbs m, float* red, int& buf) {
+  float v[1] = {__int_as_float(min(m.hi, 0x7f000000))};
+  reduce<NW, 1, true>(v, red, buf);
+  return __float_as_int(v[0]);
+}
+constexpr int kHi1e30 = 0x46293e59;  // high word of 1e30
+
+// The exponent of a right-hand side whose largest high word is hi, within the normal range, and
+// the power of two of one: right-hand sides are scaled to a maximum of 1 to 2 before they become
+// FP32, whatever the state's scale.
+__device__ __forceinline__ int exponent_of(int hi) { return max((hi >> 20) - 1023, -1022); }
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+
 }  // namespace nl
 }  // namespace ridg
