@@ -269,8 +269,9 @@ int ridg_profile_step(ridg_t* h, int n, ridg_profile_t* out);
  * fastest (tile shapes and schedules per polynomial order).  Tuned now: for the 3D mixed
  * path the depth of the GEMM's operand ring (the slots that fit, up to 8) and the
  * correction's block size (64, 128, 256 threads); for a nonlinear
- * flux the persistent Newton grid (1, 2, 4 or 8 CTAs per 4 SMs: fewer CTAs keep more of
- * their block storage in L2).  Each candidate runs a few real steps (CUDA events around
+ * flux in 2D the persistent grid of the block elimination (1, 2, 4 or 8 CTAs per 4 SMs: fewer
+ * CTAs keep more of their block storage in L2), if the iterative solver leaves regions of the
+ * current state to it; else that grid stays the largest and nothing is stored.  Each candidate runs a few real steps (CUDA events around
  * each launch); the state, t and the step count are restored afterwards, and captured
  * graphs are dropped.  The choices go into the process-wide cache under keys naming the
  * kernel family, degree, slices / conserved variables and precision, which ridg_create and
@@ -281,7 +282,7 @@ int ridg_profile_step(ridg_t* h, int n, ridg_profile_t* out);
 int ridg_autotune(ridg_t* h, const char* cache_path);
 
 /* The handle's current launch choices (any pointer may be NULL): 3D GEMM ring cap (0 = as
- * many slots as fit), 3D correction block size, Newton grid in CTAs.                      */
+ * many slots as fit), 3D correction block size, block elimination grid in CTAs.           */
 int ridg_get_tuning(ridg_t* h, int* gemm3_slots, int* corr3_block, int* newton_grid);
 
 /* Merge the "key value" lines of a cache file into the process-wide cache

@@ -84,8 +84,10 @@ std::string key_batch(const ridg_t* h) {
   return "batch.schedule flux" + std::to_string(h->flux.kind) + " prec" +
          std::to_string(h->opt.precision);
 }
+// (the grid of the regions that the iterative solver leaves; a value that an earlier version stored
+// as newton.grid, when every region or none went there, is not read)
 std::string key_newton(const ridg_t* h) {
-  return "newton.grid nb" + std::to_string(h->nb) + " m" + std::to_string(h->m) + " flux" +
+  return "newton.list_grid nb" + std::to_string(h->nb) + " m" + std::to_string(h->m) + " flux" +
          std::to_string(h->flux.kind) + " prec" + std::to_string(h->opt.precision);
 }
 
@@ -1134,13 +1136,23 @@ int ridg_autotune(ridg_t* h, const char* cache_path) {
       }
     }
     if (!rc && newton) {
-      // the persistent Newton grid in CTAs per 4 SMs: fewer CTAs keep more of their block
-      // storage in L2, more hide the latency of the pivot chains
+      // The persistent grid of the block elimination (2D) in CTAs per 4 SMs: fewer CTAs keep more
+      // of their block storage in L2, more hide the latency of the pivot chains.  Timed only if
+      // the iterative solver leaves regions of this state to it; else the candidates differ by
+      // noise, and the grid stays the largest.
+      h->nl_grid = h->nl_grid_max;
+      int listed = 0;
+      double t0p = 0, t0c = 0;
+      rc = measure(1, &t0p, &t0c);
+      if (!rc && (cudaMemcpyAsync(&listed, h->nl_list, sizeof(int), cudaMemcpyDeviceToHost,
+                                  h->stream) != cudaSuccess ||
+                  cudaStreamSynchronize(h->stream) != cudaSuccess))
+        rc = set_err(h, RIDG_ECUDA, "autotune: listed regions");
       const int per4 = std::max(1, h->nl_grid_max * 4 / std::max(1, sm_count()));
       int best_q = per4;
       double best = 1e300;
       for (int q : {1, 2, 4, 8}) {
-        if (q > per4) break;
+        if (rc || listed == 0 || q > per4) break;
         h->nl_grid = newton_grid_of(h, q);
         double tp = 0, tc = 0;
         if ((rc = measure(1, &tp, &tc))) break;
@@ -1149,8 +1161,8 @@ int ridg_autotune(ridg_t* h, const char* cache_path) {
           best_q = q;
         }
       }
-      h->nl_grid = newton_grid_of(h, best_q);
-      if (!rc) ridg::tune_put(key_newton(h), best_q);
+      if (listed > 0) h->nl_grid = newton_grid_of(h, best_q);
+      if (!rc && listed > 0) ridg::tune_put(key_newton(h), best_q);
     }
     const int rr = restore();
     dev_free(h, save);
