@@ -126,9 +126,10 @@ void drop_graphs(ridg_t* h) {
 // 3D, Burgers Q1 on 10 x 11 x 9 cells: 1014 -> 972 us).  A linear step's kernels are as short as
 // their launches and its dt stays: a graph from the start.  So are calls of more launches than
 // the stream takes without blocking the caller (about a thousand; half of it is left free).  A
-// capturing stream goes the graph's way, which refuses it before anything of the step is recorded.
+// capturing stream and the legacy default stream go the graph's way, which refuses them before
+// anything of the step is recorded.
 bool run_direct(std::set<int>& counts_run, int n, size_t launches_per_step, cudaStream_t s) {
-  if (n > 512 / (int)launches_per_step) return false;
+  if (n > 512 / (int)launches_per_step || s == cudaStreamLegacy) return false;
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;
   return counts_run.insert(n).second;
