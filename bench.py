@@ -318,12 +318,14 @@ def ensemble_section(R, I, steps, cpu_cells, rank=0, ws=1):
                         "left over, one for every instance's correction"
                         if sched["schedule"] == 1 else
                         "two Newton launches per degree + one correction per instance"),
-           "launches_per_step": sched["launches_per_step"],
+           # the schedule's elimination and correction launches, and one of the iterative
+           # solver per degree ahead of them
+           "launches_per_step": sched["launches_per_step"] + len({w["M"] for w in ens}),
            "newton_unconverged": sum(inf["newton_unconverged"] for inf in infos),
            "status": [int(x) for x in status],
            "newton_iters_total": sum(inf["newton_iters_total"] for inf in infos),
            "roofline": {"bound": "alu", "kernel": "newton_mf_kernel (FP64 residuals, all degrees)",
-                        "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
+                        "operations": "three residuals per region, a lower bound", "achieved": ach, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                         "frac": ach / FP64_PEAK_TFLOPS, "traffic": None,
                         "peak_source": "nominal: FP64 FMA pipes x 2 flop x 2.07 GHz"}}
     out["accuracy"] = ensemble_accuracy(R, I, R.RIDG_PREC_MIXED_TF32)
@@ -492,8 +494,10 @@ def residual_fp64_ops(M, m, first=False):
 
 
 def region_fp64_ops(M, m, iters=None):
-    """FP64 operations of one region's Newton solve: the residuals of its iterates.  The mixed
-    forms take three (the initial iterate's and two more); iters: of an FP64 solve."""
+    """FP64 operations of one region's Newton solve: the residuals of its iterates.  For the mixed
+    forms a fixed three, the fewest of an ordinary region (the initial iterate's and two more; a
+    region may take up to seven), whatever the run took: the rate made from it is a lower bound
+    of the executed one.  iters: of an FP64 solve."""
     full = 2 if iters is None else max(iters - 1, 0)
     return residual_fp64_ops(M, m, first=True) + full * residual_fp64_ops(M, m)
 
@@ -516,7 +520,7 @@ def newton_section(R, I, steps, cpu_cells):
         q = I.initial_state(w)
         s.set_state(q)
         if AUTOTUNE[0]:
-            s.autotune()                         # the Newton grid for this precision
+            s.autotune()                         # the grid of the regions left over, if any
         s.profile_step(1)                        # warm-up
         p = s.profile_step(steps)
         info = s.info()
@@ -531,9 +535,12 @@ def newton_section(R, I, steps, cpu_cells):
              "correct_ms": p["correct_ms"],
              "value": cells * 4 * (w["M"] + 1) ** 2 / (p["step_ms"] * 1e-3),
              "unit": "element-DOF updates/s", "newton_iters_per_cell": iters / cells,
-             "newton_iters_max": info["newton_iters_max"], "newton_grid_ctas": grid,
+             "newton_iters_max": info["newton_iters_max"],
+             "elimination_grid_ctas": grid,         # of the regions left over
              "roofline": {"bound": "alu", "kernel": "newton_mf_kernel (FP64 residuals)",
-                          "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+                          "operations": ("three residuals per region, a lower bound"
+                                         if tag.startswith("mixed") else
+                                         "one residual per Newton iteration"), "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                           "traffic": (_recorded_traffic("newton_" + tag[6:], iters)
                                       if tag.startswith("mixed") else None),
                           "peak_source": "nominal: FP64 FMA pipes x 2 flop x 2.07 GHz"}}

@@ -75,9 +75,9 @@ typedef struct {
 } ridg_flux;
 
 enum {
-  RIDG_PREC_FP64 = 0,        /* every step of the path to FP64 accuracy (2D Newton: each
-                                linear system by FP32 iterations refined against its FP64
-                                residual down to round-off, or FP64 block elimination)    */
+  RIDG_PREC_FP64 = 0,        /* every step of the path to FP64 accuracy (Newton: each linear
+                                system by FP32 iterations refined against its FP64 residual
+                                down to round-off, or FP64 block elimination; 3D: LU)     */
   RIDG_PREC_MIXED_BF16 = 1,  /* linear prediction as a sliced BF16 tensor-core contraction
                                 with FP32 accumulation recombined into double-float pairs
                                 (split-operand refinement); in the step the contraction
@@ -309,13 +309,13 @@ ridg_t* ridg_batch_instance(ridg_batch_t* b, int i);
 int ridg_batch_set_state(ridg_batch_t* b, int i, const double* q, int on_device);
 int ridg_batch_get_state(ridg_batch_t* b, int i, double* q, int on_device);
 int ridg_batch_step(ridg_batch_t* b, int n);
-/* The batch's schedule for a nonlinear flux (1: the whole ensemble's Newton prediction in one
- * launch -- every degree's regions, highest degree first, each CTA moving to the next
- * degree's queue as one runs out -- and every instance's correction in one more launch;
- * 0: one Newton launch per degree and one correction per instance) and the prediction and
- * correction launches of one step.  Each Newton launch is the block elimination of the regions
- * that the iterative solver, one more launch per degree ahead of it, left; those are not
- * counted.  Burgers batches default to 1 unless the autotuner recorded otherwise.         */
+/* The batch's schedule for a nonlinear flux and its prediction and correction launches per step.
+ * In both the iterative Newton solver runs first, one launch per degree, and takes every region
+ * it can; these launches are not counted.  1: the block elimination of the regions left over in
+ * one launch -- every degree's list, highest degree first, each CTA moving to the next as one
+ * runs out -- and every instance's correction in one more; 0: one elimination launch per degree
+ * and one correction per instance.  Burgers batches default to 1 unless the autotuner recorded
+ * otherwise.                                                                            */
 int ridg_batch_schedule(ridg_batch_t* b, int* schedule, int* launches_per_step);
 /* Time one step in each schedule from the instances' current states (restored afterwards,
  * graphs dropped) and keep the faster; the choice goes into the autotuner's cache (and to

@@ -1277,7 +1277,7 @@ int ridg_l2_error(ridg_t* h, const double* x, int on_device, double* err) {
 // batched ensemble: independent instances sharing one stream; n steps of all of them are
 // captured into a single graph and replayed.
 // ------------------------------------------------------------------------------------------
-// Instances of a nonlinear batch with the same degree: one persistent Newton launch covers
+// Instances of a nonlinear batch with the same degree: one launch of each Newton solver covers
 // all their regions (instance table on the device, one region counter).
 struct NlGroup {
   std::vector<int> idx;                // instances of the group, in batch order
@@ -1299,9 +1299,9 @@ struct ridg_batch {
   std::set<int> counts_run;  // step counts that have run (run_direct)
   std::map<int, cudaGraph_t> defs;
   std::vector<unsigned long long> gens;  // operator generation of each instance at capture
-  // nonlinear flux: one Newton launch over every degree's regions and one correction launch
-  // over every instance's cells (schedule 1, the default) or one launch per degree and per
-  // instance (schedule 0); the autotuner may pick either
+  // nonlinear flux, after the iterative solver's launch per degree: one elimination launch over
+  // every degree's listed regions and one correction launch over every instance's cells (schedule
+  // 1, the default) or one per degree and per instance (schedule 0); the autotuner may pick either
   int schedule = 1;
   std::vector<ridg::CorrInst> corr_host;  // all instances, block0 increasing
   ridg::CorrInst* corr_table = nullptr;
@@ -1390,7 +1390,8 @@ ridg::NewtonArgs group_args(ridg_batch_t* b, const NlGroup& g) {
   return a;
 }
 
-// One persistent Newton launch over every region of the group's instances.
+// The iterative solver over every region of the group's instances, and one persistent launch for
+// those it leaves over.
 int enqueue_newton_group(ridg_batch_t* b, const NlGroup& g) {
   ridg_t* h = b->inst[g.idx[0]];
   ridg::NewtonArgs a = group_args(b, g);
@@ -1400,8 +1401,9 @@ int enqueue_newton_group(ridg_batch_t* b, const NlGroup& g) {
   return RIDG_OK;
 }
 
-// The whole ensemble's Newton prediction in one launch (the degrees' queues, highest degree
-// first), then every instance's correction in one launch.
+// The block elimination of the whole ensemble's listed regions in one launch (the degrees'
+// queues, highest degree first), after one launch of the iterative solver per degree, then every
+// instance's correction in one launch.
 int upload_batch_multi(ridg_batch_t* b) {
   ridg::NewtonMulti& m = b->multi_host;
   std::memset(&m, 0, sizeof(m));
@@ -1608,8 +1610,8 @@ static int batch_step(ridg_batch_t* b, int n, bool may_direct) {
           if (rc) break;
         }
       } else {
-        // nonlinear flux: the whole ensemble in two launches, or one Newton launch per
-        // degree over all its instances, then the instances' corrections
+        // nonlinear flux: the iterative solver per degree, then the regions it left over and the
+        // corrections of the whole ensemble in one launch each, or per degree and per instance
         if (b->schedule == 1 && b->corr_table) {
           rc = enqueue_batch_multi(b);
           continue;

@@ -432,8 +432,12 @@ PredictGrid predict_grid(long long ncell, int K, int nout, int rows) {
   return p;
 }
 
-// The correction's form: a thread per mode below ~45 cells per SM (2D Q3, 24 cells per SM: 10.9
-// against 17.4 us; 66: 19.1 against 17.0), and where a cell's time means do not fit a thread.
+// The correction's form: a thread per mode below ~45 cells per SM, and where a cell's time means do
+// not fit a thread.  The line lies between the sides at every degree (thread per mode against per
+// cell, in us; 2D at 44 and 79 cells per SM, 3D at 38 and 70: 2D Q1 7.6 / 8.9 and 8.8 / 8.9, Q2 10.9 /
+// 10.9 and 13.0 / 10.9, Q3 14.9 / 17.0 and 19.5 / 17.1, Q4 21.1 / 21.2 and 31.5 / 21.2, Q5 29.6 / 28.1
+// and 48.0 / 29.3; 3D Q1 10.9 / 13.0 and 13.1 / 13.0, Q2 21.3 / 27.9 and 31.3 / 28.6, Q3 46.2 / 64.1 and
+// 78.5 / 64.5).
 bool correct_by_modes(int dim, int nb, long long ncell) {
   return (dim == 3 && nb >= 5) || ncell < 45LL * device_sms();
 }

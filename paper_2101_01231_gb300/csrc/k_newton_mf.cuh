@@ -23,7 +23,7 @@
 // Measured against the block elimination alone (one step with its correction, tensor-core /
 // FP32 solves): Euler Q2 160^2 214 -> 12.6 ms (the residuals' FP64 operations alone: 8.8 ms),
 // Euler Q1 67 x 90 7.7 -> 0.91 ms, eight Burgers problems of up to 72^2 at degrees 1 .. 4
-// 227 -> 10.0 ms; FP64, Burgers Q2 45 x 33 31.7 -> 0.55 ms.
+// 227 -> 9.7 ms; FP64, Burgers Q2 45 x 33 31.7 -> 0.55 ms.
 //
 // The initial iterate is Q^n extended constant in time, so the first residual is evaluated
 // with one time mode and one time point.
@@ -67,8 +67,13 @@ struct Cfg {
   static constexpr int FL = 24 * NB;                // face lines: 24 faces, NB lines each
   static constexpr int NG = MV == 1 ? 1 : 2;        // Burgers: one flux for both directions
   static_assert(FL <= NT, "one thread per face line");
-  // CTAs per SM that the registers are held to: the best of a sweep (Euler Q2: 3 and 2 leave no
-  // spills, 4.53 against 5.02 ms at 96^2 with 4; Burgers Q3: 6, 2.26 against 2.37 ms with 4)
+  // CTAs per SM that the registers are held to, the best of a sweep for every degree and
+  // precision (predictions with one CTA fewer / these / one more, in us.  FP32 solves: Burgers Q1
+  // 128 x 120 573 / 554 / 572, Q2 96 x 100 1231 / 1136 / 1158, Q3 72 x 64 1277 / 1232 / 1236, Q4 60 x 50
+  // 2868 / 2203 / 2249, Euler Q1 90 x 96 1245 / 1164 / 1217, Q2 96^2 5354 / 4559 / 5050; FP64: Burgers Q4
+  // 7368 / 5690 / 6467, Euler Q2 15665 / 15676 / 18090, the others within 3% but for Q2's 2770 /
+  // 2621 / 2646).  They cost 76 to 356 bytes of spills for Euler Q2, Burgers Q3 and Q4, and Euler Q1
+  // in FP64.
   static constexpr int MINB = MV == 4 ? (NB == 2 ? 5 : F64 ? 2 : 3) : (NB == 2 ? 9 : NB == 3 ? 5 : NB == 4 ? 6 : 2);
   // FP64 arena: B1, B2 (line buffers), face fluxes; the face traces share B2
   static constexpr int nB = C * NB * NQ * NQ, nTr = 4 * C * NB * NQ, nH = 24 * MV * NB * NQ;
