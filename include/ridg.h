@@ -271,7 +271,7 @@ int ridg_profile_step(ridg_t* h, int n, ridg_profile_t* out);
  * correction's block size (64, 128, 256 threads); for a nonlinear
  * flux in 2D the persistent grid of the block elimination (1, 2, 4 or 8 CTAs per 4 SMs: fewer
  * CTAs keep more of their block storage in L2), if the iterative solver leaves regions of the
- * current state to it; else that grid stays the largest and nothing is stored.  Each candidate runs a few real steps (CUDA events around
+ * current state to it; else that grid stays as it is and nothing is stored.  Each candidate runs a few real steps (CUDA events around
  * each launch); the state, t and the step count are restored afterwards, and captured
  * graphs are dropped.  The choices go into the process-wide cache under keys naming the
  * kernel family, degree, slices / conserved variables and precision, which ridg_create and

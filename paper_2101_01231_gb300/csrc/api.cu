@@ -1140,8 +1140,8 @@ int ridg_autotune(ridg_t* h, const char* cache_path) {
       // The persistent grid of the block elimination (2D) in CTAs per 4 SMs: fewer CTAs keep more
       // of their block storage in L2, more hide the latency of the pivot chains.  Timed only if
       // the iterative solver leaves regions of this state to it; else the candidates differ by
-      // noise, and the grid stays the largest.
-      h->nl_grid = h->nl_grid_max;
+      // noise, and the grid stays as it is.
+      const int grid = h->nl_grid;
       int listed = 0;
       double t0p = 0, t0c = 0;
       rc = measure(1, &t0p, &t0c);
@@ -1162,7 +1162,7 @@ int ridg_autotune(ridg_t* h, const char* cache_path) {
           best_q = q;
         }
       }
-      if (listed > 0) h->nl_grid = newton_grid_of(h, best_q);
+      h->nl_grid = listed > 0 ? newton_grid_of(h, best_q) : grid;
       if (!rc && listed > 0) ridg::tune_put(key_newton(h), best_q);
     }
     const int rr = restore();

@@ -47,4 +47,7 @@ def test_grid_is_tuned_only_for_listed_regions(tmp_path):
     s.close()
     s, _ = _solver(R)
     assert s.tuning()["newton_grid"] == g
+    s.set_state(q)
+    s.autotune()
+    assert s.tuning()["newton_grid"] == g       # (nothing listed: a stored choice stays)
     s.close()
